@@ -220,7 +220,11 @@ rgs_status rgs_render_backward(rgs_ctx* ctx, uint64_t state, const rgs_image_gra
 rgs_status rgs_autotune(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera* cams,
                         int32_t n_views, rgs_config* cfg, float* ms_out, void* stream);
 
-/* Frees a state's device memory (after its queued work completes). */
+/* Ends a state; its handle is unknown from then on. The context keeps the memory of the last two
+ * states released (together at most 1/16 of the device's) for the states that later forwards
+ * create, which run after the work queued on it on whatever stream; the call does not wait. A
+ * larger state, and one that a forward or backward under stream capture has used, is freed (after
+ * the device's queued work). What is kept is freed by rgs_destroy, or when an allocation fails. */
 rgs_status rgs_release_state(rgs_ctx* ctx, uint64_t state);
 
 /* Grows a state's pair-list capacity to at least `pair_capacity` entries (0 = leave), so that a

@@ -132,6 +132,16 @@ struct State {
   cudaEvent_t ev[kNumEvents] = {};
   bool fwd_timed = false, bwd_timed = false;
   uint32_t fwd_launches = 0, bwd_launches = 0;
+  // Reuse after release. `done` follows the last complete forward or backward; `open` marks a
+  // call that has queued work and not yet recorded it; `captured` a state that a graph may refer
+  // to.
+  cudaEvent_t done = nullptr;
+  bool open = false, captured = false;
+
+  size_t bytes() const {
+    return r_vn.bytes + r_n.bytes + r_pix.bytes + r_tile.bytes + r_pair.bytes + r_scratch.bytes +
+           r_pose.bytes + r_counters.bytes;
+  }
 };
 
 }  // namespace
@@ -170,6 +180,13 @@ struct rgs_ctx {
   std::string last_error;
   std::map<uint64_t, State*> states;
   uint64_t next_id = 1;
+  // Released states kept for the next one (oldest first): at most kSpareStates of them, together
+  // at most spare_limit bytes. A forward that creates its state (every `render` call does) then
+  // takes buffers that are already there: allocating and freeing them with a device
+  // synchronisation cost 0.55 ms of a 0.82 ms 1200x680 frame and 1.0 ms of a 1.7 ms ten-view
+  // training step. Freed with the context, and whenever one of its allocations fails.
+  std::vector<State*> spare;
+  size_t spare_limit = 0;
   Counters* host_counters = nullptr;  // pinned
   double* track_sums = nullptr;       // device [kMaxViews][4]: exposure-fit sums
   Region r_seed;                      // seed-initialisation scratch, grown on demand
@@ -199,10 +216,19 @@ void free_region(Region& r) {
   r.bytes = 0;
 }
 
-cudaError_t alloc_region(Region& r, size_t bytes) {
+constexpr size_t kSpareStates = 2;
+
+void drop_spares(rgs_ctx* ctx);
+
+cudaError_t alloc_region(rgs_ctx* ctx, Region& r, size_t bytes) {
   free_region(r);
   if (bytes == 0) return cudaSuccess;
   cudaError_t e = cudaMalloc(&r.base, bytes);
+  if (e == cudaErrorMemoryAllocation && !ctx->spare.empty()) {
+    cudaGetLastError();
+    drop_spares(ctx);
+    e = cudaMalloc(&r.base, bytes);
+  }
   if (e != cudaSuccess) {
     r.base = nullptr;
     return e;
@@ -237,7 +263,7 @@ rgs_status ensure_scratch(rgs_ctx* ctx, State& s, int64_t items, bool capturing)
   if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "scratch too small during stream capture");
   RGS_CUDA(cudaDeviceSynchronize(), "sync before scratch growth");
   const size_t bytes = align_up(sizeof(uint32_t) * hist) + align_up(sizeof(uint32_t) * sums);
-  RGS_CUDA(alloc_region(s.r_scratch, bytes), "allocate sort scratch");
+  RGS_CUDA(alloc_region(ctx, s.r_scratch, bytes), "allocate sort scratch");
   char* p = static_cast<char*>(s.r_scratch.base);
   s.hist = carve<uint32_t>(p, hist);
   s.block_sums = carve<uint32_t>(p, sums);
@@ -251,7 +277,7 @@ rgs_status ensure_vn(rgs_ctx* ctx, State& s, int64_t vn, int64_t n, int64_t pose
   if (n > s.n_cap) {
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "per-Gaussian buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
-    RGS_CUDA(alloc_region(s.r_n, sizeof(unsigned long long) * n), "allocate visibility masks");
+    RGS_CUDA(alloc_region(ctx, s.r_n, sizeof(unsigned long long) * n), "allocate visibility masks");
     s.vis_mask = static_cast<unsigned long long*>(s.r_n.base);
     RGS_CUDA(cudaMemsetAsync(s.vis_mask, 0, sizeof(unsigned long long) * n, stream),
              "zero visibility masks");
@@ -264,7 +290,7 @@ rgs_status ensure_vn(rgs_ctx* ctx, State& s, int64_t vn, int64_t n, int64_t pose
     size_t bytes = 3 * align_up(sizeof(float4) * cap) + 7 * align_up(sizeof(uint32_t) * cap) +
                    align_up(sizeof(float) * kG2Stride * cap) +
                    align_up(sizeof(uint32_t) * vis_bit_words_cap(cap));
-    RGS_CUDA(alloc_region(s.r_vn, bytes), "allocate per-Gaussian buffers");
+    RGS_CUDA(alloc_region(ctx, s.r_vn, bytes), "allocate per-Gaussian buffers");
     char* p = static_cast<char*>(s.r_vn.base);
     s.rec0 = carve<float4>(p, cap);
     s.rec1 = carve<float4>(p, cap);
@@ -285,7 +311,7 @@ rgs_status ensure_vn(rgs_ctx* ctx, State& s, int64_t vn, int64_t n, int64_t pose
   if (pose_entries > s.pose_cap) {
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "pose buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
-    RGS_CUDA(alloc_region(s.r_pose, sizeof(float) * pose_entries), "allocate pose partials");
+    RGS_CUDA(alloc_region(ctx, s.r_pose, sizeof(float) * pose_entries), "allocate pose partials");
     s.pose_partial = static_cast<float*>(s.r_pose.base);
     s.pose_cap = pose_entries;
   }
@@ -297,7 +323,7 @@ rgs_status ensure_pix_tiles(rgs_ctx* ctx, State& s, int64_t pixels, int64_t tile
   if (pixels > s.pix_cap) {
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "pixel buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
-    RGS_CUDA(alloc_region(s.r_pix, align_up(sizeof(float) * pixels) +
+    RGS_CUDA(alloc_region(ctx, s.r_pix, align_up(sizeof(float) * pixels) +
                                         align_up(sizeof(int32_t) * pixels)),
              "allocate pixel state");
     char* p = static_cast<char*>(s.r_pix.base);
@@ -308,7 +334,7 @@ rgs_status ensure_pix_tiles(rgs_ctx* ctx, State& s, int64_t pixels, int64_t tile
   if (tiles > s.tile_cap) {
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "tile buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
-    RGS_CUDA(alloc_region(s.r_tile, align_up(sizeof(uint2) * tiles) +
+    RGS_CUDA(alloc_region(ctx, s.r_tile, align_up(sizeof(uint2) * tiles) +
                                          4 * align_up(sizeof(uint32_t) * tiles)),
              "allocate tile ranges");
     char* p = static_cast<char*>(s.r_tile.base);
@@ -327,7 +353,7 @@ rgs_status ensure_pairs(rgs_ctx* ctx, State& s, int64_t pairs) {
   RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
   const int64_t cap = std::max<int64_t>(pairs + pairs / 4, 4096);
   if (cap >= (int64_t)UINT32_MAX) return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^32");
-  RGS_CUDA(alloc_region(s.r_pair, 4 * align_up(sizeof(uint32_t) * cap)), "allocate pair lists");
+  RGS_CUDA(alloc_region(ctx, s.r_pair, 4 * align_up(sizeof(uint32_t) * cap)), "allocate pair lists");
   char* p = static_cast<char*>(s.r_pair.base);
   s.pair_keys[0] = carve<uint32_t>(p, cap);
   s.pair_keys[1] = carve<uint32_t>(p, cap);
@@ -342,14 +368,42 @@ State* find_state(rgs_ctx* ctx, uint64_t id) {
   return it == ctx->states.end() ? nullptr : it->second;
 }
 
-rgs_status get_or_create_state(rgs_ctx* ctx, uint64_t* handle, State** out) {
+void destroy_state(State* s);
+
+// A released state for a forward of these sizes on `stream`: the smallest that holds them, else
+// the one released last, whose buffers then grow. What its earlier owner queued runs first,
+// whatever stream that was on. Null without one; a forward under stream capture takes none (an
+// event from outside the capture cannot be waited for inside it, and its buffers could not grow).
+State* take_spare(rgs_ctx* ctx, int64_t vn, int64_t n, int64_t pixels, cudaStream_t stream) {
+  int best = (int)ctx->spare.size() - 1;
+  if (best < 0) return nullptr;
+  bool fits = false;
+  for (int k = 0; k < (int)ctx->spare.size(); ++k) {
+    const State* s = ctx->spare[k];
+    if (s->vn_cap < vn || s->n_cap < n || s->pix_cap < pixels) continue;
+    if (!fits || s->bytes() < ctx->spare[best]->bytes()) best = k;
+    fits = true;
+  }
+  State* s = ctx->spare[best];
+  if (cudaStreamWaitEvent(stream, s->done, 0) != cudaSuccess) return nullptr;
+  ctx->spare.erase(ctx->spare.begin() + best);
+  s->has_forward = s->fwd_timed = s->bwd_timed = false;
+  s->fwd_launches = s->bwd_launches = 0;
+  return s;
+}
+
+// The named state, or for handle 0 a new one (`spare`, if given, serves as the new one).
+rgs_status get_or_create_state(rgs_ctx* ctx, uint64_t* handle, State** out,
+                               State* spare = nullptr) {
   if (!handle) return fail(ctx, RGS_ERR_INVALID_ARG, "state handle pointer is null");
   if (*handle == 0) {
-    State* s = new State();
-    for (cudaEvent_t& e : s->ev) {
-      if (cudaEventCreate(&e) != cudaSuccess) {
-        e = nullptr;
-        delete s;
+    State* s = spare;
+    if (!s) {
+      s = new State();
+      bool ok = cudaEventCreateWithFlags(&s->done, cudaEventDisableTiming) == cudaSuccess;
+      for (cudaEvent_t& e : s->ev) ok = ok && cudaEventCreate(&e) == cudaSuccess;
+      if (!ok) {
+        destroy_state(s);
         return fail(ctx, RGS_ERR_CUDA, "cudaEventCreate failed");
       }
     }
@@ -368,6 +422,7 @@ rgs_status get_or_create_state(rgs_ctx* ctx, uint64_t* handle, State** out) {
 void destroy_state(State* s) {
   for (cudaEvent_t& e : s->ev)
     if (e) cudaEventDestroy(e);
+  if (s->done) cudaEventDestroy(s->done);
   free_region(s->r_vn);
   free_region(s->r_n);
   free_region(s->r_pix);
@@ -378,6 +433,24 @@ void destroy_state(State* s) {
   free_region(s->r_counters);
   free_region(s->r_reg);
   delete s;
+}
+
+void drop_spares(rgs_ctx* ctx) {
+  if (ctx->spare.empty()) return;
+  cudaDeviceSynchronize();  // queued work may still use their buffers
+  for (State* s : ctx->spare) destroy_state(s);
+  ctx->spare.clear();
+}
+
+// Brackets the work that a forward or backward queues on a state.
+void open_state(State& s, bool capturing) {
+  s.open = true;
+  s.captured = s.captured || capturing;
+}
+cudaError_t close_state(State& s, bool capturing, cudaStream_t stream) {
+  const cudaError_t e = capturing ? cudaSuccess : cudaEventRecord(s.done, stream);
+  s.open = e != cudaSuccess;
+  return e;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -517,6 +590,8 @@ rgs_status rgs_create(rgs_ctx** out, int device) {
     delete ctx;
     return RGS_ERR_NOMEM;
   }
+  size_t free_bytes = 0, total_bytes = 0;
+  if (cudaMemGetInfo(&free_bytes, &total_bytes) == cudaSuccess) ctx->spare_limit = total_bytes / 16;
   *out = ctx;
   return RGS_OK;
 }
@@ -527,6 +602,7 @@ void rgs_destroy(rgs_ctx* ctx) {
   cudaDeviceSynchronize();
   for (auto& kv : ctx->states) destroy_state(kv.second);
   ctx->states.clear();
+  drop_spares(ctx);
   if (ctx->host_counters) cudaFreeHost(ctx->host_counters);
   if (ctx->track_sums) cudaFree(ctx->track_sums);
   free_region(ctx->r_seed);
@@ -680,9 +756,26 @@ rgs_status rgs_release_state(rgs_ctx* ctx, uint64_t handle) {
   State* s = find_state(ctx, handle);
   if (!s) return fail(ctx, RGS_ERR_STATE, "unknown state handle");
   cudaSetDevice(ctx->device);
-  cudaDeviceSynchronize();  // queued work may still read the state's buffers
-  destroy_state(s);
   ctx->states.erase(handle);
+  const size_t bytes = s->bytes();
+  // Kept for the next state, unless a graph may still refer to its buffers, the end of its work
+  // was not recorded (it failed half-way, or never ran), or it alone exceeds the bound.
+  if (s->captured || s->open || !s->has_forward || bytes > ctx->spare_limit) {
+    cudaDeviceSynchronize();  // queued work may still read the state's buffers
+    destroy_state(s);
+    return RGS_OK;
+  }
+  size_t held = bytes;
+  for (const State* o : ctx->spare) held += o->bytes();
+  while (!ctx->spare.empty() &&
+         (ctx->spare.size() >= kSpareStates || held > ctx->spare_limit)) {
+    State* oldest = ctx->spare.front();
+    held -= oldest->bytes();
+    cudaEventSynchronize(oldest->done);  // the last work queued on it
+    destroy_state(oldest);
+    ctx->spare.erase(ctx->spare.begin());
+  }
+  ctx->spare.push_back(s);
   return RGS_OK;
 }
 
@@ -755,9 +848,13 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
     return fail(ctx, RGS_ERR_CUDA, "cudaSetDevice failed");
   const bool capturing = is_capturing(stream);
   State* s = nullptr;
-  st = get_or_create_state(ctx, handle, &s);
+  State* spare = handle && *handle == 0 && !capturing
+                     ? take_spare(ctx, vn, g->n, views.total_pixels, stream)
+                     : nullptr;
+  st = get_or_create_state(ctx, handle, &s, spare);
   if (st != RGS_OK) return st;
   s->has_forward = false;
+  open_state(*s, capturing);
   const int64_t pose_entries = (int64_t)preprocess_backward_blocks(vn) * n_views * 6;
   st = ensure_vn(ctx, *s, vn, g->n, pose_entries, capturing, stream);
   if (st != RGS_OK) return st;
@@ -773,7 +870,7 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
   if (s->r_counters.bytes < pose_bytes + reset_bytes) {
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "counters grow during capture");
     if (s->r_counters.base) RGS_CUDA(cudaDeviceSynchronize(), "sync before counters growth");
-    RGS_CUDA(alloc_region(s->r_counters, pose_bytes + reset_bytes), "allocate counters");
+    RGS_CUDA(alloc_region(ctx, s->r_counters, pose_bytes + reset_bytes), "allocate counters");
   }
   s->pose_records = static_cast<float*>(s->r_counters.base);
   s->counters = reinterpret_cast<Counters*>(static_cast<char*>(s->r_counters.base) + pose_bytes);
@@ -811,20 +908,21 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
                                   lookback_at(lb_area, &cnt->status, s->vn_cap), stream),
            "compact");
   RGS_CUDA(mark(ctx, *s, 2, stream, capturing), "event");
-  // Size the sorted list of visible entries (outside capture: read the count back; under
+  // Size the sorted list of visible entries (outside capture: the count itself, read back; under
   // capture the capacity of the last eager call holds, and a larger count is clamped to it and
   // recorded in the status word).
+  int64_t vis_cap = 0;
   if (!capturing) {
     RGS_CUDA(cudaMemcpyAsync(ctx->host_counters, cnt, sizeof(Counters), cudaMemcpyDeviceToHost,
                              stream),
              "read counters");
     RGS_CUDA(cudaStreamSynchronize(stream), "sync for visible count");
-    const int64_t nv = ctx->host_counters->n_visible;
-    if (nv > s->vis_cap) s->vis_cap = std::max<int64_t>(nv + nv / 4, 1024);
-  } else if (s->vis_cap == 0) {
-    s->vis_cap = vn;
+    vis_cap = ctx->host_counters->n_visible;
+    if (vis_cap > s->vis_cap) s->vis_cap = std::max<int64_t>(vis_cap + vis_cap / 4, 1024);
+  } else {
+    if (s->vis_cap == 0) s->vis_cap = vn;
+    vis_cap = std::min<int64_t>(s->vis_cap, vn);
   }
-  const int64_t vis_cap = std::min<int64_t>(s->vis_cap, vn);
   // 3. Stable sort by depth (positive float bits order like the values; the sign bit is 0).
   bool alt = false;
   RGS_CUDA(launch_radix_sort(s->vis_keys[0], s->vis_vals[0], s->vis_keys[1], s->vis_vals[1],
@@ -897,6 +995,7 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
            "blend forward");
   RGS_CUDA(mark(ctx, *s, 8, stream, capturing), "event");
   s->fwd_launches = (uint32_t)(launch_counter() - launches0);
+  RGS_CUDA(close_state(*s, capturing, stream), "record the end of the forward");
   s->has_forward = true;
   return RGS_OK;
 }
@@ -976,7 +1075,7 @@ rgs_status render_backward(rgs_ctx* ctx, uint64_t handle, const rgs_image_grads*
         if (capturing)
           return fail(ctx, RGS_ERR_CAPACITY, "regulariser scratch: make a first call outside capture");
         free_region(s->r_reg);
-        RGS_CUDA(alloc_region(s->r_reg, sizeof(float) * (size_t)n), "allocate regulariser scratch");
+        RGS_CUDA(alloc_region(ctx, s->r_reg, sizeof(float) * (size_t)n), "allocate regulariser scratch");
         s->reg_vals = static_cast<float*>(s->r_reg.base);
         s->reg_cap = n;
       }
@@ -984,6 +1083,7 @@ rgs_status render_backward(rgs_ctx* ctx, uint64_t handle, const rgs_image_grads*
     }
   }
   const uint64_t launches0 = launch_counter();
+  open_state(*s, capturing);
   s->bwd_timed = ctx->timing;
   RGS_CUDA(mark(ctx, *s, kEvBwd0, stream, capturing), "event");
   RGS_CUDA(launch_blend(false, s->views, s->consts, s->ranges, s->sorted_vals, s->rec0, s->rec1,
@@ -998,6 +1098,7 @@ rgs_status render_backward(rgs_ctx* ctx, uint64_t handle, const rgs_image_grads*
            "preprocess backward");
   RGS_CUDA(mark(ctx, *s, kEvBwd0 + 2, stream, capturing), "event");
   s->bwd_launches = (uint32_t)(launch_counter() - launches0);
+  RGS_CUDA(close_state(*s, capturing, stream), "record the end of the backward");
   return RGS_OK;
 }
 }  // namespace
@@ -1035,9 +1136,7 @@ rgs_status rgs_query_stats(rgs_ctx* ctx, uint64_t handle, rgs_stats* out, void* 
   if (!s) return fail(ctx, RGS_ERR_STATE, "unknown state handle");
   std::memset(out, 0, sizeof(*out));
   out->pair_capacity = s->pair_cap;
-  out->state_bytes = (int64_t)(s->r_vn.bytes + s->r_n.bytes + s->r_pix.bytes + s->r_tile.bytes +
-                               s->r_pair.bytes + s->r_scratch.bytes + s->r_pose.bytes +
-                               s->r_counters.bytes);
+  out->state_bytes = (int64_t)s->bytes();
   if (!s->counters) return RGS_OK;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);
   cudaSetDevice(ctx->device);
@@ -1424,7 +1523,7 @@ rgs_status rgs_init_seeds(rgs_ctx* ctx, const rgs_camera* cams, int32_t n_views,
   // The scratch region is kept in the context and only grows: repeated calls (one per new
   // keyframe) neither allocate nor free.
   if (ctx->r_seed.bytes < bytes)
-    RGS_CUDA(alloc_region(ctx->r_seed, bytes), "allocate seeding scratch");
+    RGS_CUDA(alloc_region(ctx, ctx->r_seed, bytes), "allocate seeding scratch");
   char* p = static_cast<char*>(ctx->r_seed.base);
   uint32_t* flags = carve<uint32_t>(p, m);
   uint32_t* pos = carve<uint32_t>(p, m);
