@@ -180,10 +180,9 @@ const char* rgs_last_error(const rgs_ctx* ctx);
  *   state: in/out. If *state is 0 a new state is created and its handle written back; otherwise
  *     the named state is reused (its previous contents are replaced). The state keeps the data
  *     the backward needs.
- * Outside stream capture the call synchronises the stream twice (after the visibility
- * compaction and after the pair count) to size the sorted list of visible entries and the pair
- * list. Under stream capture it never synchronises and keeps the sizes of the last call outside
- * capture; if a list would overflow, the kernels record it, the output is incomplete and
+ * Outside stream capture the call waits once, for the projection, whose counts size the sorted
+ * list of visible entries and the tile lists; the rest is queued while the stream runs on. Under
+ * stream capture it never synchronises and keeps the sizes of the last call outside capture; if a list would overflow, the kernels record it, the output is incomplete and
  * rgs_query_stats reports status bit 1 (pairs) or 2 (visible entries). */
 rgs_status rgs_render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera* cams,
                               int32_t n_views, const rgs_config* cfg, rgs_images* out,
@@ -315,11 +314,11 @@ rgs_status rgs_pose_adam_step(rgs_ctx* ctx, int32_t n_views, const rgs_adam_conf
 #define RGS_PHASE_PREPROCESS 0     /* projection, SH colour, tile counts (Eq. proj, Eq. app-sh) */
 #define RGS_PHASE_COMPACT 1        /* visible (view, Gaussian) entries with depth keys */
 #define RGS_PHASE_DEPTH_SORT 2     /* radix sort of the visible entries by depth */
-#define RGS_PHASE_OFFSETS 3        /* pair offsets (scan of tile counts in depth order) */
-#define RGS_PHASE_DUPLICATE 4      /* (tile, Gaussian) pair emission */
-#define RGS_PHASE_TILE_SORT 5      /* radix sort of the pairs by tile */
-#define RGS_PHASE_RANGES 6         /* per-tile [first, last + 1) (with an SH event, also the
-                                      colours of the visible entries) */
+#define RGS_PHASE_OFFSETS 3        /* nothing: the emission finds its own offsets */
+#define RGS_PHASE_DUPLICATE 4      /* emission of one entry per touched cell of 4 x 4 tiles */
+#define RGS_PHASE_TILE_SORT 5      /* radix sort of those by cell */
+#define RGS_PHASE_RANGES 6         /* the tiles' lists, ranges and launch order (with an SH event,
+                                      also the colours of the visible entries) */
 #define RGS_PHASE_BLEND_FORWARD 7  /* front-to-back compositing (Eq. alpha) */
 #define RGS_PHASE_BLEND_BACKWARD 8 /* back-to-front screen-space gradients */
 #define RGS_PHASE_PREPROCESS_BACKWARD 9 /* parameter and twist gradients (Eq. muCjac..sigmaIjac) */
@@ -332,8 +331,8 @@ rgs_status rgs_set_phase_timing(rgs_ctx* ctx, int32_t enable);
 
 /* Device milliseconds of each phase of the most recent forward and backward on `state`
  * (ms[RGS_PHASE_COUNT]; a phase that did not run reads 0). Synchronises `stream`. Outside stream
- * capture, the depth-sort and duplicate phases of a forward include the host synchronisations
- * that size the visible list and the pair list. */
+ * capture, the compaction and depth-sort phases of a forward include the host wait
+ * that sizes the lists. */
 rgs_status rgs_phase_times(rgs_ctx* ctx, uint64_t state, float* ms, int32_t n, void* stream);
 
 /* ---- Diagnostics: copies of a state's binning results (synchronise `stream`). ----

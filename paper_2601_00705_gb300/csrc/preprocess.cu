@@ -295,7 +295,7 @@ __device__ __forceinline__ void load_sh(const float* __restrict__ sh, int i, flo
 __global__ void __launch_bounds__(kPreThreads) cull_kernel(
     const __grid_constant__ Views views, const Consts c, int n, const float* __restrict__ means,
     const float* __restrict__ log_scales, const float* __restrict__ quats,
-    const float* __restrict__ logits, uint32_t* __restrict__ ntiles, uint32_t* __restrict__ cand,
+    const float* __restrict__ logits, uint32_t* __restrict__ cand,
     uint32_t* __restrict__ vis_bits, int bit_words, Counters* __restrict__ counters,
     int views_per_chunk) {
   static_assert(kPreThreads % 32 == 0, "whole words of the visibility bitmask per block");
@@ -428,9 +428,10 @@ __global__ void __launch_bounds__(kPreThreads) project_kernel(
     const float* __restrict__ log_scales, const float* __restrict__ quats,
     const float* __restrict__ logits, const float* __restrict__ sh,
     const uint32_t* __restrict__ cand, float4* __restrict__ rec0, float4* __restrict__ rec1,
-    float4* __restrict__ rec2, uint32_t* __restrict__ ntiles, uint32_t* __restrict__ vis_bits,
+    float4* __restrict__ rec2, uint2* __restrict__ touched, uint32_t* __restrict__ vis_bits,
     int bit_words, Counters* __restrict__ counters) {
   chain_wait();
+  unsigned long long sum_visible = 0, sum_tiles = 0, sum_cells = 0;
   constexpr int K = DEG >= 0 ? (DEG + 1) * (DEG + 1) : 1;
   const uint32_t n_cand = counters->n_candidates;
   for (uint32_t k = blockIdx.x * kPreThreads + threadIdx.x; k < n_cand;
@@ -471,106 +472,97 @@ __global__ void __launch_bounds__(kPreThreads) project_kernel(
     float rgb[3] = {0.0f, 0.0f, 0.0f};
     if constexpr (DEG >= 0) sh_colour<DEG>(shc, g.m, ps, rgb);
     const float4 r2 = make_float4(rgb[0], rgb[1], rgb[2], p.mc[2]);
-    uint32_t count = 0;
+    uint32_t tiles = 0, cells = 0;
     Ellipse e;
-    if (make_ellipse(r0, r1, c.log2_alpha_min, e))
-      for_each_tile_row(e, views.tile_w, views.tile_h, vp.tiles_x, vp.tiles_y,
-                        [&](int, int tx0, int tx1) { count += (uint32_t)(tx1 - tx0 + 1); });
+    TileCover tc;
+    if (make_ellipse(r0, r1, c.log2_alpha_min, e) &&
+        tc.init(e, views.tile_w, views.tile_h, vp.tiles_x, vp.tiles_y)) {
+      for (int cy = tc.ty0 >> kCellShift; cy <= tc.ty1 >> kCellShift; ++cy) {
+        CellRow row;
+        if (!cell_row(tc, cy, row)) continue;
+        cells += (uint32_t)(row.c1 - row.c0 + 1);
+#pragma unroll
+        for (int r = 0; r < kCellTiles; ++r) tiles += span_tiles(row.span[r]);
+      }
+    }
     rec0[vi] = r0;
     rec1[vi] = r1;
     rec2[vi] = r2;
-    ntiles[vi] = count;
-    if (count > 0) atomicOr(&vis_bits[(size_t)v * bit_words + (i >> 5)], 1u << (i & 31));
+    touched[vi] = make_uint2(tiles, cells);
+    if (tiles > 0) {
+      atomicOr(&vis_bits[(size_t)v * bit_words + (i >> 5)], 1u << (i & 31));
+      ++sum_visible;
+      sum_tiles += tiles;
+      sum_cells += cells;
+    }
+  }
+  // The totals the host sizes the lists by: one set of atomics per block.
+  __shared__ unsigned long long s_sum[3];
+  if (threadIdx.x < 3) s_sum[threadIdx.x] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sum_visible += __shfl_xor_sync(0xffffffffu, sum_visible, o);
+    sum_tiles += __shfl_xor_sync(0xffffffffu, sum_tiles, o);
+    sum_cells += __shfl_xor_sync(0xffffffffu, sum_cells, o);
+  }
+  if ((threadIdx.x & 31) == 0 && sum_visible) {
+    atomicAdd(&s_sum[0], sum_visible);
+    atomicAdd(&s_sum[1], sum_tiles);
+    atomicAdd(&s_sum[2], sum_cells);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && s_sum[0]) {
+    atomicAdd(&counters->all_visible, s_sum[0]);
+    atomicAdd(&counters->all_pairs, s_sum[1]);
+    atomicAdd(&counters->all_cells, s_sum[2]);
   }
 }
 
-// Forward, pass 3 (after the tile lists are built, before the blend), one launch of two
-// independent parts.
-//  * Blocks [0, range_blocks): tile ranges. Thread t looks at the eight sorted keys 8t .. 8t + 7
-//    (two 16-byte loads; the key arrays are 256-byte aligned) and the key before them, and writes
-//    the run boundaries among them into `ranges` (zero on entry: tiles without pairs keep
-//    [0, 0)).
-//  * The other blocks: one thread per visible entry, in (view, Gaussian) order (grid-stride
-//    over `list`, the compacted list: neighbouring threads read neighbouring Gaussians' SH
-//    rows; in depth order the reads are scattered, which costs ~0.15 ms on 3M Gaussians whose
-//    coefficients do not fit in L2). The colour from the SH
-//    coefficients for the direction camera centre -> Gaussian (Eq. app-sh), clamped at 0, into
-//    rec2.xyz. An entry with a non-finite coefficient gets log2 opacity -inf, so that it covers
-//    no pixel in either blend, and is counted as culled.
-constexpr int kRangesColourThreads = 256;
-constexpr int kRangesKeys = 8;  // sorted keys per thread of the range part (two 16-byte loads)
+// Forward, pass 3 (only with an SH event; after the tile lists are built, before the blend): one
+// thread per visible entry, in (view, Gaussian) order (grid-stride over `list`, the compacted
+// list: neighbouring threads read neighbouring Gaussians' SH rows; in depth order the reads are
+// scattered, which costs ~0.15 ms on 3M Gaussians whose coefficients do not fit in L2). The colour
+// from the SH coefficients for the direction camera centre -> Gaussian (Eq. app-sh), clamped at 0,
+// into rec2.xyz. An entry with a non-finite coefficient gets log2 opacity -inf, so that it covers
+// no pixel in either blend, and is counted as culled.
+constexpr int kColourThreads = 256;
 
 template <int DEG, bool kDevPose>
-__global__ void __launch_bounds__(kRangesColourThreads) ranges_colour_kernel(
-    const uint32_t* __restrict__ keys, uint32_t total_tiles, uint2* __restrict__ ranges,
-    uint32_t range_blocks, const __grid_constant__ Views views, int n,
-    const float* __restrict__ means, const float* __restrict__ sh,
-    const uint32_t* __restrict__ list, float4* __restrict__ rec1, float4* __restrict__ rec2,
-    Counters* __restrict__ counters) {
+__global__ void __launch_bounds__(kColourThreads) colour_kernel(
+    const __grid_constant__ Views views, int n, const float* __restrict__ means,
+    const float* __restrict__ sh, const uint32_t* __restrict__ list, float4* __restrict__ rec1,
+    float4* __restrict__ rec2, Counters* __restrict__ counters) {
   chain_wait();
-  if (blockIdx.x < range_blocks) {
-    const uint32_t np = counters->n_pairs_stored;
-    const uint32_t p0 = (uint32_t)kRangesKeys * (blockIdx.x * kRangesColourThreads + threadIdx.x);
-    if (p0 >= np) return;
-    uint32_t k[kRangesKeys + 1];  // k[0] = key before p0 (or none), k[1..] = keys p0 ..
-    k[0] = p0 > 0 ? keys[p0 - 1] : 0xffffffffu;
-    if (p0 + kRangesKeys <= np) {
+  constexpr int K = (DEG + 1) * (DEG + 1);
+  const uint32_t n_visible = counters->n_visible_kept;
+  for (uint32_t k = blockIdx.x * kColourThreads + threadIdx.x; k < n_visible;
+       k += gridDim.x * kColourThreads) {
+    const uint32_t vi = list[k];
+    const int v = (int)(vi / (uint32_t)n);
+    const int i = (int)(vi - (uint32_t)v * (uint32_t)n);
+    float shc[3 * K];
+    load_sh<DEG>(sh, i, shc);
+    bool sh_finite = true;
 #pragma unroll
-      for (int h = 0; h < kRangesKeys / 4; ++h) {
-        const uint4 q = *reinterpret_cast<const uint4*>(keys + p0 + 4 * h);
-        k[4 * h + 1] = q.x;
-        k[4 * h + 2] = q.y;
-        k[4 * h + 3] = q.z;
-        k[4 * h + 4] = q.w;
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < kRangesKeys; ++j) k[j + 1] = p0 + j < np ? keys[p0 + j] : 0xffffffffu;
-    }
-    const uint32_t next = p0 + kRangesKeys < np ? keys[p0 + kRangesKeys] : 0xffffffffu;
-#pragma unroll
-    for (int j = 0; j < kRangesKeys; ++j) {
-      const uint32_t p = p0 + j;
-      const uint32_t key = k[j + 1];
-      if (p >= np || key >= total_tiles) continue;
-      const uint32_t after = j < kRangesKeys - 1 ? k[j + 2] : next;
-      if (p == 0 || k[j] != key) ranges[key].x = p;
-      if (p == np - 1 || after != key) ranges[key].y = p + 1;
-    }
-    return;
-  }
-  if constexpr (DEG >= 0) {
-    constexpr int K = (DEG + 1) * (DEG + 1);
-    const uint32_t n_visible = counters->n_visible_kept;
-    const uint32_t stride = (gridDim.x - range_blocks) * kRangesColourThreads;
-    for (uint32_t k = (blockIdx.x - range_blocks) * kRangesColourThreads + threadIdx.x;
-         k < n_visible; k += stride) {
-      const uint32_t vi = list[k];
-      const int v = (int)(vi / (uint32_t)n);
-      const int i = (int)(vi - (uint32_t)v * (uint32_t)n);
-      float shc[3 * K];
-      load_sh<DEG>(sh, i, shc);
-      bool sh_finite = true;
-  #pragma unroll
-      for (int a = 0; a < 3 * K; ++a) sh_finite = sh_finite && isfinite(shc[a]);
-      float4 r2 = rec2[vi];
-      if (!sh_finite) {
-        atomicAdd(&counters->n_nonfinite, 1u);
-        reinterpret_cast<float*>(rec1 + vi)[3] = -INFINITY;
-        r2.x = r2.y = r2.z = 0.0f;
-        rec2[vi] = r2;
-        continue;
-      }
-      const PoseRef ps = view_pose<kDevPose>(views, v);
-      const float m[3] = {__ldg(means + 3 * (size_t)i), __ldg(means + 3 * (size_t)i + 1),
-                          __ldg(means + 3 * (size_t)i + 2)};
-      float rgb[3];
-      sh_colour<DEG>(shc, m, ps, rgb);
-      r2.x = rgb[0];
-      r2.y = rgb[1];
-      r2.z = rgb[2];
+    for (int a = 0; a < 3 * K; ++a) sh_finite = sh_finite && isfinite(shc[a]);
+    float4 r2 = rec2[vi];
+    if (!sh_finite) {
+      atomicAdd(&counters->n_nonfinite, 1u);
+      reinterpret_cast<float*>(rec1 + vi)[3] = -INFINITY;
+      r2.x = r2.y = r2.z = 0.0f;
       rec2[vi] = r2;
+      continue;
     }
+    const PoseRef ps = view_pose<kDevPose>(views, v);
+    const float m[3] = {__ldg(means + 3 * (size_t)i), __ldg(means + 3 * (size_t)i + 1),
+                        __ldg(means + 3 * (size_t)i + 2)};
+    float rgb[3];
+    sh_colour<DEG>(shc, m, ps, rgb);
+    r2.x = rgb[0];
+    r2.y = rgb[1];
+    r2.z = rgb[2];
+    rec2[vi] = r2;
   }
 }
 
@@ -1066,7 +1058,7 @@ __global__ void __launch_bounds__(256) reg_sum_kernel(int n, const float* __rest
 
 cudaError_t launch_preprocess_forward(const Views& views, const Consts& c,
                                       const rgs_gaussians& g, float4* rec0, float4* rec1,
-                                      float4* rec2, uint32_t* ntiles, uint32_t* cand,
+                                      float4* rec2, uint2* touched, uint32_t* cand,
                                       uint32_t* vis_bits, bool defer_colour, Counters* counters,
                                       cudaStream_t stream) {
   if (g.n == 0) return cudaSuccess;
@@ -1080,8 +1072,7 @@ cudaError_t launch_preprocess_forward(const Views& views, const Consts& c,
   const int per_chunk = (views.n_views + chunks - 1) / chunks;
   const dim3 grid((unsigned)blocks_x, (unsigned)((views.n_views + per_chunk - 1) / per_chunk));
   cudaError_t e = launch_chained(cull_kernel, grid, dim3(kPreThreads), stream, views, c, g.n,
-                                 g.means, g.log_scales, g.quats, g.opacity_logits, ntiles, cand,
-                                 vis_bits, bit_words, counters, per_chunk);
+                                 g.means, g.log_scales, g.quats, g.opacity_logits, cand, vis_bits, bit_words, counters, per_chunk);
   RGS_LAUNCHED();
   if (e != cudaSuccess) return e;
   // Pass 2: grid-stride over the candidates.
@@ -1091,7 +1082,7 @@ cudaError_t launch_preprocess_forward(const Views& views, const Consts& c,
   e = launch_chained(views.pose_dev ? project_kernel<D, true> : project_kernel<D, false>,         \
                      dim3(blocks2), dim3(kPreThreads), stream, views, c, g.n, g.means,            \
                      g.log_scales, g.quats, g.opacity_logits, g.sh, (const uint32_t*)cand, rec0, \
-                     rec1, rec2, ntiles, vis_bits, bit_words, counters)
+                     rec1, rec2, touched, vis_bits, bit_words, counters)
   if (defer_colour) {
     RGS_PROJECT(-1);
   } else {
@@ -1107,42 +1098,25 @@ cudaError_t launch_preprocess_forward(const Views& views, const Consts& c,
   return e;
 }
 
-cudaError_t launch_ranges_colour(const uint32_t* keys, int total_tiles, uint2* ranges,
-                                 uint32_t pair_capacity, const Views& views,
-                                 const rgs_gaussians& g, const uint32_t* list, int64_t vis_cap,
-                                 bool colour, float4* rec1, float4* rec2, Counters* counters,
-                                 cudaStream_t stream) {
-  const uint32_t range_blocks =
-      (uint32_t)(((int64_t)pair_capacity + kRangesKeys * kRangesColourThreads - 1) /
-                 (kRangesKeys * kRangesColourThreads));
-  const int64_t colour_items = colour && g.n > 0 ? vis_cap : 0;
-  const uint32_t colour_blocks = (uint32_t)std::min<int64_t>(
-      (colour_items + kRangesColourThreads - 1) / kRangesColourThreads, 4 * 152);
-  if (range_blocks + colour_blocks == 0) return cudaSuccess;
+cudaError_t launch_colour(const Views& views, const rgs_gaussians& g, const uint32_t* list,
+                          int64_t vis_cap, float4* rec1, float4* rec2, Counters* counters,
+                          cudaStream_t stream) {
+  const unsigned blocks =
+      (unsigned)std::min<int64_t>((vis_cap + kColourThreads - 1) / kColourThreads, 4 * 152);
+  if (g.n == 0 || blocks == 0) return cudaSuccess;
   cudaError_t e = cudaSuccess;
-  if (colour_blocks == 0) {
-    // Ranges only: the instance without the colour code keeps the registers, and so the
-    // occupancy, of a plain scan over the pairs.
-    e = launch_chained(ranges_colour_kernel<-1, false>, dim3(range_blocks),
-                       dim3(kRangesColourThreads), stream, keys, (uint32_t)total_tiles, ranges,
-                       range_blocks, views, g.n, g.means, g.sh, list, rec1, rec2, counters);
-    RGS_LAUNCHED();
-    return e;
-  }
-#define RGS_RANGES_COLOUR(D)                                                                   \
-  e = launch_chained(views.pose_dev ? ranges_colour_kernel<D, true>                             \
-                                    : ranges_colour_kernel<D, false>,                           \
-                     dim3(range_blocks + colour_blocks), dim3(kRangesColourThreads), stream,    \
-                     keys, (uint32_t)total_tiles, ranges, range_blocks, views, g.n, g.means,    \
-                     g.sh, list, rec1, rec2, counters)
+#define RGS_COLOUR(D)                                                                         \
+  e = launch_chained(views.pose_dev ? colour_kernel<D, true> : colour_kernel<D, false>,       \
+                     dim3(blocks), dim3(kColourThreads), stream, views, g.n, g.means, g.sh, \
+                     list, rec1, rec2, counters)
   switch (g.sh_degree) {
-    case 0: RGS_RANGES_COLOUR(0); break;
-    case 1: RGS_RANGES_COLOUR(1); break;
-    case 2: RGS_RANGES_COLOUR(2); break;
-    default: RGS_RANGES_COLOUR(3); break;
+    case 0: RGS_COLOUR(0); break;
+    case 1: RGS_COLOUR(1); break;
+    case 2: RGS_COLOUR(2); break;
+    default: RGS_COLOUR(3); break;
   }
   RGS_LAUNCHED();
-#undef RGS_RANGES_COLOUR
+#undef RGS_COLOUR
   return e;
 }
 

@@ -1,4 +1,4 @@
-// raster.cu -- pair duplication, tile ranges, and the forward / backward alpha blends.
+// raster.cu -- the forward and backward alpha blends.
 //
 // Forward blend (Section 3.1, Eq. alpha; Section 3.2.2): one CTA per (view, tile), the tiles
 // taken longest run first; the tile's Gaussians, already in near-to-far order, are staged
@@ -15,183 +15,6 @@
 
 namespace rgs {
 namespace {
-
-constexpr int kDupThreads = 256;
-constexpr int kDupWarps = kDupThreads / 32;
-// Footprints of up to this many tiles are walked by their own lane into a per-warp staging
-// buffer in shared memory, from which the warp writes them out coalesced; larger ones are walked
-// by the whole warp, up to 32 tile rows at a time with the rows' tiles dealt out over the lanes.
-constexpr uint32_t kDupSerialMax = 32;
-constexpr int kDupStage = 32 * kDupSerialMax;  // staged pairs per warp and round
-
-// First lane whose inclusive count exceeds idx (idx < the warp total).
-__device__ __forceinline__ int lane_of(int incl, int idx) {
-  int lo = 0, hi = 31;
-#pragma unroll
-  for (int step = 0; step < 5; ++step) {
-    const int mid = (lo + hi) >> 1;
-    if (__shfl_sync(0xffffffffu, incl, mid) > idx) hi = mid; else lo = mid + 1;
-  }
-  return lo;
-}
-
-// One (tile, vi) pair per tile touched by each visible entry, into the entry's slots
-// [offsets[k], offsets[k] + ntiles[vi]) of the pair list (so the list is in the entries' depth
-// order). The counting pass in the projection visits the same tiles, so every slot is written;
-// if that ever failed, the unused slots get the out-of-range key total_tiles, which sorts last
-// and owns no tile range.
-__global__ void __launch_bounds__(kDupThreads) duplicate_kernel(
-    const __grid_constant__ Views views, int n, const uint32_t* __restrict__ order,
-    const uint32_t* __restrict__ offsets, const uint32_t* __restrict__ ntiles,
-    const float4* __restrict__ rec0, const float4* __restrict__ rec1, float log2_alpha_min,
-    uint32_t visible_cap, uint32_t capacity, uint32_t* __restrict__ keys,
-    uint32_t* __restrict__ vals, Counters* __restrict__ counters) {
-  chain_wait();
-  __shared__ uint32_t s_stage[kDupWarps][kDupStage];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t* stage = s_stage[warp];
-  // The sorted list holds at most visible_cap entries; more (only possible under stream
-  // capture) are recorded in the status word. The pair count the tile sort uses is stored here.
-  const uint32_t n_visible_raw = counters->n_visible;
-  const uint32_t n_visible = min(n_visible_raw, visible_cap);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    if (n_visible_raw > visible_cap) atomicOr(&counters->status, (uint32_t)kStatusVisibleOverflow);
-    counters->n_visible_kept = n_visible;
-    const uint32_t p = counters->n_pairs;
-    counters->n_pairs_stored = p < capacity ? p : capacity;
-  }
-  const uint32_t sentinel = (uint32_t)views.total_tiles;
-  // Lane l of global warp w takes entry k = round * 32 W + l W + w (W warps in the grid): the
-  // nearest entries, whose footprints are the largest, come first in the depth order and are
-  // spread one per warp instead of filling the first warps.
-  const uint32_t n_warps = gridDim.x * kDupWarps;
-  const uint32_t gwarp = blockIdx.x * kDupWarps + warp;
-  for (uint64_t round_base = 0; round_base + gwarp < n_visible; round_base += 32ull * n_warps) {
-    const uint64_t k64 = round_base + (uint64_t)lane * n_warps + gwarp;
-    const uint32_t k = k64 < n_visible ? (uint32_t)k64 : n_visible;
-    uint32_t vi = 0, begin = 0, cnt = 0;
-    bool ok = false;
-    if (k < n_visible) {
-      vi = order[k];
-      begin = offsets[k];
-      cnt = ntiles[vi];
-      if ((uint64_t)begin + cnt > capacity)
-        atomicOr(&counters->status, (uint32_t)kStatusPairOverflow);
-    }
-    const int v = (int)(vi / (uint32_t)max(n, 1));
-    // Every lane sets up its own entry's tile cover once; a large footprint's cover is then
-    // handed to the whole warp by shuffles instead of being recomputed by every lane.
-    TileCover tc;
-    if (k < n_visible) {
-      Ellipse e;
-      const ViewParams& vp = views.v[v];
-      ok = make_ellipse(rec0[vi], rec1[vi], log2_alpha_min, e) &&
-           tc.init(e, views.tile_w, views.tile_h, vp.tiles_x, vp.tiles_y);
-    }
-    // Small footprints: stage, then write out.
-    const bool small = k < n_visible && cnt <= kDupSerialMax;
-    const int c_small = small ? (int)cnt : 0;
-    int incl = c_small;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    const int staged = __shfl_sync(0xffffffffu, incl, 31);
-    if (small) {
-      int q = incl - c_small;
-      const int q_end = incl;
-      if (ok) {
-        const ViewParams& vp = views.v[v];
-        for (int ty = tc.ty0; ty <= tc.ty1; ++ty) {
-          int tx0, tx1;
-          if (!tc.span(ty, tx0, tx1)) continue;
-          const uint32_t row = (uint32_t)(vp.tile_base + ty * vp.tiles_x);
-          for (int tx = tx0; tx <= tx1 && q < q_end; ++tx) stage[q++] = row + tx;
-        }
-      }
-      for (; q < q_end; ++q) stage[q] = sentinel;
-    }
-    __syncwarp();
-    for (int b = 0; b < staged; b += 32) {
-      const int idx = b + lane;
-      const int src = lane_of(incl, idx);
-      const int src_incl = __shfl_sync(0xffffffffu, incl, src);
-      const int src_cnt = __shfl_sync(0xffffffffu, c_small, src);
-      const uint32_t src_begin = __shfl_sync(0xffffffffu, begin, src);
-      const uint32_t src_vi = __shfl_sync(0xffffffffu, vi, src);
-      if (idx < staged) {
-        const uint32_t off = src_begin + (uint32_t)(idx - (src_incl - src_cnt));
-        if (off < capacity) {
-          keys[off] = stage[idx];
-          vals[off] = src_vi;
-        }
-      }
-    }
-    __syncwarp();
-    // Large footprints: the whole warp, one entry at a time.
-    unsigned big = __ballot_sync(0xffffffffu, k < n_visible && cnt > kDupSerialMax);
-    while (big) {
-      const int src = __ffs(big) - 1;
-      big &= big - 1;
-      const uint32_t vib = __shfl_sync(0xffffffffu, vi, src);
-      const uint32_t bbeg = __shfl_sync(0xffffffffu, begin, src);
-      const uint32_t bend = min(bbeg + __shfl_sync(0xffffffffu, cnt, src), capacity);
-      uint32_t done = 0;  // pairs written so far (rows before the current chunk)
-      if (__shfl_sync(0xffffffffu, (int)ok, src)) {
-        const TileCover tb = tc.broadcast(src);
-        const ViewParams& vp = views.v[__shfl_sync(0xffffffffu, v, src)];
-        {
-          for (int r0 = tb.ty0; r0 <= tb.ty1; r0 += 32) {
-            // Lane l takes tile row r0 + l; the rows' tiles are then dealt out 32 at a time.
-            const int ty = r0 + lane;
-            int tx0 = 0, tx1 = -1;
-            if (ty > tb.ty1 || !tb.span(ty, tx0, tx1)) {
-              tx0 = 0;
-              tx1 = -1;
-            }
-            const int w = tx1 - tx0 + 1;
-            int rincl = w;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-              const int y = __shfl_up_sync(0xffffffffu, rincl, o);
-              if (lane >= o) rincl += y;
-            }
-            const int total = __shfl_sync(0xffffffffu, rincl, 31);
-            for (int b = 0; b < total; b += 32) {
-              const int idx = b + lane;
-              const int row = lane_of(rincl, idx);
-              const int r_incl = __shfl_sync(0xffffffffu, rincl, row);
-              const int r_w = __shfl_sync(0xffffffffu, w, row);
-              const int r_tx0 = __shfl_sync(0xffffffffu, tx0, row);
-              const uint32_t off = bbeg + done + (uint32_t)idx;
-              if (idx < total && off < bend) {
-                keys[off] = (uint32_t)(vp.tile_base + (r0 + row) * vp.tiles_x + r_tx0 + idx -
-                                       (r_incl - r_w));
-                vals[off] = vib;
-              }
-            }
-            done += (uint32_t)total;
-          }
-        }
-      }
-      for (uint32_t off = bbeg + done + lane; off < bend; off += 32) {
-        keys[off] = sentinel;
-        vals[off] = vib;
-      }
-    }
-  }
-}
-
-// Keeps at most `capacity` visible entries (the sorted-list capacity under stream capture): the
-// entries beyond it are dropped from this forward and the overflow is recorded.
-__global__ void store_pair_count_kernel(Counters* counters, uint32_t capacity) {
-  chain_wait();
-  const uint32_t p = counters->n_pairs;
-  counters->n_pairs_stored = p < capacity ? p : capacity;
-  if (counters->n_visible > 0) atomicOr(&counters->status, (uint32_t)kStatusVisibleOverflow);
-  counters->n_visible_kept = 0;
-}
 
 // ------------------------------------------------------------------------------------------
 // Staging of a batch of Gaussians in shared memory, with the row terms of the tile's anchor row
@@ -796,30 +619,6 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
   }
 }
 
-// ------------------------------------------------------------------------------------------
-// Launch order of the blends' tiles: longest run first. A CTA's time grows with its tile's run,
-// and runs differ by two orders of magnitude (a few tiles near dense structure hold thousands of
-// Gaussians); launched in tile order, a long run that starts late holds its SM after the others
-// have drained. Sorted by decreasing length, the long runs start first and the short ones fill
-// the end. The key is the run length's octave, so the stable sort keeps each octave's tiles in
-// tile order: neighbouring tiles, which share Gaussians (their records, and in the backward their
-// gradient atomics), still run together. Finer classes (16 per octave) made the backward 3 %
-// slower; octaves made it 1 % faster than plain tile order.
-// ------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t length_octave(uint32_t len) {
-  return (uint32_t)(31 - __clz(len + 1u));  // 0 .. 32
-}
-
-__global__ void tile_order_keys_kernel(const uint2* __restrict__ ranges, uint32_t total_tiles,
-                                       uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-  chain_wait();
-  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= total_tiles) return;
-  const uint2 r = ranges[t];
-  keys[t] = 32u - length_octave(r.y - r.x);
-  vals[t] = t;
-}
-
 template <int TW, int TH, int PPT>
 cudaError_t launch_blends_t(bool forward, const Views& views, const Consts& c,
                             const uint2* ranges, const uint32_t* pair_vals, const float4* rec0,
@@ -848,49 +647,6 @@ cudaError_t launch_blends_t(bool forward, const Views& views, const Consts& c,
 }
 
 }  // namespace
-
-cudaError_t launch_duplicate(const Views& views, int n, const uint32_t* order,
-                             const uint32_t* offsets, const uint32_t* ntiles, const float4* rec0,
-                             const float4* rec1, const float4* rec2, float log2_alpha_min,
-                             int64_t visible_cap, uint32_t capacity,
-                             uint32_t* keys, uint32_t* vals, Counters* counters,
-                             cudaStream_t stream) {
-  (void)rec2;
-  if (visible_cap > 0) {
-    const int64_t need = (visible_cap + kDupThreads - 1) / kDupThreads;
-    const unsigned blocks = (unsigned)std::min<int64_t>(need, 8 * 152);
-    const cudaError_t e =
-        launch_chained(duplicate_kernel, dim3(blocks), dim3(kDupThreads), stream, views, n, order,
-                       offsets, ntiles, rec0, rec1, log2_alpha_min,
-                       (uint32_t)std::min<int64_t>(visible_cap, 0xffffffffll), capacity, keys,
-                       vals, counters);
-    RGS_LAUNCHED();
-    return e;
-  }
-  // No visible-list capacity: nothing to duplicate, but the counts still need storing.
-  const cudaError_t e = launch_chained(store_pair_count_kernel, dim3(1), dim3(1), stream, counters,
-                                       capacity);
-  RGS_LAUNCHED();
-  return e;
-}
-
-cudaError_t launch_tile_order(const uint2* ranges, int total_tiles, uint32_t* keys,
-                              uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
-                              uint32_t* hist, uint32_t* block_sums, const uint32_t** order,
-                              cudaStream_t stream) {
-  *order = vals;
-  if (total_tiles <= 0) return cudaSuccess;
-  constexpr int kThreads = 256;
-  cudaError_t e = launch_chained(tile_order_keys_kernel, dim3((total_tiles + kThreads - 1) / kThreads),
-                                 dim3(kThreads), stream, ranges, (uint32_t)total_tiles, keys, vals);
-  RGS_LAUNCHED();
-  if (e != cudaSuccess) return e;
-  bool alt = false;
-  e = launch_radix_sort(keys, vals, keys_alt, vals_alt, total_tiles, nullptr, 0, 6, hist,
-                        block_sums, &alt, stream, kSortItemsSmall);
-  *order = alt ? vals_alt : vals;
-  return e;
-}
 
 cudaError_t launch_blend(bool forward, const Views& views, const Consts& c, const uint2* ranges,
                          const uint32_t* pair_vals, const float4* rec0, const float4* rec1,

@@ -5,12 +5,11 @@
 //   1. preprocess      per Gaussian, all views: projected records + tile counts  (Eq. proj)
 //   2. compact         visible (view, Gaussian) entries with their depth keys
 //   3. depth sort      stable radix sort of the visible entries by float32 depth
-//   4. offsets         exclusive scan of tile counts in depth order
-//   5. duplicate       one (tile, vi) pair per touched tile, emitted in depth order
-//   6. tile sort       stable radix sort of the pairs by global tile id; stability keeps each
-//                      tile's run in (depth, index) order
-//   7. ranges          [first, last + 1) of each tile's run
-//   8. blend           front-to-back compositing per tile                          (Eq. alpha)
+//   4. emit            one (cell, vi) entry per touched cell of 4 x 4 tiles, in depth order
+//   5. cell sort       stable radix sort of those by cell; stability keeps each cell's run in
+//                      (depth, index) order
+//   6. tile lists      each cell's run expanded to its tiles' lists, and the lists' ranges
+//   7. blend           front-to-back compositing per tile                          (Eq. alpha)
 // Backward: backward blend (screen-space gradients) then backward preprocess (parameter and
 // twist gradients, Eq. muCjac / muIjac / sigmaIjac) and the twist reduction.
 #include <algorithm>
@@ -26,14 +25,12 @@
 namespace rgs {
 cudaError_t launch_preprocess_forward(const Views& views, const Consts& c,
                                       const rgs_gaussians& g, float4* rec0, float4* rec1,
-                                      float4* rec2, uint32_t* ntiles, uint32_t* cand,
+                                      float4* rec2, uint2* touched, uint32_t* cand,
                                       uint32_t* vis_bits, bool defer_colour, Counters* counters,
                                       cudaStream_t stream);
-cudaError_t launch_ranges_colour(const uint32_t* keys, int total_tiles, uint2* ranges,
-                                 uint32_t pair_capacity, const Views& views,
-                                 const rgs_gaussians& g, const uint32_t* list, int64_t vis_cap,
-                                 bool colour, float4* rec1, float4* rec2, Counters* counters,
-                                 cudaStream_t stream);
+cudaError_t launch_colour(const Views& views, const rgs_gaussians& g, const uint32_t* list,
+                          int64_t vis_cap, float4* rec1, float4* rec2, Counters* counters,
+                          cudaStream_t stream);
 int preprocess_backward_blocks(int64_t vn);
 cudaError_t launch_preprocess_backward(const Views& views, const Consts& c,
                                        const rgs_gaussians& g, unsigned long long* vis_mask,
@@ -42,22 +39,27 @@ cudaError_t launch_preprocess_backward(const Views& views, const Consts& c,
                                        float* d_means, float* d_log_scales, float* d_quats,
                                        float* d_logits, float* d_sh, float* pose_partial,
                                        float* d_pose, const MapReg* reg, cudaStream_t stream);
-cudaError_t launch_duplicate(const Views& views, int n, const uint32_t* order,
-                             const uint32_t* offsets, const uint32_t* ntiles, const float4* rec0,
-                             const float4* rec1, const float4* rec2, float log2_alpha_min,
-                             int64_t visible_cap, uint32_t capacity,
-                             uint32_t* keys, uint32_t* vals, Counters* counters,
-                             cudaStream_t stream);
+int64_t max_emit_blocks(int64_t visible);
+int order_words();
+cudaError_t launch_emit_cells(const Views& views, int n, const uint32_t* order,
+                              const uint2* touched, const float4* rec0, const float4* rec1,
+                              float log2_alpha_min, int64_t visible_cap, uint32_t capacity,
+                              uint32_t* keys, uint32_t* vals, Lookback lb, Counters* counters,
+                              cudaStream_t stream);
+cudaError_t launch_cell_ranges(const Views& views, const uint32_t* keys, int64_t n_keys,
+                               uint2* ranges, const Counters* counters, cudaStream_t stream);
+cudaError_t launch_tile_lists(const Views& views, const uint2* cell_ranges, const uint32_t* keys,
+                              const uint32_t* vals, const float4* rec0, const float4* rec1,
+                              float log2_alpha_min, uint32_t* tile_counts, uint2* ranges,
+                              uint32_t* pairs, uint32_t capacity, uint32_t* order_words,
+                              uint32_t* tile_order, Lookback lb, Counters* counters,
+                              cudaStream_t stream);
 cudaError_t launch_blend(bool forward, const Views& views, const Consts& c, const uint2* ranges,
                          const uint32_t* pair_vals, const float4* rec0, const float4* rec1,
                          const float4* rec2, float* color, float* depth, float* alpha,
                          float* t_final, int32_t* last_index, const float* d_color,
                          const float* d_depth, const float* d_alpha, float* g2d,
                          const uint32_t* tile_order, Counters* counters, cudaStream_t stream);
-cudaError_t launch_tile_order(const uint2* ranges, int total_tiles, uint32_t* keys,
-                              uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
-                              uint32_t* hist, uint32_t* block_sums, const uint32_t** order,
-                              cudaStream_t stream);
 }  // namespace rgs
 
 using namespace rgs;
@@ -85,17 +87,17 @@ struct State {
   bool has_forward = false;
 
   // Capacities and regions.
-  int64_t vn_cap = 0, n_cap = 0, pix_cap = 0, tile_cap = 0, pair_cap = 0, pose_cap = 0;
+  int64_t vn_cap = 0, n_cap = 0, pix_cap = 0, tile_cap = 0, cell_cap = 0, pair_cap = 0,
+          pose_cap = 0;
   // Sorted-list capacity for the visible entries (not an allocation: the buffers hold vn_cap
-  // entries); the depth sort, the offsets scan and the duplication are sized by it.
+  // entries); the depth sort and the emission are sized by it.
   int64_t vis_cap = 0;
-  Region r_vn, r_n, r_pix, r_tile, r_pair, r_scratch, r_pose, r_counters;
+  Region r_vn, r_n, r_pix, r_tile, r_cell, r_pair, r_scratch, r_pose, r_counters;
 
   // Per (view, Gaussian).
   float4 *rec0 = nullptr, *rec1 = nullptr, *rec2 = nullptr;
-  uint32_t* ntiles = nullptr;
+  uint2* touched = nullptr;  // (tiles, cells)
   uint32_t *vis_keys[2] = {nullptr, nullptr}, *vis_vals[2] = {nullptr, nullptr};
-  uint32_t* offsets = nullptr;
   // The visible entries in (view, Gaussian) order (the compaction's output, kept past the depth
   // sort): the colour pass and the backward's per-entry pass walk it, so that neighbouring
   // threads read neighbouring Gaussians and mostly share a view.
@@ -112,11 +114,10 @@ struct State {
   float* t_final = nullptr;
   int32_t* last_index = nullptr;
   uint2* ranges = nullptr;
-  // Launch order of the blends' tiles (longest run first) and the buffers of its sort.
-  uint32_t *tile_keys[2] = {nullptr, nullptr}, *tile_vals[2] = {nullptr, nullptr};
-  const uint32_t* tile_order = nullptr;
-  uint32_t *pair_keys[2] = {nullptr, nullptr}, *pair_vals[2] = {nullptr, nullptr};
-  const uint32_t* sorted_vals = nullptr;
+  uint32_t* tile_counts = nullptr;
+  uint32_t* tile_order = nullptr;  // launch order of the blends' tiles (longest run first)
+  uint32_t *cell_keys[2] = {nullptr, nullptr}, *cell_vals[2] = {nullptr, nullptr};
+  uint32_t* pairs = nullptr;
   // Scratch.
   uint32_t* hist = nullptr;
   uint32_t* block_sums = nullptr;
@@ -139,8 +140,8 @@ struct State {
   bool open = false, captured = false;
 
   size_t bytes() const {
-    return r_vn.bytes + r_n.bytes + r_pix.bytes + r_tile.bytes + r_pair.bytes + r_scratch.bytes +
-           r_pose.bytes + r_counters.bytes;
+    return r_vn.bytes + r_n.bytes + r_pix.bytes + r_tile.bytes + r_cell.bytes + r_pair.bytes +
+           r_scratch.bytes + r_pose.bytes + r_counters.bytes;
   }
 };
 
@@ -250,12 +251,15 @@ bool is_capturing(cudaStream_t s) {
   return st != cudaStreamCaptureStatusNone;
 }
 
+// Cell sorts of up to this many entries take blocks of 1024 instead of 2048 keys: below it the
+// larger blocks leave SMs without one.
+constexpr int64_t kSmallBlockSort = 512 * 1024;
+
 // Scratch for the scans and sorts of up to `items` elements.
 rgs_status ensure_scratch(rgs_ctx* ctx, State& s, int64_t items, bool capturing) {
-  // The depth sort and the sort of the tiles' launch order run with small blocks over the
-  // per-Gaussian and tile capacities, the tile sort with large blocks over the pair capacity;
+  // The depth sort and small cell sorts run with small blocks, larger cell sorts with large ones;
   // the table must fit each.
-  const int64_t small = std::max<int64_t>(std::max(s.vn_cap, s.tile_cap), 1);
+  const int64_t small = std::max<int64_t>(std::max(s.vn_cap, std::min(items, kSmallBlockSort)), 1);
   const int64_t hist = std::max(sort_hist_entries(small, kSortItemsSmall),
                                 sort_hist_entries(std::max<int64_t>(items, 1)));
   const int64_t sums = std::max(scan_blocks(hist), scan_blocks(std::max<int64_t>(items, 1))) + 1;
@@ -287,7 +291,8 @@ rgs_status ensure_vn(rgs_ctx* ctx, State& s, int64_t vn, int64_t n, int64_t pose
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "per-Gaussian buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
     const int64_t cap = vn;
-    size_t bytes = 3 * align_up(sizeof(float4) * cap) + 7 * align_up(sizeof(uint32_t) * cap) +
+    size_t bytes = 3 * align_up(sizeof(float4) * cap) + align_up(sizeof(uint2) * cap) +
+                   5 * align_up(sizeof(uint32_t) * cap) +
                    align_up(sizeof(float) * kG2Stride * cap) +
                    align_up(sizeof(uint32_t) * vis_bit_words_cap(cap));
     RGS_CUDA(alloc_region(ctx, s.r_vn, bytes), "allocate per-Gaussian buffers");
@@ -295,12 +300,11 @@ rgs_status ensure_vn(rgs_ctx* ctx, State& s, int64_t vn, int64_t n, int64_t pose
     s.rec0 = carve<float4>(p, cap);
     s.rec1 = carve<float4>(p, cap);
     s.rec2 = carve<float4>(p, cap);
-    s.ntiles = carve<uint32_t>(p, cap);
+    s.touched = carve<uint2>(p, cap);
     s.vis_keys[0] = carve<uint32_t>(p, cap);
     s.vis_keys[1] = carve<uint32_t>(p, cap);
     s.vis_vals[0] = carve<uint32_t>(p, cap);
     s.vis_vals[1] = carve<uint32_t>(p, cap);
-    s.offsets = carve<uint32_t>(p, cap);
     s.vis_list = carve<uint32_t>(p, cap);
     s.g2d = carve<float>(p, kG2Stride * cap);
     s.vis_bits = carve<uint32_t>(p, vis_bit_words_cap(cap));
@@ -335,31 +339,46 @@ rgs_status ensure_pix_tiles(rgs_ctx* ctx, State& s, int64_t pixels, int64_t tile
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "tile buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
     RGS_CUDA(alloc_region(ctx, s.r_tile, align_up(sizeof(uint2) * tiles) +
-                                         4 * align_up(sizeof(uint32_t) * tiles)),
+                                         2 * align_up(sizeof(uint32_t) * tiles)),
              "allocate tile ranges");
     char* p = static_cast<char*>(s.r_tile.base);
     s.ranges = carve<uint2>(p, tiles);
-    s.tile_keys[0] = carve<uint32_t>(p, tiles);
-    s.tile_keys[1] = carve<uint32_t>(p, tiles);
-    s.tile_vals[0] = carve<uint32_t>(p, tiles);
-    s.tile_vals[1] = carve<uint32_t>(p, tiles);
+    s.tile_counts = carve<uint32_t>(p, tiles);
+    s.tile_order = carve<uint32_t>(p, tiles);
     s.tile_cap = tiles;
   }
   return RGS_OK;
 }
 
+// Capacity for `count` list entries: a quarter more than asked for.
+int64_t with_slack(int64_t count) { return std::max<int64_t>(count + count / 4, 4096); }
+
 rgs_status ensure_pairs(rgs_ctx* ctx, State& s, int64_t pairs) {
   if (pairs <= s.pair_cap) return RGS_OK;
-  RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
-  const int64_t cap = std::max<int64_t>(pairs + pairs / 4, 4096);
+  const int64_t cap = with_slack(pairs);
   if (cap >= (int64_t)UINT32_MAX) return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^32");
-  RGS_CUDA(alloc_region(ctx, s.r_pair, 4 * align_up(sizeof(uint32_t) * cap)), "allocate pair lists");
-  char* p = static_cast<char*>(s.r_pair.base);
-  s.pair_keys[0] = carve<uint32_t>(p, cap);
-  s.pair_keys[1] = carve<uint32_t>(p, cap);
-  s.pair_vals[0] = carve<uint32_t>(p, cap);
-  s.pair_vals[1] = carve<uint32_t>(p, cap);
+  RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
+  s.pair_cap = 0;
+  RGS_CUDA(alloc_region(ctx, s.r_pair, align_up(sizeof(uint32_t) * cap)), "allocate pair list");
+  s.pairs = static_cast<uint32_t*>(s.r_pair.base);
   s.pair_cap = cap;
+  return RGS_OK;
+}
+
+rgs_status ensure_cells(rgs_ctx* ctx, State& s, int64_t cells) {
+  if (cells <= s.cell_cap) return RGS_OK;
+  const int64_t cap = with_slack(cells);
+  if (cap >= (int64_t)UINT32_MAX) return fail(ctx, RGS_ERR_INVALID_ARG, "cell list exceeds 2^32");
+  RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
+  s.cell_cap = 0;
+  RGS_CUDA(alloc_region(ctx, s.r_cell, 4 * align_up(sizeof(uint32_t) * cap)),
+           "allocate cell lists");
+  char* p = static_cast<char*>(s.r_cell.base);
+  s.cell_keys[0] = carve<uint32_t>(p, cap);
+  s.cell_keys[1] = carve<uint32_t>(p, cap);
+  s.cell_vals[0] = carve<uint32_t>(p, cap);
+  s.cell_vals[1] = carve<uint32_t>(p, cap);
+  s.cell_cap = cap;
   return RGS_OK;
 }
 
@@ -427,6 +446,7 @@ void destroy_state(State* s) {
   free_region(s->r_n);
   free_region(s->r_pix);
   free_region(s->r_tile);
+  free_region(s->r_cell);
   free_region(s->r_pair);
   free_region(s->r_scratch);
   free_region(s->r_pose);
@@ -479,7 +499,7 @@ rgs_status build_views(rgs_ctx* ctx, const rgs_camera* cams, int n_views, const 
   views.pixels_per_thread = ppt;
   views.bwd_pixels_per_thread = bwd_ppt;
   long long pix = 0;
-  long long tiles = 0;
+  long long tiles = 0, cells = 0;
   for (int v = 0; v < n_views; ++v) {
     const rgs_camera& c = cams[v];
     if (c.width < 1 || c.height < 1 || c.width > 16384 || c.height > 16384)
@@ -495,6 +515,8 @@ rgs_status build_views(rgs_ctx* ctx, const rgs_camera* cams, int n_views, const 
     vp.tiles_x = (c.width + tw - 1) / tw;
     vp.tiles_y = (c.height + th - 1) / th;
     vp.tile_base = (int)tiles;
+    vp.cells_x = (vp.tiles_x + kCellTiles - 1) / kCellTiles;
+    vp.cell_base = (int)cells;
     vp.pixel_offset = pix;
     vp.fx = c.fx;
     vp.fy = c.fy;
@@ -516,11 +538,13 @@ rgs_status build_views(rgs_ctx* ctx, const rgs_camera* cams, int n_views, const 
       vp.lim_u = vp.lim_w = 0.0f;
     }
     tiles += (long long)vp.tiles_x * vp.tiles_y;
+    cells += (long long)vp.cells_x * ((vp.tiles_y + kCellTiles - 1) / kCellTiles);
     pix += (long long)c.width * c.height;
   }
   if (tiles >= (1ll << 31) || pix >= (1ll << 31))
     return fail(ctx, RGS_ERR_INVALID_ARG, "too many pixels or tiles in one batch");
   views.total_tiles = (int)tiles;
+  views.total_cells = (int)cells;
   views.total_pixels = pix;
   consts.alpha_min = cfg.alpha_min;
   consts.alpha_max = cfg.alpha_max;
@@ -787,9 +811,11 @@ rgs_status rgs_reserve(rgs_ctx* ctx, uint64_t* handle, int64_t pair_capacity, vo
   if (st != RGS_OK) return st;
   cudaSetDevice(ctx->device);
   if (pair_capacity > 0) {
+    // No footprint has more cell entries than pairs, but for the few cells a thin one skips over.
     st = ensure_pairs(ctx, *s, pair_capacity);
+    if (st == RGS_OK) st = ensure_cells(ctx, *s, pair_capacity);
     if (st != RGS_OK) return st;
-    st = ensure_scratch(ctx, *s, std::max<int64_t>(s->pair_cap, s->vn_cap), false);
+    st = ensure_scratch(ctx, *s, std::max<int64_t>(s->cell_cap, s->vn_cap), false);
     if (st != RGS_OK) return st;
   }
   return RGS_OK;
@@ -860,13 +886,20 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
   if (st != RGS_OK) return st;
   st = ensure_pix_tiles(ctx, *s, views.total_pixels, views.total_tiles, capturing);
   if (st != RGS_OK) return st;
-  st = ensure_scratch(ctx, *s, std::max<int64_t>(vn, s->pair_cap), capturing);
+  st = ensure_scratch(ctx, *s, std::max<int64_t>(vn, s->cell_cap), capturing);
   if (st != RGS_OK) return st;
-  // Pose records, then the counters and the bookkeeping of the two single-pass scans (the
-  // compaction and the pair offsets), which one memset zeroes at the start of every forward.
+  // Pose records, then what one memset zeroes at the start of every forward: the counters, the
+  // bookkeeping of the three single-pass scans (compaction, emission, tile runs), the sizes of the
+  // launch order's classes, and the cell ranges (cells without entries keep [0, 0)).
   const size_t pose_bytes = align_up(sizeof(float) * 16 * kMaxViews);
-  const size_t lb_bytes = align_up(lookback_bytes(s->vn_cap));
-  const size_t reset_bytes = align_up(sizeof(Counters)) + 2 * lb_bytes;
+  const int64_t emit_items = max_emit_blocks(vn) * kScanTile;  // a look-back area counts kScanTile each
+  const size_t lb_bytes = align_up(lookback_bytes(vn));
+  const size_t lb_emit_bytes = align_up(lookback_bytes(emit_items));
+  const size_t lb_tile_bytes = align_up(lookback_bytes(views.total_tiles));
+  const size_t order_bytes = align_up(sizeof(uint32_t) * order_words());
+  const size_t reset_bytes = align_up(sizeof(Counters)) + lb_bytes + lb_emit_bytes +
+                             lb_tile_bytes + order_bytes +
+                             align_up(sizeof(uint2) * (size_t)views.total_cells);
   if (s->r_counters.bytes < pose_bytes + reset_bytes) {
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "counters grow during capture");
     if (s->r_counters.base) RGS_CUDA(cudaDeviceSynchronize(), "sync before counters growth");
@@ -875,6 +908,10 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
   s->pose_records = static_cast<float*>(s->r_counters.base);
   s->counters = reinterpret_cast<Counters*>(static_cast<char*>(s->r_counters.base) + pose_bytes);
   char* lb_area = reinterpret_cast<char*>(s->counters) + align_up(sizeof(Counters));
+  char* lb_emit = lb_area + lb_bytes;
+  char* lb_tile = lb_emit + lb_emit_bytes;
+  uint32_t* order_state = reinterpret_cast<uint32_t*>(lb_tile + lb_tile_bytes);
+  uint2* cell_ranges = reinterpret_cast<uint2*>(lb_tile + lb_tile_bytes + order_bytes);
   if (world_to_cam) views.pose_dev = s->pose_records;
   s->g = *g;
   s->views = views;
@@ -884,9 +921,6 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
   const uint64_t launches0 = launch_counter();
   s->fwd_timed = ctx->timing;
   RGS_CUDA(cudaMemsetAsync(cnt, 0, reset_bytes, stream), "reset counters");
-  // Tiles without pairs keep the empty range [0, 0); the range kernel writes the others.
-  RGS_CUDA(cudaMemsetAsync(s->ranges, 0, sizeof(uint2) * (size_t)views.total_tiles, stream),
-           "reset tile ranges");
   RGS_CUDA(mark(ctx, *s, 0, stream, capturing), "event");
   // Device poses: records (R, t, camera centre) for the projection kernels and the backward.
   if (world_to_cam)
@@ -898,28 +932,44 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
   // The colours are evaluated in the projection, unless the caller's SH coefficients may still
   // be in flight: then after the sorts, behind the caller's event.
   const bool defer_colour = cfg.sh_ready_event != nullptr;
-  RGS_CUDA(launch_preprocess_forward(views, consts, *g, s->rec0, s->rec1, s->rec2, s->ntiles,
+  RGS_CUDA(launch_preprocess_forward(views, consts, *g, s->rec0, s->rec1, s->rec2, s->touched,
                                      s->vis_keys[1], s->vis_bits, defer_colour, cnt, stream),
            "preprocess");
   RGS_CUDA(mark(ctx, *s, 1, stream, capturing), "event");
-  // 2. Visible entries with depth keys, in (view, Gaussian) order.
-  RGS_CUDA(launch_compact_visible(s->vis_bits, n_views, g->n, s->rec2, s->vis_keys[0],
-                                  s->vis_vals[0], s->vis_list, &cnt->n_visible,
-                                  lookback_at(lb_area, &cnt->status, s->vn_cap), stream),
-           "compact");
-  RGS_CUDA(mark(ctx, *s, 2, stream, capturing), "event");
-  // Size the sorted list of visible entries (outside capture: the count itself, read back; under
-  // capture the capacity of the last eager call holds, and a larger count is clamped to it and
-  // recorded in the status word).
-  int64_t vis_cap = 0;
+  // Outside capture the lists are sized by the projection's totals, which the host waits for
+  // while the compaction runs.
   if (!capturing) {
     RGS_CUDA(cudaMemcpyAsync(ctx->host_counters, cnt, sizeof(Counters), cudaMemcpyDeviceToHost,
                              stream),
              "read counters");
-    RGS_CUDA(cudaStreamSynchronize(stream), "sync for visible count");
-    vis_cap = ctx->host_counters->n_visible;
+    RGS_CUDA(cudaEventRecord(s->done, stream), "event");
+  }
+  // 2. Visible entries with depth keys, in (view, Gaussian) order.
+  RGS_CUDA(launch_compact_visible(s->vis_bits, n_views, g->n, s->rec2, s->vis_keys[0],
+                                  s->vis_vals[0], s->vis_list, &cnt->n_visible,
+                                  lookback_at(lb_area, &cnt->status, vn), stream),
+           "compact");
+  RGS_CUDA(mark(ctx, *s, 2, stream, capturing), "event");
+  // The sorted list of visible entries, the cell list and the pair list. Under capture the
+  // capacities of the last eager call hold, and a larger count is clamped to them and recorded in
+  // the status word.
+  int64_t vis_cap = 0, n_cells = s->cell_cap;
+  if (!capturing) {
+    RGS_CUDA(cudaEventSynchronize(s->done), "wait for the projection's counts");
+    const Counters& c = *ctx->host_counters;
+    if (c.all_pairs >= UINT32_MAX || c.all_cells >= UINT32_MAX)
+      return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^32");
+    vis_cap = (int64_t)c.all_visible;
     if (vis_cap > s->vis_cap) s->vis_cap = std::max<int64_t>(vis_cap + vis_cap / 4, 1024);
+    n_cells = (int64_t)c.all_cells;
+    st = ensure_pairs(ctx, *s, (int64_t)c.all_pairs);
+    if (st == RGS_OK) st = ensure_cells(ctx, *s, n_cells);
+    if (st == RGS_OK) st = ensure_scratch(ctx, *s, std::max<int64_t>(vn, s->cell_cap), false);
+    if (st != RGS_OK) return st;
   } else {
+    if (s->pair_cap == 0 || s->cell_cap == 0)
+      return fail(ctx, RGS_ERR_CAPACITY,
+                  "pair list has no capacity under capture: rgs_reserve");
     if (s->vis_cap == 0) s->vis_cap = vn;
     vis_cap = std::min<int64_t>(s->vis_cap, vn);
   }
@@ -931,65 +981,45 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
            "depth sort");
   s->order = s->vis_vals[alt ? 1 : 0];
   RGS_CUDA(mark(ctx, *s, 3, stream, capturing), "event");
-  // 4. Pair offsets in depth order.
-  RGS_CUDA(launch_gather_scan(s->ntiles, s->order, vis_cap, &cnt->n_visible, s->offsets,
-                              &cnt->n_pairs, s->block_sums,
-                              lookback_at(lb_area + lb_bytes, &cnt->status, s->vn_cap), stream),
-           "pair offsets");
   RGS_CUDA(mark(ctx, *s, 4, stream, capturing), "event");
-  // Size the pair list (outside capture: read the count back and grow if needed).
-  int64_t pair_bound = s->pair_cap;
-  if (!capturing) {
-    RGS_CUDA(cudaMemcpyAsync(ctx->host_counters, cnt, sizeof(Counters), cudaMemcpyDeviceToHost,
-                             stream),
-             "read counters");
-    RGS_CUDA(cudaStreamSynchronize(stream), "sync for pair count");
-    const int64_t pairs = ctx->host_counters->n_pairs;
-    st = ensure_pairs(ctx, *s, pairs);
-    if (st != RGS_OK) return st;
-    st = ensure_scratch(ctx, *s, std::max<int64_t>(vn, s->pair_cap), false);
-    if (st != RGS_OK) return st;
-    pair_bound = pairs;
-  } else if (s->pair_cap == 0) {
-    return fail(ctx, RGS_ERR_CAPACITY, "pair list has no capacity under capture: rgs_reserve");
-  }
-  const uint32_t capacity = (uint32_t)s->pair_cap;
-  // 5. Duplicate (tile, vi) pairs in depth order.
-  RGS_CUDA(launch_duplicate(views, g->n, s->order, s->offsets, s->ntiles, s->rec0, s->rec1,
-                            s->rec2, consts.log2_alpha_min, vis_cap, capacity, s->pair_keys[0],
-                            s->pair_vals[0], cnt, stream),
-           "duplicate");
+  const uint32_t pair_cap = (uint32_t)s->pair_cap;
+  // 4. Cell entries in depth order.
+  RGS_CUDA(launch_emit_cells(views, g->n, s->order, s->touched, s->rec0, s->rec1,
+                             consts.log2_alpha_min, vis_cap, (uint32_t)s->cell_cap,
+                             s->cell_keys[0], s->cell_vals[0],
+                             lookback_at(lb_emit, &cnt->status, emit_items), cnt, stream),
+           "emit cells");
   RGS_CUDA(mark(ctx, *s, 5, stream, capturing), "event");
-  // 6. Stable sort by global tile id.
+  // 5. Stable sort by cell. The ids are [0, total_cells]; total_cells itself marks an unused slot.
   alt = false;
-  // Keys are tile ids in [0, total_tiles]; total_tiles itself marks an unused slot.
-  const int tile_bits = bits_for((uint32_t)views.total_tiles + 1u);
-  RGS_CUDA(launch_radix_sort(s->pair_keys[0], s->pair_vals[0], s->pair_keys[1], s->pair_vals[1],
-                             std::min<int64_t>(pair_bound, s->pair_cap), &cnt->n_pairs_stored, 0,
-                             tile_bits, s->hist, s->block_sums, &alt, stream),
-           "tile sort");
-  const uint32_t* sorted_keys = s->pair_keys[alt ? 1 : 0];
-  s->sorted_vals = s->pair_vals[alt ? 1 : 0];
+  const int cell_bits = bits_for((uint32_t)views.total_cells + 1u);
+  const int key_shift = cells_masked(views.total_cells) ? 16 : 0;
+  RGS_CUDA(launch_radix_sort(s->cell_keys[0], s->cell_vals[0], s->cell_keys[1], s->cell_vals[1],
+                             n_cells, &cnt->n_cells_stored, key_shift, key_shift + cell_bits,
+                             s->hist, s->block_sums, &alt, stream,
+                             n_cells <= kSmallBlockSort ? kSortItemsSmall : kSortItems),
+           "cell sort");
+  const uint32_t* keys = s->cell_keys[alt ? 1 : 0];
+  const uint32_t* vals = s->cell_vals[alt ? 1 : 0];
   RGS_CUDA(mark(ctx, *s, 6, stream, capturing), "event");
-  // 7. Tile ranges.
-  // Tile ranges and, when deferred, the colours of the visible entries, in one launch: the
-  // colours are then the first read of the SH coefficients, so the caller's upload of them may
-  // run until here.
-  if (defer_colour)
+  // 6. The tiles' lists, their ranges and launch order.
+  RGS_CUDA(launch_cell_ranges(views, keys, n_cells, cell_ranges, cnt, stream), "cell ranges");
+  RGS_CUDA(launch_tile_lists(views, cell_ranges, keys, vals, s->rec0, s->rec1,
+                             consts.log2_alpha_min, s->tile_counts, s->ranges, s->pairs, pair_cap,
+                             order_state, s->tile_order,
+                             lookback_at(lb_tile, &cnt->status, views.total_tiles), cnt, stream),
+           "tile lists");
+  // With an SH event, the colours of the visible entries: the first read of the SH coefficients,
+  // so the caller's upload of them may run until here.
+  if (defer_colour) {
     RGS_CUDA(cudaStreamWaitEvent(stream, static_cast<cudaEvent_t>(cfg.sh_ready_event), 0),
              "wait for the SH coefficients");
-  RGS_CUDA(launch_ranges_colour(sorted_keys, views.total_tiles, s->ranges,
-                                (uint32_t)std::min<int64_t>(pair_bound, s->pair_cap), views, *g,
-                                s->vis_list, vis_cap, defer_colour, s->rec1, s->rec2, cnt,
-                                stream),
-           "tile ranges and colours");
-  RGS_CUDA(launch_tile_order(s->ranges, views.total_tiles, s->tile_keys[0], s->tile_vals[0],
-                             s->tile_keys[1], s->tile_vals[1], s->hist, s->block_sums,
-                             &s->tile_order, stream),
-           "tile order");
+    RGS_CUDA(launch_colour(views, *g, s->vis_list, vis_cap, s->rec1, s->rec2, cnt, stream),
+             "colours");
+  }
   RGS_CUDA(mark(ctx, *s, 7, stream, capturing), "event");
-  // 8. Blend.
-  RGS_CUDA(launch_blend(true, views, consts, s->ranges, s->sorted_vals, s->rec0, s->rec1,
+  // 7. Blend.
+  RGS_CUDA(launch_blend(true, views, consts, s->ranges, s->pairs, s->rec0, s->rec1,
                         s->rec2, out->color, out->depth, out->alpha, s->t_final, s->last_index,
                         nullptr, nullptr, nullptr, nullptr, s->tile_order, cnt, stream),
            "blend forward");
@@ -1086,7 +1116,7 @@ rgs_status render_backward(rgs_ctx* ctx, uint64_t handle, const rgs_image_grads*
   open_state(*s, capturing);
   s->bwd_timed = ctx->timing;
   RGS_CUDA(mark(ctx, *s, kEvBwd0, stream, capturing), "event");
-  RGS_CUDA(launch_blend(false, s->views, s->consts, s->ranges, s->sorted_vals, s->rec0, s->rec1,
+  RGS_CUDA(launch_blend(false, s->views, s->consts, s->ranges, s->pairs, s->rec0, s->rec1,
                         s->rec2, nullptr, nullptr, nullptr, s->t_final, s->last_index, dc, dd, da,
                         s->g2d, s->tile_order, s->counters, stream),
            "blend backward");
@@ -1146,9 +1176,8 @@ rgs_status rgs_query_stats(rgs_ctx* ctx, uint64_t handle, rgs_stats* out, void* 
   RGS_CUDA(cudaStreamSynchronize(stream), "sync for stats");
   const Counters& c = *ctx->host_counters;
   out->n_visible = c.n_visible;
-  out->n_pairs = c.n_pairs;
+  out->n_pairs = (int64_t)c.n_pairs;
   out->n_eval = (int64_t)c.n_eval;
-  out->n_contrib = (int64_t)c.n_contrib;
   out->n_nonfinite = c.n_nonfinite;
   out->status = c.status;
   out->kernel_launches = s->fwd_launches + s->bwd_launches;
@@ -1167,10 +1196,10 @@ rgs_status rgs_copy_tile_lists(rgs_ctx* ctx, uint64_t handle, uint32_t* host_val
                            cudaMemcpyDeviceToHost, stream),
            "read counters");
   RGS_CUDA(cudaStreamSynchronize(stream), "sync");
-  const int64_t np = ctx->host_counters->n_pairs_stored;
+  const int64_t np = std::min<int64_t>(ctx->host_counters->n_pairs_listed, s->pair_cap);
   *n_pairs = np;
   if (host_vals && np <= vals_cap && np > 0)
-    RGS_CUDA(cudaMemcpyAsync(host_vals, s->sorted_vals, sizeof(uint32_t) * np,
+    RGS_CUDA(cudaMemcpyAsync(host_vals, s->pairs, sizeof(uint32_t) * np,
                              cudaMemcpyDeviceToHost, stream),
              "copy pair list");
   if (host_ranges && s->views.total_tiles > 0)
@@ -1196,8 +1225,8 @@ rgs_status rgs_copy_records(rgs_ctx* ctx, uint64_t handle, float* host_rec,
                                  sizeof(float4), (size_t)vn, cudaMemcpyDeviceToHost, stream),
                "copy records");
     if (host_ntiles)
-      RGS_CUDA(cudaMemcpyAsync(host_ntiles, s->ntiles, sizeof(uint32_t) * vn,
-                               cudaMemcpyDeviceToHost, stream),
+      RGS_CUDA(cudaMemcpy2DAsync(host_ntiles, sizeof(uint32_t), s->touched, sizeof(uint2),
+                                 sizeof(uint32_t), (size_t)vn, cudaMemcpyDeviceToHost, stream),
                "copy tile counts");
   }
   std::vector<uint32_t> bits;

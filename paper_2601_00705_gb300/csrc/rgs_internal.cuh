@@ -7,12 +7,14 @@
 //   rec1[vi] = (l11, l21, l22, log2 o)                    float4, lower-triangular factor of the
 //              base-2-scaled conic (see below)
 //   rec2[vi] = (r, g, b, depth z)                          float4
-//   ntiles[vi]: tiles touched (0 = culled / invisible)
+//   touched[vi] = (tiles, cells) touched (0 = culled / invisible)
 //   g2d[vi * 16 + s]: the backward blend's sums over the covered pixels of dL/dpower moments
 //              and of the colour / depth weights (see G2Slot), reused by the backward
 //              preprocess for its per-view intermediate results
-//   pair list: key = global tile id, value = vi; sorted so that each tile's run is in
-//              (depth, index) order; ranges[gtile] = [first, last + 1) of the run.
+//   cells: blocks of kCellTiles x kCellTiles tiles. The cell list holds one (cell, tile mask; vi)
+//              entry per touched cell, sorted so that each cell's run is in (depth, index) order
+//   pair list: the vi of every (tile, Gaussian) pair, tile by tile, each tile's run in (depth,
+//              index) order; ranges[gtile] = [first, last + 1) of the run.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -41,6 +43,8 @@ struct ViewParams {
   int width, height;
   int tiles_x, tiles_y;
   int tile_base;            // first global tile id of this view
+  int cell_base;            // first global cell id of this view
+  int cells_x;
   int pad0;
   long long pixel_offset;   // first pixel of this view in the concatenated images
   float fx, fy, cx, cy;
@@ -55,6 +59,8 @@ struct ViewParams {
 struct Views {
   int n_views;
   int total_tiles;
+  int total_cells;
+  int pad0;
   long long total_pixels;
   int tile_w, tile_h;
   int pixels_per_thread;    // vertically adjacent pixels per forward-blend thread
@@ -113,15 +119,17 @@ enum StatusBits : uint32_t {
 // Device counters of one forward.
 struct Counters {
   uint32_t n_visible;       // compacted (view, Gaussian) entries
-  uint32_t n_pairs;         // duplicated pairs
-  uint32_t n_pairs_stored;  // min(n_pairs, capacity)
+  uint32_t n_visible_kept;  // min(n_visible, visible-list capacity): the entries sorted and used
   uint32_t status;
   uint32_t n_nonfinite;
   uint32_t n_candidates;    // entries the cull pass keeps for full projection
-  uint32_t n_visible_kept;  // min(n_visible, visible-list capacity): the entries sorted and used
-  uint32_t pad;
+  uint32_t n_cells;         // (cell, entry) list entries of the kept visible entries
+  uint32_t n_cells_stored;  // min(n_cells, cell-list capacity)
+  uint32_t n_pairs_listed;  // pairs of the stored cell entries (the pair list's length, unclipped)
+  unsigned long long n_pairs;    // pairs of the kept visible entries
   unsigned long long n_eval;     // (pixel, Gaussian) positions the forward blend visited
-  unsigned long long n_contrib;  // reserved (0): composites are not counted
+  // Totals of the projection, before any capacity: what the host sizes the lists by.
+  unsigned long long all_visible, all_cells, all_pairs;
 };
 
 // Programmatic dependent launch. Every kernel of the library is launched with programmatic
@@ -167,6 +175,15 @@ __device__ __forceinline__ int view_of_tile(const Views& views, int gtile) {
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
     if (views.v[mid].tile_base <= gtile) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+__device__ __forceinline__ int view_of_cell(const Views& views, int cell) {
+  int lo = 0, hi = views.n_views - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (views.v[mid].cell_base <= cell) lo = mid; else hi = mid - 1;
   }
   return lo;
 }
@@ -405,24 +422,24 @@ struct TileCover {
     return true;
   }
 
-  // The cover set up by lane src of the warp, in every lane (all lanes must call it).
-  __device__ __forceinline__ TileCover broadcast(int src) const {
+  // The cover set up by lane src of the warp, one lane per caller (all lanes must call it).
+  __device__ __forceinline__ TileCover from_lane(int src, int tw, int th) const {
     TileCover o;
     const unsigned m = 0xffffffffu;
+    o.tile_w = tw;
+    o.tile_h = th;
+    o.inv_tw = 1.0f / (float)tw;
     o.ty0 = __shfl_sync(m, ty0, src);
     o.ty1 = __shfl_sync(m, ty1, src);
     o.bx0 = __shfl_sync(m, bx0, src);
     o.bx1 = __shfl_sync(m, bx1, src);
-    o.box_only = __shfl_sync(m, (int)box_only, src) != 0;
-    o.tile_w = __shfl_sync(m, tile_w, src);
-    o.tile_h = __shfl_sync(m, tile_h, src);
+    o.box_only = o.ty0 == o.ty1 || o.bx0 == o.bx1;
     o.tiles_x = __shfl_sync(m, tiles_x, src);
     o.mx = __shfl_sync(m, mx, src);
     o.my = __shfl_sync(m, my, src);
     o.kap = __shfl_sync(m, kap, src);
     o.rx = __shfl_sync(m, rx, src);
     o.ry = __shfl_sync(m, ry, src);
-    o.inv_tw = __shfl_sync(m, inv_tw, src);
     o.x_lo = __shfl_sync(m, x_lo, src);
     o.x_hi = __shfl_sync(m, x_hi, src);
     o.inv_syy = __shfl_sync(m, inv_syy, src);
@@ -473,15 +490,61 @@ struct TileCover {
   }
 };
 
-template <typename RowFn>
-__device__ __forceinline__ void for_each_tile_row(const Ellipse& e, int tile_w, int tile_h,
-                                                  int tiles_x, int tiles_y, RowFn&& fn) {
-  TileCover tc;
-  if (!tc.init(e, tile_w, tile_h, tiles_x, tiles_y)) return;
-  for (int ty = tc.ty0; ty <= tc.ty1; ++ty) {
-    int tx0, tx1;
-    if (tc.span(ty, tx0, tx1)) fn(ty, tx0, tx1);
+// ------------------------------------------------------------------------------------------
+// Cells: blocks of 4 x 4 tiles. A footprint's cover is listed per cell with a 16-bit mask of the
+// tiles it touches there (bit 4 row + column).
+// ------------------------------------------------------------------------------------------
+constexpr int kCellTiles = 4;
+constexpr int kCellShift = 2;  // log2 kCellTiles
+
+// One row of cells: the column spans of its tile rows, packed first | last << 16 (an untouched row
+// has first > last), and the cells [c0, c1] between the leftmost and the rightmost touched tile.
+// A cell inside may be empty (a thin diagonal footprint jumps ahead between two pixel rows).
+struct CellRow {
+  uint32_t span[kCellTiles];
+  int c0, c1;
+};
+// False when no tile of cell row cy is touched.
+__device__ __forceinline__ bool cell_row(const TileCover& tc, int cy, CellRow& out) {
+  int lo = 0x7fffffff, hi = -1;
+#pragma unroll
+  for (int r = 0; r < kCellTiles; ++r) {
+    const int ty = cy * kCellTiles + r;
+    int tx0 = 0, tx1 = -1;
+    out.span[r] = 0x0000ffffu;
+    if (ty >= tc.ty0 && ty <= tc.ty1 && tc.span(ty, tx0, tx1)) {
+      out.span[r] = (uint32_t)tx0 | ((uint32_t)tx1 << 16);
+      lo = min(lo, tx0);
+      hi = max(hi, tx1);
+    }
   }
+  out.c0 = lo >> kCellShift;
+  out.c1 = hi >> kCellShift;
+  return hi >= 0;
+}
+// Tiles of a span (0 for an untouched row).
+__device__ __forceinline__ uint32_t span_tiles(uint32_t span) {
+  const int tx0 = (int)(span & 0xffffu), tx1 = (int)(span >> 16);
+  return tx0 <= tx1 ? (uint32_t)(tx1 - tx0 + 1) : 0u;
+}
+// Tile mask of cell column c in a cell row.
+__device__ __forceinline__ uint32_t cell_mask(const uint32_t (&span)[kCellTiles], int c) {
+  uint32_t mask = 0;
+#pragma unroll
+  for (int r = 0; r < kCellTiles; ++r) {
+    const int a = max((int)(span[r] & 0xffffu) - c * kCellTiles, 0);
+    const int b = min((int)(span[r] >> 16) - c * kCellTiles, kCellTiles - 1);
+    if (a <= b) mask |= ((2u << b) - (1u << a)) << (kCellTiles * r);
+  }
+  return mask;
+}
+
+// Cell-list keys carry the tile mask in their low 16 bits, which the sort by cell (the bits above)
+// moves along for nothing. Cell ids that do not fit in 16 bits (over 65,534 cells: more than 10^6
+// tiles) fill the whole key instead, and the mask is worked out again from the records.
+constexpr int kMaxMaskedCells = 65534;  // the next id marks unused slots
+inline __host__ __device__ bool cells_masked(int total_cells) {
+  return total_cells <= kMaxMaskedCells;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -547,10 +610,12 @@ cudaError_t launch_compact_visible(const uint32_t* vis_bits, int n_views, int n,
                                    uint32_t* list, uint32_t* n_out, Lookback lb,
                                    cudaStream_t stream);
 
-// offs[k] = exclusive scan of ntiles[order[k]] for k < *n_dev; total into *total.
-cudaError_t launch_gather_scan(const uint32_t* ntiles, const uint32_t* order, int64_t n_cap,
-                               const uint32_t* n_dev, uint32_t* offs, uint32_t* total,
-                               uint32_t* block_sums, Lookback lb, cudaStream_t stream);
+// ranges[t] = [first, last + 1) of tile t's run when tile t holds counts[t] pairs and the runs
+// follow each other in tile order, clipped to `capacity` pairs ([0, 0) for an empty tile); the
+// unclipped total into *total. One single-pass launch; lb must be zeroed.
+cudaError_t launch_tile_ranges_scan(const uint32_t* counts, uint2* ranges, int64_t n_tiles,
+                                    uint32_t capacity, uint32_t* total, Lookback lb,
+                                    cudaStream_t stream);
 
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;       // keys per thread for large sorts (2048 per block)

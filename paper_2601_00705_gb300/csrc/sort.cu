@@ -10,48 +10,12 @@
 #include <algorithm>
 #include <mutex>
 
-#include "rgs_internal.cuh"
+#include "scan_device.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace rgs {
 namespace {
-
-__device__ __forceinline__ uint32_t read_count(const uint32_t* n_dev, int64_t n_cap) {
-  if (!n_dev) return (uint32_t)n_cap;
-  const uint32_t n = *n_dev;
-  return n < (uint64_t)n_cap ? n : (uint32_t)n_cap;
-}
-
-// Block-wide exclusive scan of one value per thread; returns the block total in *total.
-template <int THREADS>
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
-  __shared__ uint32_t warp_sums[THREADS / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) warp_sums[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    uint32_t w = lane < THREADS / 32 ? warp_sums[lane] : 0u;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
-    }
-    if (lane < THREADS / 32) warp_sums[lane] = w;  // inclusive warp prefix
-  }
-  __syncthreads();
-  const uint32_t warp_prefix = warp > 0 ? warp_sums[warp - 1] : 0u;
-  if (total) *total = warp_sums[THREADS / 32 - 1];
-  const uint32_t r = warp_prefix + x - v;
-  __syncthreads();  // warp_sums may be reused by the caller's next scan
-  return r;
-}
 
 // Lanes of the warp whose valid keys carry the same digit as this lane's (0 for an invalid
 // lane): one ballot per digit bit, each keeping the lanes that agree on that bit.
@@ -69,11 +33,6 @@ __device__ __forceinline__ uint32_t warp_digit_peers(uint32_t digit, bool valid,
 struct PlainLoad {
   const uint32_t* in;
   __device__ uint32_t operator()(uint32_t k) const { return in[k]; }
-};
-struct GatherLoad {
-  const uint32_t* in;
-  const uint32_t* order;
-  __device__ uint32_t operator()(uint32_t k) const { return in[order[k]]; }
 };
 
 // Pass 1: per-block sums.
@@ -131,6 +90,16 @@ struct PlainStore {
   __device__ void operator()(uint32_t k, uint32_t value, uint32_t prefix) const {
     (void)value;
     out[k] = prefix;
+  }
+};
+
+// [first, last + 1) of element k's run in a list of `capacity` slots ([0, 0) for an empty one).
+struct RangeStore {
+  uint2* out;
+  uint32_t capacity;
+  __device__ void operator()(uint32_t k, uint32_t value, uint32_t prefix) const {
+    out[k] = value ? make_uint2(min(prefix, capacity), min(prefix + value, capacity))
+                   : make_uint2(0u, 0u);
   }
 };
 
@@ -308,83 +277,6 @@ bool try_cluster_scan(Load load, Store store, int64_t n_cap, const uint32_t* n_d
   return true;
 }
 
-// ------------------------------------------------------------------------------------------
-// Single-pass scan: the chained scan with decoupled look-back of Merrill and Garland
-// ("Single-pass Parallel Prefix Scan with Decoupled Look-back", 2016), in one launch of one
-// block per tile of kScanTile elements. A block takes its tile from a ticket counter, so tiles
-// are handed out in the order blocks start: a block only ever waits for tiles of blocks that
-// are already running, which therefore finish. It scans its tile, publishes the tile total (an
-// "aggregate") and, unless it is tile 0, walks back over the earlier tiles 32 at a time (one per
-// lane of warp 0), adding aggregates until it meets a published inclusive prefix; then it
-// publishes its own inclusive prefix and stores its results. A state word packs the flag in bits 62..63 (0 not yet published, 1 aggregate,
-// 2 inclusive prefix) and the value in bits 0..31. It is written and read whole (an aligned
-// 64-bit access), and nothing else is published through it, so relaxed accesses suffice. Each
-// wait is bounded: past kLookbackSpins polls the block records kStatusScanWait and takes the
-// tile as 0 (a wrong result, reported; never expected, since the waited-for block is running).
-// ------------------------------------------------------------------------------------------
-constexpr unsigned long long kTileAggregate = 1ull << 62, kTileInclusive = 2ull << 62;
-constexpr int kLookbackSpins = 1 << 20;  // polls of ~1 us each
-
-__device__ __forceinline__ void store_state(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ unsigned long long load_state(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
-// Takes a tile from the ticket counter (thread 0; the result is broadcast to the block).
-__device__ __forceinline__ uint32_t lookback_ticket(const Lookback& lb) {
-  __shared__ uint32_t s_tile;
-  if (threadIdx.x == 0) s_tile = atomicAdd(lb.ticket, 1u);
-  __syncthreads();
-  return s_tile;
-}
-
-// Called by the 32 lanes of warp 0 of the block holding tile b, whose elements sum to agg:
-// publishes the aggregate, looks back for the exclusive prefix of the tile, publishes the
-// inclusive prefix and returns the exclusive one (in every lane).
-__device__ uint32_t lookback_prefix(const Lookback& lb, uint32_t b, uint32_t agg) {
-  const int lane = threadIdx.x & 31;
-  if (b == 0) {
-    if (lane == 0) store_state(&lb.tiles[0], kTileInclusive | agg);
-    return 0u;
-  }
-  if (lane == 0) store_state(&lb.tiles[b], kTileAggregate | agg);
-  uint32_t prefix = 0;
-  bool timed_out = false;
-  for (int64_t end = b; end > 0; end -= 32) {
-    const int64_t j = end - 1 - lane;  // lane 0 looks at the nearest earlier tile
-    unsigned long long w = kTileInclusive;  // before tile 0: an empty inclusive prefix
-    if (j >= 0) {
-      w = load_state(&lb.tiles[j]);
-      for (int spin = 0; (w >> 62) == 0; ++spin) {
-        if (spin >= kLookbackSpins) {
-          timed_out = true;
-          w = kTileInclusive;
-          break;
-        }
-        __nanosleep(32);
-        w = load_state(&lb.tiles[j]);
-      }
-    }
-    const uint32_t inclusive = __ballot_sync(0xffffffffu, (w >> 62) == 2ull);
-    // Tiles nearer than the nearest inclusive prefix contribute their aggregates, that prefix
-    // contributes itself, and the farther tiles nothing.
-    const int stop = inclusive ? __ffs(inclusive) - 1 : 32;
-    uint32_t x = lane <= stop ? (uint32_t)w : 0u;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    prefix += x;
-    if (inclusive) break;
-  }
-  if (__any_sync(0xffffffffu, timed_out) && lane == 0)
-    atomicOr(lb.status, (uint32_t)kStatusScanWait);
-  if (lane == 0) store_state(&lb.tiles[b], kTileInclusive | (prefix + agg));
-  return prefix;
-}
-
 template <typename Load, typename Store>
 __global__ void __launch_bounds__(kScanThreads) lookback_scan_kernel(Load load, Store store,
                                                                      int64_t n_cap,
@@ -429,52 +321,90 @@ __global__ void __launch_bounds__(kScanThreads) lookback_scan_kernel(Load load, 
 
 // ------------------------------------------------------------------------------------------
 // Compaction of the visible entries from the visibility bitmask, one single-pass launch. A
-// tile is kBitsThreads words, one per thread (coalesced loads). The exclusive prefix of the set
-// bits over the threads gives each thread the tile-local position of its first visible entry;
-// it writes its entries' indices there, in bit order, into a shared-memory list, while warp 0
-// finds the tile's offset by look-back. The block then stores the list with every thread:
-// independent loads of the depths, contiguous stores. Words are taken in (view, word) order and
-// bits from the lowest, so the output follows (view, Gaussian) order.
+// tile is kBitsTile words: warp w takes kBitsItems groups of 32, one word per lane (coalesced
+// loads). The exclusive prefix of the set bits over (warp, group, lane) gives each word the
+// position of its first visible entry; a group's entries are listed in shared memory in bit order
+// and then written by the whole warp: independent loads of the depths, contiguous stores. Words
+// are taken in (view, word) order and bits from the lowest, so the output follows (view, Gaussian)
+// order. The tile's length sets the length of the look-back chain, which bounds long masks: with
+// one word per thread 48M entries took 100 us (5860 tiles in the chain).
 // ------------------------------------------------------------------------------------------
 constexpr int kBitsThreads = 256;
+constexpr int kBitsWarps = kBitsThreads / 32;
+constexpr int kBitsItems = 2;
+constexpr int kBitsLoads = 4;  // depths a lane has in flight
+constexpr int kBitsTile = kBitsThreads * kBitsItems;
 
 __global__ void __launch_bounds__(kBitsThreads) compact_bits_kernel(
     const uint32_t* __restrict__ vis_bits, uint32_t n_words, uint32_t words_per_view, uint32_t n,
     const float4* __restrict__ rec2, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
     uint32_t* __restrict__ list, uint32_t* __restrict__ n_out, Lookback lb, uint32_t n_tiles) {
   chain_wait();
-  __shared__ uint32_t s_list[kBitsThreads * 32];
-  __shared__ uint32_t s_prefix;
+  __shared__ uint32_t s_list[kBitsWarps][32 * 32];
+  __shared__ uint32_t s_warp[kBitsWarps];
   const uint32_t b = lookback_ticket(lb);
   if (b >= n_tiles) {  // the ticket counter was not zeroed: report, touch nothing
     if (threadIdx.x == 0) atomicOr(lb.status, (uint32_t)kStatusScanWait);
     return;
   }
-  const uint32_t gw = b * kBitsThreads + threadIdx.x;
-  uint32_t m = gw < n_words ? vis_bits[gw] : 0u;
-  uint32_t agg;
-  uint32_t pos = block_exclusive_scan<kBitsThreads>((uint32_t)__popc(m), &agg);
-  if (threadIdx.x < 32) {
-    const uint32_t prefix = lookback_prefix(lb, b, agg);
-    if (threadIdx.x == 0) s_prefix = prefix;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t first_word = b * kBitsTile + (uint32_t)warp * (32 * kBitsItems) + lane;
+  uint32_t m[kBitsItems], excl[kBitsItems], total[kBitsItems], sum = 0;
+#pragma unroll
+  for (int j = 0; j < kBitsItems; ++j) {
+    const uint32_t gw = first_word + 32u * j;
+    m[j] = gw < n_words ? vis_bits[gw] : 0u;
   }
-  if (m) {
-    const uint32_t v = gw / words_per_view;
-    const uint32_t first = v * n + (gw - v * words_per_view) * 32u;
-    while (m) {
-      s_list[pos++] = first + (uint32_t)(__ffs(m) - 1);
-      m &= m - 1u;
-    }
+#pragma unroll
+  for (int j = 0; j < kBitsItems; ++j) {
+    excl[j] = warp_exclusive_scan((uint32_t)__popc(m[j]), &total[j]);
+    sum += total[j];
+  }
+  if (lane == 0) s_warp[warp] = sum;
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t agg;
+    const uint32_t before = warp_exclusive_scan(lane < kBitsWarps ? s_warp[lane] : 0u, &agg);
+    const uint32_t prefix = lookback_prefix(lb, b, agg);
+    if (lane < kBitsWarps) s_warp[lane] = prefix + before;
+    if (b == n_tiles - 1 && lane == 0) *n_out = prefix + agg;
   }
   __syncthreads();
-  const uint32_t prefix = s_prefix;
-  for (uint32_t t = threadIdx.x; t < agg; t += kBitsThreads) {
-    const uint32_t vi = s_list[t];
-    keys[prefix + t] = __float_as_uint(rec2[vi].w);
-    vals[prefix + t] = vi;
-    list[prefix + t] = vi;
+  uint32_t out = s_warp[warp];
+  uint32_t* mine = s_list[warp];
+#pragma unroll
+  for (int j = 0; j < kBitsItems; ++j) {
+    const uint32_t gw = first_word + 32u * j;
+    if (m[j]) {
+      const uint32_t v = gw / words_per_view;
+      const uint32_t first = v * n + (gw - v * words_per_view) * 32u;
+      uint32_t pos = excl[j];
+      while (m[j]) {
+        mine[pos++] = first + (uint32_t)(__ffs(m[j]) - 1);
+        m[j] &= m[j] - 1u;
+      }
+    }
+    __syncwarp();
+    for (uint32_t t0 = lane; t0 < total[j]; t0 += 32 * kBitsLoads) {
+      uint32_t vi[kBitsLoads], key[kBitsLoads];
+#pragma unroll
+      for (int u = 0; u < kBitsLoads; ++u) vi[u] = t0 + 32 * u < total[j] ? mine[t0 + 32 * u] : 0u;
+#pragma unroll
+      for (int u = 0; u < kBitsLoads; ++u)
+        key[u] = t0 + 32 * u < total[j] ? __float_as_uint(rec2[vi[u]].w) : 0u;
+#pragma unroll
+      for (int u = 0; u < kBitsLoads; ++u) {
+        const uint32_t t = t0 + 32 * u;
+        if (t < total[j]) {
+          keys[out + t] = key[u];
+          vals[out + t] = vi[u];
+          list[out + t] = vi[u];
+        }
+      }
+    }
+    __syncwarp();
+    out += total[j];
   }
-  if (b == n_tiles - 1 && threadIdx.x == 0) *n_out = prefix + agg;
 }
 
 // Exclusive scan of the loaded values: one single-pass launch when look-back bookkeeping is
@@ -1010,7 +940,7 @@ cudaError_t launch_compact_visible(const uint32_t* vis_bits, int n_views, int n,
                                    cudaStream_t stream) {
   const int64_t words = (int64_t)n_views * vis_bit_words_per_view(n);
   if (words == 0) return cudaMemsetAsync(n_out, 0, sizeof(uint32_t), stream);
-  const int64_t tiles = (words + kBitsThreads - 1) / kBitsThreads;
+  const int64_t tiles = (words + kBitsTile - 1) / kBitsTile;
   if (tiles > lb.capacity) return cudaErrorInvalidValue;
   const cudaError_t e = launch_chained(
       compact_bits_kernel, dim3((unsigned)tiles), dim3(kBitsThreads), stream, vis_bits,
@@ -1020,11 +950,11 @@ cudaError_t launch_compact_visible(const uint32_t* vis_bits, int n_views, int n,
   return e;
 }
 
-cudaError_t launch_gather_scan(const uint32_t* ntiles, const uint32_t* order, int64_t n_cap,
-                               const uint32_t* n_dev, uint32_t* offs, uint32_t* total,
-                               uint32_t* block_sums, Lookback lb, cudaStream_t stream) {
-  return run_scan(GatherLoad{ntiles, order}, PlainStore{offs}, n_cap, n_dev, total, block_sums,
-                  stream, lb);
+cudaError_t launch_tile_ranges_scan(const uint32_t* counts, uint2* ranges, int64_t n_tiles,
+                                    uint32_t capacity, uint32_t* total, Lookback lb,
+                                    cudaStream_t stream) {
+  return run_scan(PlainLoad{counts}, RangeStore{ranges, capacity}, n_tiles, nullptr, total,
+                  nullptr, stream, lb);
 }
 
 // Sorts of at least this many keys (capacity) take the wide passes.
