@@ -41,17 +41,6 @@ constexpr uint32_t kEmitStage = 512;  // cell entries a warp stages per round
 
 int emit_items(int64_t visible) { return visible > kEmitLong ? kEmitItems : 1; }
 
-// First lane whose inclusive count exceeds idx (31 past the warp total).
-__device__ __forceinline__ int lane_of(uint32_t incl, uint32_t idx) {
-  int lo = 0, hi = 31;
-#pragma unroll
-  for (int step = 0; step < 5; ++step) {
-    const int mid = (lo + hi) >> 1;
-    if (__shfl_sync(0xffffffffu, incl, mid) > idx) hi = mid; else lo = mid + 1;
-  }
-  return min(lo, 31);
-}
-
 template <bool kMasks>
 __device__ __forceinline__ uint32_t cell_key(uint32_t cell, uint32_t mask) {
   return kMasks ? (cell << 16) | mask : cell;

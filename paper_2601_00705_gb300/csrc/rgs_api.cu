@@ -1543,69 +1543,66 @@ rgs_status rgs_init_seeds(rgs_ctx* ctx, const rgs_camera* cams, int32_t n_views,
     return fail(ctx, RGS_ERR_CUDA, "cudaSetDevice failed");
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);
   const int sh_k = (sh_degree + 1) * (sh_degree + 1);
-  const int64_t hist = sort_hist_entries(m);
+  const int64_t hist = sort_hist_entries(m, kSortItemsSmall);
   const int64_t sums = std::max(scan_blocks(hist), scan_blocks(m)) + 1;
-  const size_t bytes = 12 * align_up(sizeof(uint32_t) * m) + align_up(sizeof(uint32_t) * hist) +
-                       align_up(sizeof(uint32_t) * sums) + align_up(sizeof(uint64_t) * m) +
-                       align_up(sizeof(double) * 3 * m) +
-                       align_up(sizeof(float) * (size_t)m * (3 + 3 + 4 + 1 + 3 + 3 * sh_k));
+  const size_t lb_bytes = align_up(lookback_bytes(m));
+  const size_t reset_bytes = align_up(sizeof(SeedCounts)) + 2 * lb_bytes;
+  const size_t bytes = reset_bytes + 8 * align_up(sizeof(uint32_t) * m) +
+                       align_up(sizeof(uint32_t) * hist) + align_up(sizeof(uint32_t) * sums) +
+                       align_up(sizeof(uint64_t) * m) + align_up(sizeof(double) * 3 * m) +
+                       align_up(sizeof(float4) * m) + align_up(sizeof(double) * 10 * m);
   // The scratch region is kept in the context and only grows: repeated calls (one per new
   // keyframe) neither allocate nor free.
   if (ctx->r_seed.bytes < bytes)
     RGS_CUDA(alloc_region(ctx, ctx->r_seed, bytes), "allocate seeding scratch");
+  SeedScratch w;
   char* p = static_cast<char*>(ctx->r_seed.base);
-  uint32_t* flags = carve<uint32_t>(p, m);
-  uint32_t* pos = carve<uint32_t>(p, m);
-  uint32_t* vidx = carve<uint32_t>(p, m);
-  uint32_t* lo = carve<uint32_t>(p, m);
-  uint32_t* hi = carve<uint32_t>(p, m);
-  uint32_t* slot = carve<uint32_t>(p, m);
-  uint32_t* t0 = carve<uint32_t>(p, m);
-  uint32_t* t1 = carve<uint32_t>(p, m);
-  uint32_t* keep = carve<uint32_t>(p, m);
-  uint32_t* kpos = carve<uint32_t>(p, m);
-  uint32_t* totals = carve<uint32_t>(p, m);  // [0]: accepted points, [1]: kept seeds
-  carve<uint32_t>(p, m);                     // spare
-  uint32_t* h = carve<uint32_t>(p, hist);
-  uint32_t* bs = carve<uint32_t>(p, sums);
-  unsigned long long* skey = carve<unsigned long long>(p, m);
-  double* sX = carve<double>(p, 3 * m);
-  float* f_means = carve<float>(p, 3 * m);
-  float* f_ls = carve<float>(p, 3 * m);
-  float* f_q = carve<float>(p, 4 * m);
-  float* f_o = carve<float>(p, m);
-  float* f_n = carve<float>(p, 3 * m);
-  float* f_sh = carve<float>(p, 3 * sh_k * m);
-  rgs_status result = RGS_OK;
-  uint32_t host_tot[2] = {0, 0};
-  do {
-    cudaError_t e = launch_seed_flags(m, n_views, valid, ref_view, flags, stream);
-    if (e == cudaSuccess) e = launch_exclusive_scan(flags, pos, m, nullptr, totals, bs, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(host_tot, totals, sizeof(uint32_t),
-                                              cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    if (e != cudaSuccess) { result = cuda_fail(ctx, e, "seed compaction"); break; }
-    const int s = (int)host_tot[0];
-    e = launch_compact_points(m, flags, pos, vidx, stream);
-    if (e == cudaSuccess)
-      e = launch_seed_points(sc, c, s, k, sh_k, vidx, ref_view, nb_view, X, err, angle, kappa,
-                             observed, gain_bias, lo, hi, slot, t0, t1, h, bs, skey, sX, f_means,
-                             f_ls, f_q, f_o, f_sh, f_n, keep, stream);
-    if (e == cudaSuccess && s > 0)
-      e = launch_exclusive_scan(keep, kpos, s, nullptr, totals + 1, bs, stream);
-    if (e == cudaSuccess && s > 0)
-      e = cudaMemcpyAsync(host_tot + 1, totals + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost,
-                          stream);
-    if (e == cudaSuccess)
-      e = launch_scatter_seeds(s, sh_k, keep, kpos, vidx, f_means, f_ls, f_q, f_o, f_sh, f_n,
-                               index, means, log_scales, quats, opacity_logits, sh, normals,
-                               stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    if (e != cudaSuccess) { result = cuda_fail(ctx, e, "seed initialisation"); break; }
-    *n_seeds = s > 0 ? (int64_t)host_tot[1] : 0;
-  } while (false);
-  cudaStreamSynchronize(stream);
-  return result;
+  w.counts = carve<SeedCounts>(p, 1);
+  w.reset_bytes = reset_bytes;
+  // The scans report an abandoned wait in a word that nothing else uses.
+  w.lb[0] = lookback_at(p, &w.counts->scan_status, m);
+  w.lb[1] = lookback_at(p + lb_bytes, &w.counts->scan_status, m);
+  p += 2 * lb_bytes;
+  uint32_t** words[] = {&w.flags, &w.pos, &w.vidx, &w.lo, &w.hi, &w.slot, &w.t0, &w.t1};
+  for (uint32_t** q : words) *q = carve<uint32_t>(p, m);
+  w.hist = carve<uint32_t>(p, hist);
+  w.block_sums = carve<uint32_t>(p, sums);
+  w.skey = carve<unsigned long long>(p, m);
+  w.sX = carve<double>(p, 3 * m);
+  w.local = carve<float4>(p, m);
+  w.mom = carve<double>(p, 10 * m);
+  SeedCounts host{};
+  // The accepted points; their number and the box of their cells size what follows.
+  RGS_CUDA(launch_accept_points(w, m, n_views, valid, ref_view, X, c.plane_radius, c.voxel,
+                                stream),
+           "seed compaction");
+  RGS_CUDA(cudaMemcpyAsync(&host, w.counts, sizeof(host), cudaMemcpyDeviceToHost, stream),
+           "read the accepted points' count");
+  RGS_CUDA(cudaStreamSynchronize(stream), "seed compaction");
+  if (host.scan_status) return fail(ctx, RGS_ERR_CUDA, "a scan gave up waiting");
+  const int s = (int)host.accepted;
+  CellPack pack[2];
+  for (int g = 0; g < 2; ++g) {
+    int bits = 0;
+    for (int a = 0; a < 3; ++a) {
+      pack[g].corner[a] = 2097151 - (int)host.box[g][a];
+      const uint32_t extent = host.box[g][3 + a] - (uint32_t)pack[g].corner[a];
+      pack[g].bits[a] = extent ? bits_for(extent + 1u) : 0;
+      bits += pack[g].bits[a];
+    }
+    pack[g].on = bits <= 32;
+  }
+  RGS_CUDA(launch_seeds(w, sc, c, pack, s, k, sh_k, ref_view, nb_view, X, err, angle, kappa,
+                        observed, gain_bias, index, means, log_scales, quats, opacity_logits, sh,
+                        normals, stream),
+           "seed initialisation");
+  if (s > 0 && c.voxel > 0.0)
+    RGS_CUDA(cudaMemcpyAsync(&host, w.counts, sizeof(host), cudaMemcpyDeviceToHost, stream),
+             "read the seed count");
+  RGS_CUDA(cudaStreamSynchronize(stream), "seed initialisation");
+  if (host.scan_status) return fail(ctx, RGS_ERR_CUDA, "a scan gave up waiting");
+  *n_seeds = s > 0 && c.voxel > 0.0 ? (int64_t)host.kept : (int64_t)s;
+  return RGS_OK;
 }
 
 rgs_status rgs_covisibility(rgs_ctx* ctx, const float* alpha_a, const float* alpha_b, int64_t n,

@@ -664,26 +664,40 @@ cudaError_t launch_triangulate(const SeedCams& cams, const SeedConsts& c, int64_
                                const int32_t* nb_view, const double* nb_xy, const float* nb_conf,
                                uint32_t* valid, double* X, int32_t* best, double* err,
                                double* angle, float* kappa, cudaStream_t stream);
-cudaError_t launch_seed_flags(int64_t m, int n_views, const uint32_t* valid,
-                              const int32_t* ref_view, uint32_t* flags, cudaStream_t stream);
-cudaError_t launch_compact_points(int64_t m, const uint32_t* valid, const uint32_t* pos,
-                                  uint32_t* vidx, cudaStream_t stream);
-cudaError_t launch_seed_points(const SeedCams& cams, const SeedConsts& c, int s, int k, int sh_k,
-                               const uint32_t* vidx, const int32_t* ref_view,
-                               const int32_t* nb_view, const double* X, const double* err,
-                               const double* angle, const float* kappa, const float* obs,
-                               const float* gain_bias, uint32_t* lo, uint32_t* hi,
-                               uint32_t* slot, uint32_t* t0, uint32_t* t1, uint32_t* hist,
-                               uint32_t* block_sums, unsigned long long* skey, double* sX,
-                               float* means, float* log_scales, float* quats, float* logits,
-                               float* sh, float* normals, uint32_t* keep, cudaStream_t stream);
-cudaError_t launch_scatter_seeds(int s, int sh_k, const uint32_t* keep, const uint32_t* pos,
-                                 const uint32_t* vidx, const float* means,
-                                 const float* log_scales, const float* quats,
-                                 const float* logits, const float* sh, const float* normals,
-                                 int32_t* o_index, float* o_means, float* o_log_scales,
-                                 float* o_quats, float* o_logits, float* o_sh, float* o_normals,
-                                 cudaStream_t stream);
+// What the seed initialisation counts on the device: accepted and kept points, and per grid (plane
+// radius, voxel) the box of their cells, per axis the maximum of (2^21 - 1 - cell) and of cell.
+struct SeedCounts {
+  uint32_t accepted, kept;
+  uint32_t scan_status;  // kStatusScanWait: a scan gave up a bounded wait
+  uint32_t box[2][6];
+};
+// Cells relative to a corner, packed into one word of bits[0] + bits[1] + bits[2] <= 32 bits.
+struct CellPack {
+  int on;
+  int corner[3], bits[3];
+};
+// Device scratch of the seed initialisation for m points (u32 [m] each unless noted). The first
+// reset_bytes from `counts` on are zeroed at the start of every call.
+struct SeedScratch {
+  SeedCounts* counts;
+  size_t reset_bytes;
+  Lookback lb[2];
+  uint32_t *flags, *pos, *vidx, *lo, *hi, *slot, *t0, *t1, *hist, *block_sums;
+  unsigned long long* skey;  // [m] sorted cell keys
+  double* sX;                // [m][3] points in sorted order
+  float4* local;             // [m] the same in cell units
+  double* mom;               // [m][10] neighbourhood moments, in compact order
+};
+cudaError_t launch_accept_points(const SeedScratch& w, int64_t m, int n_views,
+                                 const uint32_t* valid, const int32_t* ref_view, const double* X,
+                                 double plane_radius, double voxel, cudaStream_t stream);
+cudaError_t launch_seeds(const SeedScratch& w, const SeedCams& cams, const SeedConsts& c,
+                         const CellPack (&pack)[2], int s, int k, int sh_k,
+                         const int32_t* ref_view, const int32_t* nb_view, const double* X,
+                         const double* err, const double* angle, const float* kappa,
+                         const float* obs, const float* gain_bias, int32_t* index, float* means,
+                         float* log_scales, float* quats, float* logits, float* sh,
+                         float* normals, cudaStream_t stream);
 
 // Largest n the single-cluster sort takes on `device` (0: cluster launches unavailable); sorts
 // with n_cap up to it run as one launch and always return their result in the alternate buffers.

@@ -56,6 +56,17 @@ __device__ __forceinline__ uint32_t warp_exclusive_scan(uint32_t v, uint32_t* to
   return x - v;
 }
 
+// First lane whose inclusive count exceeds idx (31 past the warp total).
+__device__ __forceinline__ int lane_of(uint32_t incl, uint32_t idx) {
+  int lo = 0, hi = 31;
+#pragma unroll
+  for (int step = 0; step < 5; ++step) {
+    const int mid = (lo + hi) >> 1;
+    if (__shfl_sync(0xffffffffu, incl, mid) > idx) hi = mid; else lo = mid + 1;
+  }
+  return min(lo, 31);
+}
+
 // ------------------------------------------------------------------------------------------
 // Single-pass scan: the chained scan with decoupled look-back of Merrill and Garland
 // ("Single-pass Parallel Prefix Scan with Decoupled Look-back", 2016), in one launch of one
