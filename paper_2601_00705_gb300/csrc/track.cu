@@ -14,6 +14,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "rgs_internal.cuh"
 
@@ -21,6 +22,9 @@ namespace rgs {
 namespace {
 
 constexpr int kTrackThreads = 256;
+// Blocks per SM of the two loss passes: enough loads in flight, and few double-precision atomics
+// on each view's sums.
+constexpr int kTrackBlocksPerSm = 4;
 
 // ------------------------------------------------------------------------------------------
 // Pose records: R (9), t (3), c = -R^T t (3), pad. The centre is accumulated in double and
@@ -97,17 +101,69 @@ __global__ void __launch_bounds__(kTrackThreads) grad_weight_kernel(
   }
 }
 
-// Block-wide sum of NV values per thread, in double, into (double) accumulators with atomics.
+// The pixels of view v dealt out over the blocks of grid row v: `four(p)` for groups of four
+// pixels that start at a multiple of four in the concatenated images (their colours are then three
+// aligned 16-byte words), `one(p)` for the pixels before and after them; `one` for all when the
+// arrays are not 16-byte aligned (vec 0).
+template <typename One, typename Four>
+__device__ __forceinline__ void for_pixels(const Views& views, int v, int vec, One&& one,
+                                           Four&& four) {
+  long long first;
+  int count, W, H;
+  view_pixels(views, v, first, count, W, H);
+  const int t = blockIdx.x * kTrackThreads + threadIdx.x, step = gridDim.x * kTrackThreads;
+  int head = count, groups = 0;
+  if (vec) {
+    head = min((int)(-first & 3), count);
+    groups = (count - head) >> 2;
+  }
+  for (int k = t; k < groups; k += step) four(first + head + 4ll * k);
+  // At most six pixels are left with groups, all of them without.
+  const int rest = count - 4 * groups;
+  for (int k = t; k < rest; k += step) one(first + (k < head ? k : k + 4 * groups));
+}
+
+__device__ __forceinline__ void load12(const float* __restrict__ p, float (&x)[12]) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float4 w = reinterpret_cast<const float4*>(p)[q];
+    x[4 * q] = w.x;
+    x[4 * q + 1] = w.y;
+    x[4 * q + 2] = w.z;
+    x[4 * q + 3] = w.w;
+  }
+}
+
+// A sum of floats as an unevaluated pair, each addition exact to about 2^-48 of the sum (Knuth's
+// two-sum): the partial sums lose nothing to their length, and, unlike doubles, cost a handful of
+// FP32 operations (a double addition costs a warp 64 cycles).
+struct PairSum {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    float e;
+    two_sum(hi, x, hi, e);
+    lo = __fadd_rn(lo, e);
+  }
+  __device__ __forceinline__ void add(float h, float l) {
+    add(h);
+    lo = __fadd_rn(lo, l);
+  }
+};
+
+// Block-wide sum of NV pair sums per thread into (double) accumulators with atomics.
 template <int NV>
-__device__ __forceinline__ void block_sum_to(const float (&x)[NV], double* __restrict__ acc) {
+__device__ __forceinline__ void block_sum_to(PairSum (&x)[NV], double* __restrict__ acc) {
   __shared__ double s_part[kTrackThreads / 32][NV];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int j = 0; j < NV; ++j) {
-    float v = x[j];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) s_part[warp][j] = (double)v;
+    for (int o = 16; o > 0; o >>= 1) {
+      const float h = __shfl_xor_sync(0xffffffffu, x[j].hi, o);
+      const float l = __shfl_xor_sync(0xffffffffu, x[j].lo, o);
+      x[j].add(h, l);
+    }
+    if (lane == 0) s_part[warp][j] = (double)x[j].hi + (double)x[j].lo;
   }
   __syncthreads();
   if (threadIdx.x < NV) {
@@ -120,30 +176,41 @@ __device__ __forceinline__ void block_sum_to(const float (&x)[NV], double* __res
 
 // ------------------------------------------------------------------------------------------
 // Exposure fit, pass 1 (Eq. app-ls): per view, sum r, sum r^2, sum o, sum r o over the three
-// channels of every pixel (r rendered, o observed). Per-thread partial sums in FP32 over a few
-// dozen values, FP64 from the warp totals on.
+// channels of every pixel (r rendered, o observed). Four pixels are summed in FP32, everything from
+// there on in pair sums, and FP64 from the warp totals on.
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kTrackThreads) track_sums_kernel(
     const __grid_constant__ Views views, const float* __restrict__ color,
-    const float* __restrict__ obs, double* __restrict__ sums) {
+    const float* __restrict__ obs, int vec, double* __restrict__ sums,
+    double* __restrict__ loss) {
   chain_wait();
   const int v = blockIdx.y;
-  long long first;
-  int count, W, H;
-  view_pixels(views, v, first, count, W, H);
-  float x[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  for (int k = blockIdx.x * kTrackThreads + threadIdx.x; k < count;
-       k += gridDim.x * kTrackThreads) {
-    const long long p = first + k;
+  if (blockIdx.x == 0 && threadIdx.x == 0) loss[v] = 0.0;  // for the next pass
+  PairSum x[4];
+  // The sums of a few values, added to the thread's.
+  auto add = [&](const float* r, const float* o, auto count) {
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-      const float r = color[3 * p + ch], o = obs[3 * p + ch];
-      x[0] += r;
-      x[1] = fmaf(r, r, x[1]);
-      x[2] += o;
-      x[3] = fmaf(r, o, x[3]);
+    for (int e = 0; e < decltype(count)::value; ++e) {
+      s[0] += r[e];
+      s[1] = fmaf(r[e], r[e], s[1]);
+      s[2] += o[e];
+      s[3] = fmaf(r[e], o[e], s[3]);
     }
-  }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[q].add(s[q]);
+  };
+  for_pixels(
+      views, v, vec,
+      [&](long long p) {
+        add(color + 3 * p, obs + 3 * p, std::integral_constant<int, 3>{});
+      },
+      [&](long long p) {
+        float r[12], o[12];
+        load12(color + 3 * p, r);
+        load12(obs + 3 * p, o);
+        add(r, o, std::integral_constant<int, 12>{});
+      });
   block_sum_to<4>(x, sums + 4 * v);
 }
 
@@ -178,36 +245,67 @@ __global__ void __launch_bounds__(kTrackThreads) track_loss_kernel(
     const __grid_constant__ Views views, const float* __restrict__ color,
     const float* __restrict__ alpha, const float* __restrict__ obs,
     const float* __restrict__ w_grad, const double* __restrict__ sums, float inv_tau_alpha,
-    int fit_exposure, float* __restrict__ d_color, double* __restrict__ loss,
+    int fit_exposure, int vec, float* __restrict__ d_color, double* __restrict__ loss,
     float* __restrict__ gain_bias) {
   chain_wait();
   const int v = blockIdx.y;
-  long long first;
-  int count, W, H;
-  view_pixels(views, v, first, count, W, H);
   double gd, bd;
-  exposure_of(sums + 4 * v, 3.0 * (double)count, fit_exposure != 0, gd, bd);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    gain_bias[2 * v] = (float)gd;
-    gain_bias[2 * v + 1] = (float)bd;
+  // One thread fits the exposure: a double-precision instruction costs a warp 64 cycles.
+  __shared__ float s_fit[2];
+  if (threadIdx.x == 0) {
+    exposure_of(sums + 4 * v, 3.0 * (double)views.v[v].width * (double)views.v[v].height,
+                fit_exposure != 0, gd, bd);
+    s_fit[0] = (float)gd;
+    s_fit[1] = (float)bd;
+    if (blockIdx.x == 0) {
+      gain_bias[2 * v] = (float)gd;
+      gain_bias[2 * v + 1] = (float)bd;
+    }
   }
-  const float g = (float)gd, b = (float)bd;
-  float part[1] = {0.0f};
-  for (int k = blockIdx.x * kTrackThreads + threadIdx.x; k < count;
-       k += gridDim.x * kTrackThreads) {
-    const long long p = first + k;
-    float w = fminf(fmaxf(alpha[p] * inv_tau_alpha, 0.0f), 1.0f);
-    if (w_grad) w *= w_grad[p];
+  __syncthreads();
+  const float g = s_fit[0], b = s_fit[1];
+  PairSum part[1];
+  // One pixel's gradient, and its share of the loss, from its residuals (r rendered, o observed).
+  auto pixel = [&](float a, float wg, const float* r, const float* o, float* d) {
+    const float w = fminf(fmaxf(a * inv_tau_alpha, 0.0f), 1.0f) * wg;
     float l1 = 0.0f;
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) {
-      const float res = obs[3 * p + ch] - fmaf(g, color[3 * p + ch], b);
+      const float res = o[ch] - fmaf(g, r[ch], b);
       l1 += fabsf(res);
       const float sg = res > 0.0f ? 1.0f : (res < 0.0f ? -1.0f : 0.0f);
-      d_color[3 * p + ch] = -w * g * sg;
+      d[ch] = -w * g * sg;
     }
-    part[0] = fmaf(w, l1, part[0]);
-  }
+    return w * l1;
+  };
+  for_pixels(
+      views, v, vec,
+      [&](long long p) {
+        float r[3], o[3], d[3];
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) {
+          r[ch] = color[3 * p + ch];
+          o[ch] = obs[3 * p + ch];
+        }
+        part[0].add(pixel(alpha[p], w_grad ? w_grad[p] : 1.0f, r, o, d));
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) d_color[3 * p + ch] = d[ch];
+      },
+      [&](long long p) {
+        float r[12], o[12], d[12];
+        load12(color + 3 * p, r);
+        load12(obs + 3 * p, o);
+        const float4 a = *reinterpret_cast<const float4*>(alpha + p);
+        const float4 wg = w_grad ? *reinterpret_cast<const float4*>(w_grad + p)
+                                 : make_float4(1.0f, 1.0f, 1.0f, 1.0f);
+        const float l01 = pixel(a.x, wg.x, r, o, d) + pixel(a.y, wg.y, r + 3, o + 3, d + 3);
+        const float l23 = pixel(a.z, wg.z, r + 6, o + 6, d + 6) + pixel(a.w, wg.w, r + 9, o + 9, d + 9);
+        part[0].add(l01 + l23);
+        float4* out = reinterpret_cast<float4*>(d_color + 3 * p);
+        out[0] = make_float4(d[0], d[1], d[2], d[3]);
+        out[1] = make_float4(d[4], d[5], d[6], d[7]);
+        out[2] = make_float4(d[8], d[9], d[10], d[11]);
+      });
   block_sum_to<1>(part, loss + v);
 }
 
@@ -220,79 +318,107 @@ __global__ void __launch_bounds__(kTrackThreads) track_loss_kernel(
 // (k = 0, 1, ...) is lr * (1 + cos(pi min(k, K) / K)) / 2 with K = iterations, or lr when
 // K = 0. In FP64; the pose is stored back in FP32.
 // ------------------------------------------------------------------------------------------
+// Six lanes per view (five views per warp), lane j with component j: a double-precision
+// instruction costs a warp 64 cycles whatever its lanes do, so the views' components go through
+// each one together and what a view shares is computed by its six lanes alike (27 us with a thread
+// per view and the pow, sin and cos of the general case, 6 us).
+constexpr int kAdamViews = 5;  // views per warp
+
+// x^n for n >= 0, by squaring.
+__device__ __forceinline__ double power(double x, int n) {
+  double r = 1.0;
+  for (; n; n >>= 1) {
+    if (n & 1) r *= x;
+    x *= x;
+  }
+  return r;
+}
+
 __global__ void pose_adam_kernel(int n_views, float lr, float beta1, float beta2, float eps,
                                  int iterations, const float* __restrict__ d_pose,
                                  float* __restrict__ adam_state, int32_t* __restrict__ step,
                                  float* __restrict__ world_to_cam) {
   chain_wait();
-  const int v = threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int j = lane % 6, first = lane - j;
+  const int v = (threadIdx.x >> 5) * kAdamViews + lane / 6;
+  const bool on = lane < 6 * kAdamViews && v < n_views;
   const int k = *step;
   __syncthreads();  // every thread has read the step count before it advances
-  if (v < n_views) {
-    double lr_k = lr;
-    if (iterations > 0) {
-      const double kk = (double)(k < iterations ? k : iterations);
-      lr_k = 0.5 * (double)lr * (1.0 + cos(M_PI * kk / (double)iterations));
-    }
-    const double c1 = 1.0 - pow((double)beta1, (double)(k + 1));
-    const double c2 = 1.0 - pow((double)beta2, (double)(k + 1));
-    double xi[6];
+  double lr_k = lr;
+  if (iterations > 0)
+    lr_k = 0.5 * (double)lr * (1.0 + cospi((double)min(k, iterations) / (double)iterations));
+  // Even lanes hold 1 - beta1^(k + 1), odd ones 1 - beta2^(k + 1).
+  const double bias = 1.0 - power((lane & 1) ? (double)beta2 : (double)beta1, k + 1);
+  const double c1 = __shfl_sync(0xffffffffu, bias, 0), c2 = __shfl_sync(0xffffffffu, bias, 1);
+  double xi = 0.0;
+  if (on) {
     float* m = adam_state + 12 * v;
-    float* s2 = m + 6;
-    for (int j = 0; j < 6; ++j) {
-      const double gj = d_pose[6 * v + j];
-      const double mj = (double)beta1 * m[j] + (1.0 - (double)beta1) * gj;
-      const double vj = (double)beta2 * s2[j] + (1.0 - (double)beta2) * gj * gj;
-      m[j] = (float)mj;
-      s2[j] = (float)vj;
-      xi[j] = -lr_k * (mj / c1) / (sqrt(vj / c2) + (double)eps);
-    }
-    const double w0 = xi[3], w1 = xi[4], w2 = xi[5];
-    const double th2 = w0 * w0 + w1 * w1 + w2 * w2;
-    double A, B, C;
-    if (th2 < 1e-10) {
-      A = 1.0 - th2 / 6.0;
-      B = 0.5 - th2 / 24.0;
-      C = 1.0 / 6.0 - th2 / 120.0;
-    } else {
-      const double th = sqrt(th2);
-      A = sin(th) / th;
-      B = (1.0 - cos(th)) / th2;
-      C = (th - sin(th)) / (th2 * th);
-    }
-    // W = [omega]_x and W^2.
-    const double Wm[9] = {0.0, -w2, w1, w2, 0.0, -w0, -w1, w0, 0.0};
-    double W2[9];
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) {
-        double s = 0.0;
-        for (int c = 0; c < 3; ++c) s += Wm[3 * a + c] * Wm[3 * c + b];
-        W2[3 * a + b] = s;
-      }
-    double Rd[9], Vm[9];
-    for (int j = 0; j < 9; ++j) {
-      const double id = (j % 4 == 0) ? 1.0 : 0.0;
-      Rd[j] = id + A * Wm[j] + B * W2[j];
-      Vm[j] = id + B * Wm[j] + C * W2[j];
-    }
-    float* T = world_to_cam + 12 * v;
-    double R[9], t[3];
-    for (int a = 0; a < 3; ++a) {
-      for (int b = 0; b < 3; ++b) R[3 * a + b] = T[4 * a + b];
-      t[a] = T[4 * a + 3];
-    }
-    for (int a = 0; a < 3; ++a) {
-      double tn = 0.0;
-      for (int b = 0; b < 3; ++b) {
-        double rn = 0.0;
-        for (int c = 0; c < 3; ++c) rn += Rd[3 * a + c] * R[3 * c + b];
-        T[4 * a + b] = (float)rn;
-        tn += Rd[3 * a + b] * t[b] + Vm[3 * a + b] * xi[b];
-      }
-      T[4 * a + 3] = (float)tn;
-    }
+    const double gj = d_pose[6 * v + j];
+    const double mj = (double)beta1 * m[j] + (1.0 - (double)beta1) * gj;
+    const double vj = (double)beta2 * m[6 + j] + (1.0 - (double)beta2) * gj * gj;
+    m[j] = (float)mj;
+    m[6 + j] = (float)vj;
+    xi = -lr_k * (mj / c1) / (sqrt(vj / c2) + (double)eps);
   }
-  __syncthreads();
+  double rho[3], w[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    rho[a] = __shfl_sync(0xffffffffu, xi, first + a);
+    w[a] = __shfl_sync(0xffffffffu, xi, (first + 3 + a) & 31);
+  }
+  const double th2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
+  // A = sin(th) / th, B = (1 - cos(th)) / th^2, C = (th - sin(th)) / th^3: their Taylor series up
+  // to th = 1/2 (eight terms leave 1e-17; no cancellation for small th), else sin and cos.
+  double A, B, C;
+  if (th2 <= 0.25) {
+    A = B = C = 0.0;
+#pragma unroll
+    for (int q = 7; q >= 0; --q) {  // coefficients (-1)^q / (2q + 1)!, (2q + 2)!, (2q + 3)!
+      constexpr double kFact[18] = {1., 1., 2., 6., 24., 120., 720., 5040., 40320., 362880.,
+                                    3628800., 39916800., 479001600., 6227020800., 87178291200.,
+                                    1307674368000., 20922789888000., 355687428096000.};
+      const double sg = (q & 1) ? -1.0 : 1.0;
+      A = fma(A, th2, sg / kFact[2 * q + 1]);
+      B = fma(B, th2, sg / kFact[2 * q + 2]);
+      C = fma(C, th2, sg / kFact[2 * q + 3]);
+    }
+  } else {
+    const double th = sqrt(th2);
+    double sn, cs;
+    sincos(th, &sn, &cs);
+    A = sn / th;
+    B = (1.0 - cs) / th2;
+    C = (th - sn) / (th2 * th);
+  }
+  // Lane j answers for two entries of row a = j / 2 of the new pose: columns 0 and 1, or column 2
+  // and the translation. Row a of W = [omega]_x and of W^2 = omega omega^T - th^2 I.
+  const int a = j >> 1;
+  const double wa = a == 0 ? w[0] : a == 1 ? w[1] : w[2];
+  const double W[3] = {a == 0 ? 0.0 : a == 1 ? w[2] : -w[1], a == 0 ? -w[2] : a == 1 ? 0.0 : w[0],
+                       a == 0 ? w[1] : a == 1 ? -w[0] : 0.0};
+  double Rd[3], Vm[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    const double id = a == b ? 1.0 : 0.0;
+    const double W2 = wa * w[b] - id * th2;
+    Rd[b] = id + A * W[b] + B * W2;
+    Vm[b] = id + B * W[b] + C * W2;
+  }
+  float* T = world_to_cam + 12 * (on ? v : 0);
+  double n0 = 0.0, n1 = 0.0;
+  const int col = (j & 1) ? 2 : 0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    n0 += Rd[c] * (double)T[4 * c + col];
+    n1 += Rd[c] * (double)T[4 * c + col + 1];
+    if (j & 1) n1 += Vm[c] * rho[c];
+  }
+  __syncthreads();  // every lane of a view has read the old pose
+  if (on) {
+    T[4 * a + col] = (float)n0;
+    T[4 * a + col + 1] = (float)n1;
+  }
   if (threadIdx.x == 0) *step = k + 1;
 }
 
@@ -310,12 +436,24 @@ __global__ void __launch_bounds__(kTrackThreads) covis_count_kernel(
   const float* a = alpha_a + (size_t)j * n;
   const float* b = alpha_b + (size_t)j * n;
   unsigned long long inter = 0, uni = 0;
-  for (int64_t p = (int64_t)blockIdx.x * kTrackThreads + threadIdx.x; p < n;
-       p += (int64_t)gridDim.x * kTrackThreads) {
-    const bool va = a[p] > tau, vb = b[p] > tau;
+  auto add = [&](float x, float y) {
+    const bool va = x > tau, vb = y > tau;
     inter += (va && vb) ? 1u : 0u;
     uni += (va || vb) ? 1u : 0u;
+  };
+  // Four pixels per load where both images start on 16 bytes.
+  const bool vec = ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
+  const int64_t t = (int64_t)blockIdx.x * kTrackThreads + threadIdx.x,
+                step = (int64_t)gridDim.x * kTrackThreads, groups = vec ? n >> 2 : 0;
+  for (int64_t p = t; p < groups; p += step) {
+    const float4 x = reinterpret_cast<const float4*>(a)[p];
+    const float4 y = reinterpret_cast<const float4*>(b)[p];
+    add(x.x, y.x);
+    add(x.y, y.y);
+    add(x.z, y.z);
+    add(x.w, y.w);
   }
+  for (int64_t p = 4 * groups + t; p < n; p += step) add(a[p], b[p]);
   __shared__ unsigned long long s_i[kTrackThreads / 32], s_u[kTrackThreads / 32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -346,15 +484,18 @@ __global__ void covis_iou_kernel(int n_pairs, const unsigned long long* __restri
     iou[j] = counts[2 * j + 1] ? (float)((double)counts[2 * j] / (double)counts[2 * j + 1]) : 0.0f;
 }
 
-// Grid rows per view, columns enough to cover the largest view (at most 2 waves of blocks).
-dim3 view_grid(const Views& views) {
+// Grid rows per view, columns enough to cover the largest view four pixels a thread, at most
+// `waves` blocks per SM over all views.
+dim3 view_grid(const Views& views, int waves) {
   int max_px = 1;
   for (int v = 0; v < views.n_views; ++v)
     max_px = max(max_px, views.v[v].width * views.v[v].height);
   const int want = (max_px + kTrackThreads * 4 - 1) / (kTrackThreads * 4);
-  const int cap = max(1, 2 * 152 * 4 / views.n_views);
+  const int cap = max(1, waves * 152 / views.n_views);
   return dim3((unsigned)min(want, cap), (unsigned)views.n_views);
 }
+
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
 
@@ -368,7 +509,7 @@ cudaError_t launch_pose_prepare(const float* world_to_cam, int n_views, float* r
 
 cudaError_t launch_grad_weight(const Views& views, const float* obs, float tau_grad, float* w_out,
                                cudaStream_t stream) {
-  const cudaError_t e = launch_chained(grad_weight_kernel, view_grid(views), dim3(kTrackThreads),
+  const cudaError_t e = launch_chained(grad_weight_kernel, view_grid(views, 8), dim3(kTrackThreads),
                                        stream, views, obs, 1.0f / tau_grad, w_out);
   RGS_LAUNCHED();
   return e;
@@ -379,19 +520,23 @@ cudaError_t launch_track_loss(const Views& views, const float* color, const floa
                               bool fit_exposure, double* sums, float* d_color, double* loss,
                               float* gain_bias, cudaStream_t stream) {
   const int V = views.n_views;
-  cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(double) * 4 * V, stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, sizeof(double) * V, stream);
-  if (e != cudaSuccess) return e;
-  const dim3 grid = view_grid(views);
+  const dim3 grid = view_grid(views, kTrackBlocksPerSm);
+  const int vec = aligned16(color) && aligned16(alpha) && aligned16(obs) && aligned16(d_color) &&
+                  (!w_grad || aligned16(w_grad));
+  cudaError_t e;
   if (fit_exposure) {
-    e = launch_chained(track_sums_kernel, grid, dim3(kTrackThreads), stream, views, color, obs,
-                       sums);
-    RGS_LAUNCHED();
+    e = cudaMemsetAsync(sums, 0, sizeof(double) * 4 * V, stream);
     if (e != cudaSuccess) return e;
+    e = launch_chained(track_sums_kernel, grid, dim3(kTrackThreads), stream, views, color, obs,
+                       vec, sums, loss);
+    RGS_LAUNCHED();
+  } else {
+    e = cudaMemsetAsync(loss, 0, sizeof(double) * V, stream);
   }
+  if (e != cudaSuccess) return e;
   e = launch_chained(track_loss_kernel, grid, dim3(kTrackThreads), stream, views, color, alpha,
                      obs, w_grad, (const double*)sums, 1.0f / tau_alpha, fit_exposure ? 1 : 0,
-                     d_color, loss, gain_bias);
+                     vec, d_color, loss, gain_bias);
   RGS_LAUNCHED();
   return e;
 }
@@ -402,7 +547,7 @@ cudaError_t launch_covisibility(const float* alpha_a, const float* alpha_b, int6
   cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(unsigned long long) * 2 * n_pairs, stream);
   if (e != cudaSuccess || n_pairs == 0) return e;
   if (n > 0) {
-    const int64_t want = (n + kTrackThreads * 8 - 1) / (kTrackThreads * 8);
+    const int64_t want = (n + kTrackThreads * 4 - 1) / (kTrackThreads * 4);
     const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, 4 * 152 / n_pairs + 1));
     e = launch_chained(covis_count_kernel, dim3(gx, (unsigned)n_pairs), dim3(kTrackThreads),
                        stream, alpha_a, alpha_b, n, tau, counts);
@@ -418,8 +563,9 @@ cudaError_t launch_covisibility(const float* alpha_a, const float* alpha_b, int6
 cudaError_t launch_pose_adam(int n_views, float lr, float beta1, float beta2, float eps,
                              int iterations, const float* d_pose, float* adam_state,
                              int32_t* step, float* world_to_cam, cudaStream_t stream) {
-  const cudaError_t e = launch_chained(pose_adam_kernel, dim3(1), dim3(kMaxViews), stream,
-                                       n_views, lr, beta1, beta2, eps, iterations, d_pose,
+  const cudaError_t e = launch_chained(pose_adam_kernel, dim3(1),
+                                       dim3(32 * ((n_views + kAdamViews - 1) / kAdamViews)),
+                                       stream, n_views, lr, beta1, beta2, eps, iterations, d_pose,
                                        adam_state, step, world_to_cam);
   RGS_LAUNCHED();
   return e;

@@ -42,7 +42,7 @@ class MapRegularizer:
         ls = log_scales.detach().to(torch.float32).contiguous()
         lg = opacity_logits.detach().to(torch.float32).contiguous()
         keep = torch.empty(self.n, dtype=torch.uint8, device=ls.device)
-        n_keep = torch.zeros(1, dtype=torch.int32, device=ls.device)
+        n_keep = torch.empty(1, dtype=torch.int32, device=ls.device)
         self.ctx.prune_mask(self.n, ls.data_ptr(), lg.data_ptr(), self.obs_count.data_ptr(),
                             self.vis_score.data_ptr(), binding.default_prune_config(**bounds),
                             keep.data_ptr(), n_keep.data_ptr(), stream)
