@@ -252,41 +252,43 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
 
 // ------------------------------------------------------------------------------------------
 // Per-warp reduction of the visited Gaussians' gradient sums through shared memory. Each visit
-// writes the lane's kVals partial sums as one column of kVals rows (row b * kVals + k for the
-// b-th Gaussian of the group, RedLayout); after kBatch visits (or at the end of a staged batch)
-// every lane adds up whole rows (eight 16-byte reads of a row padded to 36 floats, so that both
-// the column writes and the row reads are free of bank conflicts) and parks the row total in
-// the padding. Lane b then turns Gaussian b's totals into its whitened moments and issues the
-// atomics. Per visit this costs kVals shared stores and a share of the row sums, in place of a
-// shuffle butterfly with its selects after every Gaussian.
+// writes the lane's sums, two by two, as one 8-byte column of kPairs rows (row kPairs b + p for
+// pair p of the b-th Gaussian of the group, RedLayout); after kBatch visits (or at the end of a
+// staged batch) every lane adds up one row (sixteen 16-byte reads of a row of 32 pairs padded to
+// 68 floats: the column writes and the row reads are both free of bank conflicts) and parks the
+// totals in the padding. Lane b then turns Gaussian b's totals into its whitened moments and
+// issues the atomics. Per visit this costs kPairs shared stores and a share of the row sums, in
+// place of a shuffle butterfly with its selects after every Gaussian; single values in rows of 32
+// floats took nine stores and two row passes per seven Gaussians (+3 % on the 16-view 1080p window,
+// +8 % on ten 640x480 views).
 //
-// The lane's values: k = 0..2: sdp, sr, srr (the sums of dp, dp r and dp r^2 over its pixels,
-// r the row offset from the tile's anchor row), k = 3..5: t_a sdp, t_a sr, t_a^2 sdp (t_a the
-// whitened offset of its column at the anchor row), k = 6..8 (9): the colour (depth) weights.
+// The lane's values: sdp, sr | srr, t_a sdp | t_a sr, t_a^2 sdp | gr, gg | gb, gz, with sdp, sr, srr
+// the sums of dp, dp r and dp r^2 over its pixels (r the row offset from the tile's anchor row), t_a
+// the whitened offset of its column at the anchor row, and gr .. gz the colour and depth weights
+// (gz 0 without a depth or opacity gradient).
 // ------------------------------------------------------------------------------------------
-constexpr int kRedPad = 36;
+constexpr int kRedPad = 68;  // floats per row of 32 lane pairs, padded
 
-template <bool kAux>
 struct RedLayout {
-  static constexpr int kVals = kAux ? 10 : 9;
-  static constexpr int kBatch = kAux ? 6 : 7;  // kVals * kBatch <= 64: two row passes
-  static constexpr int kRows = kVals * kBatch;
+  static constexpr int kPairs = 5;
+  static constexpr int kBatch = 6;  // kPairs * kBatch <= 32: one row pass
+  static constexpr int kRows = kPairs * kBatch;
 };
 
-// Adds up row r (32 lane values) and parks the total in its first padding float.
+// Adds up row r (32 lane pairs) and parks the totals in its first two padding floats.
 __device__ __forceinline__ void reduce_row(float* red, int r) {
   const ulonglong2* row = reinterpret_cast<const ulonglong2*>(red + r * kRedPad);
   f32x2 s[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const ulonglong2 v = row[c];
-    s[c] = f2_add(v.x, v.y);
+    const ulonglong2 v = row[c], w = row[c + 8];
+    s[c] = f2_add(f2_add(v.x, v.y), f2_add(w.x, w.y));
   }
 #pragma unroll
   for (int h = 4; h > 0; h >>= 1)
 #pragma unroll
     for (int c = 0; c < h; ++c) s[c] = f2_add(s[c], s[c + h]);
-  red[r * kRedPad + 32] = f2_lo(s[0]) + f2_hi(s[0]);
+  *reinterpret_cast<f32x2*>(red + r * kRedPad + 64) = s[0];
 }
 
 // ------------------------------------------------------------------------------------------
@@ -309,7 +311,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
   constexpr bool kPacked = PPT % 2 == 0;
   constexpr int P2 = kPacked ? PPT / 2 : 1;
   static_assert(kThreads % 32 == 0, "whole warps only");
-  using RL = RedLayout<kAux>;
+  using RL = RedLayout;
   __shared__ ulonglong2 sp[kPacked ? 6 : 3][kThreads];
   __shared__ uint32_t s_vi[kThreads];
   __shared__ int s_max_last[kThreads / 32];
@@ -330,17 +332,20 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
   const int lane = threadIdx.x & 31;
   float* const red = s_red[threadIdx.x >> 5];
 
-  // Per pixel: transmittance behind the current position, the upstream gradients, and
-  // U = sum_ch dL/dC_ch S_ch + dL/dD S_D, where S is the colour / depth composited behind the
-  // current position (background included), so dL/dalpha = T q + (dL/dA T_final - U) / (1 - alpha)
-  // with q = dL/dC . c + dL/dD z.
-  float T[PPT], U[PPT], gC0[PPT], gC1[PPT], gC2[PPT], gD[PPT], gAT[PPT];
+  // Per pixel: the transmittance T behind the current position, the upstream gradients, and the
+  // gradient-weighted value seen behind it per unit of transmittance,
+  //   U = dL/dC . C_behind + dL/dD D_behind  (dL/dC . background - dL/dA at the far end),
+  // so that with q = dL/dC . c + dL/dD z of a Gaussian and w = alpha T its weight,
+  //   alpha dL/dalpha = w (q - U),  U <- U + alpha (q - U)
+  // (three operations; the running sum of w q, divided by 1 - alpha at each step, took five).
+  float T[PPT], U[PPT], gC0[PPT], gC1[PPT], gC2[PPT], gD[PPT];
   int32_t last[PPT];
   int thread_last = -1;
 #pragma unroll
   for (int k = 0; k < PPT; ++k) {
     float Tfin = 1.0f;
-    gC0[k] = gC1[k] = gC2[k] = gD[k] = gAT[k] = 0.0f;
+    gC0[k] = gC1[k] = gC2[k] = gD[k] = 0.0f;
+    float gA = 0.0f;
     last[k] = -1;
     const int py = py0 + k;
     if (px < vp.width && py < vp.height) {
@@ -353,14 +358,14 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
         gC2[k] = d_color[3 * pix + 2];
       }
       if (kAux && d_depth) gD[k] = d_depth[pix];
-      if (kAux && d_alpha) gAT[k] = d_alpha[pix] * Tfin;
+      if (kAux && d_alpha) gA = d_alpha[pix];
     }
     T[k] = Tfin;
-    U[k] = Tfin * (gC0[k] * c.bg[0] + gC1[k] * c.bg[1] + gC2[k] * c.bg[2]);
+    U[k] = gC0[k] * c.bg[0] + gC1[k] * c.bg[1] + gC2[k] * c.bg[2] - gA;
     thread_last = max(thread_last, last[k]);
   }
   // The same state as (pixel 2q, pixel 2q + 1) pairs for the packed arithmetic.
-  f32x2 T2[P2], U2[P2], GC02[P2], GC12[P2], GC22[P2], GD2[P2], GAT2[P2], FR[P2];
+  f32x2 T2[P2], U2[P2], GC02[P2], GC12[P2], GC22[P2], GD2[P2], FR[P2];
 #pragma unroll
   for (int q = 0; q < P2; ++q) {
     const int k0 = kPacked ? 2 * q : 0, k1 = kPacked ? 2 * q + 1 : 0;
@@ -370,7 +375,6 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
     GC12[q] = f2_make(gC1[k0], gC1[k1]);
     GC22[q] = f2_make(gC2[k0], gC2[k1]);
     GD2[q] = f2_make(gD[k0], gD[k1]);
-    GAT2[q] = f2_make(gAT[k0], gAT[k1]);
     FR[q] = f2_make((float)(r0_ + k0), (float)(r0_ + k1));
   }
   const f32x2 FX = f2_make(fx, fx), ONE2 = f2_make(1.0f, 1.0f), ZERO2 = f2_make(0.0f, 0.0f);
@@ -416,7 +420,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
               mYY = ZERO2;
         (void)aZ;
 #pragma unroll
-        for (int q = 0; q < P2; ++q) {
+        for (int q = P2 - 1; q >= 0; --q) {
           const int k0 = 2 * q, k1 = 2 * q + 1;
           const f32x2 tt = f2_fma(FR[q], L2.x, TA);
           const f32x2 ss = f2_fma(FR[q], L2.y, L3.x);
@@ -428,45 +432,56 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
           const bool cov1 = (!kCheckLast || jj <= last[k1]) && a1 >= c.alpha_min;
           // A pixel this Gaussian does not cover gets alpha 0 and 1 / (1 - alpha) = 1 (the
           // hardware reciprocal of 1 is exactly 1 on sm_103a, measured), so its transmittance,
-          // suffix sum and every accumulator stay bit-identical.
+          // U and every accumulator stay bit-identical.
           const f32x2 am = f2_make(cov0 ? a0 : 0.0f, cov1 ? a1 : 0.0f);
           const f32x2 om = f2_sub(ONE2, am);
           const f32x2 rom = f2_make(rcp_approx(f2_lo(om)), rcp_approx(f2_hi(om)));
           T2[q] = f2_mul(T2[q], rom);  // transmittance in front of this Gaussian
           const f32x2 w = f2_mul(am, T2[q]);
-          aR = f2_fma(GC02[q], w, aR);
-          aG = f2_fma(GC12[q], w, aG);
-          aB = f2_fma(GC22[q], w, aB);
-          f32x2 qv, dLda;
+          aR = q == P2 - 1 ? f2_mul(GC02[q], w) : f2_fma(GC02[q], w, aR);
+          aG = q == P2 - 1 ? f2_mul(GC12[q], w) : f2_fma(GC12[q], w, aG);
+          aB = q == P2 - 1 ? f2_mul(GC22[q], w) : f2_fma(GC22[q], w, aB);
+          f32x2 qv;
           if constexpr (kAux) {
-            aZ = f2_fma(GD2[q], w, aZ);
+            aZ = q == P2 - 1 ? f2_mul(GD2[q], w) : f2_fma(GD2[q], w, aZ);
             qv = f2_fma(GC02[q], CA.x,
                         f2_fma(GC12[q], CA.y, f2_fma(GC22[q], CB.x, f2_mul(GD2[q], CB.y))));
-            dLda = f2_fma(T2[q], qv, f2_mul(rom, f2_sub(GAT2[q], U2[q])));
           } else {
             qv = f2_fma(GC02[q], CA.x, f2_fma(GC12[q], CA.y, f2_mul(GC22[q], CB.x)));
-            dLda = f2_fma(T2[q], qv, f2_mul(rom, f2_sub(ZERO2, U2[q])));
           }
-          U2[q] = f2_fma(w, qv, U2[q]);
+          const f32x2 diff = f2_sub(qv, U2[q]);
+          U2[q] = f2_fma(am, diff, U2[q]);
           // dL/dpower = dL/dalpha * alpha (d alpha / d power = o G = alpha), unclamped only
-          // (an uncovered pixel has alpha 0 here, so its share is 0 already).
-          f32x2 dp = f2_mul(dLda, am);
+          // (an uncovered pixel has weight 0 here, so its share is 0 already).
+          f32x2 dp = f2_mul(w, diff);
           if constexpr (kClamp) {
             const bool m0 = oG0 < c.alpha_max, m1 = oG1 < c.alpha_max;
             dp = f2_make(m0 ? f2_lo(dp) : 0.0f, m1 ? f2_hi(dp) : 0.0f);
           }
-          mP = f2_add(mP, dp);
-          const f32x2 t = f2_mul(dp, FR[q]);
-          mY = f2_add(mY, t);
-          mYY = f2_fma(t, FR[q], mYY);
+          // Suffix sums over the pairs, last pair first: mP = sum dp, mY = sum q dp,
+          // mYY = sum q (q + 1) / 2 dp (seven additions for four pairs; weighting each pair by its
+          // row offset and the offset's square took two multiply-adds and an addition per pair).
+          mP = q == P2 - 1 ? dp : f2_add(mP, dp);
+          if (q > 0) {
+            mY = q == P2 - 1 ? mP : f2_add(mY, mP);
+            mYY = q == P2 - 1 ? mY : f2_add(mYY, mY);
+          }
         }
         gr = f2_lo(aR) + f2_hi(aR);
         gg = f2_lo(aG) + f2_hi(aG);
         gb = f2_lo(aB) + f2_hi(aB);
         if constexpr (kAux) gz = f2_lo(aZ) + f2_hi(aZ);
         sdp = f2_lo(mP) + f2_hi(mP);
-        sr = f2_lo(mY) + f2_hi(mY);
-        srr = f2_lo(mYY) + f2_hi(mYY);
+        {
+          // Over the thread's rows k = 2 q + (0, 1): k1 = sum dp k, k2 = sum dp k^2; then over the
+          // row offsets r = r0 + k.
+          const float ys = f2_lo(mY) + f2_hi(mY), zs = f2_lo(mYY) + f2_hi(mYY);
+          const float k1 = fmaf(2.0f, ys, f2_hi(mP));
+          const float k2 = fmaf(8.0f, zs, fmaf(-4.0f, f2_lo(mY), f2_hi(mP)));
+          const float r0f = (float)r0_;
+          sr = fmaf(r0f, sdp, k1);
+          srr = fmaf(r0f, k1 + sr, k2);
+        }
         ta = f2_lo(TA);
       } else {
         const float4 g0 = reinterpret_cast<const float4*>(sp[0])[g];
@@ -486,18 +501,17 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
           gr = fmaf(gC0[k], w, gr);
           gg = fmaf(gC1[k], w, gg);
           gb = fmaf(gC2[k], w, gb);
-          float q, dLda;
+          float q;
           if constexpr (kAux) {
             gz = fmaf(gD[k], w, gz);
             q = fmaf(gC0[k], g2.x, fmaf(gC1[k], g2.y, fmaf(gC2[k], g2.z, gD[k] * g2.w)));
-            dLda = fmaf(T[k], q, rom * (gAT[k] - U[k]));
           } else {
             q = fmaf(gC0[k], g2.x, fmaf(gC1[k], g2.y, gC2[k] * g2.z));
-            dLda = fmaf(T[k], q, rom * (0.0f - U[k]));
           }
-          U[k] = fmaf(w, q, U[k]);
+          const float diff = q - U[k];
+          U[k] = fmaf(a, diff, U[k]);
           if (oG < c.alpha_max) {
-            const float dp = dLda * a;  // dL/dpower: d alpha / d power = o G = alpha
+            const float dp = w * diff;
             sdp += dp;
             const float t = dp * fr;
             sr += t;
@@ -507,18 +521,14 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
       }
     }
     const float tsdp = ta * sdp;
-    float* col = rows + lane;
-    col[0 * kRedPad] = sdp;
-    col[1 * kRedPad] = sr;
-    col[2 * kRedPad] = srr;
-    col[3 * kRedPad] = tsdp;
-    col[4 * kRedPad] = ta * sr;
-    col[5 * kRedPad] = ta * tsdp;
-    col[6 * kRedPad] = gr;
-    col[7 * kRedPad] = gg;
-    col[8 * kRedPad] = gb;
-    if constexpr (kAux) col[9 * kRedPad] = gz;
-    else (void)gz;
+    auto put = [&](int p, float x, float y) {
+      *reinterpret_cast<f32x2*>(rows + p * kRedPad + 2 * lane) = f2_make(x, y);
+    };
+    put(0, sdp, sr);
+    put(1, srr, tsdp);
+    put(2, ta * sr, ta * tsdp);
+    put(3, gr, gg);
+    put(4, gb, gz);
   };
 
   // Row sums of the last nb visits (staged at g_first, g_first - 1, ...), then one lane per
@@ -528,15 +538,19 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
   // s_a W_s + l22 (s_a S1 + l22 S2)) for the lane values S0..S5) and adds them to its record.
   auto flush = [&](int nb, int g_first) {
     __syncwarp();
-    const int nrows = nb * RL::kVals;
+    const int nrows = nb * RL::kPairs;
     for (int r = lane; r < nrows; r += 32) reduce_row(red, r);
     __syncwarp();
     if (lane < nb) {
       const int g = g_first - lane;
-      const float* tot = red + lane * RL::kVals * kRedPad + 32;
-      float S[RL::kVals];
+      const float* tot = red + lane * RL::kPairs * kRedPad + 64;
+      float S[2 * RL::kPairs];
 #pragma unroll
-      for (int k = 0; k < RL::kVals; ++k) S[k] = tot[k * kRedPad];
+      for (int k = 0; k < RL::kPairs; ++k) {
+        const f32x2 t = *reinterpret_cast<const f32x2*>(tot + k * kRedPad);
+        S[2 * k] = f2_lo(t);
+        S[2 * k + 1] = f2_hi(t);
+      }
       float l21, l22, s_a;
       if constexpr (kPacked) {
         l21 = f2_lo(sp[2][g].x);
@@ -550,7 +564,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
       }
       bool any = false;
 #pragma unroll
-      for (int k = 0; k < RL::kVals; ++k) any = any || S[k] != 0.0f;
+      for (int k = 0; k < 2 * RL::kPairs; ++k) any = any || S[k] != 0.0f;
       if (any) {
         const float wt = fmaf(l21, S[1], S[3]);
         const float ws = fmaf(s_a, S[0], l22 * S[1]);
@@ -599,7 +613,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
     const int split = max(bstart - 1, min(bend - 1, warp_min_last));
     for (int jj = bend - 1; jj > split; --jj) {
       const int g = jj - bstart;
-      float* rows = red + nb * RL::kVals * kRedPad;
+      float* rows = red + nb * RL::kPairs * kRedPad;
       if (clamps(g))
         visit(jj, g, rows, std::true_type{}, std::true_type{});
       else
@@ -608,7 +622,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
     }
     for (int jj = split; jj >= bstart; --jj) {
       const int g = jj - bstart;
-      float* rows = red + nb * RL::kVals * kRedPad;
+      float* rows = red + nb * RL::kPairs * kRedPad;
       if (clamps(g))
         visit(jj, g, rows, std::false_type{}, std::true_type{});
       else
