@@ -14,7 +14,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "rgs_internal.cuh"
 
@@ -22,9 +21,6 @@ namespace rgs {
 namespace {
 
 constexpr int kTrackThreads = 256;
-// Blocks per SM of the two loss passes: enough loads in flight, and few double-precision atomics
-// on each view's sums.
-constexpr int kTrackBlocksPerSm = 4;
 
 // ------------------------------------------------------------------------------------------
 // Pose records: R (9), t (3), c = -R^T t (3), pad. The centre is accumulated in double and
@@ -101,26 +97,35 @@ __global__ void __launch_bounds__(kTrackThreads) grad_weight_kernel(
   }
 }
 
-// The pixels of view v dealt out over the blocks of grid row v: `four(p)` for groups of four
-// pixels that start at a multiple of four in the concatenated images (their colours are then three
-// aligned 16-byte words), `one(p)` for the pixels before and after them; `one` for all when the
-// arrays are not 16-byte aligned (vec 0).
+// ------------------------------------------------------------------------------------------
+// The two loss passes walk the images four consecutive pixels a thread: kLossThreads threads take
+// kTrackThreads pixels of a row of blocks at a time, so that a colour quadruple is three 16-byte
+// words (where the quadruple starts on 16 bytes). Each of the four keeps its own FP32 partial sums,
+// and a group of eight threads adds its 32 as a warp with one pixel per thread would (offsets 16,
+// 8, 4 across the threads, 2 and 1 inside), so every sum is the same float as pixel by pixel; FP64
+// from there on.
+// ------------------------------------------------------------------------------------------
+constexpr int kLossThreads = kTrackThreads / 4;
+
+// Calls one(p, e) for every pixel p (index e of its quadruple) or four(p) for whole quadruples
+// that start on 16 bytes (vec: the arrays do).
 template <typename One, typename Four>
-__device__ __forceinline__ void for_pixels(const Views& views, int v, int vec, One&& one,
-                                           Four&& four) {
+__device__ __forceinline__ void for_quads(const Views& views, int v, int vec, One&& one,
+                                          Four&& four) {
   long long first;
   int count, W, H;
   view_pixels(views, v, first, count, W, H);
-  const int t = blockIdx.x * kTrackThreads + threadIdx.x, step = gridDim.x * kTrackThreads;
-  int head = count, groups = 0;
-  if (vec) {
-    head = min((int)(-first & 3), count);
-    groups = (count - head) >> 2;
+  const bool wide = vec && (first & 3) == 0;
+  for (int k = 4 * (blockIdx.x * kLossThreads + threadIdx.x); k < count;
+       k += gridDim.x * kTrackThreads) {
+    if (wide && k + 3 < count) {
+      four(first + k);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (k + e < count) one(first + k + e, e);
+    }
   }
-  for (int k = t; k < groups; k += step) four(first + head + 4ll * k);
-  // At most six pixels are left with groups, all of them without.
-  const int rest = count - 4 * groups;
-  for (int k = t; k < rest; k += step) one(first + (k < head ? k : k + 4 * groups));
 }
 
 __device__ __forceinline__ void load12(const float* __restrict__ p, float (&x)[12]) {
@@ -134,82 +139,63 @@ __device__ __forceinline__ void load12(const float* __restrict__ p, float (&x)[1
   }
 }
 
-// A sum of floats as an unevaluated pair, each addition exact to about 2^-48 of the sum (Knuth's
-// two-sum): the partial sums lose nothing to their length, and, unlike doubles, cost a handful of
-// FP32 operations (a double addition costs a warp 64 cycles).
-struct PairSum {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float x) {
-    float e;
-    two_sum(hi, x, hi, e);
-    lo = __fadd_rn(lo, e);
-  }
-  __device__ __forceinline__ void add(float h, float l) {
-    add(h);
-    lo = __fadd_rn(lo, l);
-  }
-};
-
-// Block-wide sum of NV pair sums per thread into (double) accumulators with atomics.
+// Block-wide sums of NV values of each of a thread's four pixels, into (double) accumulators with
+// atomics.
 template <int NV>
-__device__ __forceinline__ void block_sum_to(PairSum (&x)[NV], double* __restrict__ acc) {
-  __shared__ double s_part[kTrackThreads / 32][NV];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void block_sum_to(const float (&x)[4][NV], double* __restrict__ acc) {
+  constexpr int kGroups = kLossThreads / 8;
+  __shared__ double s_part[kGroups][NV];
 #pragma unroll
   for (int j = 0; j < NV; ++j) {
+    float q[4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float h = __shfl_xor_sync(0xffffffffu, x[j].hi, o);
-      const float l = __shfl_xor_sync(0xffffffffu, x[j].lo, o);
-      x[j].add(h, l);
+    for (int e = 0; e < 4; ++e) {
+      q[e] = x[e][j];
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) q[e] += __shfl_xor_sync(0xffffffffu, q[e], o);
     }
-    if (lane == 0) s_part[warp][j] = (double)x[j].hi + (double)x[j].lo;
+    const float sum = (q[0] + q[2]) + (q[1] + q[3]);
+    if ((threadIdx.x & 7) == 0) s_part[threadIdx.x >> 3][j] = (double)sum;
   }
   __syncthreads();
   if (threadIdx.x < NV) {
     double t = 0.0;
 #pragma unroll
-    for (int w = 0; w < kTrackThreads / 32; ++w) t += s_part[w][threadIdx.x];
+    for (int g = 0; g < kGroups; ++g) t += s_part[g][threadIdx.x];
     atomicAdd(acc + threadIdx.x, t);
   }
 }
 
 // ------------------------------------------------------------------------------------------
 // Exposure fit, pass 1 (Eq. app-ls): per view, sum r, sum r^2, sum o, sum r o over the three
-// channels of every pixel (r rendered, o observed). Four pixels are summed in FP32, everything from
-// there on in pair sums, and FP64 from the warp totals on.
+// channels of every pixel (r rendered, o observed).
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kTrackThreads) track_sums_kernel(
+__global__ void __launch_bounds__(kLossThreads) track_sums_kernel(
     const __grid_constant__ Views views, const float* __restrict__ color,
     const float* __restrict__ obs, int vec, double* __restrict__ sums,
     double* __restrict__ loss) {
   chain_wait();
   const int v = blockIdx.y;
   if (blockIdx.x == 0 && threadIdx.x == 0) loss[v] = 0.0;  // for the next pass
-  PairSum x[4];
-  // The sums of a few values, added to the thread's.
-  auto add = [&](const float* r, const float* o, auto count) {
-    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-    for (int e = 0; e < decltype(count)::value; ++e) {
-      s[0] += r[e];
-      s[1] = fmaf(r[e], r[e], s[1]);
-      s[2] += o[e];
-      s[3] = fmaf(r[e], o[e], s[3]);
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) x[q].add(s[q]);
+  float x[4][4] = {};
+  auto add = [](float (&s)[4], float r, float o) {
+    s[0] += r;
+    s[1] = fmaf(r, r, s[1]);
+    s[2] += o;
+    s[3] = fmaf(r, o, s[3]);
   };
-  for_pixels(
+  for_quads(
       views, v, vec,
-      [&](long long p) {
-        add(color + 3 * p, obs + 3 * p, std::integral_constant<int, 3>{});
+      [&](long long p, int e) {
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) add(x[e], color[3 * p + ch], obs[3 * p + ch]);
       },
       [&](long long p) {
         float r[12], o[12];
         load12(color + 3 * p, r);
         load12(obs + 3 * p, o);
-        add(r, o, std::integral_constant<int, 12>{});
+#pragma unroll
+        for (int e = 0; e < 12; ++e) add(x[e / 3], r[e], o[e]);
       });
   block_sum_to<4>(x, sums + 4 * v);
 }
@@ -241,7 +227,7 @@ __device__ __forceinline__ void exposure_of(const double* s, double n, bool fit,
 // with (g, b) and w held fixed (they are re-estimated from every render, and no gradient flows
 // into them). Writes the upstream colour gradient, the loss per view and (g, b) per view.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kTrackThreads) track_loss_kernel(
+__global__ void __launch_bounds__(kLossThreads) track_loss_kernel(
     const __grid_constant__ Views views, const float* __restrict__ color,
     const float* __restrict__ alpha, const float* __restrict__ obs,
     const float* __restrict__ w_grad, const double* __restrict__ sums, float inv_tau_alpha,
@@ -264,9 +250,10 @@ __global__ void __launch_bounds__(kTrackThreads) track_loss_kernel(
   }
   __syncthreads();
   const float g = s_fit[0], b = s_fit[1];
-  PairSum part[1];
-  // One pixel's gradient, and its share of the loss, from its residuals (r rendered, o observed).
-  auto pixel = [&](float a, float wg, const float* r, const float* o, float* d) {
+  float part[4][1] = {};
+  // Pixel e of the quadruple: gradient and share of the loss, from its residuals (r rendered, o
+  // observed).
+  auto pixel = [&](int e, float a, float wg, const float* r, const float* o, float* d) {
     const float w = fminf(fmaxf(a * inv_tau_alpha, 0.0f), 1.0f) * wg;
     float l1 = 0.0f;
 #pragma unroll
@@ -276,18 +263,18 @@ __global__ void __launch_bounds__(kTrackThreads) track_loss_kernel(
       const float sg = res > 0.0f ? 1.0f : (res < 0.0f ? -1.0f : 0.0f);
       d[ch] = -w * g * sg;
     }
-    return w * l1;
+    part[e][0] = fmaf(w, l1, part[e][0]);
   };
-  for_pixels(
+  for_quads(
       views, v, vec,
-      [&](long long p) {
+      [&](long long p, int e) {
         float r[3], o[3], d[3];
 #pragma unroll
         for (int ch = 0; ch < 3; ++ch) {
           r[ch] = color[3 * p + ch];
           o[ch] = obs[3 * p + ch];
         }
-        part[0].add(pixel(alpha[p], w_grad ? w_grad[p] : 1.0f, r, o, d));
+        pixel(e, alpha[p], w_grad ? w_grad[p] : 1.0f, r, o, d);
 #pragma unroll
         for (int ch = 0; ch < 3; ++ch) d_color[3 * p + ch] = d[ch];
       },
@@ -298,9 +285,10 @@ __global__ void __launch_bounds__(kTrackThreads) track_loss_kernel(
         const float4 a = *reinterpret_cast<const float4*>(alpha + p);
         const float4 wg = w_grad ? *reinterpret_cast<const float4*>(w_grad + p)
                                  : make_float4(1.0f, 1.0f, 1.0f, 1.0f);
-        const float l01 = pixel(a.x, wg.x, r, o, d) + pixel(a.y, wg.y, r + 3, o + 3, d + 3);
-        const float l23 = pixel(a.z, wg.z, r + 6, o + 6, d + 6) + pixel(a.w, wg.w, r + 9, o + 9, d + 9);
-        part[0].add(l01 + l23);
+        pixel(0, a.x, wg.x, r, o, d);
+        pixel(1, a.y, wg.y, r + 3, o + 3, d + 3);
+        pixel(2, a.z, wg.z, r + 6, o + 6, d + 6);
+        pixel(3, a.w, wg.w, r + 9, o + 9, d + 9);
         float4* out = reinterpret_cast<float4*>(d_color + 3 * p);
         out[0] = make_float4(d[0], d[1], d[2], d[3]);
         out[1] = make_float4(d[4], d[5], d[6], d[7]);
@@ -484,14 +472,14 @@ __global__ void covis_iou_kernel(int n_pairs, const unsigned long long* __restri
     iou[j] = counts[2 * j + 1] ? (float)((double)counts[2 * j] / (double)counts[2 * j + 1]) : 0.0f;
 }
 
-// Grid rows per view, columns enough to cover the largest view four pixels a thread, at most
-// `waves` blocks per SM over all views.
-dim3 view_grid(const Views& views, int waves) {
+// Grid rows per view, columns enough to cover the largest view (at most 2 waves of blocks). The
+// loss passes' partial sums follow this grid.
+dim3 view_grid(const Views& views) {
   int max_px = 1;
   for (int v = 0; v < views.n_views; ++v)
     max_px = max(max_px, views.v[v].width * views.v[v].height);
   const int want = (max_px + kTrackThreads * 4 - 1) / (kTrackThreads * 4);
-  const int cap = max(1, waves * 152 / views.n_views);
+  const int cap = max(1, 2 * 152 * 4 / views.n_views);
   return dim3((unsigned)min(want, cap), (unsigned)views.n_views);
 }
 
@@ -509,7 +497,7 @@ cudaError_t launch_pose_prepare(const float* world_to_cam, int n_views, float* r
 
 cudaError_t launch_grad_weight(const Views& views, const float* obs, float tau_grad, float* w_out,
                                cudaStream_t stream) {
-  const cudaError_t e = launch_chained(grad_weight_kernel, view_grid(views, 8), dim3(kTrackThreads),
+  const cudaError_t e = launch_chained(grad_weight_kernel, view_grid(views), dim3(kTrackThreads),
                                        stream, views, obs, 1.0f / tau_grad, w_out);
   RGS_LAUNCHED();
   return e;
@@ -520,21 +508,21 @@ cudaError_t launch_track_loss(const Views& views, const float* color, const floa
                               bool fit_exposure, double* sums, float* d_color, double* loss,
                               float* gain_bias, cudaStream_t stream) {
   const int V = views.n_views;
-  const dim3 grid = view_grid(views, kTrackBlocksPerSm);
+  const dim3 grid = view_grid(views);
   const int vec = aligned16(color) && aligned16(alpha) && aligned16(obs) && aligned16(d_color) &&
                   (!w_grad || aligned16(w_grad));
   cudaError_t e;
   if (fit_exposure) {
     e = cudaMemsetAsync(sums, 0, sizeof(double) * 4 * V, stream);
     if (e != cudaSuccess) return e;
-    e = launch_chained(track_sums_kernel, grid, dim3(kTrackThreads), stream, views, color, obs,
+    e = launch_chained(track_sums_kernel, grid, dim3(kLossThreads), stream, views, color, obs,
                        vec, sums, loss);
     RGS_LAUNCHED();
   } else {
     e = cudaMemsetAsync(loss, 0, sizeof(double) * V, stream);
   }
   if (e != cudaSuccess) return e;
-  e = launch_chained(track_loss_kernel, grid, dim3(kTrackThreads), stream, views, color, alpha,
+  e = launch_chained(track_loss_kernel, grid, dim3(kLossThreads), stream, views, color, alpha,
                      obs, w_grad, (const double*)sums, 1.0f / tau_alpha, fit_exposure ? 1 : 0,
                      vec, d_color, loss, gain_bias);
   RGS_LAUNCHED();
