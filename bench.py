@@ -51,7 +51,7 @@ L2_FLUSH_BYTES = 256 << 20
 # recovery and screen-space gradients, 40 FP32 operations (plus two MUFU operations and the
 # atomics after the warp reduction).
 # Sorts of at least this many pairs take the library's wide radix passes (9-bit digits).
-WIDE_SORT_MIN_PAIRS = 4 << 20
+WIDE_SORT_MIN_PAIRS = 1 << 20
 FWD_FLOP_PER_EVAL = 15
 BWD_FLOP_PER_EVAL = 40
 

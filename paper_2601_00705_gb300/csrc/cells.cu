@@ -49,8 +49,7 @@ __device__ __forceinline__ uint32_t cell_key(uint32_t cell, uint32_t mask) {
 template <bool kMasks, int ITEMS>
 __global__ void __launch_bounds__(kEmitThreads) emit_cells_kernel(
     const __grid_constant__ Views views, int n, const uint32_t* __restrict__ order,
-    const uint2* __restrict__ touched, const float4* __restrict__ rec0,
-    const float4* __restrict__ rec1, float log2_alpha_min, uint32_t visible_cap,
+    const Record* __restrict__ rec, float log2_alpha_min, uint32_t visible_cap,
     uint32_t capacity, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, Lookback lb,
     uint32_t n_blocks, Counters* __restrict__ counters) {
   chain_wait();
@@ -77,7 +76,7 @@ __global__ void __launch_bounds__(kEmitThreads) emit_cells_kernel(
   for (int j = 0; j < ITEMS; ++j) vi[j] = first + 32u * j < n_visible ? order[first + 32u * j] : 0u;
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) {
-    const uint2 t = first + 32u * j < n_visible ? touched[vi[j]] : make_uint2(0u, 0u);
+    const uint2 t = first + 32u * j < n_visible ? rec[vi[j]].touched : make_uint2(0u, 0u);
     tiles += t.x;
     total[j] = __reduce_add_sync(0xffffffffu, t.y);
     sum += total[j];
@@ -126,7 +125,7 @@ __global__ void __launch_bounds__(kEmitThreads) emit_cells_kernel(
       const ViewParams& vp = views.v[my_vi / (uint32_t)max(n, 1)];
       cell_base = vp.cell_base;
       cells_x = vp.cells_x;
-      if (make_ellipse(rec0[my_vi], rec1[my_vi], log2_alpha_min, e) &&
+      if (make_ellipse(rec[my_vi].mean, rec[my_vi].conic, log2_alpha_min, e) &&
           tc.init(e, views.tile_w, views.tile_h, vp.tiles_x, vp.tiles_y))
         rows = (uint32_t)((tc.ty1 >> kCellShift) - (tc.ty0 >> kCellShift) + 1);
     }
@@ -250,15 +249,15 @@ __device__ __forceinline__ int tile_of(const CellPlace& p, int t) {
 // Tile mask of list entry (key, vi) in the cell.
 template <bool kMasks>
 __device__ __forceinline__ uint32_t entry_mask(const Views& views, const CellPlace& p,
-                                               uint32_t key, uint32_t vi, const float4* rec0,
-                                               const float4* rec1, float log2_alpha_min) {
+                                               uint32_t key, uint32_t vi, const Record* rec,
+                                               float log2_alpha_min) {
   if constexpr (kMasks) {
     return key & 0xffffu;
   } else {
     Ellipse e;
     TileCover tc;
     CellRow row;
-    if (!make_ellipse(rec0[vi], rec1[vi], log2_alpha_min, e) ||
+    if (!make_ellipse(rec[vi].mean, rec[vi].conic, log2_alpha_min, e) ||
         !tc.init(e, views.tile_w, views.tile_h, p.vp->tiles_x, p.vp->tiles_y) ||
         !cell_row(tc, p.cy, row))
       return 0u;
@@ -284,7 +283,7 @@ template <bool kMasks>
 __global__ void __launch_bounds__(kCellThreads) cell_count_kernel(
     const __grid_constant__ Views views, const uint2* __restrict__ cell_ranges,
     const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals,
-    const float4* __restrict__ rec0, const float4* __restrict__ rec1, float log2_alpha_min,
+    const Record* __restrict__ rec, float log2_alpha_min,
     uint32_t* __restrict__ tile_counts, uint32_t* __restrict__ class_sizes) {
   chain_wait();
   __shared__ uint32_t s_mask[2][kCellThreads];  // the chunk in use and the next
@@ -294,8 +293,8 @@ __global__ void __launch_bounds__(kCellThreads) cell_count_kernel(
   const uint2 range = cell_ranges[blockIdx.x];
   uint32_t n0 = 0, n1 = 0;
   auto load = [&](uint32_t p) {
-    return p < range.y ? entry_mask<kMasks>(views, place, keys[p], kMasks ? 0u : vals[p], rec0,
-                                            rec1, log2_alpha_min)
+    return p < range.y ? entry_mask<kMasks>(views, place, keys[p], kMasks ? 0u : vals[p], rec,
+                                            log2_alpha_min)
                        : 0u;
   };
   uint32_t m = load(range.x + threadIdx.x);
@@ -333,7 +332,7 @@ template <bool kMasks>
 __global__ void __launch_bounds__(kCellThreads) cell_expand_kernel(
     const __grid_constant__ Views views, const uint2* __restrict__ cell_ranges,
     const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals,
-    const float4* __restrict__ rec0, const float4* __restrict__ rec1, float log2_alpha_min,
+    const Record* __restrict__ rec, float log2_alpha_min,
     const uint32_t* __restrict__ tile_counts, const uint2* __restrict__ ranges,
     uint32_t* __restrict__ pairs, uint32_t capacity, const uint32_t* __restrict__ class_sizes,
     uint32_t* __restrict__ class_taken, uint32_t* __restrict__ tile_order,
@@ -369,7 +368,7 @@ __global__ void __launch_bounds__(kCellThreads) cell_expand_kernel(
     m = val = 0;
     if (p < range.y) {
       val = vals[p];
-      m = entry_mask<kMasks>(views, place, kMasks ? keys[p] : 0u, val, rec0, rec1, log2_alpha_min);
+      m = entry_mask<kMasks>(views, place, kMasks ? keys[p] : 0u, val, rec, log2_alpha_min);
     }
   };
   load(range.x + threadIdx.x);
@@ -408,8 +407,7 @@ int64_t max_emit_blocks(int64_t visible) {
 int order_words() { return 2 * kOrderClasses; }
 
 cudaError_t launch_emit_cells(const Views& views, int n, const uint32_t* order,
-                              const uint2* touched, const float4* rec0, const float4* rec1,
-                              float log2_alpha_min, int64_t visible_cap, uint32_t capacity,
+                              const Record* rec, float log2_alpha_min, int64_t visible_cap, uint32_t capacity,
                               uint32_t* keys, uint32_t* vals, Lookback lb, Counters* counters,
                               cudaStream_t stream) {
   const int64_t blocks = emit_blocks(visible_cap);
@@ -425,7 +423,7 @@ cudaError_t launch_emit_cells(const Views& views, int n, const uint32_t* order,
                       : (masks ? emit_cells_kernel<true, kEmitItems>
                                : emit_cells_kernel<false, kEmitItems>);
     e = launch_chained(kernel, dim3((unsigned)blocks), dim3(kEmitThreads), stream, views, n, order,
-                       touched, rec0, rec1, log2_alpha_min,
+                       rec, log2_alpha_min,
                        (uint32_t)std::min<int64_t>(visible_cap, 0xffffffffll), capacity, keys,
                        vals, lb, (uint32_t)blocks, counters);
   }
@@ -446,15 +444,14 @@ cudaError_t launch_cell_ranges(const Views& views, const uint32_t* keys, int64_t
 }
 
 cudaError_t launch_tile_lists(const Views& views, const uint2* cell_ranges, const uint32_t* keys,
-                              const uint32_t* vals, const float4* rec0, const float4* rec1,
-                              float log2_alpha_min, uint32_t* tile_counts, uint2* ranges,
+                              const uint32_t* vals, const Record* rec, float log2_alpha_min, uint32_t* tile_counts, uint2* ranges,
                               uint32_t* pairs, uint32_t capacity, uint32_t* order_words,
                               uint32_t* tile_order, Lookback lb, Counters* counters,
                               cudaStream_t stream) {
   const dim3 grid(views.total_cells), block(kCellThreads);
   const bool masks = cells_masked(views.total_cells);
   cudaError_t e = launch_chained(masks ? cell_count_kernel<true> : cell_count_kernel<false>, grid,
-                                 block, stream, views, cell_ranges, keys, vals, rec0, rec1,
+                                 block, stream, views, cell_ranges, keys, vals, rec,
                                  log2_alpha_min, tile_counts, order_words);
   RGS_LAUNCHED();
   if (e == cudaSuccess)
@@ -462,7 +459,7 @@ cudaError_t launch_tile_lists(const Views& views, const uint2* cell_ranges, cons
                                 &counters->n_pairs_listed, lb, stream);
   if (e == cudaSuccess) {
     e = launch_chained(masks ? cell_expand_kernel<true> : cell_expand_kernel<false>, grid, block,
-                       stream, views, cell_ranges, keys, vals, rec0, rec1, log2_alpha_min,
+                       stream, views, cell_ranges, keys, vals, rec, log2_alpha_min,
                        (const uint32_t*)tile_counts, (const uint2*)ranges, pairs, capacity,
                        (const uint32_t*)order_words, order_words + kOrderClasses, tile_order,
                        counters);

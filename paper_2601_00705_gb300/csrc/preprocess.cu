@@ -286,29 +286,76 @@ __device__ __forceinline__ void load_sh(const float* __restrict__ sh, int i, flo
   }
 }
 
-// Forward, pass 1 (cull): one thread per (Gaussian, chunk of views). Only the camera-space mean,
-// the projected centre and the footprint-radius bound of project_view are computed, and the
-// entries that may touch the image are appended to `cand` (gathered in
-// shared memory, then one global atomic per block; their order does not matter). Pass 2 then
-// projects only those, so its warps are not held up by the large majority of entries that fall
-// outside the image.
+// Forward, pass 1 (cull): one thread per (Gaussian, chunk of views). The entries that may touch the
+// image are appended to `cand` (gathered per warp in shared memory, then one global atomic per
+// block; their order does not matter). Pass 2 then projects only those, so its warps are not held
+// up by the large majority of entries that fall outside the image.
+//
+// The pass is bound by instruction issue, so an entry is tested by planes: with
+// (x, y, z) = R m + t, the centre lies at pixel (fx x / z + cx, fy y / z + cy), and the
+// alpha >= alpha_min footprint reaches at most
+//   rad = sqrt(kappa (|J|_F^2 smax^2 + eps)) <= sqrt(kappa) (F smax / z + sqrt(eps)),
+// since the largest eigenvalue of Sigma^I is at most |J|_F^2 smax^2 + eps and |J|_F <= F / z with
+// F^2 = fx^2 (1 + lim_u^2) + fy^2 (1 + lim_w^2) for the guard-banded J. Times z > 0, "mx + rad < 0"
+// and its three siblings become linear in m and z, with no division or square root per entry:
+// three dot products and four comparisons (about 20 instructions; the exact radius took 60: 137 us
+// for 24 views of a million Gaussians, 258 us for 16 of three). rad is widened by 2 % and 4 px,
+// beyond the 1-px padding of the tile coverage and the rounding here. Without a guard band |J|_F
+// has no such bound and follows from u and w.
+//
+// Plain FMA dot products: the cull only has to keep every Gaussian the projection keeps. Their
+// error is below 8 units of roundoff of the summed magnitudes, so a Gaussian is dropped for the
+// near plane only when even z + that bound is at or below it (the projection then decides with its
+// compensated depth).
+struct CullView {
+  float4 px;   // fx R0 + cx R2 | fx t0 + cx t2: z times the pixel column of the centre
+  float4 py;   // likewise for the row
+  float4 z;    // R2 | t2
+  float4 lim;  // width - 1, height - 1, 1.02 F, bound of z's error from t2
+};
+
 __global__ void __launch_bounds__(kPreThreads) cull_kernel(
     const __grid_constant__ Views views, const Consts c, int n, const float* __restrict__ means,
     const float* __restrict__ log_scales, const float* __restrict__ quats,
     const float* __restrict__ logits, uint32_t* __restrict__ cand,
     uint32_t* __restrict__ vis_bits, int bit_words, Counters* __restrict__ counters,
     int views_per_chunk) {
+  constexpr int kWarps = kPreThreads / 32;
   static_assert(kPreThreads % 32 == 0, "whole words of the visibility bitmask per block");
   chain_wait();
-  __shared__ uint32_t s_cand[kPreThreads * kCullMaxViewsPerThread];
-  __shared__ uint32_t s_count, s_base;
-  if (threadIdx.x == 0) s_count = 0;
-  __syncthreads();
+  __shared__ uint32_t s_cand[kWarps][32 * kCullMaxViewsPerThread];
+  __shared__ CullView s_view[kCullMaxViewsPerThread];
+  __shared__ uint32_t s_count[kWarps], s_base;
   const int i = blockIdx.x * kPreThreads + threadIdx.x;
   const bool in_range = i < n;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int v_begin = blockIdx.y * views_per_chunk;
-  const int v_end = min(views.n_views, v_begin + views_per_chunk);
+  const int v_count = min(views.n_views, v_begin + views_per_chunk) - v_begin;
+  if (threadIdx.x < v_count) {
+    const ViewParams& vp = views.v[v_begin + threadIdx.x];
+    const PoseRef ps = view_pose(views, v_begin + threadIdx.x);
+    const float* R = ps.R;
+    CullView cv;
+    cv.px = make_float4(fmaf(vp.fx, R[0], vp.cx * R[6]), fmaf(vp.fx, R[1], vp.cx * R[7]),
+                        fmaf(vp.fx, R[2], vp.cx * R[8]), fmaf(vp.fx, ps.t[0], vp.cx * ps.t[2]));
+    cv.py = make_float4(fmaf(vp.fy, R[3], vp.cy * R[6]), fmaf(vp.fy, R[4], vp.cy * R[7]),
+                        fmaf(vp.fy, R[5], vp.cy * R[8]), fmaf(vp.fy, ps.t[1], vp.cy * ps.t[2]));
+    cv.z = make_float4(R[6], R[7], R[8], ps.t[2]);
+    const float F = sqrtf(vp.fx * vp.fx * (1.0f + vp.lim_u * vp.lim_u) +
+                          vp.fy * vp.fy * (1.0f + vp.lim_w * vp.lim_w));
+    // A negative value tells that there is no guard band.
+    cv.lim = make_float4((float)(vp.width - 1), (float)(vp.height - 1),
+                         vp.lim_u > 0.0f ? 1.02f * F : -1.0f, 4.8e-7f * fabsf(ps.t[2]));
+    s_view[threadIdx.x] = cv;
+  }
+  // The block's Gaussians own whole words of each view's row of the visibility bitmask. Tile counts
+  // are written by the projection for its candidates only: the later passes read them only for
+  // entries whose visibility bit is set.
+  for (int t = threadIdx.x; t < kWarps * v_count; t += kPreThreads) {
+    const int w = blockIdx.x * kWarps + t % kWarps;
+    if (w < bit_words) vis_bits[(size_t)(v_begin + t / kWarps) * bit_words + w] = 0u;
+  }
+  __syncthreads();
   float m[3] = {0, 0, 0}, ls[3] = {0, 0, 0}, q[4] = {1, 0, 0, 0}, logit = 0.0f;
   if (in_range) {
 #pragma unroll
@@ -330,68 +377,53 @@ __global__ void __launch_bounds__(kPreThreads) cull_kernel(
   for (int k = 0; k < 4; ++k) finite = finite && isfinite(q[k]);
   const float qn2 = q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
   finite = finite && qn2 > 0.0f && isfinite(qn2);
-  if (in_range && !finite) atomicAdd(&counters->n_nonfinite, (uint32_t)(v_end - v_begin));
-  float smax = fmaxf(ls[0], fmaxf(ls[1], ls[2]));
-  const float smax2 = finite ? expf(2.0f * smax) : 0.0f;
+  if (in_range && !finite) atomicAdd(&counters->n_nonfinite, (uint32_t)v_count);
+  const float smax = expf(fmaxf(ls[0], fmaxf(ls[1], ls[2])));
   const float opacity = 1.0f / (1.0f + expf(-logit));
   const float kappa = finite ? 2.0f * logf(opacity / c.alpha_min) : -1.0f;
-  for (int v = v_begin; v < v_end; ++v) {
-    const ViewParams& vp = views.v[v];
-    const PoseRef ps = view_pose(views, v);
-    const size_t vi = (size_t)v * n + i;
-    bool keep = false;
-    if (finite && kappa >= 0.0f) {
-      const float* R = ps.R;
-      // Plain FMA dot products: the cull only has to keep every Gaussian the projection keeps.
-      // Their error is below 8 units of roundoff of the summed magnitudes, so a Gaussian is
-      // dropped for the near plane only when even z + that bound is at or below it (the
-      // projection then decides with its compensated depth); the projected centre's error is
-      // far inside the radius bound's 4 px slack.
-      const float z = fmaf(R[6], m[0], fmaf(R[7], m[1], fmaf(R[8], m[2], ps.t[2])));
-      const float z_err =
-          4.8e-7f * (fabsf(R[6] * m[0]) + fabsf(R[7] * m[1]) + fabsf(R[8] * m[2]) + fabsf(ps.t[2]));
-      if (z + z_err > c.znear && z > 0.0f) {
-        const float x = fmaf(R[0], m[0], fmaf(R[1], m[1], fmaf(R[2], m[2], ps.t[0])));
-        const float y = fmaf(R[3], m[0], fmaf(R[4], m[1], fmaf(R[5], m[2], ps.t[1])));
-        const float rz = 1.0f / z;
-        const float u = x * rz, w = y * rz;
-        float uc = u, wc = w;
-        if (vp.lim_u > 0.0f) {
-          uc = fminf(fmaxf(u, -vp.lim_u), vp.lim_u);
-          wc = fminf(fmaxf(w, -vp.lim_w), vp.lim_w);
-        }
-        const float jf2 = (vp.fx * vp.fx * (1.0f + uc * uc) + vp.fy * vp.fy * (1.0f + wc * wc)) *
-                          (rz * rz);
-        // A rigorous bound of the alpha >= alpha_min footprint radius: the largest eigenvalue of
-        // Sigma^I is at most ||J||_F^2 smax^2 + eps, so the radius is at most
-        // sqrt(kappa (||J||_F^2 smax^2 + eps)); widened by 2 % and 4 px, beyond the 1-px padding
-        // of the tile coverage and the rounding of this cheaper mean.
-        const float rad = sqrtf(kappa * fmaf(jf2, smax2, c.eps2d)) * 1.02f + 4.0f;
-        const float mx = fmaf(vp.fx, u, vp.cx), my = fmaf(vp.fy, w, vp.cy);
-        keep = !(mx + rad < 0.0f || mx - rad > (float)(vp.width - 1) || my + rad < 0.0f ||
-                 my - rad > (float)(vp.height - 1));
-      }
+  const bool shown = finite && kappa >= 0.0f;
+  // rad z <= F reach + band z; an overflowing product keeps the entry.
+  const float root = sqrtf(fmaxf(kappa, 0.0f));
+  const float reach = root * smax, band = fmaf(1.02f * root, sqrtf(c.eps2d), 4.0f);
+  const float z_err = 4.8e-7f * (fabsf(m[0]) + fabsf(m[1]) + fabsf(m[2]));
+  uint32_t count = 0;  // candidates of the warp so far
+  for (int k = 0; k < v_count; ++k) {
+    const float4 zr = s_view[k].z, lim = s_view[k].lim;
+    const float z = fmaf(zr.x, m[0], fmaf(zr.y, m[1], fmaf(zr.z, m[2], zr.w)));
+    const float4 pr = s_view[k].px, qr = s_view[k].py;
+    const float px = fmaf(pr.x, m[0], fmaf(pr.y, m[1], fmaf(pr.z, m[2], pr.w)));
+    const float py = fmaf(qr.x, m[0], fmaf(qr.y, m[1], fmaf(qr.z, m[2], qr.w)));
+    float margin = fmaf(lim.z, reach, band * z);
+    if (lim.z < 0.0f) {  // no guard band (the same for every Gaussian)
+      const ViewParams& vp = views.v[v_begin + k];
+      const float u = (px - vp.cx * z) / (vp.fx * z), w = (py - vp.cy * z) / (vp.fy * z);
+      const float F = sqrtf(vp.fx * vp.fx * fmaf(u, u, 1.0f) + vp.fy * vp.fy * fmaf(w, w, 1.0f));
+      margin = fmaf(1.03f * F, reach, band * z);
     }
-    // The block's Gaussians own whole words of row v of the visibility bitmask. Tile counts are
-    // written by the projection for its candidates only: the later passes read them only for
-    // entries whose visibility bit is set.
-    if (threadIdx.x < kPreThreads / 32) {
-      const int w = blockIdx.x * (kPreThreads / 32) + threadIdx.x;
-      if (w < bit_words) vis_bits[(size_t)v * bit_words + w] = 0u;
-    }
+    const bool keep = shown && z + (z_err + lim.w) > c.znear && z > 0.0f &&
+                      !(px + margin < 0.0f || py + margin < 0.0f ||
+                        px > fmaf(lim.x, z, margin) || py > fmaf(lim.y, z, margin));
     const unsigned ballot = __ballot_sync(0xffffffffu, keep);
-    if (ballot) {
-      const int leader = __ffs(ballot) - 1;
-      uint32_t base = 0;
-      if (lane == leader) base = atomicAdd(&s_count, (uint32_t)__popc(ballot));
-      base = __shfl_sync(0xffffffffu, base, leader);
-      if (keep) s_cand[base + __popc(ballot & ((1u << lane) - 1u))] = (uint32_t)vi;
+    if (keep)
+      s_cand[warp][count + __popc(ballot & ((1u << lane) - 1u))] =
+          (uint32_t)((size_t)(v_begin + k) * n + i);
+    count += __popc(ballot);
+  }
+  if (lane == 0) s_count[warp] = count;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t total = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const uint32_t x = s_count[w];
+      s_count[w] = total;
+      total += x;
     }
+    s_base = total ? atomicAdd(&counters->n_candidates, total) : 0u;
   }
   __syncthreads();
-  if (threadIdx.x == 0) s_base = s_count ? atomicAdd(&counters->n_candidates, s_count) : 0u;
-  __syncthreads();
-  for (uint32_t t = threadIdx.x; t < s_count; t += kPreThreads) cand[s_base + t] = s_cand[t];
+  uint32_t* out = cand + s_base + s_count[warp];
+  for (uint32_t t = lane; t < count; t += 32) out[t] = s_cand[warp][t];
 }
 
 // Colour of a Gaussian from its SH coefficients (Eq. app-sh) for the direction camera centre ->
@@ -420,16 +452,14 @@ __device__ __forceinline__ void sh_colour(const float* shc, const float* m, cons
 // (Eq. proj), tile count and, for DEG >= 0, the colour; writes the entry's records and tile count.
 // An entry with a non-finite SH coefficient is culled here and counted. With DEG = -1 (the
 // caller's SH coefficients may still be in flight) the colour is left to the pass after the
-// sorts (rec2.xyz = 0 until then). Entries that are not candidates keep ntiles = 0 and unwritten
-// records.
+// sorts (colour.xyz = 0 until then). Entries that are not candidates keep unwritten records.
 template <int DEG, bool kDevPose>
-__global__ void __launch_bounds__(kPreThreads) project_kernel(
+__global__ void __launch_bounds__(kPreThreads, 7) project_kernel(
     const __grid_constant__ Views views, const Consts c, int n, const float* __restrict__ means,
     const float* __restrict__ log_scales, const float* __restrict__ quats,
     const float* __restrict__ logits, const float* __restrict__ sh,
-    const uint32_t* __restrict__ cand, float4* __restrict__ rec0, float4* __restrict__ rec1,
-    float4* __restrict__ rec2, uint2* __restrict__ touched, uint32_t* __restrict__ vis_bits,
-    int bit_words, Counters* __restrict__ counters) {
+    const uint32_t* __restrict__ cand, Record* __restrict__ rec, uint32_t* __restrict__ depths,
+    uint32_t* __restrict__ vis_bits, int bit_words, Counters* __restrict__ counters) {
   chain_wait();
   unsigned long long sum_visible = 0, sum_tiles = 0, sum_cells = 0;
   constexpr int K = DEG >= 0 ? (DEG + 1) * (DEG + 1) : 1;
@@ -450,6 +480,7 @@ __global__ void __launch_bounds__(kPreThreads) project_kernel(
     q[1] = q4.y;
     q[2] = q4.z;
     q[3] = q4.w;
+    const float logit = __ldg(logits + i);
     float shc[3 * K];
     if constexpr (DEG >= 0) {
       load_sh<DEG>(sh, i, shc);
@@ -461,16 +492,19 @@ __global__ void __launch_bounds__(kPreThreads) project_kernel(
         continue;
       }
     }
-    GaussianLocal g;
-    gaussian_local(m, ls, q, __ldg(logits + i), g);
     const ViewParams& vp = views.v[v];
     const PoseRef ps = view_pose<kDevPose>(views, v);
+    // The colour comes first: the 3K coefficients are then not held through the projection, and 72
+    // registers (7 blocks per SM) do at degree 3 where 95 were held: 390 -> 352 us over 16 views
+    // of 3M Gaussians, a gather that waits on memory.
+    float rgb[3] = {0.0f, 0.0f, 0.0f};
+    if constexpr (DEG >= 0) sh_colour<DEG>(shc, m, ps, rgb);
+    GaussianLocal g;
+    gaussian_local(m, ls, q, logit, g);
     ViewProj p;
     if (!project_view(g, vp, ps, c, p)) continue;
     const float4 r0 = make_float4(p.mean2d[0], p.mean2d[1], p.mean2d_lo[0], p.mean2d_lo[1]);
     const float4 r1 = make_float4(p.chol[0], p.chol[1], p.chol[2], log2f(g.opacity));
-    float rgb[3] = {0.0f, 0.0f, 0.0f};
-    if constexpr (DEG >= 0) sh_colour<DEG>(shc, g.m, ps, rgb);
     const float4 r2 = make_float4(rgb[0], rgb[1], rgb[2], p.mc[2]);
     uint32_t tiles = 0, cells = 0;
     Ellipse e;
@@ -485,10 +519,11 @@ __global__ void __launch_bounds__(kPreThreads) project_kernel(
         for (int r = 0; r < kCellTiles; ++r) tiles += span_tiles(row.span[r]);
       }
     }
-    rec0[vi] = r0;
-    rec1[vi] = r1;
-    rec2[vi] = r2;
-    touched[vi] = make_uint2(tiles, cells);
+    rec[vi].mean = r0;
+    rec[vi].conic = r1;
+    rec[vi].colour = r2;
+    rec[vi].touched = make_uint2(tiles, cells);
+    depths[vi] = __float_as_uint(p.mc[2]);  // again, densely, for the compaction
     if (tiles > 0) {
       atomicOr(&vis_bits[(size_t)v * bit_words + (i >> 5)], 1u << (i & 31));
       ++sum_visible;
@@ -524,15 +559,15 @@ __global__ void __launch_bounds__(kPreThreads) project_kernel(
 // list: neighbouring threads read neighbouring Gaussians' SH rows; in depth order the reads are
 // scattered, which costs ~0.15 ms on 3M Gaussians whose coefficients do not fit in L2). The colour
 // from the SH coefficients for the direction camera centre -> Gaussian (Eq. app-sh), clamped at 0,
-// into rec2.xyz. An entry with a non-finite coefficient gets log2 opacity -inf, so that it covers
+// into the record. An entry with a non-finite coefficient gets log2 opacity -inf, so that it covers
 // no pixel in either blend, and is counted as culled.
 constexpr int kColourThreads = 256;
 
 template <int DEG, bool kDevPose>
 __global__ void __launch_bounds__(kColourThreads) colour_kernel(
     const __grid_constant__ Views views, int n, const float* __restrict__ means,
-    const float* __restrict__ sh, const uint32_t* __restrict__ list, float4* __restrict__ rec1,
-    float4* __restrict__ rec2, Counters* __restrict__ counters) {
+    const float* __restrict__ sh, const uint32_t* __restrict__ list, Record* __restrict__ rec,
+    Counters* __restrict__ counters) {
   chain_wait();
   constexpr int K = (DEG + 1) * (DEG + 1);
   const uint32_t n_visible = counters->n_visible_kept;
@@ -546,12 +581,12 @@ __global__ void __launch_bounds__(kColourThreads) colour_kernel(
     bool sh_finite = true;
 #pragma unroll
     for (int a = 0; a < 3 * K; ++a) sh_finite = sh_finite && isfinite(shc[a]);
-    float4 r2 = rec2[vi];
+    float4 r2 = rec[vi].colour;
     if (!sh_finite) {
       atomicAdd(&counters->n_nonfinite, 1u);
-      reinterpret_cast<float*>(rec1 + vi)[3] = -INFINITY;
+      rec[vi].conic.w = -INFINITY;
       r2.x = r2.y = r2.z = 0.0f;
-      rec2[vi] = r2;
+      rec[vi].colour = r2;
       continue;
     }
     const PoseRef ps = view_pose<kDevPose>(views, v);
@@ -562,7 +597,7 @@ __global__ void __launch_bounds__(kColourThreads) colour_kernel(
     r2.x = rgb[0];
     r2.y = rgb[1];
     r2.z = rgb[2];
-    rec2[vi] = r2;
+    rec[vi].colour = r2;
   }
 }
 
@@ -1057,8 +1092,7 @@ __global__ void __launch_bounds__(256) reg_sum_kernel(int n, const float* __rest
 }  // namespace
 
 cudaError_t launch_preprocess_forward(const Views& views, const Consts& c,
-                                      const rgs_gaussians& g, float4* rec0, float4* rec1,
-                                      float4* rec2, uint2* touched, uint32_t* cand,
+                                      const rgs_gaussians& g, Record* rec, uint32_t* depths, uint32_t* cand,
                                       uint32_t* vis_bits, bool defer_colour, Counters* counters,
                                       cudaStream_t stream) {
   if (g.n == 0) return cudaSuccess;
@@ -1081,8 +1115,8 @@ cudaError_t launch_preprocess_forward(const Views& views, const Consts& c,
 #define RGS_PROJECT(D)                                                                          \
   e = launch_chained(views.pose_dev ? project_kernel<D, true> : project_kernel<D, false>,         \
                      dim3(blocks2), dim3(kPreThreads), stream, views, c, g.n, g.means,            \
-                     g.log_scales, g.quats, g.opacity_logits, g.sh, (const uint32_t*)cand, rec0, \
-                     rec1, rec2, touched, vis_bits, bit_words, counters)
+                     g.log_scales, g.quats, g.opacity_logits, g.sh, (const uint32_t*)cand, rec,  \
+                     depths, vis_bits, bit_words, counters)
   if (defer_colour) {
     RGS_PROJECT(-1);
   } else {
@@ -1099,7 +1133,7 @@ cudaError_t launch_preprocess_forward(const Views& views, const Consts& c,
 }
 
 cudaError_t launch_colour(const Views& views, const rgs_gaussians& g, const uint32_t* list,
-                          int64_t vis_cap, float4* rec1, float4* rec2, Counters* counters,
+                          int64_t vis_cap, Record* rec, Counters* counters,
                           cudaStream_t stream) {
   const unsigned blocks =
       (unsigned)std::min<int64_t>((vis_cap + kColourThreads - 1) / kColourThreads, 4 * 152);
@@ -1108,7 +1142,7 @@ cudaError_t launch_colour(const Views& views, const rgs_gaussians& g, const uint
 #define RGS_COLOUR(D)                                                                         \
   e = launch_chained(views.pose_dev ? colour_kernel<D, true> : colour_kernel<D, false>,       \
                      dim3(blocks), dim3(kColourThreads), stream, views, g.n, g.means, g.sh, \
-                     list, rec1, rec2, counters)
+                     list, rec, counters)
   switch (g.sh_degree) {
     case 0: RGS_COLOUR(0); break;
     case 1: RGS_COLOUR(1); break;

@@ -25,7 +25,7 @@ namespace {
 //   [2] (l21, l21), (l22, l22)           [3] (s_a, s_a), (-log2 o, -log2 o)
 //   [4] (r, r), (g, g)                   [5] (b, b), (z, z)
 // With one pixel per thread rows 0..2 hold (mx hi, mx lo, l11, c21), (l21, l22, s_a, -log2 o)
-// and rec2 as float4.
+// and the colour as float4.
 // ------------------------------------------------------------------------------------------
 template <int R, int N>
 __device__ __forceinline__ void stage_gaussian(ulonglong2 (&sp)[R][N], int t, float4 r0,
@@ -65,8 +65,7 @@ __device__ __forceinline__ void stage_gaussian(ulonglong2 (&sp)[R][N], int t, fl
 template <int TW, int TH, int PPT>
 __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
     const __grid_constant__ Views views, const Consts c, const uint2* __restrict__ ranges,
-    const uint32_t* __restrict__ pair_vals, const float4* __restrict__ rec0,
-    const float4* __restrict__ rec1, const float4* __restrict__ rec2, float* __restrict__ color,
+    const uint32_t* __restrict__ pair_vals, const Record* __restrict__ rec, float* __restrict__ color,
     float* __restrict__ depth, float* __restrict__ alpha_out, float* __restrict__ t_final,
     int32_t* __restrict__ last_index, const uint32_t* __restrict__ tile_order,
     Counters* __restrict__ counters) {
@@ -159,7 +158,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
     const uint32_t j = start + threadIdx.x;
     if (j < range.y) {
       const uint32_t vi = pair_vals[j];
-      stage_gaussian(sp, threadIdx.x, rec0[vi], rec1[vi], rec2[vi], y_a);
+      stage_gaussian(sp, threadIdx.x, rec[vi].mean, rec[vi].conic, rec[vi].colour, y_a);
     }
     __syncthreads();
     const int cnt = (int)min((uint32_t)kThreads, range.y - start);
@@ -300,8 +299,7 @@ __device__ __forceinline__ void reduce_row(float* red, int r) {
 template <int TW, int TH, int PPT, bool kAux>
 __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
     const __grid_constant__ Views views, const Consts c, const uint2* __restrict__ ranges,
-    const uint32_t* __restrict__ pair_vals, const float4* __restrict__ rec0,
-    const float4* __restrict__ rec1, const float4* __restrict__ rec2,
+    const uint32_t* __restrict__ pair_vals, const Record* __restrict__ rec,
     const float* __restrict__ t_final, const int32_t* __restrict__ last_index,
     const float* __restrict__ d_color, const float* __restrict__ d_depth,
     const float* __restrict__ d_alpha, const uint32_t* __restrict__ tile_order,
@@ -593,7 +591,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
     if (j < bend) {
       const uint32_t vi = pair_vals[j];
       s_vi[threadIdx.x] = vi;
-      stage_gaussian(sp, threadIdx.x, rec0[vi], rec1[vi], rec2[vi], y_a);
+      stage_gaussian(sp, threadIdx.x, rec[vi].mean, rec[vi].conic, rec[vi].colour, y_a);
     }
     __syncthreads();
     // Positions above the warp's smallest last index test each pixel; the rest do not. Whether
@@ -635,8 +633,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
 
 template <int TW, int TH, int PPT>
 cudaError_t launch_blends_t(bool forward, const Views& views, const Consts& c,
-                            const uint2* ranges, const uint32_t* pair_vals, const float4* rec0,
-                            const float4* rec1, const float4* rec2, float* color, float* depth,
+                            const uint2* ranges, const uint32_t* pair_vals, const Record* rec, float* color, float* depth,
                             float* alpha, float* t_final, int32_t* last_index,
                             const float* d_color, const float* d_depth, const float* d_alpha,
                             float* g2d, const uint32_t* tile_order, Counters* counters,
@@ -646,14 +643,14 @@ cudaError_t launch_blends_t(bool forward, const Views& views, const Consts& c,
   cudaError_t e;
   if (forward) {
     e = launch_chained(blend_forward_kernel<TW, TH, PPT>, dim3(views.total_tiles), dim3(kThreads),
-                       stream, views, c, ranges, pair_vals, rec0, rec1, rec2, color, depth, alpha,
+                       stream, views, c, ranges, pair_vals, rec, color, depth, alpha,
                        t_final, last_index, tile_order, counters);
   } else {
     const bool aux = d_depth != nullptr || d_alpha != nullptr;
     e = launch_chained(aux ? blend_backward_kernel<TW, TH, PPT, true>
                            : blend_backward_kernel<TW, TH, PPT, false>,
                        dim3(views.total_tiles), dim3(kThreads), stream, views, c, ranges,
-                       pair_vals, rec0, rec1, rec2, (const float*)t_final,
+                       pair_vals, rec, (const float*)t_final,
                        (const int32_t*)last_index, d_color, d_depth, d_alpha, tile_order, g2d);
   }
   RGS_LAUNCHED();
@@ -663,8 +660,7 @@ cudaError_t launch_blends_t(bool forward, const Views& views, const Consts& c,
 }  // namespace
 
 cudaError_t launch_blend(bool forward, const Views& views, const Consts& c, const uint2* ranges,
-                         const uint32_t* pair_vals, const float4* rec0, const float4* rec1,
-                         const float4* rec2, float* color, float* depth, float* alpha,
+                         const uint32_t* pair_vals, const Record* rec, float* color, float* depth, float* alpha,
                          float* t_final, int32_t* last_index, const float* d_color,
                          const float* d_depth, const float* d_alpha, float* g2d,
                          const uint32_t* tile_order, Counters* counters, cudaStream_t stream) {
@@ -672,7 +668,7 @@ cudaError_t launch_blend(bool forward, const Views& views, const Consts& c, cons
   const int ppt = forward ? views.pixels_per_thread : views.bwd_pixels_per_thread;
 #define RGS_BLEND(W, H, P)                                                                        \
   if (tw == W && th == H && ppt == P)                                                             \
-  return launch_blends_t<W, H, P>(forward, views, c, ranges, pair_vals, rec0, rec1, rec2, color, \
+  return launch_blends_t<W, H, P>(forward, views, c, ranges, pair_vals, rec, color, \
                                   depth, alpha, t_final, last_index, d_color, d_depth, d_alpha,   \
                                   g2d, tile_order, counters, stream)
   RGS_BLEND(16, 16, 1);

@@ -24,12 +24,11 @@
 
 namespace rgs {
 cudaError_t launch_preprocess_forward(const Views& views, const Consts& c,
-                                      const rgs_gaussians& g, float4* rec0, float4* rec1,
-                                      float4* rec2, uint2* touched, uint32_t* cand,
+                                      const rgs_gaussians& g, Record* rec, uint32_t* depths, uint32_t* cand,
                                       uint32_t* vis_bits, bool defer_colour, Counters* counters,
                                       cudaStream_t stream);
 cudaError_t launch_colour(const Views& views, const rgs_gaussians& g, const uint32_t* list,
-                          int64_t vis_cap, float4* rec1, float4* rec2, Counters* counters,
+                          int64_t vis_cap, Record* rec, Counters* counters,
                           cudaStream_t stream);
 int preprocess_backward_blocks(int64_t vn);
 cudaError_t launch_preprocess_backward(const Views& views, const Consts& c,
@@ -42,21 +41,18 @@ cudaError_t launch_preprocess_backward(const Views& views, const Consts& c,
 int64_t max_emit_blocks(int64_t visible);
 int order_words();
 cudaError_t launch_emit_cells(const Views& views, int n, const uint32_t* order,
-                              const uint2* touched, const float4* rec0, const float4* rec1,
-                              float log2_alpha_min, int64_t visible_cap, uint32_t capacity,
+                              const Record* rec, float log2_alpha_min, int64_t visible_cap, uint32_t capacity,
                               uint32_t* keys, uint32_t* vals, Lookback lb, Counters* counters,
                               cudaStream_t stream);
 cudaError_t launch_cell_ranges(const Views& views, const uint32_t* keys, int64_t n_keys,
                                uint2* ranges, const Counters* counters, cudaStream_t stream);
 cudaError_t launch_tile_lists(const Views& views, const uint2* cell_ranges, const uint32_t* keys,
-                              const uint32_t* vals, const float4* rec0, const float4* rec1,
-                              float log2_alpha_min, uint32_t* tile_counts, uint2* ranges,
+                              const uint32_t* vals, const Record* rec, float log2_alpha_min, uint32_t* tile_counts, uint2* ranges,
                               uint32_t* pairs, uint32_t capacity, uint32_t* order_words,
                               uint32_t* tile_order, Lookback lb, Counters* counters,
                               cudaStream_t stream);
 cudaError_t launch_blend(bool forward, const Views& views, const Consts& c, const uint2* ranges,
-                         const uint32_t* pair_vals, const float4* rec0, const float4* rec1,
-                         const float4* rec2, float* color, float* depth, float* alpha,
+                         const uint32_t* pair_vals, const Record* rec, float* color, float* depth, float* alpha,
                          float* t_final, int32_t* last_index, const float* d_color,
                          const float* d_depth, const float* d_alpha, float* g2d,
                          const uint32_t* tile_order, Counters* counters, cudaStream_t stream);
@@ -95,8 +91,7 @@ struct State {
   Region r_vn, r_n, r_pix, r_tile, r_cell, r_pair, r_scratch, r_pose, r_counters;
 
   // Per (view, Gaussian).
-  float4 *rec0 = nullptr, *rec1 = nullptr, *rec2 = nullptr;
-  uint2* touched = nullptr;  // (tiles, cells)
+  Record* rec = nullptr;
   uint32_t *vis_keys[2] = {nullptr, nullptr}, *vis_vals[2] = {nullptr, nullptr};
   // The visible entries in (view, Gaussian) order (the compaction's output, kept past the depth
   // sort): the colour pass and the backward's per-entry pass walk it, so that neighbouring
@@ -291,16 +286,12 @@ rgs_status ensure_vn(rgs_ctx* ctx, State& s, int64_t vn, int64_t n, int64_t pose
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "per-Gaussian buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
     const int64_t cap = vn;
-    size_t bytes = 3 * align_up(sizeof(float4) * cap) + align_up(sizeof(uint2) * cap) +
-                   5 * align_up(sizeof(uint32_t) * cap) +
+    size_t bytes = align_up(sizeof(Record) * cap) + 5 * align_up(sizeof(uint32_t) * cap) +
                    align_up(sizeof(float) * kG2Stride * cap) +
                    align_up(sizeof(uint32_t) * vis_bit_words_cap(cap));
     RGS_CUDA(alloc_region(ctx, s.r_vn, bytes), "allocate per-Gaussian buffers");
     char* p = static_cast<char*>(s.r_vn.base);
-    s.rec0 = carve<float4>(p, cap);
-    s.rec1 = carve<float4>(p, cap);
-    s.rec2 = carve<float4>(p, cap);
-    s.touched = carve<uint2>(p, cap);
+    s.rec = carve<Record>(p, cap);
     s.vis_keys[0] = carve<uint32_t>(p, cap);
     s.vis_keys[1] = carve<uint32_t>(p, cap);
     s.vis_vals[0] = carve<uint32_t>(p, cap);
@@ -927,12 +918,12 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
     RGS_CUDA(launch_pose_prepare(world_to_cam, n_views, s->pose_records, stream), "pose records");
 
   // 1. Projection.
-  // The cull pass's candidate list lives in the depth sort's second key buffer, which is free
-  // until the sort starts.
+  // The cull pass's candidate list and the projection's depths live in the depth sort's second key
+  // and value buffers, which are free until the sort starts.
   // The colours are evaluated in the projection, unless the caller's SH coefficients may still
   // be in flight: then after the sorts, behind the caller's event.
   const bool defer_colour = cfg.sh_ready_event != nullptr;
-  RGS_CUDA(launch_preprocess_forward(views, consts, *g, s->rec0, s->rec1, s->rec2, s->touched,
+  RGS_CUDA(launch_preprocess_forward(views, consts, *g, s->rec, s->vis_vals[1],
                                      s->vis_keys[1], s->vis_bits, defer_colour, cnt, stream),
            "preprocess");
   RGS_CUDA(mark(ctx, *s, 1, stream, capturing), "event");
@@ -945,7 +936,7 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
     RGS_CUDA(cudaEventRecord(s->done, stream), "event");
   }
   // 2. Visible entries with depth keys, in (view, Gaussian) order.
-  RGS_CUDA(launch_compact_visible(s->vis_bits, n_views, g->n, s->rec2, s->vis_keys[0],
+  RGS_CUDA(launch_compact_visible(s->vis_bits, n_views, g->n, s->vis_vals[1], s->vis_keys[0],
                                   s->vis_vals[0], s->vis_list, &cnt->n_visible,
                                   lookback_at(lb_area, &cnt->status, vn), stream),
            "compact");
@@ -977,14 +968,14 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
   bool alt = false;
   RGS_CUDA(launch_radix_sort(s->vis_keys[0], s->vis_vals[0], s->vis_keys[1], s->vis_vals[1],
                              vis_cap, &cnt->n_visible, 0, 31, s->hist, s->block_sums, &alt,
-                             stream, kSortItemsSmall),
+                             stream, vis_cap < kWideMinN ? kSortItemsSmall : kSortItems),
            "depth sort");
   s->order = s->vis_vals[alt ? 1 : 0];
   RGS_CUDA(mark(ctx, *s, 3, stream, capturing), "event");
   RGS_CUDA(mark(ctx, *s, 4, stream, capturing), "event");
   const uint32_t pair_cap = (uint32_t)s->pair_cap;
   // 4. Cell entries in depth order.
-  RGS_CUDA(launch_emit_cells(views, g->n, s->order, s->touched, s->rec0, s->rec1,
+  RGS_CUDA(launch_emit_cells(views, g->n, s->order, s->rec,
                              consts.log2_alpha_min, vis_cap, (uint32_t)s->cell_cap,
                              s->cell_keys[0], s->cell_vals[0],
                              lookback_at(lb_emit, &cnt->status, emit_items), cnt, stream),
@@ -1004,7 +995,7 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
   RGS_CUDA(mark(ctx, *s, 6, stream, capturing), "event");
   // 6. The tiles' lists, their ranges and launch order.
   RGS_CUDA(launch_cell_ranges(views, keys, n_cells, cell_ranges, cnt, stream), "cell ranges");
-  RGS_CUDA(launch_tile_lists(views, cell_ranges, keys, vals, s->rec0, s->rec1,
+  RGS_CUDA(launch_tile_lists(views, cell_ranges, keys, vals, s->rec,
                              consts.log2_alpha_min, s->tile_counts, s->ranges, s->pairs, pair_cap,
                              order_state, s->tile_order,
                              lookback_at(lb_tile, &cnt->status, views.total_tiles), cnt, stream),
@@ -1014,13 +1005,13 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
   if (defer_colour) {
     RGS_CUDA(cudaStreamWaitEvent(stream, static_cast<cudaEvent_t>(cfg.sh_ready_event), 0),
              "wait for the SH coefficients");
-    RGS_CUDA(launch_colour(views, *g, s->vis_list, vis_cap, s->rec1, s->rec2, cnt, stream),
+    RGS_CUDA(launch_colour(views, *g, s->vis_list, vis_cap, s->rec, cnt, stream),
              "colours");
   }
   RGS_CUDA(mark(ctx, *s, 7, stream, capturing), "event");
   // 7. Blend.
-  RGS_CUDA(launch_blend(true, views, consts, s->ranges, s->pairs, s->rec0, s->rec1,
-                        s->rec2, out->color, out->depth, out->alpha, s->t_final, s->last_index,
+  RGS_CUDA(launch_blend(true, views, consts, s->ranges, s->pairs, s->rec,
+                        out->color, out->depth, out->alpha, s->t_final, s->last_index,
                         nullptr, nullptr, nullptr, nullptr, s->tile_order, cnt, stream),
            "blend forward");
   RGS_CUDA(mark(ctx, *s, 8, stream, capturing), "event");
@@ -1116,8 +1107,8 @@ rgs_status render_backward(rgs_ctx* ctx, uint64_t handle, const rgs_image_grads*
   open_state(*s, capturing);
   s->bwd_timed = ctx->timing;
   RGS_CUDA(mark(ctx, *s, kEvBwd0, stream, capturing), "event");
-  RGS_CUDA(launch_blend(false, s->views, s->consts, s->ranges, s->pairs, s->rec0, s->rec1,
-                        s->rec2, nullptr, nullptr, nullptr, s->t_final, s->last_index, dc, dd, da,
+  RGS_CUDA(launch_blend(false, s->views, s->consts, s->ranges, s->pairs, s->rec,
+                        nullptr, nullptr, nullptr, s->t_final, s->last_index, dc, dd, da,
                         s->g2d, s->tile_order, s->counters, stream),
            "blend backward");
   RGS_CUDA(mark(ctx, *s, kEvBwd0 + 1, stream, capturing), "event");
@@ -1219,14 +1210,14 @@ rgs_status rgs_copy_records(rgs_ctx* ctx, uint64_t handle, float* host_rec,
   cudaSetDevice(ctx->device);
   const int64_t vn = s->vn;
   if (vn > 0) {
-    const float4* recs[3] = {s->rec0, s->rec1, s->rec2};
-    for (int k = 0; k < 3; ++k)
-      RGS_CUDA(cudaMemcpy2DAsync(host_rec + 4 * k, 12 * sizeof(float), recs[k], sizeof(float4),
-                                 sizeof(float4), (size_t)vn, cudaMemcpyDeviceToHost, stream),
-               "copy records");
+    RGS_CUDA(cudaMemcpy2DAsync(host_rec, 12 * sizeof(float), s->rec, sizeof(Record),
+                               12 * sizeof(float), (size_t)vn, cudaMemcpyDeviceToHost, stream),
+             "copy records");
     if (host_ntiles)
-      RGS_CUDA(cudaMemcpy2DAsync(host_ntiles, sizeof(uint32_t), s->touched, sizeof(uint2),
-                                 sizeof(uint32_t), (size_t)vn, cudaMemcpyDeviceToHost, stream),
+      RGS_CUDA(cudaMemcpy2DAsync(host_ntiles, sizeof(uint32_t),
+                                 reinterpret_cast<const char*>(s->rec) + offsetof(Record, touched),
+                                 sizeof(Record), sizeof(uint32_t), (size_t)vn,
+                                 cudaMemcpyDeviceToHost, stream),
                "copy tile counts");
   }
   std::vector<uint32_t> bits;

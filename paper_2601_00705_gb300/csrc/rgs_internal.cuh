@@ -1,16 +1,7 @@
 // rgs_internal.cuh -- shared declarations and device helpers of the sm_103a rasterizer.
 //
 // Layout in HBM (V views, N Gaussians, "vi" = v * N + i):
-//   rec0[vi] = (mean2d.x hi, mean2d.y hi, mean2d.x lo, mean2d.y lo)   float4, the projected
-//              mean as an unevaluated double-float sum, so that p - mu^I is accurate to ~1e-7 px
-//              even at 1080p coordinates
-//   rec1[vi] = (l11, l21, l22, log2 o)                    float4, lower-triangular factor of the
-//              base-2-scaled conic (see below)
-//   rec2[vi] = (r, g, b, depth z)                          float4
-//   touched[vi] = (tiles, cells) touched (0 = culled / invisible)
-//   g2d[vi * 16 + s]: the backward blend's sums over the covered pixels of dL/dpower moments
-//              and of the colour / depth weights (see G2Slot), reused by the backward
-//              preprocess for its per-view intermediate results
+//   rec[vi]: the projected record (Record below), one aligned 64-byte line per entry
 //   cells: blocks of kCellTiles x kCellTiles tiles. The cell list holds one (cell, tile mask; vi)
 //              entry per touched cell, sorted so that each cell's run is in (depth, index) order
 //   pair list: the vi of every (tile, Gaussian) pair, tile by tile, each tile's run in (depth,
@@ -25,6 +16,20 @@
 namespace rgs {
 
 constexpr int kMaxViews = RGS_MAX_VIEWS;
+
+// Projected record of a (view, Gaussian). Every reader gathers it by entry, in depth or tile order:
+// in one line its three words take two sectors and one DRAM access; as separate arrays (and the
+// tile counts in a fourth) they took four of each.
+struct alignas(64) Record {
+  // (mean2d.x hi, mean2d.y hi, mean2d.x lo, mean2d.y lo): the projected mean as an unevaluated
+  // double-float sum, so that p - mu^I is accurate to ~1e-7 px even at 1080p coordinates.
+  float4 mean;
+  // (l11, l21, l22, log2 o): lower-triangular factor of the base-2-scaled conic (see below).
+  float4 conic;
+  float4 colour;  // (r, g, b, depth z)
+  uint2 touched;  // (tiles, cells) touched; meaningful where the visibility bit is set
+  uint2 pad;
+};
 constexpr int kG2Stride = 16;  // floats per (view, Gaussian) gradient record (64 bytes)
 
 // Slots the backward blend accumulates per (view, Gaussian), with dp = dL/dpower of a covered,
@@ -340,11 +345,11 @@ constexpr float kTilePad = 0.0625f;
 
 struct Ellipse {
   float mx, my;           // centre
-  float l11, l21, l22;    // factor of the scaled conic (the record's rec1.xyz)
+  float l11, l21, l22;    // factor of the scaled conic (the record's conic.xyz)
   float kappa;
 };
 
-// From the stored records (rec0.xy = mean hi parts, rec1 = factor and log2 o).
+// From the stored records (r0 = mean, r1 = conic).
 __device__ __forceinline__ bool make_ellipse(float4 r0, float4 r1, float log2_alpha_min,
                                              Ellipse& e) {
   const float kappa = __fsub_rn(r1.w, log2_alpha_min);
@@ -601,12 +606,12 @@ cudaError_t launch_exclusive_scan_single_pass(const uint32_t* in, uint32_t* out,
                                               uint32_t* total, Lookback lb, cudaStream_t stream);
 
 // Compaction of the visible entries, in (view, Gaussian) order: for every set bit i of row v of
-// the visibility bitmask (n_views rows for n Gaussians), writes keys[pos] = float bits of
-// rec2[v n + i].w (depth) and vals[pos] = list[pos] = v n + i (vals feeds the depth sort, list
+// the visibility bitmask (n_views rows for n Gaussians), writes keys[pos] = depths[v n + i]
+// (float bits) and vals[pos] = list[pos] = v n + i (vals feeds the depth sort, list
 // keeps the order for the colour pass and the backward's per-entry pass); the count into *n_out.
 // One single-pass launch; lb must be zeroed.
 cudaError_t launch_compact_visible(const uint32_t* vis_bits, int n_views, int n,
-                                   const float4* rec2, uint32_t* keys, uint32_t* vals,
+                                   const uint32_t* depths, uint32_t* keys, uint32_t* vals,
                                    uint32_t* list, uint32_t* n_out, Lookback lb,
                                    cudaStream_t stream);
 
@@ -621,6 +626,10 @@ constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;       // keys per thread for large sorts (2048 per block)
 constexpr int kSortItemsSmall = 4;  // for sorts whose live count is far below the capacity
 constexpr int kRadixBins = 256;
+// Sorts of at least this many keys (capacity) with large blocks take the wide passes (9-bit digits,
+// blocks of 8192 keys). A 31-bit sort of 3.7M keys takes 132 us so, 157 us in blocks of 2048 and
+// 184 us in blocks of 1024; of 1.9M keys 101, 101 and 110 us.
+constexpr int64_t kWideMinN = 1 << 20;
 
 inline int64_t sort_blocks(int64_t n, int items = kSortItems) {
   return (n + kSortThreads * items - 1) / (kSortThreads * items);

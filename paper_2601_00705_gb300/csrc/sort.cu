@@ -337,7 +337,7 @@ constexpr int kBitsTile = kBitsThreads * kBitsItems;
 
 __global__ void __launch_bounds__(kBitsThreads) compact_bits_kernel(
     const uint32_t* __restrict__ vis_bits, uint32_t n_words, uint32_t words_per_view, uint32_t n,
-    const float4* __restrict__ rec2, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
+    const uint32_t* __restrict__ depths, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
     uint32_t* __restrict__ list, uint32_t* __restrict__ n_out, Lookback lb, uint32_t n_tiles) {
   chain_wait();
   __shared__ uint32_t s_list[kBitsWarps][32 * 32];
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kBitsThreads) compact_bits_kernel(
       for (int u = 0; u < kBitsLoads; ++u) vi[u] = t0 + 32 * u < total[j] ? mine[t0 + 32 * u] : 0u;
 #pragma unroll
       for (int u = 0; u < kBitsLoads; ++u)
-        key[u] = t0 + 32 * u < total[j] ? __float_as_uint(rec2[vi[u]].w) : 0u;
+        key[u] = t0 + 32 * u < total[j] ? depths[vi[u]] : 0u;
 #pragma unroll
       for (int u = 0; u < kBitsLoads; ++u) {
         const uint32_t t = t0 + 32 * u;
@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_downsweep_kernel(
 }
 
 // ------------------------------------------------------------------------------------------
-// Wide radix passes for large sorts (the pair list: 10^7 - 10^8 keys): digits of up to 9 bits,
+// Wide radix passes for large sorts (10^6 - 10^8 keys): digits of up to 9 bits,
 // so that the 17-bit tile ids of a 16-view 1080p window sort in two passes instead of three, and
 // blocks of kWideTile = 8192 keys (512 threads x 16), so that each digit's run inside a block is
 // long enough for coalesced stores. The same three kernels per pass as above:
@@ -935,7 +935,7 @@ cudaError_t launch_exclusive_scan_single_pass(const uint32_t* in, uint32_t* out,
 }
 
 cudaError_t launch_compact_visible(const uint32_t* vis_bits, int n_views, int n,
-                                   const float4* rec2, uint32_t* keys, uint32_t* vals,
+                                   const uint32_t* depths, uint32_t* keys, uint32_t* vals,
                                    uint32_t* list, uint32_t* n_out, Lookback lb,
                                    cudaStream_t stream) {
   const int64_t words = (int64_t)n_views * vis_bit_words_per_view(n);
@@ -944,7 +944,7 @@ cudaError_t launch_compact_visible(const uint32_t* vis_bits, int n_views, int n,
   if (tiles > lb.capacity) return cudaErrorInvalidValue;
   const cudaError_t e = launch_chained(
       compact_bits_kernel, dim3((unsigned)tiles), dim3(kBitsThreads), stream, vis_bits,
-      (uint32_t)words, (uint32_t)vis_bit_words_per_view(n), (uint32_t)n, rec2, keys, vals, list,
+      (uint32_t)words, (uint32_t)vis_bit_words_per_view(n), (uint32_t)n, depths, keys, vals, list,
       n_out, lb, (uint32_t)tiles);
   RGS_LAUNCHED();
   return e;
@@ -956,9 +956,6 @@ cudaError_t launch_tile_ranges_scan(const uint32_t* counts, uint2* ranges, int64
   return run_scan(PlainLoad{counts}, RangeStore{ranges, capacity}, n_tiles, nullptr, total,
                   nullptr, stream, lb);
 }
-
-// Sorts of at least this many keys (capacity) take the wide passes.
-constexpr int64_t kWideMinN = 4 << 20;
 
 cudaError_t radix_sort_wide(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
                             int64_t n_cap, const uint32_t* n_dev, int begin_bit, int end_bit,
