@@ -23,11 +23,12 @@ namespace {
 // operands straight from shared memory:
 //   [0] (mx hi, mx hi), (mx lo, mx lo)   [1] (l11, l11), (c21, c21)
 //   [2] (l21, l21), (l22, l22)           [3] (s_a, s_a), (-log2 o, -log2 o)
-//   [4] (r, r), (g, g)                   [5] (b, b), (z, z)
+//   [4] (r, r), (g, g)                   [5] (b, b), (z, z); for the backward (b, b), (z, r_g)
+// with r_g the row of the tile nearest to the Gaussian's centre, relative to the anchor row.
 // With one pixel per thread rows 0..2 hold (mx hi, mx lo, l11, c21), (l21, l22, s_a, -log2 o)
 // and the colour as float4.
 // ------------------------------------------------------------------------------------------
-template <int R, int N>
+template <int kTileH, bool kBackward, int R, int N>
 __device__ __forceinline__ void stage_gaussian(ulonglong2 (&sp)[R][N], int t, float4 r0,
                                                float4 r1, float4 r2, float y_a) {
   const AnchorTerms at = anchor_terms(r0, r1, y_a);
@@ -38,7 +39,10 @@ __device__ __forceinline__ void stage_gaussian(ulonglong2 (&sp)[R][N], int t, fl
     sp[2][t] = make_ulonglong2(f2_make(r1.y, r1.y), f2_make(r1.z, r1.z));
     sp[3][t] = make_ulonglong2(f2_make(at.s_a, at.s_a), f2_make(nlo, nlo));
     sp[4][t] = make_ulonglong2(f2_make(r2.x, r2.x), f2_make(r2.y, r2.y));
-    sp[5][t] = make_ulonglong2(f2_make(r2.z, r2.z), f2_make(r2.w, r2.w));
+    float last = r2.w;
+    if constexpr (kBackward)
+      last = fminf(fmaxf(rintf(-at.dya), (float)(-kTileH / 2)), (float)(kTileH - 1 - kTileH / 2));
+    sp[5][t] = make_ulonglong2(f2_make(r2.z, r2.z), f2_make(r2.w, last));
   } else {
     reinterpret_cast<float4*>(sp[0])[t] = make_float4(r0.x, r0.z, r1.x, at.c21);
     reinterpret_cast<float4*>(sp[1])[t] = make_float4(r1.y, r1.z, at.s_a, nlo);
@@ -141,8 +145,6 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
         FR[q] = f2_make(stop0 ? kFarRow : f2_lo(FR[q]), stop1 ? kFarRow : f2_hi(FR[q]));
         if (stop0) visited_end[k0] = pos + 1;
         if (stop1) visited_end[k1] = pos + 1;
-        done[k0] = done[k0] || stop0;
-        done[k1] = done[k1] || stop1;
         live -= (int)stop0 + (int)stop1;
       }
       C02[q] = f2_fma(w, CA.x, C02[q]);
@@ -158,7 +160,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
     const uint32_t j = start + threadIdx.x;
     if (j < range.y) {
       const uint32_t vi = pair_vals[j];
-      stage_gaussian(sp, threadIdx.x, rec[vi].mean, rec[vi].conic, rec[vi].colour, y_a);
+      stage_gaussian<TH, false>(sp, threadIdx.x, rec[vi].mean, rec[vi].conic, rec[vi].colour, y_a);
     }
     __syncthreads();
     const int cnt = (int)min((uint32_t)kThreads, range.y - start);
@@ -206,6 +208,8 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
   if constexpr (kPacked) {
 #pragma unroll
     for (int q = 0; q < P2; ++q) {
+      done[2 * q] = f2_lo(FR[q]) == kFarRow;
+      done[2 * q + 1] = f2_hi(FR[q]) == kFarRow;
       T[2 * q] = f2_lo(T2[q]);
       T[2 * q + 1] = f2_hi(T2[q]);
       C0[2 * q] = f2_lo(C02[q]);
@@ -262,8 +266,9 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
 // +8 % on ten 640x480 views).
 //
 // The lane's values: sdp, sr | srr, t_a sdp | t_a sr, t_a^2 sdp | gr, gg | gb, gz, with sdp, sr, srr
-// the sums of dp, dp r and dp r^2 over its pixels (r the row offset from the tile's anchor row), t_a
-// the whitened offset of its column at the anchor row, and gr .. gz the colour and depth weights
+// the sums of dp, dp r and dp r^2 over its pixels (r the row offset from the tile row nearest to the
+// Gaussian's centre; from the tile's anchor row with one pixel per thread), t_a the whitened offset
+// of its column at that row, and gr .. gz the colour and depth weights
 // (gz 0 without a depth or opacity gradient).
 // ------------------------------------------------------------------------------------------
 constexpr int kRedPad = 68;  // floats per row of 32 lane pairs, padded
@@ -403,8 +408,9 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
     constexpr bool kClamp = decltype(clamp_tag)::value;
     (void)kClamp;  // the one-pixel path always clamps
     // Per-thread sums of dp = dL/dpower over the thread's pixels, weighted by their row offset
-    // r from the anchor row: sdp = sum dp, sr = sum dp r, srr = sum dp r^2. Every pixel of the
-    // column has w = (t, s) = (t_a + r l21, s_a + r l22), so the whitened moments follow from
+    // r from row r_g (0, the anchor row, with one pixel per thread): sdp = sum dp, sr = sum dp r,
+    // srr = sum dp r^2. Every pixel of the column has w = (t, s) = (t_a + r l21, s_a + r l22) with
+    // t_a, s_a at that row, so the whitened moments follow from
     // these three and t_a once per Gaussian.
     float sdp = 0.0f, sr = 0.0f, srr = 0.0f, ta = 0.0f, gr = 0.0f, gg = 0.0f, gb = 0.0f,
           gz = 0.0f;
@@ -414,8 +420,9 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
         const ulonglong2 CA = sp[4 % (kPacked ? 6 : 3)][g], CB = sp[5 % (kPacked ? 6 : 3)][g];
         const f32x2 dx2 = f2_sub(f2_sub(FX, X.x), X.y);
         const f32x2 TA = f2_fma(L1.x, dx2, L1.y);
-        f32x2 aR = ZERO2, aG = ZERO2, aB = ZERO2, aZ = ZERO2, mP = ZERO2, mY = ZERO2,
-              mYY = ZERO2;
+        const f32x2 Z2 = f2_make(f2_lo(CB.y), f2_lo(CB.y));
+        (void)Z2;
+        f32x2 aR = ZERO2, aG = ZERO2, aB = ZERO2, aZ = ZERO2, dps[P2];
         (void)aZ;
 #pragma unroll
         for (int q = P2 - 1; q >= 0; --q) {
@@ -443,7 +450,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
           if constexpr (kAux) {
             aZ = q == P2 - 1 ? f2_mul(GD2[q], w) : f2_fma(GD2[q], w, aZ);
             qv = f2_fma(GC02[q], CA.x,
-                        f2_fma(GC12[q], CA.y, f2_fma(GC22[q], CB.x, f2_mul(GD2[q], CB.y))));
+                        f2_fma(GC12[q], CA.y, f2_fma(GC22[q], CB.x, f2_mul(GD2[q], Z2))));
           } else {
             qv = f2_fma(GC02[q], CA.x, f2_fma(GC12[q], CA.y, f2_mul(GC22[q], CB.x)));
           }
@@ -456,31 +463,43 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
             const bool m0 = oG0 < c.alpha_max, m1 = oG1 < c.alpha_max;
             dp = f2_make(m0 ? f2_lo(dp) : 0.0f, m1 ? f2_hi(dp) : 0.0f);
           }
-          // Suffix sums over the pairs, last pair first: mP = sum dp, mY = sum q dp,
-          // mYY = sum q (q + 1) / 2 dp (seven additions for four pairs; weighting each pair by its
-          // row offset and the offset's square took two multiply-adds and an addition per pair).
-          mP = q == P2 - 1 ? dp : f2_add(mP, dp);
-          if (q > 0) {
-            mY = q == P2 - 1 ? mP : f2_add(mY, mP);
-            mYY = q == P2 - 1 ? mY : f2_add(mYY, mY);
-          }
+          dps[q] = dp;
         }
         gr = f2_lo(aR) + f2_hi(aR);
         gg = f2_lo(aG) + f2_hi(aG);
         gb = f2_lo(aB) + f2_hi(aB);
         if constexpr (kAux) gz = f2_lo(aZ) + f2_hi(aZ);
-        sdp = f2_lo(mP) + f2_hi(mP);
-        {
-          // Over the thread's rows k = 2 q + (0, 1): k1 = sum dp k, k2 = sum dp k^2; then over the
-          // row offsets r = r0 + k.
-          const float ys = f2_lo(mY) + f2_hi(mY), zs = f2_lo(mYY) + f2_hi(mYY);
-          const float k1 = fmaf(2.0f, ys, f2_hi(mP));
-          const float k2 = fmaf(8.0f, zs, fmaf(-4.0f, f2_lo(mY), f2_hi(mP)));
-          const float r0f = (float)r0_;
-          sr = fmaf(r0f, sdp, k1);
-          srr = fmaf(r0f, k1 + sr, k2);
+        // Moments about the middle of the thread's rows, folded by symmetry: pair q's middle lies
+        // p_q = 2 q - (P2 - 1) rows from there and its pixels half a row to either side, so with
+        // mP = sum dp, mF = sum p_q dp, mQ = sum p_q^2 dp the first and second moments are
+        // k1 = sum mF + (hi - lo) mP / 2 and k2 = sum mQ + (hi - lo) mF + sum mP / 4 (seven
+        // packed operations for four pairs). Sums from the thread's first row took as many and
+        // cancelled up to 225 : 1 in the shift to another row, these 64 : 1.
+        f32x2 mP, mF = ZERO2, mQ = ZERO2;
+        if constexpr (P2 == 4) {
+          const f32x2 A = f2_add(dps[3 % P2], dps[0]), B = f2_add(dps[2 % P2], dps[1 % P2]);
+          const f32x2 C = f2_sub(dps[3 % P2], dps[0]), D = f2_sub(dps[2 % P2], dps[1 % P2]);
+          mP = f2_add(A, B);
+          mF = f2_fma(f2_make(3.0f, 3.0f), C, D);
+          mQ = f2_fma(f2_make(9.0f, 9.0f), A, B);
+        } else if constexpr (P2 == 2) {
+          mP = mQ = f2_add(dps[1 % P2], dps[0]);
+          mF = f2_sub(dps[1 % P2], dps[0]);
+        } else {
+          mP = dps[0];
         }
-        ta = f2_lo(TA);
+        sdp = f2_lo(mP) + f2_hi(mP);
+        const float k1 = fmaf(0.5f, f2_hi(mP) - f2_lo(mP), f2_lo(mF) + f2_hi(mF));
+        const float k2 =
+            fmaf(0.25f, sdp, (f2_lo(mQ) + f2_hi(mQ)) + (f2_hi(mF) - f2_lo(mF)));
+        // Then over the rows' offsets r - r_g from the tile row nearest to the Gaussian's centre:
+        // the lanes' sums and the whitened moments formed from them are then about the size of
+        // the result. About the tile's middle row a Gaussian seven rows away cancelled 50 : 1.
+        const float r_g = f2_hi(CB.y);
+        const float rc = ((float)r0_ + 0.5f * (float)(PPT - 1)) - r_g;
+        sr = fmaf(rc, sdp, k1);
+        srr = fmaf(rc, k1 + sr, k2);
+        ta = fmaf(r_g, f2_lo(L2.x), f2_lo(TA));
       } else {
         const float4 g0 = reinterpret_cast<const float4*>(sp[0])[g];
         const float4 g1 = reinterpret_cast<const float4*>(sp[1])[g];
@@ -553,7 +572,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
       if constexpr (kPacked) {
         l21 = f2_lo(sp[2][g].x);
         l22 = f2_lo(sp[2][g].y);
-        s_a = f2_lo(sp[3][g].x);
+        s_a = fmaf(f2_hi(sp[5 % (kPacked ? 6 : 3)][g].y), l22, f2_lo(sp[3][g].x));
       } else {
         const float4 g1 = reinterpret_cast<const float4*>(sp[1])[g];
         l21 = g1.x;
@@ -591,7 +610,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
     if (j < bend) {
       const uint32_t vi = pair_vals[j];
       s_vi[threadIdx.x] = vi;
-      stage_gaussian(sp, threadIdx.x, rec[vi].mean, rec[vi].conic, rec[vi].colour, y_a);
+      stage_gaussian<TH, true>(sp, threadIdx.x, rec[vi].mean, rec[vi].conic, rec[vi].colour, y_a);
     }
     __syncthreads();
     // Positions above the warp's smallest last index test each pixel; the rest do not. Whether

@@ -263,11 +263,11 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // its tile row, so both blends take identical coverage decisions whatever their pixels per
 // thread.
 struct AnchorTerms {
-  float c21, s_a;
+  float c21, s_a, dya;  // dya: the anchor row's offset from the Gaussian's centre
 };
 __device__ __forceinline__ AnchorTerms anchor_terms(float4 r0, float4 r1, float y_a) {
   const float dya = __fsub_rn(__fsub_rn(y_a, r0.y), r0.w);
-  return AnchorTerms{__fmul_rn(r1.y, dya), __fmul_rn(r1.z, dya)};
+  return AnchorTerms{__fmul_rn(r1.y, dya), __fmul_rn(r1.z, dya), dya};
 }
 // t at the anchor row of column px.
 __device__ __forceinline__ float column_t(float px, float4 r0, float l11, float c21) {
