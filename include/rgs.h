@@ -98,9 +98,10 @@ typedef struct {
                                 depend on it or on the tile shape beyond atomics-order rounding of
                                 the gradients */
   int32_t backward_pixels_per_thread; /* the same for the backward blend (same rules); 0 = equal to
-                                         pixels_per_thread. The two blends share only the tile
-                                         shape: the per-pixel state between them is stored in
-                                         image order */
+                                         pixels_per_thread, or 8 in place of 4 where the batch has
+                                         tiles enough (of 16x16 or 32x8). The two
+                                         blends share only the tile shape: the per-pixel state
+                                         between them is stored in image order */
   void* sh_ready_event; /* optional cudaEvent_t, or NULL. NULL: the projection evaluates the
                            colours (Eq. app-sh) and culls entries with a non-finite coefficient.
                            An event: the forward reads the SH coefficients only after the tile

@@ -466,6 +466,14 @@ cudaError_t close_state(State& s, bool capturing, cudaStream_t stream) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Where the caller leaves the backward blend's pixels per thread open, 8 take the place of 4 from
+// this many 256-pixel tiles on. With 8 a tile is one warp, which reads every staged Gaussian once
+// and reduces its gradient sums once, but a launch needs enough tiles to occupy the SMs: 16 such
+// warps are resident per SM, and the line lies at 12. Measured with 4 -> 8 (us): 80 tiles
+// 43 -> 54, 300 tiles 35 -> 46, 1200 tiles 42 -> 44; 2400 tiles 70 -> 56, 2508 tiles 74 -> 72,
+// 3225 tiles 89 -> 81, 8160 tiles 167 -> 133, 12000 tiles 265 -> 204.
+constexpr long long kBackwardWideTiles = 12 * 152;
+
 rgs_status build_views(rgs_ctx* ctx, const rgs_camera* cams, int n_views, const rgs_config& cfg,
                        Views& views, Consts& consts) {
   if (!cams) return fail(ctx, RGS_ERR_INVALID_ARG, "cams is null");
@@ -537,6 +545,9 @@ rgs_status build_views(rgs_ctx* ctx, const rgs_camera* cams, int n_views, const 
   views.total_tiles = (int)tiles;
   views.total_cells = (int)cells;
   views.total_pixels = pix;
+  if (cfg.backward_pixels_per_thread == 0 && ppt == 4 && tw * th == 256 &&
+      tiles >= kBackwardWideTiles)
+    views.bwd_pixels_per_thread = 8;
   consts.alpha_min = cfg.alpha_min;
   consts.alpha_max = cfg.alpha_max;
   consts.t_min = cfg.t_min;
