@@ -18,36 +18,91 @@ namespace {
 
 // ------------------------------------------------------------------------------------------
 // Staging of a batch of Gaussians in shared memory, with the row terms of the tile's anchor row
-// y_a (anchor_terms). For an even number of pixels per thread every per-Gaussian operand is
-// stored twice, as (x, x) pairs, so the packed f32x2 arithmetic of two pixels reads its broadcast
-// operands straight from shared memory:
-//   [0] (mx hi, mx hi), (mx lo, mx lo)   [1] (l11, l11), (c21, c21)
-//   [2] (l21, l21), (l22, l22)           [3] (s_a, s_a), (-log2 o, -log2 o)
-//   [4] (r, r), (g, g)                   [5] (b, b), (z, z); for the backward (b, b), (z, r_g)
-// with r_g the row of the tile nearest to the Gaussian's centre, relative to the anchor row.
-// With one pixel per thread rows 0..2 hold (mx hi, mx lo, l11, c21), (l21, l22, s_a, -log2 o)
-// and the colour as float4.
+// y_a (anchor_terms), as 16-byte rows:
+//   column  (mx hi, mx lo), (l11, c21): what a thread needs once for its column
+//   shape   (l21, l22), (s_a, -log2 o)
+//   colour  (r, g), (b, z)
+// For an even number of pixels per thread the packed f32x2 arithmetic of two pixels reads shape and
+// colour as (x, x) pairs. Stored doubled (two rows in place of one) they arrive paired; stored once,
+// a thread pairs them with register moves. The blends are held up by the bytes their warps read
+// from shared memory (a 16-byte broadcast row occupies the SM's 128 bytes per cycle for four
+// cycles) as much as by issue slots, so what is best depends on how many pixel pairs share a read.
+// Blends of 16 views of 1080p, by rows per Gaussian (column row single, the others as said):
+//   forward, 4 pixels: all doubled, column row too 2.97 ms, 2.82 with it single; shape single 2.64;
+//     shape and colour single 2.86
+//   forward, 8 pixels: 2.98, 2.93, 2.81, 2.56
+//   backward, 8 pixels: 4.39, 4.32, 4.50, 4.47
+// For the backward the z of a doubled colour gives its place to r_g: (b, b), (z, r_g), with r_g the
+// row of the tile nearest to the Gaussian's centre, relative to the anchor row.
 // ------------------------------------------------------------------------------------------
-template <int kTileH, bool kBackward, int R, int N>
+template <bool kBackward, int PPT>
+struct StageLayout {
+  static constexpr bool kPacked = PPT % 2 == 0;
+  static constexpr bool kShapeTwice = kPacked && kBackward;
+  static constexpr bool kColourTwice = kPacked && (kBackward || PPT < 8);
+  static constexpr int kShape = 1;
+  static constexpr int kColour = kShape + (kShapeTwice ? 2 : 1);
+  static constexpr int kRows = kColour + (kColourTwice ? 2 : 1);
+};
+
+template <int kTileH, bool kBackward, int PPT, int R, int N>
 __device__ __forceinline__ void stage_gaussian(ulonglong2 (&sp)[R][N], int t, float4 r0,
                                                float4 r1, float4 r2, float y_a) {
+  using L = StageLayout<kBackward, PPT>;
+  static_assert(R == L::kRows, "rows of the layout");
   const AnchorTerms at = anchor_terms(r0, r1, y_a);
   const float nlo = -r1.w;
-  if constexpr (R == 6) {
-    sp[0][t] = make_ulonglong2(f2_make(r0.x, r0.x), f2_make(r0.z, r0.z));
-    sp[1][t] = make_ulonglong2(f2_make(r1.x, r1.x), f2_make(at.c21, at.c21));
-    sp[2][t] = make_ulonglong2(f2_make(r1.y, r1.y), f2_make(r1.z, r1.z));
-    sp[3][t] = make_ulonglong2(f2_make(at.s_a, at.s_a), f2_make(nlo, nlo));
-    sp[4][t] = make_ulonglong2(f2_make(r2.x, r2.x), f2_make(r2.y, r2.y));
+  sp[0][t] = make_ulonglong2(f2_make(r0.x, r0.z), f2_make(r1.x, at.c21));
+  if constexpr (L::kShapeTwice) {
+    sp[L::kShape][t] = make_ulonglong2(f2_make(r1.y, r1.y), f2_make(r1.z, r1.z));
+    sp[L::kShape + 1][t] = make_ulonglong2(f2_make(at.s_a, at.s_a), f2_make(nlo, nlo));
+  } else {
+    sp[L::kShape][t] = make_ulonglong2(f2_make(r1.y, r1.z), f2_make(at.s_a, nlo));
+  }
+  if constexpr (L::kColourTwice) {
     float last = r2.w;
     if constexpr (kBackward)
       last = fminf(fmaxf(rintf(-at.dya), (float)(-kTileH / 2)), (float)(kTileH - 1 - kTileH / 2));
-    sp[5][t] = make_ulonglong2(f2_make(r2.z, r2.z), f2_make(r2.w, last));
+    sp[L::kColour][t] = make_ulonglong2(f2_make(r2.x, r2.x), f2_make(r2.y, r2.y));
+    sp[L::kColour + 1][t] = make_ulonglong2(f2_make(r2.z, r2.z), f2_make(r2.w, last));
   } else {
-    reinterpret_cast<float4*>(sp[0])[t] = make_float4(r0.x, r0.z, r1.x, at.c21);
-    reinterpret_cast<float4*>(sp[1])[t] = make_float4(r1.y, r1.z, at.s_a, nlo);
-    reinterpret_cast<float4*>(sp[2])[t] = r2;
+    sp[L::kColour][t] = make_ulonglong2(f2_make(r2.x, r2.y), f2_make(r2.z, r2.w));
   }
+}
+
+// Two values of a row as (x, x), (y, y).
+__device__ __forceinline__ ulonglong2 f2_spread(f32x2 v) {
+  return make_ulonglong2(f2_make(f2_lo(v), f2_lo(v)), f2_make(f2_hi(v), f2_hi(v)));
+}
+// Staged Gaussian g for the packed arithmetic: column row, (l21, l22), (s_a, -log2 o), (r, g),
+// (b, z or (z, r_g)), each value of the last four twice.
+struct Staged {
+  ulonglong2 column, l2, sn, rg, bz;
+};
+template <bool kBackward, int PPT, int R, int N>
+__device__ __forceinline__ Staged staged(const ulonglong2 (&sp)[R][N], int g) {
+  using L = StageLayout<kBackward, PPT>;
+  Staged s;
+  s.column = sp[0][g];
+  s.l2 = sp[L::kShape][g];
+  if constexpr (L::kShapeTwice) {
+    s.sn = sp[L::kShape + 1][g];
+  } else {
+    s.sn = f2_spread(s.l2.y);
+    s.l2 = f2_spread(s.l2.x);
+  }
+  s.rg = sp[L::kColour][g];
+  if constexpr (L::kColourTwice) {
+    s.bz = sp[L::kColour + 1][g];
+  } else {
+    s.bz = f2_spread(s.rg.y);
+    s.rg = f2_spread(s.rg.x);
+  }
+  return s;
+}
+// t of a thread's column at the anchor row, from the column row.
+__device__ __forceinline__ float column_t(float fx, ulonglong2 x) {
+  return __fmaf_rn(f2_lo(x.y), __fsub_rn(__fsub_rn(fx, f2_lo(x.x)), f2_hi(x.x)), f2_hi(x.y));
 }
 
 // ------------------------------------------------------------------------------------------
@@ -78,7 +133,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
   constexpr bool kPacked = PPT % 2 == 0;
   constexpr int P2 = kPacked ? PPT / 2 : 1;
   static_assert(kThreads % 32 == 0, "whole warps only");
-  __shared__ ulonglong2 sp[kPacked ? 6 : 3][kThreads];
+  __shared__ ulonglong2 sp[StageLayout<false, PPT>::kRows][kThreads];
   __shared__ unsigned long long s_eval[kThreads / 32];
   const int gtile = (int)tile_order[blockIdx.x];
   const int v = view_of_tile(views, gtile);
@@ -115,21 +170,19 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
     C02[q] = C12[q] = C22[q] = D2[q] = f2_make(0.0f, 0.0f);
     FR[q] = f2_make(done[k0] ? kFarRow : (float)(r0_ + k0), done[k1] ? kFarRow : (float)(r0_ + k1));
   }
-  const f32x2 FX = f2_make(fx, fx);
 
   // One staged Gaussian (list position pos, slot g) against the thread's pixel pairs.
   auto composite_pairs = [&](uint32_t pos, int g) {
-    const ulonglong2 X = sp[0][g], L1 = sp[1][g], L2 = sp[2][g], L3 = sp[3][g];
-    const ulonglong2 CA = sp[4 % (kPacked ? 6 : 3)][g], CB = sp[5 % (kPacked ? 6 : 3)][g];
+    const Staged st = staged<false, PPT>(sp, g);
     // Whitened offset t at the anchor row of the thread's column (Eq. alpha's exponent).
-    const f32x2 dx = f2_sub(f2_sub(FX, X.x), X.y);
-    const f32x2 TA = f2_fma(L1.x, dx, L1.y);
+    const float ta = column_t(fx, st.column);
+    const f32x2 TA = f2_make(ta, ta);
 #pragma unroll
     for (int q = 0; q < P2; ++q) {
       const int k0 = 2 * q, k1 = 2 * q + 1;
-      const f32x2 tt = f2_fma(FR[q], L2.x, TA);
-      const f32x2 ss = f2_fma(FR[q], L2.y, L3.x);
-      const f32x2 nq = f2_fma(tt, tt, f2_fma(ss, ss, L3.y));  // -log2(o G)
+      const f32x2 tt = f2_fma(FR[q], st.l2.x, TA);
+      const f32x2 ss = f2_fma(FR[q], st.l2.y, st.sn.x);
+      const f32x2 nq = f2_fma(tt, tt, f2_fma(ss, ss, st.sn.y));  // -log2(o G)
       const float a0 = fminf(c.alpha_max, ex2_neg_approx(f2_lo(nq)));
       const float a1 = fminf(c.alpha_max, ex2_neg_approx(f2_hi(nq)));
       // w = alpha T and the transmittance after this Gaussian T' = T - w; an uncovered pixel
@@ -147,10 +200,10 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
         if (stop1) visited_end[k1] = pos + 1;
         live -= (int)stop0 + (int)stop1;
       }
-      C02[q] = f2_fma(w, CA.x, C02[q]);
-      C12[q] = f2_fma(w, CA.y, C12[q]);
-      C22[q] = f2_fma(w, CB.x, C22[q]);
-      D2[q] = f2_fma(w, CB.y, D2[q]);
+      C02[q] = f2_fma(w, st.rg.x, C02[q]);
+      C12[q] = f2_fma(w, st.rg.y, C12[q]);
+      C22[q] = f2_fma(w, st.bz.x, C22[q]);
+      D2[q] = f2_fma(w, st.bz.y, D2[q]);
       T2[q] = Tn;
     }
   };
@@ -160,15 +213,18 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
     const uint32_t j = start + threadIdx.x;
     if (j < range.y) {
       const uint32_t vi = pair_vals[j];
-      stage_gaussian<TH, false>(sp, threadIdx.x, rec[vi].mean, rec[vi].conic, rec[vi].colour, y_a);
+      stage_gaussian<TH, false, PPT>(sp, threadIdx.x, rec[vi].mean, rec[vi].conic,
+                                     rec[vi].colour, y_a);
     }
     __syncthreads();
     const int cnt = (int)min((uint32_t)kThreads, range.y - start);
     // The warp leaves the batch together, once none of its pixels is live: a stopped pixel
     // composites nothing more (its alpha is 0), and a loop without per-thread exits ran 9 %
-    // faster than one that let each thread leave on its own.
+    // faster than one that let each thread leave on its own. The vote is taken before a visit and
+    // followed after it, so that it waits for nothing (a view of 160x120: 33 -> 29 us; the one
+    // visit more changes nothing).
     for (int g = 0; g < cnt; ++g) {
-      if (!__any_sync(0xffffffffu, live > 0)) break;
+      const bool go_on = __any_sync(0xffffffffu, live > 0);
       const uint32_t pos = start + g;
       if constexpr (kPacked) {
         // Always with the clamp: a warp-uniform clamp-free variant (as in the backward) made
@@ -203,6 +259,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
           }
         }
       }
+      if (!go_on) break;
     }
   }
   if constexpr (kPacked) {
@@ -315,7 +372,8 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
   constexpr int P2 = kPacked ? PPT / 2 : 1;
   static_assert(kThreads % 32 == 0, "whole warps only");
   using RL = RedLayout;
-  __shared__ ulonglong2 sp[kPacked ? 6 : 3][kThreads];
+  using SL = StageLayout<true, PPT>;
+  __shared__ ulonglong2 sp[SL::kRows][kThreads];
   __shared__ uint32_t s_vi[kThreads];
   __shared__ int s_max_last[kThreads / 32];
   __shared__ __align__(16) float s_red[kThreads / 32][RL::kRows * kRedPad];
@@ -380,7 +438,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
     GD2[q] = f2_make(gD[k0], gD[k1]);
     FR[q] = f2_make((float)(r0_ + k0), (float)(r0_ + k1));
   }
-  const f32x2 FX = f2_make(fx, fx), ONE2 = f2_make(1.0f, 1.0f), ZERO2 = f2_make(0.0f, 0.0f);
+  const f32x2 ONE2 = f2_make(1.0f, 1.0f), ZERO2 = f2_make(0.0f, 0.0f);
   // Only list positions up to the largest last-contributor index of the tile matter.
   int m = thread_last;
 #pragma unroll
@@ -416,20 +474,19 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
           gz = 0.0f;
     if (!kCheckLast || jj <= thread_last) {
       if constexpr (kPacked) {
-        const ulonglong2 X = sp[0][g], L1 = sp[1][g], L2 = sp[2][g], L3 = sp[3][g];
-        const ulonglong2 CA = sp[4 % (kPacked ? 6 : 3)][g], CB = sp[5 % (kPacked ? 6 : 3)][g];
-        const f32x2 dx2 = f2_sub(f2_sub(FX, X.x), X.y);
-        const f32x2 TA = f2_fma(L1.x, dx2, L1.y);
-        const f32x2 Z2 = f2_make(f2_lo(CB.y), f2_lo(CB.y));
+        const Staged st = staged<true, PPT>(sp, g);
+        const float ta0 = column_t(fx, st.column);
+        const f32x2 TA = f2_make(ta0, ta0);
+        const f32x2 Z2 = f2_make(f2_lo(st.bz.y), f2_lo(st.bz.y));
         (void)Z2;
         f32x2 aR = ZERO2, aG = ZERO2, aB = ZERO2, aZ = ZERO2, dps[P2];
         (void)aZ;
 #pragma unroll
         for (int q = P2 - 1; q >= 0; --q) {
           const int k0 = 2 * q, k1 = 2 * q + 1;
-          const f32x2 tt = f2_fma(FR[q], L2.x, TA);
-          const f32x2 ss = f2_fma(FR[q], L2.y, L3.x);
-          const f32x2 nq = f2_fma(tt, tt, f2_fma(ss, ss, L3.y));  // -log2(o G)
+          const f32x2 tt = f2_fma(FR[q], st.l2.x, TA);
+          const f32x2 ss = f2_fma(FR[q], st.l2.y, st.sn.x);
+          const f32x2 nq = f2_fma(tt, tt, f2_fma(ss, ss, st.sn.y));  // -log2(o G)
           const float oG0 = ex2_neg_approx(f2_lo(nq)), oG1 = ex2_neg_approx(f2_hi(nq));
           const float a0 = kClamp ? fminf(c.alpha_max, oG0) : oG0;
           const float a1 = kClamp ? fminf(c.alpha_max, oG1) : oG1;
@@ -449,10 +506,11 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
           f32x2 qv;
           if constexpr (kAux) {
             aZ = q == P2 - 1 ? f2_mul(GD2[q], w) : f2_fma(GD2[q], w, aZ);
-            qv = f2_fma(GC02[q], CA.x,
-                        f2_fma(GC12[q], CA.y, f2_fma(GC22[q], CB.x, f2_mul(GD2[q], Z2))));
+            qv = f2_fma(GC02[q], st.rg.x,
+                        f2_fma(GC12[q], st.rg.y, f2_fma(GC22[q], st.bz.x, f2_mul(GD2[q], Z2))));
           } else {
-            qv = f2_fma(GC02[q], CA.x, f2_fma(GC12[q], CA.y, f2_mul(GC22[q], CB.x)));
+            qv = f2_fma(GC02[q], st.rg.x,
+                        f2_fma(GC12[q], st.rg.y, f2_mul(GC22[q], st.bz.x)));
           }
           const f32x2 diff = f2_sub(qv, U2[q]);
           U2[q] = f2_fma(am, diff, U2[q]);
@@ -495,11 +553,11 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
         // Then over the rows' offsets r - r_g from the tile row nearest to the Gaussian's centre:
         // the lanes' sums and the whitened moments formed from them are then about the size of
         // the result. About the tile's middle row a Gaussian seven rows away cancelled 50 : 1.
-        const float r_g = f2_hi(CB.y);
+        const float r_g = f2_hi(st.bz.y);
         const float rc = ((float)r0_ + 0.5f * (float)(PPT - 1)) - r_g;
         sr = fmaf(rc, sdp, k1);
         srr = fmaf(rc, k1 + sr, k2);
-        ta = fmaf(r_g, f2_lo(L2.x), f2_lo(TA));
+        ta = fmaf(r_g, f2_lo(st.l2.x), ta0);
       } else {
         const float4 g0 = reinterpret_cast<const float4*>(sp[0])[g];
         const float4 g1 = reinterpret_cast<const float4*>(sp[1])[g];
@@ -570,9 +628,9 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
       }
       float l21, l22, s_a;
       if constexpr (kPacked) {
-        l21 = f2_lo(sp[2][g].x);
-        l22 = f2_lo(sp[2][g].y);
-        s_a = fmaf(f2_hi(sp[5 % (kPacked ? 6 : 3)][g].y), l22, f2_lo(sp[3][g].x));
+        l21 = f2_lo(sp[SL::kShape][g].x);
+        l22 = f2_lo(sp[SL::kShape][g].y);
+        s_a = fmaf(f2_hi(sp[SL::kRows - 1][g].y), l22, f2_lo(sp[SL::kShape + 1][g].x));
       } else {
         const float4 g1 = reinterpret_cast<const float4*>(sp[1])[g];
         l21 = g1.x;
@@ -587,16 +645,19 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
         const float ws = fmaf(s_a, S[0], l22 * S[1]);
         const float u = fmaf(l21, S[2], S[4]);
         float* dst = g2d + (size_t)s_vi[g] * kG2Stride;
-        atomicAdd(dst + kM0, S[0]);
-        atomicAdd(dst + kWt, wt);
-        atomicAdd(dst + kWs, ws);
-        atomicAdd(dst + kWtt, fmaf(l21, S[4] + u, S[5]));
-        atomicAdd(dst + kWts, fmaf(s_a, wt, l22 * u));
-        atomicAdd(dst + kWss, fmaf(s_a, ws, l22 * fmaf(s_a, S[1], l22 * S[2])));
-        atomicAdd(dst + kGR, S[6]);
-        atomicAdd(dst + kGG, S[7]);
-        atomicAdd(dst + kGB, S[8]);
-        if constexpr (kAux) atomicAdd(dst + kGZ, S[9]);
+        // Three vector additions to the 64-byte record in place of nine or ten single ones.
+        static_assert(kM0 == 0 && kWt == 1 && kWs == 2 && kWtt == 3 && kWts == 4 && kWss == 5 &&
+                          kGR == 6 && kGG == 7 && kGB == 8 && kGZ == 9 && kG2Stride % 4 == 0,
+                      "the sums' order in the record");
+        atomicAdd(reinterpret_cast<float4*>(dst),
+                  make_float4(S[0], wt, ws, fmaf(l21, S[4] + u, S[5])));
+        atomicAdd(reinterpret_cast<float4*>(dst) + 1,
+                  make_float4(fmaf(s_a, wt, l22 * u),
+                              fmaf(s_a, ws, l22 * fmaf(s_a, S[1], l22 * S[2])), S[6], S[7]));
+        if constexpr (kAux)
+          atomicAdd(reinterpret_cast<float2*>(dst) + 4, make_float2(S[8], S[9]));
+        else
+          atomicAdd(dst + kGB, S[8]);
       }
     }
     __syncwarp();
@@ -607,17 +668,24 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
     const int bstart = max(first, bend - kThreads);
     __syncthreads();
     const int j = bstart + (int)threadIdx.x;
+    bool may_clamp = false;
     if (j < bend) {
       const uint32_t vi = pair_vals[j];
       s_vi[threadIdx.x] = vi;
-      stage_gaussian<TH, true>(sp, threadIdx.x, rec[vi].mean, rec[vi].conic, rec[vi].colour, y_a);
+      const float4 r1 = rec[vi].conic;
+      may_clamp = !(-r1.w > c.unclamped_neg_lo);
+      stage_gaussian<TH, true, PPT>(sp, threadIdx.x, rec[vi].mean, r1, rec[vi].colour, y_a);
     }
+    const unsigned clamp_bits = __ballot_sync(0xffffffffu, may_clamp);
     __syncthreads();
     // Positions above the warp's smallest last index test each pixel; the rest do not. Whether
-    // the staged Gaussian can reach alpha_max is warp-uniform (every thread reads its opacity).
+    // the staged Gaussian can reach alpha_max is warp-uniform. Where the block is one warp it is a
+    // bit of the staging vote, so that no load stands between two visits (16 views of 1080p: 4.51
+    // -> 4.40 ms); otherwise every thread reads its opacity.
     auto clamps = [&](int g) {
-      if constexpr (kPacked) return !(f2_lo(sp[3][g].y) > c.unclamped_neg_lo);
-      return true;
+      if constexpr (!kPacked) return true;
+      if constexpr (kThreads == 32) return ((clamp_bits >> g) & 1u) != 0u;
+      return !(f2_lo(sp[SL::kShape + 1][g].y) > c.unclamped_neg_lo);
     };
     int nb = 0, g_first = bend - 1 - bstart;
     auto next = [&](int g) {

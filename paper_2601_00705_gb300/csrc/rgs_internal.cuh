@@ -269,10 +269,6 @@ __device__ __forceinline__ AnchorTerms anchor_terms(float4 r0, float4 r1, float 
   const float dya = __fsub_rn(__fsub_rn(y_a, r0.y), r0.w);
   return AnchorTerms{__fmul_rn(r1.y, dya), __fmul_rn(r1.z, dya), dya};
 }
-// t at the anchor row of column px.
-__device__ __forceinline__ float column_t(float px, float4 r0, float l11, float c21) {
-  return __fmaf_rn(l11, __fsub_rn(__fsub_rn(px, r0.x), r0.z), c21);
-}
 // t^2 + s^2 - log2(o) = -log2(o G) at row offset r.
 __device__ __forceinline__ float neg_log2_og(float t_a, float s_a, float l21, float l22,
                                              float neg_lo, float r) {
