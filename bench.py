@@ -516,7 +516,11 @@ def phase_rooflines(phases, stats, n, V, K, tiles, hbm_peak, fp32_peak):
     - ranges: every pair's key read, two words written per tile, and the tile order's keys and
       values sorted (one pass, 24 B per tile);
     - preprocess backward: a 64 B record read and written per visible entry, the parameters read
-      and their gradients written once per Gaussian (11 + 3K floats each)."""
+      and their gradients written once per Gaussian (11 + 3K floats each).
+    Offsets, duplicate, tile sort and ranges are counted as a sort of every (tile, entry) pair
+    would move them. The library builds its lists in two levels (one entry per cell of 4x4 tiles is
+    sorted and then expanded) and moves fewer bytes, so their fractions compare with that sort and
+    can exceed 1."""
     nv, pairs, n_eval = stats["n_visible"], stats["n_pairs"], stats["n_eval"]
     tile_bits = max(1, int(np.ceil(np.log2(tiles + 2))))
     bytes_model = {

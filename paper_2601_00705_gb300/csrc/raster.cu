@@ -22,11 +22,12 @@ namespace {
 //   column  (mx hi, mx lo), (l11, c21): what a thread needs once for its column
 //   shape   (l21, l22), (s_a, -log2 o)
 //   colour  (r, g), (b, z)
-// For an even number of pixels per thread the packed f32x2 arithmetic of two pixels reads shape and
-// colour as (x, x) pairs. Stored doubled (two rows in place of one) they arrive paired; stored once,
-// a thread pairs them with register moves. The blends are held up by the bytes their warps read
-// from shared memory (a 16-byte broadcast row occupies the SM's 128 bytes per cycle for four
-// cycles) as much as by issue slots, so what is best depends on how many pixel pairs share a read.
+// For an even number of pixels per thread the packed f32x2 arithmetic of two pixels reads shape
+// and colour as (x, x) pairs. Stored doubled (two rows in place of one) they arrive paired; stored
+// once, a thread pairs them with register moves. The blends are bound by instruction issue and
+// wait on their shared-memory reads in between (a 16-byte broadcast row is one instruction and two
+// wavefronts of a pipe that is 44 to 52 % busy), so what is best depends on how many pixel pairs
+// share a read, and was measured:
 // Blends of 16 views of 1080p, by rows per Gaussian (column row single, the others as said):
 //   forward, 4 pixels: all doubled, column row too 2.97 ms, 2.82 with it single; shape single 2.64;
 //     shape and colour single 2.86
@@ -322,11 +323,11 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
 // floats took nine stores and two row passes per seven Gaussians (+3 % on the 16-view 1080p window,
 // +8 % on ten 640x480 views).
 //
-// The lane's values: sdp, sr | srr, t_a sdp | t_a sr, t_a^2 sdp | gr, gg | gb, gz, with sdp, sr, srr
-// the sums of dp, dp r and dp r^2 over its pixels (r the row offset from the tile row nearest to the
-// Gaussian's centre; from the tile's anchor row with one pixel per thread), t_a the whitened offset
-// of its column at that row, and gr .. gz the colour and depth weights
-// (gz 0 without a depth or opacity gradient).
+// The lane's values: sdp, sr | srr, t_a sdp | t_a sr, t_a^2 sdp | gr, gg | gb, gz, with sdp, sr,
+// srr the sums of dp, dp r and dp r^2 over its pixels (r the row offset from the tile row nearest
+// to the Gaussian's centre; from the tile's anchor row with one pixel per thread), t_a the whitened
+// offset of its column at that row, and gr .. gz the colour and depth weights (gz 0 without a depth
+// or opacity gradient).
 // ------------------------------------------------------------------------------------------
 constexpr int kRedPad = 68;  // floats per row of 32 lane pairs, padded
 
