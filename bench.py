@@ -465,11 +465,11 @@ def measure_tracking(r, params, cameras, images, hbm_peak, steps, flush):
                               "bytes_per_pixel": 68}}
 
 
-# FP64 operations of one two-view hypothesis of the triangulation (4x4 system, one-sided Jacobi,
+# FP64 operations of one two-view hypothesis of the triangulation (4x4 system, QR and Jacobi,
 # reprojection error and angle), counted from the kernel's double-precision instructions under
 # ncu on the seeding workload (FMA as 2; the division and square-root sequences included):
-# 1.772e9 over 409957 hypotheses.
-TRI_FP64_FLOP_PER_HYP = 4323
+# 7.635e8 over 409957 hypotheses.
+TRI_FP64_FLOP_PER_HYP = 1862
 FP64_NOMINAL_TFLOPS = 1.25  # GB300 dense FP64, nominal
 
 
