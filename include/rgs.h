@@ -141,7 +141,10 @@ typedef struct {
 
 /* Counters of the last forward on a state (read back with a stream synchronisation). */
 typedef struct {
-  int64_t n_visible;       /* (view, Gaussian) pairs that touch at least one tile */
+  int64_t n_visible;       /* (view, Gaussian) pairs seen: the footprint touches at least one
+                              tile, and its bounding radius sqrt(kappa (|J|_F^2 smax^2 + eps2d)),
+                              kappa = 2 ln(o / alpha_min), widened by 2 % and 4 px, reaches the
+                              image (edge tiles reach past it) */
   int64_t n_pairs;         /* duplicated (view, tile, Gaussian) entries (of the visible entries
                               kept, when status bit 2 is set) */
   int64_t n_eval;          /* (pixel, Gaussian) list positions visited by the forward blend */
@@ -373,7 +376,8 @@ typedef struct {
   float lambda_alpha;      /* weight of sum_i psi(alpha_i), psi = -log(alpha) - log(1 - alpha) */
   float lambda_mu;         /* weight of sum_i |mu_i - mu_bar_i|^2 */
   const float* ema_means;  /* DEVICE [n][3] anchor mu_bar, or NULL: no position term */
-  uint32_t* obs_count;     /* DEVICE [n] or NULL: += number of views of the forward that see i */
+  uint32_t* obs_count;     /* DEVICE [n] or NULL: += number of views of the forward that see i
+                              (as counted in rgs_stats.n_visible) */
   float* vis_score;        /* DEVICE [n] or NULL: += that number times alpha_i */
   double* value;           /* DEVICE [1] or NULL: R summed over all Gaussians */
 } rgs_map_reg;

@@ -286,32 +286,65 @@ __device__ __forceinline__ void load_sh(const float* __restrict__ sh, int i, flo
   }
 }
 
-// Forward, pass 1 (cull): one thread per (Gaussian, chunk of views). The entries that may touch the
+// Whether the footprint of an entry may reach the image: the rule, with the tile cover, of what
+// counts as seen (n_visible, the observation counts), so it must not depend on how loose the test
+// is that picks the candidates. The centre comes from plain FMA dot products and the radius from a
+// bound of the alpha >= alpha_min footprint: the largest eigenvalue of Sigma^I is at most
+// |J|_F^2 smax^2 + eps, so the radius is at most sqrt(kappa (|J|_F^2 smax^2 + eps)); widened by 2 %
+// and 4 px. An entry past the edge by less counts where a tile at the right or bottom edge reaches
+// past the image.
+__device__ __forceinline__ bool reaches_image(const ViewParams& vp, const PoseRef& ps,
+                                              const Consts& c, const float* m, const float* ls,
+                                              float logit) {
+  const float* R = ps.R;
+  const float z = fmaf(R[6], m[0], fmaf(R[7], m[1], fmaf(R[8], m[2], ps.t[2])));
+  const float z_err =
+      4.8e-7f * (fabsf(R[6] * m[0]) + fabsf(R[7] * m[1]) + fabsf(R[8] * m[2]) + fabsf(ps.t[2]));
+  if (!(z + z_err > c.znear && z > 0.0f)) return false;
+  const float smax2 = expf(2.0f * fmaxf(ls[0], fmaxf(ls[1], ls[2])));
+  const float opacity = 1.0f / (1.0f + expf(-logit));
+  const float kappa = 2.0f * logf(opacity / c.alpha_min);
+  const float x = fmaf(R[0], m[0], fmaf(R[1], m[1], fmaf(R[2], m[2], ps.t[0])));
+  const float y = fmaf(R[3], m[0], fmaf(R[4], m[1], fmaf(R[5], m[2], ps.t[1])));
+  const float rz = 1.0f / z;
+  const float u = x * rz, w = y * rz;
+  float uc = u, wc = w;
+  if (vp.lim_u > 0.0f) {
+    uc = fminf(fmaxf(u, -vp.lim_u), vp.lim_u);
+    wc = fminf(fmaxf(w, -vp.lim_w), vp.lim_w);
+  }
+  const float jf2 = (vp.fx * vp.fx * (1.0f + uc * uc) + vp.fy * vp.fy * (1.0f + wc * wc)) * (rz * rz);
+  const float rad = sqrtf(kappa * fmaf(jf2, smax2, c.eps2d)) * 1.02f + 4.0f;
+  const float mx = fmaf(vp.fx, u, vp.cx), my = fmaf(vp.fy, w, vp.cy);
+  return !(mx + rad < 0.0f || mx - rad > (float)(vp.width - 1) || my + rad < 0.0f ||
+           my - rad > (float)(vp.height - 1));
+}
+
+// Forward, pass 1 (cull): one thread per (Gaussian, chunk of views). The entries that may reach the
 // image are appended to `cand` (gathered per warp in shared memory, then one global atomic per
-// block; their order does not matter). Pass 2 then projects only those, so its warps are not held
-// up by the large majority of entries that fall outside the image.
+// block; their order does not matter). Pass 2 then decides on and projects only those, so its warps
+// are not held up by the large majority of entries that fall outside the image.
 //
 // The pass is bound by instruction issue, so an entry is tested by planes: with
-// (x, y, z) = R m + t, the centre lies at pixel (fx x / z + cx, fy y / z + cy), and the
-// alpha >= alpha_min footprint reaches at most
-//   rad = sqrt(kappa (|J|_F^2 smax^2 + eps)) <= sqrt(kappa) (F smax / z + sqrt(eps)),
-// since the largest eigenvalue of Sigma^I is at most |J|_F^2 smax^2 + eps and |J|_F <= F / z with
+// (x, y, z) = R m + t, the centre lies at pixel (fx x / z + cx, fy y / z + cy), and the radius of
+// reaches_image is at most 1.02 sqrt(kappa) (F smax / z + sqrt(eps)) + 4 with
 // F^2 = fx^2 (1 + lim_u^2) + fy^2 (1 + lim_w^2) for the guard-banded J. Times z > 0, "mx + rad < 0"
 // and its three siblings become linear in m and z, with no division or square root per entry:
-// three dot products and four comparisons (about 20 instructions; the exact radius took 60: 137 us
-// for 24 views of a million Gaussians, 258 us for 16 of three). rad is widened by 2 % and 4 px,
-// beyond the 1-px padding of the tile coverage and the rounding here. Without a guard band |J|_F
+// three dot products and four comparisons (about 20 instructions; the radius itself took 60: 137 us
+// for 24 views of a million Gaussians, 258 us for 16 of three). Without a guard band |J|_F
 // has no such bound and follows from u and w.
 //
-// Plain FMA dot products: the cull only has to keep every Gaussian the projection keeps. Their
-// error is below 8 units of roundoff of the summed magnitudes, so a Gaussian is dropped for the
-// near plane only when even z + that bound is at or below it (the projection then decides with its
-// compensated depth).
+// Everything that reaches_image keeps is a candidate. Both tests take the same z; their pixel
+// columns (rows) times z differ by rounding: at most 5 units of roundoff of the summed magnitudes in
+// the planes (two in the combined coefficients, three in the FMA chain), 4 + 3 in the other's centre
+// and its products, so the margin takes 16 (9.6e-7) of (f + |c|) (|m|_1 + |t|_1), which no sum
+// exceeds. The roundings of the radius itself lie below 1e-6 of it: 1.021 and 4.01 cover them.
 struct CullView {
   float4 px;   // fx R0 + cx R2 | fx t0 + cx t2: z times the pixel column of the centre
   float4 py;   // likewise for the row
   float4 z;    // R2 | t2
-  float4 lim;  // width - 1, height - 1, 1.02 F, bound of z's error from t2
+  float4 lim;  // width - 1, height - 1, 1.021 F, bound of z's error from t2
+  float2 err;  // bound of the planes' rounding per unit of |m|_1, and from t
 };
 
 __global__ void __launch_bounds__(kPreThreads) cull_kernel(
@@ -345,7 +378,9 @@ __global__ void __launch_bounds__(kPreThreads) cull_kernel(
                           vp.fy * vp.fy * (1.0f + vp.lim_w * vp.lim_w));
     // A negative value tells that there is no guard band.
     cv.lim = make_float4((float)(vp.width - 1), (float)(vp.height - 1),
-                         vp.lim_u > 0.0f ? 1.02f * F : -1.0f, 4.8e-7f * fabsf(ps.t[2]));
+                         vp.lim_u > 0.0f ? 1.021f * F : -1.0f, 4.9e-7f * fabsf(ps.t[2]));
+    cv.err.x = 9.6e-7f * fmaxf(vp.fx + fabsf(vp.cx), vp.fy + fabsf(vp.cy));
+    cv.err.y = cv.err.x * (fabsf(ps.t[0]) + fabsf(ps.t[1]) + fabsf(ps.t[2]));
     s_view[threadIdx.x] = cv;
   }
   // The block's Gaussians own whole words of each view's row of the visibility bitmask. Tile counts
@@ -382,10 +417,10 @@ __global__ void __launch_bounds__(kPreThreads) cull_kernel(
   const float opacity = 1.0f / (1.0f + expf(-logit));
   const float kappa = finite ? 2.0f * logf(opacity / c.alpha_min) : -1.0f;
   const bool shown = finite && kappa >= 0.0f;
-  // rad z <= F reach + band z; an overflowing product keeps the entry.
+  // rad z <= F reach + band z + rounding; an overflowing product keeps the entry.
   const float root = sqrtf(fmaxf(kappa, 0.0f));
-  const float reach = root * smax, band = fmaf(1.02f * root, sqrtf(c.eps2d), 4.0f);
-  const float z_err = 4.8e-7f * (fabsf(m[0]) + fabsf(m[1]) + fabsf(m[2]));
+  const float reach = root * smax, band = fmaf(1.021f * root, sqrtf(c.eps2d), 4.01f);
+  const float m1 = fabsf(m[0]) + fabsf(m[1]) + fabsf(m[2]), z_err = 4.9e-7f * m1;
   uint32_t count = 0;  // candidates of the warp so far
   for (int k = 0; k < v_count; ++k) {
     const float4 zr = s_view[k].z, lim = s_view[k].lim;
@@ -393,12 +428,14 @@ __global__ void __launch_bounds__(kPreThreads) cull_kernel(
     const float4 pr = s_view[k].px, qr = s_view[k].py;
     const float px = fmaf(pr.x, m[0], fmaf(pr.y, m[1], fmaf(pr.z, m[2], pr.w)));
     const float py = fmaf(qr.x, m[0], fmaf(qr.y, m[1], fmaf(qr.z, m[2], qr.w)));
-    float margin = fmaf(lim.z, reach, band * z);
+    const float err = fmaf(s_view[k].err.x, m1, s_view[k].err.y);
+    float margin = fmaf(lim.z, reach, fmaf(band, z, err));
     if (lim.z < 0.0f) {  // no guard band (the same for every Gaussian)
       const ViewParams& vp = views.v[v_begin + k];
-      const float u = (px - vp.cx * z) / (vp.fx * z), w = (py - vp.cy * z) / (vp.fy * z);
+      const float u = (fabsf(px - vp.cx * z) + err) / (vp.fx * z),
+                  w = (fabsf(py - vp.cy * z) + err) / (vp.fy * z);
       const float F = sqrtf(vp.fx * vp.fx * fmaf(u, u, 1.0f) + vp.fy * vp.fy * fmaf(w, w, 1.0f));
-      margin = fmaf(1.03f * F, reach, band * z);
+      margin = fmaf(1.03f * F, reach, fmaf(band, z, err));
     }
     const bool keep = shown && z + (z_err + lim.w) > c.znear && z > 0.0f &&
                       !(px + margin < 0.0f || py + margin < 0.0f ||
@@ -449,7 +486,8 @@ __device__ __forceinline__ void sh_colour(const float* shc, const float* m, cons
 }
 
 // Forward, pass 2 (project): one thread per candidate entry (grid-stride). Full projection
-// (Eq. proj), tile count and, for DEG >= 0, the colour; writes the entry's records and tile count.
+// (Eq. proj), tile count and, for DEG >= 0, the colour; writes the entry's records and tile count,
+// if its footprint may reach the image (reaches_image).
 // An entry with a non-finite SH coefficient is culled here and counted. With DEG = -1 (the
 // caller's SH coefficients may still be in flight) the colour is left to the pass after the
 // sorts (colour.xyz = 0 until then). Entries that are not candidates keep unwritten records.
@@ -481,6 +519,9 @@ __global__ void __launch_bounds__(kPreThreads, 7) project_kernel(
     q[2] = q4.z;
     q[3] = q4.w;
     const float logit = __ldg(logits + i);
+    const ViewParams& vp = views.v[v];
+    const PoseRef ps = view_pose<kDevPose>(views, v);
+    if (!reaches_image(vp, ps, c, m, ls, logit)) continue;
     float shc[3 * K];
     if constexpr (DEG >= 0) {
       load_sh<DEG>(sh, i, shc);
@@ -492,8 +533,6 @@ __global__ void __launch_bounds__(kPreThreads, 7) project_kernel(
         continue;
       }
     }
-    const ViewParams& vp = views.v[v];
-    const PoseRef ps = view_pose<kDevPose>(views, v);
     // The colour comes first: the 3K coefficients are then not held through the projection, and 72
     // registers (7 blocks per SM) do at degree 3 where 95 were held: 390 -> 352 us over 16 views
     // of 3M Gaussians, a gather that waits on memory.
