@@ -34,7 +34,12 @@ namespace {
 //   forward, 8 pixels: 2.98, 2.93, 2.81, 2.56
 //   backward, 8 pixels: 4.39, 4.32, 4.50, 4.47
 // For the backward the z of a doubled colour gives its place to r_g: (b, b), (z, r_g), with r_g the
-// row of the tile nearest to the Gaussian's centre, relative to the anchor row.
+// row of the tile nearest to where the footprint's ridge (in each column the point of largest
+// weight, dy = -l11 l21 dx / (l21^2 + l22^2)) crosses the tile's middle column, relative to the
+// anchor row. The backward sums its moments about that row: the pixels that a tilted footprint
+// covers lie around its ridge, not around its centre, which may be many tiles away. Error of the
+// second moment across thin footprints of any tilt, in units of the moment: 2.0e-6 about the
+// ridge's row, 6.0e-6 about the row nearest to the centre, 3.7e-6 about the anchor row.
 // ------------------------------------------------------------------------------------------
 template <bool kBackward, int PPT>
 struct StageLayout {
@@ -48,7 +53,7 @@ struct StageLayout {
 
 template <int kTileH, bool kBackward, int PPT, int R, int N>
 __device__ __forceinline__ void stage_gaussian(ulonglong2 (&sp)[R][N], int t, float4 r0,
-                                               float4 r1, float4 r2, float y_a) {
+                                               float4 r1, float4 r2, float x_m, float y_a) {
   using L = StageLayout<kBackward, PPT>;
   static_assert(R == L::kRows, "rows of the layout");
   const AnchorTerms at = anchor_terms(r0, r1, y_a);
@@ -62,8 +67,12 @@ __device__ __forceinline__ void stage_gaussian(ulonglong2 (&sp)[R][N], int t, fl
   }
   if constexpr (L::kColourTwice) {
     float last = r2.w;
-    if constexpr (kBackward)
-      last = fminf(fmaxf(rintf(-at.dya), (float)(-kTileH / 2)), (float)(kTileH - 1 - kTileH / 2));
+    if constexpr (kBackward) {
+      // An undefined quotient (an exponent that underflows) leaves the tile's first row.
+      const float ridge = __fdividef(r1.x * r1.y * (r0.x - x_m), fmaf(r1.y, r1.y, r1.z * r1.z));
+      last = fminf(fmaxf(rintf(ridge - at.dya), (float)(-kTileH / 2)),
+                   (float)(kTileH - 1 - kTileH / 2));
+    }
     sp[L::kColour][t] = make_ulonglong2(f2_make(r2.x, r2.x), f2_make(r2.y, r2.y));
     sp[L::kColour + 1][t] = make_ulonglong2(f2_make(r2.z, r2.z), f2_make(r2.w, last));
   } else {
@@ -145,7 +154,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
   const int py0 = ty * TH + (int)(threadIdx.x / TW) * PPT;
   const float fx = (float)px;
   // Anchor row of the tile's row terms, and the thread's first row relative to it.
-  const float y_a = (float)(ty * TH + TH / 2);
+  const float x_m = (float)(tx * TW) + 0.5f * (float)(TW - 1), y_a = (float)(ty * TH + TH / 2);
   const int r0_ = (int)(threadIdx.x / TW) * PPT - TH / 2;
   const uint2 range = ranges[gtile];
 
@@ -215,7 +224,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
     if (j < range.y) {
       const uint32_t vi = pair_vals[j];
       stage_gaussian<TH, false, PPT>(sp, threadIdx.x, rec[vi].mean, rec[vi].conic,
-                                     rec[vi].colour, y_a);
+                                     rec[vi].colour, x_m, y_a);
     }
     __syncthreads();
     const int cnt = (int)min((uint32_t)kThreads, range.y - start);
@@ -324,9 +333,8 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_forward_kernel(
 // +8 % on ten 640x480 views).
 //
 // The lane's values: sdp, sr | srr, t_a sdp | t_a sr, t_a^2 sdp | gr, gg | gb, gz, with sdp, sr,
-// srr the sums of dp, dp r and dp r^2 over its pixels (r the row offset from the tile row nearest
-// to the Gaussian's centre; from the tile's anchor row with one pixel per thread), t_a the whitened
-// offset of its column at that row, and gr .. gz the colour and depth weights (gz 0 without a depth
+// srr the sums of dp, dp r and dp r^2 over its pixels (r the row offset from row r_g; from the
+// tile's anchor row with one pixel per thread), t_a the whitened offset of its column at that row, and gr .. gz the colour and depth weights (gz 0 without a depth
 // or opacity gradient).
 // ------------------------------------------------------------------------------------------
 constexpr int kRedPad = 68;  // floats per row of 32 lane pairs, padded
@@ -388,7 +396,7 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
   const float fx = (float)px;
   // Anchor row of the tile's row terms, and the thread's first row relative to it (as in the
   // forward, so both blends compute every pixel's exponent to the same bits).
-  const float y_a = (float)(ty * TH + TH / 2);
+  const float x_m = (float)(tx * TW) + 0.5f * (float)(TW - 1), y_a = (float)(ty * TH + TH / 2);
   const int r0_ = (int)(threadIdx.x / TW) * PPT - TH / 2;
   const uint2 range = ranges[gtile];
   const int lane = threadIdx.x & 31;
@@ -551,9 +559,9 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
         const float k1 = fmaf(0.5f, f2_hi(mP) - f2_lo(mP), f2_lo(mF) + f2_hi(mF));
         const float k2 =
             fmaf(0.25f, sdp, (f2_lo(mQ) + f2_hi(mQ)) + (f2_hi(mF) - f2_lo(mF)));
-        // Then over the rows' offsets r - r_g from the tile row nearest to the Gaussian's centre:
-        // the lanes' sums and the whitened moments formed from them are then about the size of
-        // the result. About the tile's middle row a Gaussian seven rows away cancelled 50 : 1.
+        // Then over the rows' offsets r - r_g from the row of the footprint's ridge: the lanes'
+        // sums and the whitened moments formed from them are then about the size of the result.
+        // About the tile's middle row a footprint seven rows away cancelled 50 : 1.
         const float r_g = f2_hi(st.bz.y);
         const float rc = ((float)r0_ + 0.5f * (float)(PPT - 1)) - r_g;
         sr = fmaf(rc, sdp, k1);
@@ -675,7 +683,8 @@ __global__ void __launch_bounds__(TW * TH / PPT) blend_backward_kernel(
       s_vi[threadIdx.x] = vi;
       const float4 r1 = rec[vi].conic;
       may_clamp = !(-r1.w > c.unclamped_neg_lo);
-      stage_gaussian<TH, true, PPT>(sp, threadIdx.x, rec[vi].mean, r1, rec[vi].colour, y_a);
+      stage_gaussian<TH, true, PPT>(sp, threadIdx.x, rec[vi].mean, r1, rec[vi].colour,
+                                    x_m, y_a);
     }
     const unsigned clamp_bits = __ballot_sync(0xffffffffu, may_clamp);
     __syncthreads();
