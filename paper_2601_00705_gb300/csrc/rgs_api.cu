@@ -16,6 +16,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <map>
 #include <string>
 #include <vector>
@@ -216,7 +217,11 @@ constexpr size_t kSpareStates = 2;
 
 void drop_spares(rgs_ctx* ctx);
 
-cudaError_t alloc_region(rgs_ctx* ctx, Region& r, size_t bytes) {
+// The region anew, with `bytes` bytes. `caps`: the capacities that its contents stand for. They are
+// zero until the caller sets them, so that a failure leaves none for memory that is gone.
+cudaError_t alloc_region(rgs_ctx* ctx, Region& r, size_t bytes,
+                         std::initializer_list<int64_t*> caps = {}) {
+  for (int64_t* cap : caps) *cap = 0;
   free_region(r);
   if (bytes == 0) return cudaSuccess;
   cudaError_t e = cudaMalloc(&r.base, bytes);
@@ -262,7 +267,7 @@ rgs_status ensure_scratch(rgs_ctx* ctx, State& s, int64_t items, bool capturing)
   if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "scratch too small during stream capture");
   RGS_CUDA(cudaDeviceSynchronize(), "sync before scratch growth");
   const size_t bytes = align_up(sizeof(uint32_t) * hist) + align_up(sizeof(uint32_t) * sums);
-  RGS_CUDA(alloc_region(ctx, s.r_scratch, bytes), "allocate sort scratch");
+  RGS_CUDA(alloc_region(ctx, s.r_scratch, bytes, {&s.hist_cap, &s.sums_cap}), "allocate sort scratch");
   char* p = static_cast<char*>(s.r_scratch.base);
   s.hist = carve<uint32_t>(p, hist);
   s.block_sums = carve<uint32_t>(p, sums);
@@ -276,7 +281,8 @@ rgs_status ensure_vn(rgs_ctx* ctx, State& s, int64_t vn, int64_t n, int64_t pose
   if (n > s.n_cap) {
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "per-Gaussian buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
-    RGS_CUDA(alloc_region(ctx, s.r_n, sizeof(unsigned long long) * n), "allocate visibility masks");
+    RGS_CUDA(alloc_region(ctx, s.r_n, sizeof(unsigned long long) * n, {&s.n_cap}),
+             "allocate visibility masks");
     s.vis_mask = static_cast<unsigned long long*>(s.r_n.base);
     RGS_CUDA(cudaMemsetAsync(s.vis_mask, 0, sizeof(unsigned long long) * n, stream),
              "zero visibility masks");
@@ -289,7 +295,7 @@ rgs_status ensure_vn(rgs_ctx* ctx, State& s, int64_t vn, int64_t n, int64_t pose
     size_t bytes = align_up(sizeof(Record) * cap) + 5 * align_up(sizeof(uint32_t) * cap) +
                    align_up(sizeof(float) * kG2Stride * cap) +
                    align_up(sizeof(uint32_t) * vis_bit_words_cap(cap));
-    RGS_CUDA(alloc_region(ctx, s.r_vn, bytes), "allocate per-Gaussian buffers");
+    RGS_CUDA(alloc_region(ctx, s.r_vn, bytes, {&s.vn_cap}), "allocate per-Gaussian buffers");
     char* p = static_cast<char*>(s.r_vn.base);
     s.rec = carve<Record>(p, cap);
     s.vis_keys[0] = carve<uint32_t>(p, cap);
@@ -306,7 +312,8 @@ rgs_status ensure_vn(rgs_ctx* ctx, State& s, int64_t vn, int64_t n, int64_t pose
   if (pose_entries > s.pose_cap) {
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "pose buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
-    RGS_CUDA(alloc_region(ctx, s.r_pose, sizeof(float) * pose_entries), "allocate pose partials");
+    RGS_CUDA(alloc_region(ctx, s.r_pose, sizeof(float) * pose_entries, {&s.pose_cap}),
+             "allocate pose partials");
     s.pose_partial = static_cast<float*>(s.r_pose.base);
     s.pose_cap = pose_entries;
   }
@@ -319,7 +326,7 @@ rgs_status ensure_pix_tiles(rgs_ctx* ctx, State& s, int64_t pixels, int64_t tile
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "pixel buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
     RGS_CUDA(alloc_region(ctx, s.r_pix, align_up(sizeof(float) * pixels) +
-                                        align_up(sizeof(int32_t) * pixels)),
+                                            align_up(sizeof(int32_t) * pixels), {&s.pix_cap}),
              "allocate pixel state");
     char* p = static_cast<char*>(s.r_pix.base);
     s.t_final = carve<float>(p, pixels);
@@ -330,7 +337,7 @@ rgs_status ensure_pix_tiles(rgs_ctx* ctx, State& s, int64_t pixels, int64_t tile
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "tile buffers grow during capture");
     RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
     RGS_CUDA(alloc_region(ctx, s.r_tile, align_up(sizeof(uint2) * tiles) +
-                                         2 * align_up(sizeof(uint32_t) * tiles)),
+                                             2 * align_up(sizeof(uint32_t) * tiles), {&s.tile_cap}),
              "allocate tile ranges");
     char* p = static_cast<char*>(s.r_tile.base);
     s.ranges = carve<uint2>(p, tiles);
@@ -349,8 +356,8 @@ rgs_status ensure_pairs(rgs_ctx* ctx, State& s, int64_t pairs) {
   const int64_t cap = with_slack(pairs);
   if (cap >= (int64_t)UINT32_MAX) return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^32");
   RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
-  s.pair_cap = 0;
-  RGS_CUDA(alloc_region(ctx, s.r_pair, align_up(sizeof(uint32_t) * cap)), "allocate pair list");
+  RGS_CUDA(alloc_region(ctx, s.r_pair, align_up(sizeof(uint32_t) * cap), {&s.pair_cap}),
+           "allocate pair list");
   s.pairs = static_cast<uint32_t*>(s.r_pair.base);
   s.pair_cap = cap;
   return RGS_OK;
@@ -361,8 +368,7 @@ rgs_status ensure_cells(rgs_ctx* ctx, State& s, int64_t cells) {
   const int64_t cap = with_slack(cells);
   if (cap >= (int64_t)UINT32_MAX) return fail(ctx, RGS_ERR_INVALID_ARG, "cell list exceeds 2^32");
   RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
-  s.cell_cap = 0;
-  RGS_CUDA(alloc_region(ctx, s.r_cell, 4 * align_up(sizeof(uint32_t) * cap)),
+  RGS_CUDA(alloc_region(ctx, s.r_cell, 4 * align_up(sizeof(uint32_t) * cap), {&s.cell_cap}),
            "allocate cell lists");
   char* p = static_cast<char*>(s.r_cell.base);
   s.cell_keys[0] = carve<uint32_t>(p, cap);
@@ -905,6 +911,7 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
   if (s->r_counters.bytes < pose_bytes + reset_bytes) {
     if (capturing) return fail(ctx, RGS_ERR_CAPACITY, "counters grow during capture");
     if (s->r_counters.base) RGS_CUDA(cudaDeviceSynchronize(), "sync before counters growth");
+    s->counters = nullptr;
     RGS_CUDA(alloc_region(ctx, s->r_counters, pose_bytes + reset_bytes), "allocate counters");
   }
   s->pose_records = static_cast<float*>(s->r_counters.base);
@@ -1106,8 +1113,8 @@ rgs_status render_backward(rgs_ctx* ctx, uint64_t handle, const rgs_image_grads*
       if (s->reg_cap < n) {
         if (capturing)
           return fail(ctx, RGS_ERR_CAPACITY, "regulariser scratch: make a first call outside capture");
-        free_region(s->r_reg);
-        RGS_CUDA(alloc_region(ctx, s->r_reg, sizeof(float) * (size_t)n), "allocate regulariser scratch");
+        RGS_CUDA(alloc_region(ctx, s->r_reg, sizeof(float) * (size_t)n, {&s->reg_cap}),
+                 "allocate regulariser scratch");
         s->reg_vals = static_cast<float*>(s->r_reg.base);
         s->reg_cap = n;
       }

@@ -1,0 +1,17 @@
+// The state of a fake of the CUDA runtime, for running the library's host code without a GPU: device
+// memory is host memory whose live blocks are known, an allocation beyond `limit` fails, streams and
+// events do nothing (fake_runtime.cpp).
+#pragma once
+
+#include <cstddef>
+#include <cstdint>
+
+namespace fake {
+extern size_t live, limit, total;
+extern bool capturing;
+extern int stale;  // accesses outside live memory
+// What the projection of the next forwards counts.
+extern unsigned long long visible, cells, pairs;
+
+void check(const void* p, size_t bytes, const char* what);
+}  // namespace fake

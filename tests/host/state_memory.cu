@@ -1,0 +1,101 @@
+// Host-side scenarios of the context's states on the fake device; one per run, named by argv[1].
+#include "fake_launchers.h"
+
+using namespace rgs;
+
+namespace {
+
+struct Images {
+  std::vector<float> color, depth, alpha;
+  rgs_images get(int pixels) {
+    color.resize(3 * pixels);
+    depth.resize(pixels);
+    alpha.resize(pixels);
+    return rgs_images{color.data(), depth.data(), alpha.data()};
+  }
+};
+
+rgs_ctx* make_context() {
+  rgs_ctx* ctx = nullptr;
+  if (rgs_create(&ctx, 0) != RGS_OK) std::exit(2);
+  return ctx;
+}
+
+// A forward of `views` views of w x w pixels and n Gaussians that counts `count` of everything.
+rgs_status forward(rgs_ctx* ctx, int n, int w, unsigned long long count, uint64_t* state,
+                   int views = 1) {
+  static Images images;
+  alignas(16) static float parameters[4];
+  fake::visible = count < (unsigned long long)n * views ? count : (unsigned long long)n * views;
+  fake::cells = fake::pairs = count;
+  std::vector<rgs_camera> cams(views);
+  for (rgs_camera& c : cams) {
+    c = rgs_camera{};
+    c.width = c.height = w;
+    c.fx = c.fy = 100.0f;
+    c.world_to_cam[0] = c.world_to_cam[5] = c.world_to_cam[10] = 1.0f;
+  }
+  const rgs_gaussians g{n, 0, parameters, parameters, parameters, parameters, parameters};
+  rgs_images out = images.get(views * w * w);
+  return rgs_render_forward(ctx, &g, cams.data(), views, nullptr, &out, state, nullptr);
+}
+
+rgs_status backward(rgs_ctx* ctx, uint64_t state, bool reg = false) {
+  alignas(16) static float grads[4];
+  static double value;
+  const rgs_image_grads up{grads, nullptr, nullptr};
+  rgs_map_reg r{};
+  r.value = &value;
+  return rgs_render_backward_mapping(ctx, state, &up, RGS_GRAD_ALL, grads, grads, grads, grads,
+                                     grads, grads, reg ? &r : nullptr, nullptr);
+}
+
+int failures = 0;
+#define EXPECT(x)                                            \
+  do {                                                       \
+    if (!(x)) {                                              \
+      ++failures;                                            \
+      std::printf("line %d: %s does not hold\n", __LINE__, #x); \
+    }                                                        \
+  } while (0)
+
+// A forward that runs out of memory at any of its allocations leaves nothing behind that a later,
+// smaller forward on the same state would use.
+void failed_growth() {
+  const struct { int n, w, views; unsigned long long count; } larger[] = {
+      {5000, 64, 1, 6000},    // per Gaussian
+      {1000, 64, 8, 6000},    // per entry
+      {1000, 300, 1, 6000},   // per pixel and tile
+      {1000, 64, 1, 900000},  // the lists and the sort's scratch
+  };
+  for (const auto& l : larger) {
+    for (size_t room = 0;; room += 4096) {
+      rgs_ctx* ctx = make_context();
+      uint64_t s = 0;
+      EXPECT(forward(ctx, 1000, 64, 6000, &s) == RGS_OK);
+      EXPECT(backward(ctx, s, true) == RGS_OK);
+      fake::limit = fake::live + room;
+      const rgs_status st = forward(ctx, l.n, l.w, l.count, &s, l.views);
+      EXPECT(st == RGS_OK || st == RGS_ERR_NOMEM);
+      if (st == RGS_OK) backward(ctx, s, true);  // its scratch may fail, too
+      rgs_stats stats;
+      EXPECT(rgs_query_stats(ctx, s, &stats, nullptr) == RGS_OK);
+      fake::limit = SIZE_MAX;
+      EXPECT(forward(ctx, 1000, 64, 6000, &s) == RGS_OK);
+      EXPECT(backward(ctx, s, true) == RGS_OK);
+      rgs_destroy(ctx);
+      EXPECT(fake::live == 0);
+      if (st == RGS_OK) break;
+    }
+  }
+}
+
+}  // namespace
+
+int main(int argc, char** argv) {
+  const std::string which = argc > 1 ? argv[1] : "";
+  if (which == "failed_growth") failed_growth();
+  else return 2;
+  EXPECT(fake::stale == 0);
+  return failures ? 1 : 0;
+}
