@@ -312,14 +312,15 @@ __global__ void __launch_bounds__(kLossThreads) track_loss_kernel(
 // per view and the pow, sin and cos of the general case, 6 us).
 constexpr int kAdamViews = 5;  // views per warp
 
-// x^n for n >= 0, by squaring.
-__device__ __forceinline__ double power(double x, int n) {
+// x^n by squaring. n follows from the caller's step counter in device memory, so it may be anything:
+// the loop runs over an unsigned exponent, at most 32 times.
+__device__ __forceinline__ double power(double x, int64_t n) {
   double r = 1.0;
-  for (; n; n >>= 1) {
-    if (n & 1) r *= x;
+  for (uint32_t e = (uint32_t)(n < 0 ? -n : n); e; e >>= 1) {
+    if (e & 1) r *= x;
     x *= x;
   }
-  return r;
+  return n < 0 ? 1.0 / r : r;
 }
 
 __global__ void pose_adam_kernel(int n_views, float lr, float beta1, float beta2, float eps,
@@ -337,7 +338,7 @@ __global__ void pose_adam_kernel(int n_views, float lr, float beta1, float beta2
   if (iterations > 0)
     lr_k = 0.5 * (double)lr * (1.0 + cospi((double)min(k, iterations) / (double)iterations));
   // Even lanes hold 1 - beta1^(k + 1), odd ones 1 - beta2^(k + 1).
-  const double bias = 1.0 - power((lane & 1) ? (double)beta2 : (double)beta1, k + 1);
+  const double bias = 1.0 - power((lane & 1) ? (double)beta2 : (double)beta1, (int64_t)k + 1);
   const double c1 = __shfl_sync(0xffffffffu, bias, 0), c2 = __shfl_sync(0xffffffffu, bias, 1);
   double xi = 0.0;
   if (on) {
@@ -407,7 +408,7 @@ __global__ void pose_adam_kernel(int n_views, float lr, float beta1, float beta2
     T[4 * a + col] = (float)n0;
     T[4 * a + col + 1] = (float)n1;
   }
-  if (threadIdx.x == 0) *step = k + 1;
+  if (threadIdx.x == 0) *step = (int32_t)((uint32_t)k + 1u);
 }
 
 // ------------------------------------------------------------------------------------------
