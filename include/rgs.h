@@ -183,7 +183,8 @@ const char* rgs_last_error(const rgs_ctx* ctx);
  *   out: device output images.
  *   state: in/out. If *state is 0 a new state is created and its handle written back; otherwise
  *     the named state is reused (its previous contents are replaced). The state keeps the data
- *     the backward needs.
+ *     the backward needs. When the call fails, *state stays 0 (what it created is freed), and a
+ *     named state stays known but holds no forward.
  * Outside stream capture the call waits once, for the projection, whose counts size the sorted
  * list of visible entries and the tile lists; the rest is queued while the stream runs on. Under
  * stream capture it never synchronises and keeps the sizes of the last call outside capture; if a list would overflow, the kernels record it, the output is incomplete and

@@ -854,9 +854,31 @@ rgs_status rgs_render_forward_posed(rgs_ctx* ctx, const rgs_gaussians* g,
 }
 
 namespace {
+rgs_status forward_on_state(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera* cams,
+                            int32_t n_views, const float* world_to_cam, const rgs_config* cfg_in,
+                            rgs_images* out, uint64_t* handle, void* stream_ptr);
+
 rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera* cams,
                           int32_t n_views, const float* world_to_cam, const rgs_config* cfg_in,
                           rgs_images* out, uint64_t* handle, void* stream_ptr) {
+  const bool creates = handle && *handle == 0;
+  const rgs_status st = forward_on_state(ctx, g, cams, n_views, world_to_cam, cfg_in, out, handle,
+                                         stream_ptr);
+  if (st != RGS_OK && creates && *handle != 0) {
+    // The caller has no state from a call that failed: what it created ends here. (Under stream
+    // capture the state holds no memory, and nothing here may disturb the capture.)
+    State* s = find_state(ctx, *handle);
+    ctx->states.erase(*handle);
+    *handle = 0;
+    if (s->bytes() > 0) cudaDeviceSynchronize();  // queued work may still use its buffers
+    destroy_state(s);
+  }
+  return st;
+}
+
+rgs_status forward_on_state(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera* cams,
+                            int32_t n_views, const float* world_to_cam, const rgs_config* cfg_in,
+                            rgs_images* out, uint64_t* handle, void* stream_ptr) {
   if (!ctx) return RGS_ERR_INVALID_ARG;
   ctx->last_error.clear();
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);

@@ -15,7 +15,7 @@ static std::map<char*, size_t>& blocks() {
 }
 size_t live = 0, limit = SIZE_MAX, total = 288ull << 30;
 bool capturing = false;
-int stale = 0;
+int stale = 0, unsafe = 0;
 unsigned long long visible = 0, cells = 0, pairs = 0;
 
 void check(const void* p, size_t bytes, const char* what) {
@@ -32,6 +32,7 @@ void check(const void* p, size_t bytes, const char* what) {
 
 extern "C" {
 cudaError_t cudaMalloc(void** p, size_t bytes) {
+  fake::unsafe += fake::capturing;
   *p = nullptr;
   if (fake::live + bytes > fake::limit) return cudaErrorMemoryAllocation;
   char* base = static_cast<char*>(std::malloc(bytes));
@@ -42,6 +43,7 @@ cudaError_t cudaMalloc(void** p, size_t bytes) {
   return cudaSuccess;
 }
 cudaError_t cudaFree(void* p) {
+  fake::unsafe += fake::capturing;
   auto it = fake::blocks().find(static_cast<char*>(p));
   if (it == fake::blocks().end()) return p ? cudaErrorInvalidValue : cudaSuccess;
   fake::live -= it->second;
@@ -75,8 +77,14 @@ cudaError_t cudaHostAlloc(void** p, size_t bytes, unsigned) {
 cudaError_t cudaFreeHost(void* p) { std::free(p); return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
-cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() {
+  fake::unsafe += fake::capturing;
+  return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t) {
+  fake::unsafe += fake::capturing;
+  return cudaSuccess;
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
   *s = fake::capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;

@@ -9,7 +9,8 @@
 namespace fake {
 extern size_t live, limit, total;
 extern bool capturing;
-extern int stale;  // accesses outside live memory
+extern int stale;     // accesses outside live memory
+extern int unsafe;    // calls that would invalidate a stream capture, made during one
 // What the projection of the next forwards counts.
 extern unsigned long long visible, cells, pairs;
 

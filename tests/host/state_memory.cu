@@ -1,4 +1,6 @@
 // Host-side scenarios of the context's states on the fake device; one per run, named by argv[1].
+#include <cstring>
+
 #include "fake_launchers.h"
 
 using namespace rgs;
@@ -90,11 +92,53 @@ void failed_growth() {
   }
 }
 
+// A forward that fails after it created its state leaves none: the handle stays 0, the memory is
+// free again (a kept state that it took, too), and a capture is not disturbed.
+void failed_first() {
+  for (int kept = 0; kept < 2; ++kept) {
+    for (size_t room = 0;; room += 4096) {
+      rgs_ctx* ctx = make_context();
+      const size_t bare = fake::live;
+      uint64_t s = 0;
+      if (kept) {
+        EXPECT(forward(ctx, 1000, 64, 6000, &s) == RGS_OK);
+        EXPECT(rgs_release_state(ctx, s) == RGS_OK);
+        s = 0;
+      }
+      fake::limit = bare + room;
+      const rgs_status st = forward(ctx, 2000, 100, 20000, &s);
+      fake::limit = SIZE_MAX;
+      if (st != RGS_OK) {
+        EXPECT(st == RGS_ERR_NOMEM && s == 0 && fake::live == bare);
+        EXPECT(std::strlen(rgs_last_error(ctx)) > 0);
+      }
+      rgs_destroy(ctx);
+      if (st == RGS_OK) break;
+    }
+  }
+  rgs_ctx* ctx = make_context();
+  uint64_t s = 0;
+  fake::capturing = true;
+  EXPECT(forward(ctx, 1000, 64, 6000, &s) == RGS_ERR_CAPACITY && s == 0);
+  EXPECT(forward(ctx, 0, 64, 0, &s) == RGS_ERR_CAPACITY && s == 0);
+  EXPECT(fake::unsafe == 0);
+  fake::capturing = false;
+  // A named state outlives a call that fails on it.
+  EXPECT(forward(ctx, 1000, 64, 6000, &s) == RGS_OK);
+  fake::limit = fake::live;
+  const uint64_t named = s;
+  EXPECT(forward(ctx, 2000, 100, 20000, &s) == RGS_ERR_NOMEM && s == named);
+  fake::limit = SIZE_MAX;
+  EXPECT(rgs_release_state(ctx, s) == RGS_OK);
+  rgs_destroy(ctx);
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
   const std::string which = argc > 1 ? argv[1] : "";
   if (which == "failed_growth") failed_growth();
+  else if (which == "failed_first") failed_first();
   else return 2;
   EXPECT(fake::stale == 0);
   return failures ? 1 : 0;

@@ -32,3 +32,7 @@ def _run(program, name):
 
 def test_a_forward_that_runs_out_of_memory_leaves_nothing_stale(program):
     _run(program, "failed_growth")
+
+
+def test_a_first_forward_that_fails_leaves_no_state(program):
+    _run(program, "failed_first")
