@@ -137,7 +137,7 @@ struct State {
 
   size_t bytes() const {
     return r_vn.bytes + r_n.bytes + r_pix.bytes + r_tile.bytes + r_cell.bytes + r_pair.bytes +
-           r_scratch.bytes + r_pose.bytes + r_counters.bytes;
+           r_scratch.bytes + r_pose.bytes + r_counters.bytes + r_reg.bytes;
   }
 };
 
@@ -217,6 +217,18 @@ constexpr size_t kSpareStates = 2;
 
 void drop_spares(rgs_ctx* ctx);
 
+// Device memory. When there is none left the kept states are freed first.
+cudaError_t device_alloc(rgs_ctx* ctx, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && !ctx->spare.empty()) {
+    cudaGetLastError();
+    drop_spares(ctx);
+    e = cudaMalloc(p, bytes);
+  }
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
+
 // The region anew, with `bytes` bytes. `caps`: the capacities that its contents stand for. They are
 // zero until the caller sets them, so that a failure leaves none for memory that is gone.
 cudaError_t alloc_region(rgs_ctx* ctx, Region& r, size_t bytes,
@@ -224,18 +236,9 @@ cudaError_t alloc_region(rgs_ctx* ctx, Region& r, size_t bytes,
   for (int64_t* cap : caps) *cap = 0;
   free_region(r);
   if (bytes == 0) return cudaSuccess;
-  cudaError_t e = cudaMalloc(&r.base, bytes);
-  if (e == cudaErrorMemoryAllocation && !ctx->spare.empty()) {
-    cudaGetLastError();
-    drop_spares(ctx);
-    e = cudaMalloc(&r.base, bytes);
-  }
-  if (e != cudaSuccess) {
-    r.base = nullptr;
-    return e;
-  }
-  r.bytes = bytes;
-  return cudaSuccess;
+  const cudaError_t e = device_alloc(ctx, &r.base, bytes);
+  if (e == cudaSuccess) r.bytes = bytes;
+  return e;
 }
 
 template <typename T>
@@ -674,9 +677,9 @@ rgs_status rgs_autotune(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera* 
   const size_t bytes = align_up(sizeof(float) * 5 * pixels) + align_up(sizeof(float) * 3 * pixels) +
                        3 * align_up(sizeof(float) * 4 * n1) + align_up(sizeof(float) * n1) +
                        align_up(sizeof(float) * 3 * K * n1) + align_up(sizeof(float) * 6 * n_views);
-  char* base = nullptr;
-  RGS_CUDA(cudaMalloc(&base, bytes), "autotune scratch");
-  char* p = base;
+  void* base = nullptr;
+  RGS_CUDA(device_alloc(ctx, &base, bytes), "autotune scratch");
+  char* p = static_cast<char*>(base);
   float* img = carve<float>(p, 5 * pixels);
   float* upc = carve<float>(p, 3 * pixels);
   float* d_means = carve<float>(p, 4 * n1);
@@ -1291,11 +1294,11 @@ rgs_status rgs_radix_sort_u32(rgs_ctx* ctx, uint32_t* keys, uint32_t* vals, int6
   cudaSetDevice(ctx->device);
   const int64_t hist = sort_hist_entries(n);
   const int64_t sums = std::max(scan_blocks(hist), scan_blocks(n)) + 1;
-  char* base = nullptr;
+  void* base = nullptr;
   const size_t bytes = 2 * align_up(sizeof(uint32_t) * n) + align_up(sizeof(uint32_t) * hist) +
                        align_up(sizeof(uint32_t) * sums);
-  RGS_CUDA(cudaMalloc(&base, bytes), "allocate sort scratch");
-  char* p = base;
+  RGS_CUDA(device_alloc(ctx, &base, bytes), "allocate sort scratch");
+  char* p = static_cast<char*>(base);
   uint32_t* kalt = carve<uint32_t>(p, n);
   uint32_t* valt = carve<uint32_t>(p, n);
   uint32_t* h = carve<uint32_t>(p, hist);
@@ -1324,8 +1327,9 @@ rgs_status rgs_exclusive_scan_u32(rgs_ctx* ctx, const uint32_t* in, uint32_t* ou
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);
   cudaSetDevice(ctx->device);
   const int64_t sums = scan_blocks(n) + 1;
-  uint32_t* bs = nullptr;
-  RGS_CUDA(cudaMalloc(&bs, sizeof(uint32_t) * sums), "allocate scan scratch");
+  void* base = nullptr;
+  RGS_CUDA(device_alloc(ctx, &base, sizeof(uint32_t) * sums), "allocate scan scratch");
+  uint32_t* bs = static_cast<uint32_t*>(base);
   cudaError_t e = launch_exclusive_scan(in, out, n, nullptr, total_out, bs, stream);
   cudaError_t e2 = cudaStreamSynchronize(stream);
   cudaFree(bs);

@@ -133,12 +133,57 @@ void failed_first() {
   rgs_destroy(ctx);
 }
 
+// Every allocation of the library frees the kept states before it fails, and the bound on what is
+// kept counts all that a state holds.
+void kept_states_give_way() {
+  void *keys, *vals;
+  cudaMalloc(&keys, 4 * 5000);
+  cudaMalloc(&vals, 4 * 5000);
+  for (int call = 0; call < 3; ++call) {
+    rgs_ctx* ctx = make_context();
+    const size_t bare = fake::live;
+    uint64_t s = 0;
+    EXPECT(forward(ctx, 200000, 64, 6000, &s) == RGS_OK);
+    const size_t before = fake::live;
+    EXPECT(backward(ctx, s, true) == RGS_OK);
+    rgs_stats stats;
+    EXPECT(rgs_query_stats(ctx, s, &stats, nullptr) == RGS_OK);
+    EXPECT(fake::live - before == 4 * 200000);  // the regulariser's scratch
+    EXPECT((size_t)stats.state_bytes == fake::live - bare);
+    EXPECT(rgs_release_state(ctx, s) == RGS_OK);
+    EXPECT(fake::live > bare);
+    fake::limit = fake::live;  // nothing is left but what is kept
+    rgs_status st = RGS_ERR_INVALID_ARG;
+    uint32_t *k = static_cast<uint32_t*>(keys), *v = static_cast<uint32_t*>(vals);
+    if (call == 0) st = rgs_radix_sort_u32(ctx, k, v, 5000, 0, 32, nullptr);
+    if (call == 1) st = rgs_exclusive_scan_u32(ctx, k, v, 5000, nullptr, nullptr);
+    if (call == 2) {
+      alignas(16) static float parameters[4];
+      const rgs_gaussians g{100, 0, parameters, parameters, parameters, parameters, parameters};
+      rgs_camera cam{};
+      cam.width = cam.height = 32;
+      cam.fx = cam.fy = 100.0f;
+      rgs_config cfg;
+      rgs_config_default(&cfg);
+      fake::visible = fake::cells = fake::pairs = 100;
+      st = rgs_autotune(ctx, &g, &cam, 1, &cfg, nullptr, nullptr);
+    }
+    EXPECT(st == RGS_OK);
+    fake::limit = SIZE_MAX;
+    rgs_destroy(ctx);
+    EXPECT(fake::live == 2 * 4 * 5000);
+  }
+  cudaFree(keys);
+  cudaFree(vals);
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
   const std::string which = argc > 1 ? argv[1] : "";
   if (which == "failed_growth") failed_growth();
   else if (which == "failed_first") failed_first();
+  else if (which == "kept_states_give_way") kept_states_give_way();
   else return 2;
   EXPECT(fake::stale == 0);
   return failures ? 1 : 0;

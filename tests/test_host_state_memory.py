@@ -36,3 +36,7 @@ def test_a_forward_that_runs_out_of_memory_leaves_nothing_stale(program):
 
 def test_a_first_forward_that_fails_leaves_no_state(program):
     _run(program, "failed_first")
+
+
+def test_every_allocation_frees_the_kept_states_before_it_fails(program):
+    _run(program, "kept_states_give_way")
