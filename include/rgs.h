@@ -188,7 +188,8 @@ const char* rgs_last_error(const rgs_ctx* ctx);
  * Outside stream capture the call waits once, for the projection, whose counts size the sorted
  * list of visible entries and the tile lists; the rest is queued while the stream runs on. Under
  * stream capture it never synchronises and keeps the sizes of the last call outside capture; if a list would overflow, the kernels record it, the output is incomplete and
- * rgs_query_stats reports status bit 1 (pairs) or 2 (visible entries). */
+ * rgs_query_stats reports status bit 1 (pairs) or 2 (visible entries). More than 2^31 - 1 pairs
+ * outside capture are RGS_ERR_INVALID_ARG. */
 rgs_status rgs_render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera* cams,
                               int32_t n_views, const rgs_config* cfg, rgs_images* out,
                               uint64_t* state, void* stream);
@@ -232,7 +233,8 @@ rgs_status rgs_autotune(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera* 
 rgs_status rgs_release_state(rgs_ctx* ctx, uint64_t state);
 
 /* Grows a state's pair-list capacity to at least `pair_capacity` entries (0 = leave), so that a
- * later forward under stream capture does not overflow. Creates the state if *state is 0. */
+ * later forward under stream capture does not overflow. Creates the state if *state is 0. At most
+ * 2^31 - 1 (RGS_ERR_INVALID_ARG beyond). */
 rgs_status rgs_reserve(rgs_ctx* ctx, uint64_t* state, int64_t pair_capacity, void* stream);
 
 /* Reads the counters of the last forward on `state` (synchronises `stream`). */

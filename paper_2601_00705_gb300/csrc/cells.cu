@@ -343,8 +343,10 @@ __global__ void __launch_bounds__(kCellThreads) cell_expand_kernel(
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const CellPlace place = place_of(views, blockIdx.x);
   const uint2 range = cell_ranges[blockIdx.x];
-  if (blockIdx.x == 0 && threadIdx.x == 0 && counters->n_pairs > capacity)
+  if (blockIdx.x == 0 && threadIdx.x == 0 && counters->n_pairs > capacity) {
     atomicOr(&counters->status, (uint32_t)kStatusPairOverflow);
+    if (counters->n_pairs > 0xffffffffull) counters->n_pairs_listed = 0;  // the scan wrapped
+  }
   if (warp == 0) {
     // The cell's tiles, their runs, and their places in the launch order.
     const int tile = lane < kCellArea ? tile_of(place, lane) : -1;
@@ -456,7 +458,7 @@ cudaError_t launch_tile_lists(const Views& views, const uint2* cell_ranges, cons
   RGS_LAUNCHED();
   if (e == cudaSuccess)
     e = launch_tile_ranges_scan(tile_counts, ranges, views.total_tiles, capacity,
-                                &counters->n_pairs_listed, lb, stream);
+                                &counters->n_pairs, &counters->n_pairs_listed, lb, stream);
   if (e == cudaSuccess) {
     e = launch_chained(masks ? cell_expand_kernel<true> : cell_expand_kernel<false>, grid, block,
                        stream, views, cell_ranges, keys, vals, rec, log2_alpha_min,

@@ -351,13 +351,18 @@ rgs_status ensure_pix_tiles(rgs_ctx* ctx, State& s, int64_t pixels, int64_t tile
   return RGS_OK;
 }
 
-// Capacity for `count` list entries: a quarter more than asked for.
-int64_t with_slack(int64_t count) { return std::max<int64_t>(count + count / 4, 4096); }
+// The blends keep positions in the pair list as signed 32-bit numbers.
+constexpr int64_t kMaxListed = INT32_MAX;
+
+// Capacity for `count` <= kMaxListed list entries: a quarter more than asked for.
+int64_t with_slack(int64_t count) {
+  return std::min(std::max<int64_t>(count + count / 4, 4096), kMaxListed);
+}
 
 rgs_status ensure_pairs(rgs_ctx* ctx, State& s, int64_t pairs) {
   if (pairs <= s.pair_cap) return RGS_OK;
+  if (pairs > kMaxListed) return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^31 - 1");
   const int64_t cap = with_slack(pairs);
-  if (cap >= (int64_t)UINT32_MAX) return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^32");
   RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
   RGS_CUDA(alloc_region(ctx, s.r_pair, align_up(sizeof(uint32_t) * cap), {&s.pair_cap}),
            "allocate pair list");
@@ -368,8 +373,8 @@ rgs_status ensure_pairs(rgs_ctx* ctx, State& s, int64_t pairs) {
 
 rgs_status ensure_cells(rgs_ctx* ctx, State& s, int64_t cells) {
   if (cells <= s.cell_cap) return RGS_OK;
+  if (cells > kMaxListed) return fail(ctx, RGS_ERR_INVALID_ARG, "cell list exceeds 2^31 - 1");
   const int64_t cap = with_slack(cells);
-  if (cap >= (int64_t)UINT32_MAX) return fail(ctx, RGS_ERR_INVALID_ARG, "cell list exceeds 2^32");
   RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
   RGS_CUDA(alloc_region(ctx, s.r_cell, 4 * align_up(sizeof(uint32_t) * cap), {&s.cell_cap}),
            "allocate cell lists");
@@ -817,6 +822,8 @@ rgs_status rgs_release_state(rgs_ctx* ctx, uint64_t handle) {
 rgs_status rgs_reserve(rgs_ctx* ctx, uint64_t* handle, int64_t pair_capacity, void* stream) {
   (void)stream;
   if (!ctx) return RGS_ERR_INVALID_ARG;
+  if (pair_capacity > kMaxListed)
+    return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^31 - 1");
   State* s = nullptr;
   rgs_status st = get_or_create_state(ctx, handle, &s);
   if (st != RGS_OK) return st;
@@ -991,8 +998,8 @@ rgs_status forward_on_state(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_came
   if (!capturing) {
     RGS_CUDA(cudaEventSynchronize(s->done), "wait for the projection's counts");
     const Counters& c = *ctx->host_counters;
-    if (c.all_pairs >= UINT32_MAX || c.all_cells >= UINT32_MAX)
-      return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^32");
+    if (c.all_pairs > kMaxListed || c.all_cells > kMaxListed)
+      return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^31 - 1");
     vis_cap = (int64_t)c.all_visible;
     if (vis_cap > s->vis_cap) s->vis_cap = std::max<int64_t>(vis_cap + vis_cap / 4, 1024);
     n_cells = (int64_t)c.all_cells;

@@ -613,10 +613,12 @@ cudaError_t launch_compact_visible(const uint32_t* vis_bits, int n_views, int n,
 
 // ranges[t] = [first, last + 1) of tile t's run when tile t holds counts[t] pairs and the runs
 // follow each other in tile order, clipped to `capacity` pairs ([0, 0) for an empty tile); the
-// unclipped total into *total. One single-pass launch; lb must be zeroed.
+// unclipped total into *total. *bound is at least that total: past 32 bits every range is empty
+// (the sums would wrap; only under stream capture, where the host has not seen the counts). One
+// single-pass launch; lb must be zeroed.
 cudaError_t launch_tile_ranges_scan(const uint32_t* counts, uint2* ranges, int64_t n_tiles,
-                                    uint32_t capacity, uint32_t* total, Lookback lb,
-                                    cudaStream_t stream);
+                                    uint32_t capacity, const unsigned long long* bound,
+                                    uint32_t* total, Lookback lb, cudaStream_t stream);
 
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;       // keys per thread for large sorts (2048 per block)

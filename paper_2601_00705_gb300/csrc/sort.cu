@@ -93,13 +93,16 @@ struct PlainStore {
   }
 };
 
-// [first, last + 1) of element k's run in a list of `capacity` slots ([0, 0) for an empty one).
+// [first, last + 1) of element k's run in a list of `capacity` slots ([0, 0) for an empty one, and
+// for all when the sums do not fit in 32 bits).
 struct RangeStore {
   uint2* out;
   uint32_t capacity;
+  const unsigned long long* bound;
   __device__ void operator()(uint32_t k, uint32_t value, uint32_t prefix) const {
-    out[k] = value ? make_uint2(min(prefix, capacity), min(prefix + value, capacity))
-                   : make_uint2(0u, 0u);
+    out[k] = value && *bound <= 0xffffffffull
+                 ? make_uint2(min(prefix, capacity), min(prefix + value, capacity))
+                 : make_uint2(0u, 0u);
   }
 };
 
@@ -951,9 +954,9 @@ cudaError_t launch_compact_visible(const uint32_t* vis_bits, int n_views, int n,
 }
 
 cudaError_t launch_tile_ranges_scan(const uint32_t* counts, uint2* ranges, int64_t n_tiles,
-                                    uint32_t capacity, uint32_t* total, Lookback lb,
-                                    cudaStream_t stream) {
-  return run_scan(PlainLoad{counts}, RangeStore{ranges, capacity}, n_tiles, nullptr, total,
+                                    uint32_t capacity, const unsigned long long* bound,
+                                    uint32_t* total, Lookback lb, cudaStream_t stream) {
+  return run_scan(PlainLoad{counts}, RangeStore{ranges, capacity, bound}, n_tiles, nullptr, total,
                   nullptr, stream, lb);
 }
 

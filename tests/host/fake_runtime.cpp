@@ -1,5 +1,6 @@
 // The CUDA runtime calls of csrc/rgs_api.cu on host memory.
 #include <cuda_runtime_api.h>
+#include <sys/mman.h>
 
 #include <cstdio>
 #include <cstdlib>
@@ -35,8 +36,10 @@ cudaError_t cudaMalloc(void** p, size_t bytes) {
   fake::unsafe += fake::capturing;
   *p = nullptr;
   if (fake::live + bytes > fake::limit) return cudaErrorMemoryAllocation;
-  char* base = static_cast<char*>(std::malloc(bytes));
-  if (!base) return cudaErrorMemoryAllocation;
+  void* base_ptr = mmap(nullptr, bytes, PROT_READ | PROT_WRITE,
+                        MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
+  if (base_ptr == MAP_FAILED) return cudaErrorMemoryAllocation;
+  char* base = static_cast<char*>(base_ptr);
   fake::blocks()[base] = bytes;
   fake::live += bytes;
   *p = base;
@@ -47,8 +50,8 @@ cudaError_t cudaFree(void* p) {
   auto it = fake::blocks().find(static_cast<char*>(p));
   if (it == fake::blocks().end()) return p ? cudaErrorInvalidValue : cudaSuccess;
   fake::live -= it->second;
+  munmap(p, it->second);
   fake::blocks().erase(it);
-  std::free(p);
   return cudaSuccess;
 }
 cudaError_t cudaMemGetInfo(size_t* free_bytes, size_t* total_bytes) {

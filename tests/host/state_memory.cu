@@ -177,6 +177,28 @@ void kept_states_give_way() {
   cudaFree(vals);
 }
 
+// List positions are signed 32-bit numbers in the blends: more pairs or cell entries than those
+// hold are refused, by the forward and by rgs_reserve, and capacities with their slack stay below.
+void list_limits() {
+  const unsigned long long most = 2147483647ull;
+  rgs_ctx* ctx = make_context();
+  const size_t bare = fake::live;
+  uint64_t s = 0;
+  EXPECT(rgs_reserve(ctx, &s, (int64_t)most + 1, nullptr) == RGS_ERR_INVALID_ARG);
+  EXPECT(s == 0 && fake::live == bare);
+  for (unsigned long long count : {most + 1, 3000000000ull, 4294967294ull, 5000000000ull}) {
+    EXPECT(forward(ctx, 1000, 64, count, &s) == RGS_ERR_INVALID_ARG);
+    EXPECT(s == 0 && fake::live == bare);
+  }
+  for (unsigned long long count : {1800000000ull, most}) {
+    EXPECT(forward(ctx, 1000, 64, count, &s) == RGS_OK);
+    rgs_stats stats;
+    EXPECT(rgs_query_stats(ctx, s, &stats, nullptr) == RGS_OK);
+    EXPECT(stats.pair_capacity == (int64_t)most);
+  }
+  rgs_destroy(ctx);
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -184,6 +206,7 @@ int main(int argc, char** argv) {
   if (which == "failed_growth") failed_growth();
   else if (which == "failed_first") failed_first();
   else if (which == "kept_states_give_way") kept_states_give_way();
+  else if (which == "list_limits") list_limits();
   else return 2;
   EXPECT(fake::stale == 0);
   return failures ? 1 : 0;

@@ -40,3 +40,7 @@ def test_a_first_forward_that_fails_leaves_no_state(program):
 
 def test_every_allocation_frees_the_kept_states_before_it_fails(program):
     _run(program, "kept_states_give_way")
+
+
+def test_lists_past_the_blends_positions_are_refused(program):
+    _run(program, "list_limits")
