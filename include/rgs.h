@@ -232,8 +232,9 @@ rgs_status rgs_autotune(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera* 
  * the device's queued work). What is kept is freed by rgs_destroy, or when an allocation fails. */
 rgs_status rgs_release_state(rgs_ctx* ctx, uint64_t state);
 
-/* Grows a state's pair-list capacity to at least `pair_capacity` entries (0 = leave), so that a
- * later forward under stream capture does not overflow. Creates the state if *state is 0. At most
+/* Grows a state's pair-list capacity to at least `pair_capacity` entries (0 = leave) and the list of
+ * touched cells behind it (at most one entry per pair) to as many, so that a later forward under
+ * stream capture does not overflow. Takes 20 bytes per entry asked for (16, and a quarter more). Creates the state if *state is 0. At most
  * 2^31 - 1 (RGS_ERR_INVALID_ARG beyond). */
 rgs_status rgs_reserve(rgs_ctx* ctx, uint64_t* state, int64_t pair_capacity, void* stream);
 

@@ -113,6 +113,8 @@ struct State {
   uint32_t* tile_counts = nullptr;
   uint32_t* tile_order = nullptr;  // launch order of the blends' tiles (longest run first)
   uint32_t *cell_keys[2] = {nullptr, nullptr}, *cell_vals[2] = {nullptr, nullptr};
+  // The pair list of the last forward: in r_pair, or, where the cell list's buffers are at least as
+  // long, in the one that the cell sort leaves free.
   uint32_t* pairs = nullptr;
   // Scratch.
   uint32_t* hist = nullptr;
@@ -135,6 +137,7 @@ struct State {
   cudaEvent_t done = nullptr;
   bool open = false, captured = false;
 
+  int64_t pair_capacity() const { return std::max(pair_cap, cell_cap); }
   size_t bytes() const {
     return r_vn.bytes + r_n.bytes + r_pix.bytes + r_tile.bytes + r_cell.bytes + r_pair.bytes +
            r_scratch.bytes + r_pose.bytes + r_counters.bytes + r_reg.bytes;
@@ -359,14 +362,14 @@ int64_t with_slack(int64_t count) {
   return std::min(std::max<int64_t>(count + count / 4, 4096), kMaxListed);
 }
 
+// After ensure_cells.
 rgs_status ensure_pairs(rgs_ctx* ctx, State& s, int64_t pairs) {
-  if (pairs <= s.pair_cap) return RGS_OK;
+  if (pairs <= s.pair_capacity()) return RGS_OK;
   if (pairs > kMaxListed) return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^31 - 1");
   const int64_t cap = with_slack(pairs);
   RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
   RGS_CUDA(alloc_region(ctx, s.r_pair, align_up(sizeof(uint32_t) * cap), {&s.pair_cap}),
            "allocate pair list");
-  s.pairs = static_cast<uint32_t*>(s.r_pair.base);
   s.pair_cap = cap;
   return RGS_OK;
 }
@@ -829,9 +832,10 @@ rgs_status rgs_reserve(rgs_ctx* ctx, uint64_t* handle, int64_t pair_capacity, vo
   if (st != RGS_OK) return st;
   cudaSetDevice(ctx->device);
   if (pair_capacity > 0) {
-    // No footprint has more cell entries than pairs, but for the few cells a thin one skips over.
-    st = ensure_pairs(ctx, *s, pair_capacity);
-    if (st == RGS_OK) st = ensure_cells(ctx, *s, pair_capacity);
+    // As many cell entries, whose buffers hold the pair list too. No footprint has more cell
+    // entries than pairs, unless it skips whole cells between two pixel rows: only a needle of an
+    // opacity below 1.4 alpha_min can (the dilation makes every other one too thick).
+    st = ensure_cells(ctx, *s, pair_capacity);
     if (st != RGS_OK) return st;
     st = ensure_scratch(ctx, *s, std::max<int64_t>(s->cell_cap, s->vn_cap), false);
     if (st != RGS_OK) return st;
@@ -1003,12 +1007,12 @@ rgs_status forward_on_state(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_came
     vis_cap = (int64_t)c.all_visible;
     if (vis_cap > s->vis_cap) s->vis_cap = std::max<int64_t>(vis_cap + vis_cap / 4, 1024);
     n_cells = (int64_t)c.all_cells;
-    st = ensure_pairs(ctx, *s, (int64_t)c.all_pairs);
-    if (st == RGS_OK) st = ensure_cells(ctx, *s, n_cells);
+    st = ensure_cells(ctx, *s, n_cells);
+    if (st == RGS_OK) st = ensure_pairs(ctx, *s, (int64_t)c.all_pairs);
     if (st == RGS_OK) st = ensure_scratch(ctx, *s, std::max<int64_t>(vn, s->cell_cap), false);
     if (st != RGS_OK) return st;
   } else {
-    if (s->pair_cap == 0 || s->cell_cap == 0)
+    if (s->cell_cap == 0)
       return fail(ctx, RGS_ERR_CAPACITY,
                   "pair list has no capacity under capture: rgs_reserve");
     if (s->vis_cap == 0) s->vis_cap = vn;
@@ -1023,7 +1027,6 @@ rgs_status forward_on_state(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_came
   s->order = s->vis_vals[alt ? 1 : 0];
   RGS_CUDA(mark(ctx, *s, 3, stream, capturing), "event");
   RGS_CUDA(mark(ctx, *s, 4, stream, capturing), "event");
-  const uint32_t pair_cap = (uint32_t)s->pair_cap;
   // 4. Cell entries in depth order.
   RGS_CUDA(launch_emit_cells(views, g->n, s->order, s->rec,
                              consts.log2_alpha_min, vis_cap, (uint32_t)s->cell_cap,
@@ -1042,6 +1045,9 @@ rgs_status forward_on_state(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_came
            "cell sort");
   const uint32_t* keys = s->cell_keys[alt ? 1 : 0];
   const uint32_t* vals = s->cell_vals[alt ? 1 : 0];
+  s->pairs = s->pair_cap >= s->cell_cap ? static_cast<uint32_t*>(s->r_pair.base)
+                                        : s->cell_keys[alt ? 0 : 1];
+  const uint32_t pair_cap = (uint32_t)s->pair_capacity();
   RGS_CUDA(mark(ctx, *s, 6, stream, capturing), "event");
   // 6. The tiles' lists, their ranges and launch order.
   RGS_CUDA(launch_cell_ranges(views, keys, n_cells, cell_ranges, cnt, stream), "cell ranges");
@@ -1206,7 +1212,7 @@ rgs_status rgs_query_stats(rgs_ctx* ctx, uint64_t handle, rgs_stats* out, void* 
   State* s = find_state(ctx, handle);
   if (!s) return fail(ctx, RGS_ERR_STATE, "unknown state handle");
   std::memset(out, 0, sizeof(*out));
-  out->pair_capacity = s->pair_cap;
+  out->pair_capacity = s->pair_capacity();
   out->state_bytes = (int64_t)s->bytes();
   if (!s->counters) return RGS_OK;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);
@@ -1237,7 +1243,7 @@ rgs_status rgs_copy_tile_lists(rgs_ctx* ctx, uint64_t handle, uint32_t* host_val
                            cudaMemcpyDeviceToHost, stream),
            "read counters");
   RGS_CUDA(cudaStreamSynchronize(stream), "sync");
-  const int64_t np = std::min<int64_t>(ctx->host_counters->n_pairs_listed, s->pair_cap);
+  const int64_t np = std::min<int64_t>(ctx->host_counters->n_pairs_listed, s->pair_capacity());
   *n_pairs = np;
   if (host_vals && np <= vals_cap && np > 0)
     RGS_CUDA(cudaMemcpyAsync(host_vals, s->pairs, sizeof(uint32_t) * np,

@@ -17,7 +17,7 @@ static std::map<char*, size_t>& blocks() {
 size_t live = 0, limit = SIZE_MAX, total = 288ull << 30;
 bool capturing = false;
 int stale = 0, unsafe = 0;
-unsigned long long visible = 0, cells = 0, pairs = 0;
+unsigned long long visible = 0, cells = 0, pairs = 0, pairs_per_cell = 1;
 
 void check(const void* p, size_t bytes, const char* what) {
   char* c = static_cast<char*>(const_cast<void*>(p));

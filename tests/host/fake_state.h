@@ -12,7 +12,7 @@ extern bool capturing;
 extern int stale;     // accesses outside live memory
 extern int unsafe;    // calls that would invalidate a stream capture, made during one
 // What the projection of the next forwards counts.
-extern unsigned long long visible, cells, pairs;
+extern unsigned long long visible, cells, pairs, pairs_per_cell;
 
 void check(const void* p, size_t bytes, const char* what);
 }  // namespace fake

@@ -29,7 +29,8 @@ rgs_status forward(rgs_ctx* ctx, int n, int w, unsigned long long count, uint64_
   static Images images;
   alignas(16) static float parameters[4];
   fake::visible = count < (unsigned long long)n * views ? count : (unsigned long long)n * views;
-  fake::cells = fake::pairs = count;
+  fake::cells = count;
+  fake::pairs = fake::pairs_per_cell * count;
   std::vector<rgs_camera> cams(views);
   for (rgs_camera& c : cams) {
     c = rgs_camera{};
@@ -199,6 +200,41 @@ void list_limits() {
   rgs_destroy(ctx);
 }
 
+// Reserved pairs take 16 bytes each (and a quarter more of them), and serve forwards under capture
+// with as many pairs and cells, whichever of the two is larger, before and after eager ones.
+void reserved_pairs() {
+  const int64_t asked = 1000000;
+  rgs_ctx* ctx = make_context();
+  uint64_t s = 0;
+  EXPECT(forward(ctx, 1000, 64, 100, &s) == RGS_OK);
+  const size_t before = fake::live;
+  EXPECT(rgs_reserve(ctx, &s, asked, nullptr) == RGS_OK);
+  const size_t grown = fake::live - before;
+  const size_t scratch = 1 << 20;  // the sort's tables
+  EXPECT(grown >= 16 * (size_t)asked && grown <= 20 * (size_t)asked + scratch);
+  rgs_stats stats;
+  EXPECT(rgs_query_stats(ctx, s, &stats, nullptr) == RGS_OK);
+  EXPECT(stats.pair_capacity >= asked);
+  for (int round = 0; round < 2; ++round) {
+    fake::capturing = true;
+    EXPECT(forward(ctx, 1000, 64, asked, &s) == RGS_OK);
+    EXPECT(backward(ctx, s) == RGS_OK);
+    fake::capturing = false;
+    EXPECT(fake::live - before == grown);
+    EXPECT(forward(ctx, 1000, 64, asked, &s) == RGS_OK);  // nothing grows
+    EXPECT(backward(ctx, s) == RGS_OK);
+    EXPECT(fake::live - before == grown);
+  }
+  fake::pairs_per_cell = 8;
+  EXPECT(forward(ctx, 1000, 64, asked, &s) == RGS_OK);
+  EXPECT(rgs_query_stats(ctx, s, &stats, nullptr) == RGS_OK);
+  EXPECT(stats.pair_capacity >= 8 * asked);
+  fake::pairs_per_cell = 1;
+  EXPECT(forward(ctx, 1000, 64, asked, &s) == RGS_OK);
+  EXPECT(fake::unsafe == 0);
+  rgs_destroy(ctx);
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -207,6 +243,7 @@ int main(int argc, char** argv) {
   else if (which == "failed_first") failed_first();
   else if (which == "kept_states_give_way") kept_states_give_way();
   else if (which == "list_limits") list_limits();
+  else if (which == "reserved_pairs") reserved_pairs();
   else return 2;
   EXPECT(fake::stale == 0);
   return failures ? 1 : 0;

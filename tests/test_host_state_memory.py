@@ -44,3 +44,7 @@ def test_every_allocation_frees_the_kept_states_before_it_fails(program):
 
 def test_lists_past_the_blends_positions_are_refused(program):
     _run(program, "list_limits")
+
+
+def test_reserved_pairs_take_their_documented_memory_and_serve_captures(program):
+    _run(program, "reserved_pairs")
