@@ -226,11 +226,18 @@ rgs_status rgs_autotune(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera* 
                         int32_t n_views, rgs_config* cfg, float* ms_out, void* stream);
 
 /* Ends a state; its handle is unknown from then on. The context keeps the memory of the last two
- * states released (together at most 1/16 of the device's) for the states that later forwards
+ * states released (together at most 1/64 of the device's) for the states that later forwards
  * create, which run after the work queued on it on whatever stream; the call does not wait. A
- * larger state, and one that a forward or backward under stream capture has used, is freed (after
- * the device's queued work). What is kept is freed by rgs_destroy, or when an allocation fails. */
+ * larger state, one of 64 MB and more while less than 1/8 of the device's memory is free (those
+ * kept go then, too), and one that a forward or backward under stream capture has used, is freed
+ * (after the device's queued work). What is kept is freed by rgs_trim and rgs_destroy, and when an
+ * allocation of the context fails. */
 rgs_status rgs_release_state(rgs_ctx* ctx, uint64_t state);
+
+/* Gives back the device memory that the context keeps for later calls: that of released states and
+ * the scratch of the seed initialisation. For a caller whose own allocations need it (other
+ * allocators cannot free it). Waits for the device's queued work; not during a stream capture. */
+rgs_status rgs_trim(rgs_ctx* ctx);
 
 /* Grows a state's pair-list capacity to at least `pair_capacity` entries (0 = leave) and the list of
  * touched cells behind it (at most one entry per pair) to as many, so that a later forward under

@@ -23,7 +23,7 @@ GRAD_ALL = 63
 
 # Every function the header declares (checked by the ABI tests).
 EXPORTED = ("rgs_create", "rgs_destroy", "rgs_config_default", "rgs_last_error",
-            "rgs_render_forward", "rgs_render_backward", "rgs_release_state", "rgs_reserve",
+            "rgs_render_forward", "rgs_render_backward", "rgs_release_state", "rgs_trim", "rgs_reserve",
             "rgs_query_stats", "rgs_set_phase_timing", "rgs_phase_times", "rgs_radix_sort_u32",
             "rgs_exclusive_scan_u32", "rgs_exclusive_scan_u32_static", "rgs_copy_tile_lists",
             "rgs_copy_records", "rgs_autotune", "rgs_render_forward_posed",
@@ -137,6 +137,7 @@ def load(build_if_needed: bool = True):
             "rgs_render_backward": (S, [P, U64, ctypes.POINTER(ImageGrads), U32, P, P, P, P, P, P,
                                         P]),
             "rgs_release_state": (S, [P, U64]),
+            "rgs_trim": (S, [P]),
             "rgs_reserve": (S, [P, ctypes.POINTER(U64), I64, P]),
             "rgs_query_stats": (S, [P, U64, ctypes.POINTER(Stats), P]),
             "rgs_set_phase_timing": (S, [P, I32]),
@@ -391,6 +392,10 @@ class Context:
     def release(self, state: int):
         if state:
             self._check(self.lib.rgs_release_state(self.handle, ctypes.c_uint64(state)))
+
+    def trim(self):
+        """Gives back the device memory kept for later calls (waits for the device)."""
+        self._check(self.lib.rgs_trim(self.handle))
 
     def reserve(self, state: int, pair_capacity: int, stream: int = 0) -> int:
         h = ctypes.c_uint64(state)

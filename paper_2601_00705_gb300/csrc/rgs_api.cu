@@ -181,10 +181,12 @@ struct rgs_ctx {
   std::map<uint64_t, State*> states;
   uint64_t next_id = 1;
   // Released states kept for the next one (oldest first): at most kSpareStates of them, together
-  // at most spare_limit bytes. A forward that creates its state (every `render` call does) then
+  // at most 1/kSpareShare of the device (spare_limit). A forward that creates its state (every `render` call does) then
   // takes buffers that are already there: allocating and freeing them with a device
   // synchronisation cost 0.55 ms of a 0.82 ms 1200x680 frame and 1.0 ms of a 1.7 ms ten-view
-  // training step. Freed with the context, and whenever one of its allocations fails.
+  // training step. Freed by rgs_trim, with the context, and whenever one of its allocations fails.
+  // Other allocators of the process cannot ask for them, so a state of kSmallSpare and more is kept
+  // only while 1/kSpareFree of the device is free: a program near the limit finds nothing withheld.
   std::vector<State*> spare;
   size_t spare_limit = 0;
   Counters* host_counters = nullptr;  // pinned
@@ -217,6 +219,7 @@ void free_region(Region& r) {
 }
 
 constexpr size_t kSpareStates = 2;
+constexpr size_t kSpareShare = 64, kSpareFree = 8, kSmallSpare = 64u << 20;
 
 void drop_spares(rgs_ctx* ctx);
 
@@ -634,7 +637,8 @@ rgs_status rgs_create(rgs_ctx** out, int device) {
     return RGS_ERR_NOMEM;
   }
   size_t free_bytes = 0, total_bytes = 0;
-  if (cudaMemGetInfo(&free_bytes, &total_bytes) == cudaSuccess) ctx->spare_limit = total_bytes / 16;
+  if (cudaMemGetInfo(&free_bytes, &total_bytes) == cudaSuccess)
+    ctx->spare_limit = total_bytes / kSpareShare;
   *out = ctx;
   return RGS_OK;
 }
@@ -801,9 +805,15 @@ rgs_status rgs_release_state(rgs_ctx* ctx, uint64_t handle) {
   cudaSetDevice(ctx->device);
   ctx->states.erase(handle);
   const size_t bytes = s->bytes();
+  size_t free_bytes = 0, total_bytes = 0;
+  const bool scarce = bytes >= kSmallSpare &&
+                      (cudaMemGetInfo(&free_bytes, &total_bytes) != cudaSuccess ||
+                       free_bytes < total_bytes / kSpareFree);
   // Kept for the next state, unless a graph may still refer to its buffers, the end of its work
-  // was not recorded (it failed half-way, or never ran), or it alone exceeds the bound.
-  if (s->captured || s->open || !s->has_forward || bytes > ctx->spare_limit) {
+  // was not recorded (it failed half-way, or never ran), it alone exceeds the bound, or memory is
+  // scarce.
+  if (s->captured || s->open || !s->has_forward || bytes > ctx->spare_limit || scarce) {
+    if (scarce) drop_spares(ctx);
     cudaDeviceSynchronize();  // queued work may still read the state's buffers
     destroy_state(s);
     return RGS_OK;
@@ -819,6 +829,16 @@ rgs_status rgs_release_state(rgs_ctx* ctx, uint64_t handle) {
     ctx->spare.erase(ctx->spare.begin());
   }
   ctx->spare.push_back(s);
+  return RGS_OK;
+}
+
+rgs_status rgs_trim(rgs_ctx* ctx) {
+  if (!ctx) return RGS_ERR_INVALID_ARG;
+  ctx->last_error.clear();
+  if (cudaSetDevice(ctx->device) != cudaSuccess)
+    return fail(ctx, RGS_ERR_CUDA, "cudaSetDevice failed");
+  drop_spares(ctx);
+  free_region(ctx->r_seed);  // its calls end synchronised
   return RGS_OK;
 }
 

@@ -43,6 +43,14 @@ class Renderer:
     def stream_handle(self) -> int:
         return torch.cuda.current_stream(self.device).cuda_stream
 
+    def _empty(self, *shapes) -> list[torch.Tensor]:
+        """Outputs; when they do not fit, what the context keeps is freed and they are tried again."""
+        try:
+            return [torch.empty(s, dtype=torch.float32, device=self.device) for s in shapes]
+        except torch.cuda.OutOfMemoryError:
+            self.ctx.trim()
+            return [torch.empty(s, dtype=torch.float32, device=self.device) for s in shapes]
+
     def forward_raw(self, means, log_scales, quats, opacity_logits, sh, cameras, state: int = 0,
                     out=None, world_to_cam: torch.Tensor | None = None,
                     sh_event: "torch.cuda.Event | None" = None):
@@ -69,9 +77,7 @@ class Renderer:
         cams = cameras if hasattr(cameras, "_type_") else binding.make_cameras(cameras)
         P = sum(int(c.width) * int(c.height) for c in cams)
         if out is None:
-            color = torch.empty((P, 3), dtype=torch.float32, device=dev)
-            depth = torch.empty((P,), dtype=torch.float32, device=dev)
-            alpha = torch.empty((P,), dtype=torch.float32, device=dev)
+            color, depth, alpha = self._empty((P, 3), (P,), (P,))
         else:
             color, depth, alpha = out
         g = binding.Gaussians(n, deg, means.data_ptr(), log_scales.data_ptr(), quats.data_ptr(),
@@ -129,7 +135,7 @@ class Renderer:
                                      f"16-byte aligned float32 tensor of {shape}")
                 out[name] = t
             else:
-                out[name] = torch.empty(shape, dtype=torch.float32, device=dev)
+                out[name], = self._empty(shape)
         grads = binding.ImageGrads(d_color.data_ptr() if d_color is not None else None,
                                    d_depth.data_ptr() if d_depth is not None else None,
                                    d_alpha.data_ptr() if d_alpha is not None else None)
@@ -162,6 +168,11 @@ class Renderer:
 
     def release(self, state: int):
         self.ctx.release(state)
+
+    def trim(self):
+        """Gives back the device memory that the context keeps for later calls (that of released
+        states, outside PyTorch's allocator)."""
+        self.ctx.trim()
 
     def stats(self, state: int) -> dict:
         return self.ctx.stats(state, self.stream_handle())

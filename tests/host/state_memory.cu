@@ -235,6 +235,37 @@ void reserved_pairs() {
   rgs_destroy(ctx);
 }
 
+// What is kept after a release is bounded, is not kept while memory is scarce, and is given back.
+void kept_memory() {
+  for (size_t room : {(size_t)0, fake::total / 8 - (1u << 20), fake::total / 8 + (1u << 20)}) {
+    rgs_ctx* ctx = make_context();
+    const size_t bare = fake::live;
+    uint64_t a = 0, b = 0, c = 0;
+    EXPECT(forward(ctx, 1000, 64, 6000, &a) == RGS_OK);
+    EXPECT(forward(ctx, 1000000, 64, 6000, &b) == RGS_OK);   // 150 MB
+    EXPECT(forward(ctx, 60000000, 64, 6000, &c) == RGS_OK);  // 9 GB
+    fake::limit = fake::live + room;
+    EXPECT(rgs_release_state(ctx, a) == RGS_OK);  // small: kept
+    EXPECT(fake::live > bare + (150u << 20));
+    EXPECT(rgs_release_state(ctx, c) == RGS_OK);  // beyond the bound
+    fake::limit = fake::live + room;
+    const size_t with_b = fake::live;
+    EXPECT(rgs_release_state(ctx, b) == RGS_OK);
+    const bool scarce = room < fake::total / 8;
+    EXPECT(scarce ? fake::live == bare : fake::live == with_b);
+    EXPECT(fake::live - bare <= fake::total / 64);
+    EXPECT(rgs_trim(ctx) == RGS_OK);
+    EXPECT(fake::live == bare);
+    uint64_t s = 0;
+    fake::limit = SIZE_MAX;
+    EXPECT(forward(ctx, 1000, 64, 6000, &s) == RGS_OK);
+    EXPECT(backward(ctx, s) == RGS_OK);
+    rgs_destroy(ctx);
+    EXPECT(fake::live == 0);
+  }
+  EXPECT(rgs_trim(nullptr) == RGS_ERR_INVALID_ARG);
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -244,6 +275,7 @@ int main(int argc, char** argv) {
   else if (which == "kept_states_give_way") kept_states_give_way();
   else if (which == "list_limits") list_limits();
   else if (which == "reserved_pairs") reserved_pairs();
+  else if (which == "kept_memory") kept_memory();
   else return 2;
   EXPECT(fake::stale == 0);
   return failures ? 1 : 0;

@@ -48,3 +48,7 @@ def test_lists_past_the_blends_positions_are_refused(program):
 
 def test_reserved_pairs_take_their_documented_memory_and_serve_captures(program):
     _run(program, "reserved_pairs")
+
+
+def test_kept_memory_is_bounded_and_given_back(program):
+    _run(program, "kept_memory")
