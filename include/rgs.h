@@ -143,8 +143,9 @@ typedef struct {
 typedef struct {
   int64_t n_visible;       /* (view, Gaussian) pairs seen: the footprint touches at least one
                               tile, and its bounding radius sqrt(kappa (|J|_F^2 smax^2 + eps2d)),
-                              kappa = 2 ln(o / alpha_min), widened by 2 % and 4 px, reaches the
-                              image (edge tiles reach past it) */
+                              kappa = 2 ln(o / alpha_min), widened by 2 % and 4 px (by more where
+                              the rounding of far coordinates takes more), reaches the image (edge
+                              tiles reach past it) */
   int64_t n_pairs;         /* duplicated (view, tile, Gaussian) entries (of the visible entries
                               kept, when status bit 2 is set) */
   int64_t n_eval;          /* (pixel, Gaussian) list positions visited by the forward blend */

@@ -286,18 +286,30 @@ __device__ __forceinline__ void load_sh(const float* __restrict__ sh, int i, flo
   }
 }
 
+// Bound of the rounding of a plainly computed centre (column or row times depth) per unit of
+// |m|_1 + |t|_1: see cull_kernel.
+__device__ __forceinline__ float image_rounding(const ViewParams& vp) {
+  return 9.6e-7f * fmaxf(vp.fx + fabsf(vp.cx), vp.fy + fabsf(vp.cy));
+}
+__device__ __forceinline__ float norm1(const float* a) {
+  return fabsf(a[0]) + fabsf(a[1]) + fabsf(a[2]);
+}
+
 // Whether the footprint of an entry may reach the image: the rule, with the tile cover, of what
 // counts as seen (n_visible, the observation counts), so it must not depend on how loose the test
 // is that picks the candidates. The centre comes from plain FMA dot products and the radius from a
 // bound of the alpha >= alpha_min footprint: the largest eigenvalue of Sigma^I is at most
 // |J|_F^2 smax^2 + eps, so the radius is at most sqrt(kappa (|J|_F^2 smax^2 + eps)); widened by 2 %
 // and 4 px. An entry past the edge by less counts where a tile at the right or bottom edge reaches
-// past the image.
+// past the image. The 4 px also cover the centre's rounding, which grows with the distance of the
+// Gaussian and the camera from the origin: where its bound (image_rounding, times the depth) exceeds
+// 3 px, the planes of the cull, which take it into account, have the last word.
 __device__ __forceinline__ bool reaches_image(const ViewParams& vp, const PoseRef& ps,
                                               const Consts& c, const float* m, const float* ls,
                                               float logit) {
   const float* R = ps.R;
   const float z = fmaf(R[6], m[0], fmaf(R[7], m[1], fmaf(R[8], m[2], ps.t[2])));
+  if (image_rounding(vp) * (norm1(m) + norm1(ps.t)) > 3.0f * z) return true;
   const float z_err =
       4.8e-7f * (fabsf(R[6] * m[0]) + fabsf(R[7] * m[1]) + fabsf(R[8] * m[2]) + fabsf(ps.t[2]));
   if (!(z + z_err > c.znear && z > 0.0f)) return false;
@@ -328,23 +340,25 @@ __device__ __forceinline__ bool reaches_image(const ViewParams& vp, const PoseRe
 // The pass is bound by instruction issue, so an entry is tested by planes: with
 // (x, y, z) = R m + t, the centre lies at pixel (fx x / z + cx, fy y / z + cy), and the radius of
 // reaches_image is at most 1.02 sqrt(kappa) (F smax / z + sqrt(eps)) + 4 with
-// F^2 = fx^2 (1 + lim_u^2) + fy^2 (1 + lim_w^2) for the guard-banded J. Times z > 0, "mx + rad < 0"
+// F^2 = fx^2 (1 + lim_u^2) + fy^2 (1 + lim_w^2) for the guard-banded J. Times z, "mx + rad < 0"
 // and its three siblings become linear in m and z, with no division or square root per entry:
 // three dot products and four comparisons (about 20 instructions; the radius itself took 60: 137 us
 // for 24 views of a million Gaussians, 258 us for 16 of three). Without a guard band |J|_F
 // has no such bound and follows from u and w.
 //
-// Everything that reaches_image keeps is a candidate. Both tests take the same z; their pixel
-// columns (rows) times z differ by rounding: at most 5 units of roundoff of the summed magnitudes in
-// the planes (two in the combined coefficients, three in the FMA chain), 4 + 3 in the other's centre
-// and its products, so the margin takes 16 (9.6e-7) of (f + |c|) (|m|_1 + |t|_1), which no sum
-// exceeds. The roundings of the radius itself lie below 1e-6 of it: 1.021 and 4.01 cover them.
+// Everything that reaches_image keeps, and everything that covers a pixel, is a candidate. The
+// pixel column (row) times z differs from the exact one by at most 5 units of roundoff of the summed
+// magnitudes (two in the combined coefficients, three in the FMA chain), from reaches_image's by 4 +
+// 3 more (its centre and products), so the margin takes 16 (9.6e-7) of (f + |c|) (|m|_1 + |t|_1),
+// which no sum exceeds. Likewise the depth: z_hi = z + 4.9e-7 (|m|_1 + |t|_1) bounds it from above,
+// and takes its place where a larger depth keeps more. The roundings of the radius itself lie below
+// 1e-6 of it: 1.021 and 4.01 cover them.
 struct CullView {
   float4 px;   // fx R0 + cx R2 | fx t0 + cx t2: z times the pixel column of the centre
   float4 py;   // likewise for the row
   float4 z;    // R2 | t2
-  float4 lim;  // width - 1, height - 1, 1.021 F, bound of z's error from t2
-  float2 err;  // bound of the planes' rounding per unit of |m|_1, and from t
+  float4 lim;  // width - 1, height - 1, 1.021 F, |t|_1
+  float err;   // bound of the planes' rounding per unit of |m|_1 + |t|_1
 };
 
 __global__ void __launch_bounds__(kPreThreads) cull_kernel(
@@ -378,9 +392,8 @@ __global__ void __launch_bounds__(kPreThreads) cull_kernel(
                           vp.fy * vp.fy * (1.0f + vp.lim_w * vp.lim_w));
     // A negative value tells that there is no guard band.
     cv.lim = make_float4((float)(vp.width - 1), (float)(vp.height - 1),
-                         vp.lim_u > 0.0f ? 1.021f * F : -1.0f, 4.9e-7f * fabsf(ps.t[2]));
-    cv.err.x = 9.6e-7f * fmaxf(vp.fx + fabsf(vp.cx), vp.fy + fabsf(vp.cy));
-    cv.err.y = cv.err.x * (fabsf(ps.t[0]) + fabsf(ps.t[1]) + fabsf(ps.t[2]));
+                         vp.lim_u > 0.0f ? 1.021f * F : -1.0f, norm1(ps.t));
+    cv.err = image_rounding(vp);
     s_view[threadIdx.x] = cv;
   }
   // The block's Gaussians own whole words of each view's row of the visibility bitmask. Tile counts
@@ -420,7 +433,7 @@ __global__ void __launch_bounds__(kPreThreads) cull_kernel(
   // rad z <= F reach + band z + rounding; an overflowing product keeps the entry.
   const float root = sqrtf(fmaxf(kappa, 0.0f));
   const float reach = root * smax, band = fmaf(1.021f * root, sqrtf(c.eps2d), 4.01f);
-  const float m1 = fabsf(m[0]) + fabsf(m[1]) + fabsf(m[2]), z_err = 4.9e-7f * m1;
+  const float m1 = norm1(m);
   uint32_t count = 0;  // candidates of the warp so far
   for (int k = 0; k < v_count; ++k) {
     const float4 zr = s_view[k].z, lim = s_view[k].lim;
@@ -428,18 +441,20 @@ __global__ void __launch_bounds__(kPreThreads) cull_kernel(
     const float4 pr = s_view[k].px, qr = s_view[k].py;
     const float px = fmaf(pr.x, m[0], fmaf(pr.y, m[1], fmaf(pr.z, m[2], pr.w)));
     const float py = fmaf(qr.x, m[0], fmaf(qr.y, m[1], fmaf(qr.z, m[2], qr.w)));
-    const float err = fmaf(s_view[k].err.x, m1, s_view[k].err.y);
-    float margin = fmaf(lim.z, reach, fmaf(band, z, err));
+    const float sum = m1 + lim.w, err = s_view[k].err * sum;
+    const float z_hi = fmaf(4.9e-7f, sum, z);
+    float margin = fmaf(lim.z, reach, fmaf(band, z_hi, err));
     if (lim.z < 0.0f) {  // no guard band (the same for every Gaussian)
       const ViewParams& vp = views.v[v_begin + k];
-      const float u = (fabsf(px - vp.cx * z) + err) / (vp.fx * z),
-                  w = (fabsf(py - vp.cy * z) + err) / (vp.fy * z);
+      const float z_lo = z - (z_hi - z);
+      const float u = (fabsf(px - vp.cx * z) + 2.0f * err) / (vp.fx * z_lo),
+                  w = (fabsf(py - vp.cy * z) + 2.0f * err) / (vp.fy * z_lo);
       const float F = sqrtf(vp.fx * vp.fx * fmaf(u, u, 1.0f) + vp.fy * vp.fy * fmaf(w, w, 1.0f));
-      margin = fmaf(1.03f * F, reach, fmaf(band, z, err));
+      margin = z_lo > 0.0f ? fmaf(1.03f * F, reach, fmaf(band, z_hi, err)) : INFINITY;
     }
-    const bool keep = shown && z + (z_err + lim.w) > c.znear && z > 0.0f &&
+    const bool keep = shown && z_hi > c.znear &&
                       !(px + margin < 0.0f || py + margin < 0.0f ||
-                        px > fmaf(lim.x, z, margin) || py > fmaf(lim.y, z, margin));
+                        px > fmaf(lim.x, z_hi, margin) || py > fmaf(lim.y, z_hi, margin));
     const unsigned ballot = __ballot_sync(0xffffffffu, keep);
     if (keep)
       s_cand[warp][count + __popc(ballot & ((1u << lane) - 1u))] =
