@@ -50,10 +50,10 @@ L2_FLUSH_BYTES = 256 << 20
 # compositing, 15 FP32 operations (plus one exp); the backward's recomputation, transmittance
 # recovery and screen-space gradients, 40 FP32 operations (plus two MUFU operations and the
 # atomics after the warp reduction).
-# Sorts of at least this many pairs take the library's wide radix passes (9-bit digits).
-WIDE_SORT_MIN_PAIRS = 1 << 20
 FWD_FLOP_PER_EVAL = 15
 BWD_FLOP_PER_EVAL = 40
+# Sorts of at least this many keys take the library's wide radix passes (9-bit digits).
+WIDE_SORT_MIN_PAIRS = 1 << 20
 
 # DRAM bytes (read + written) per launch of a dominant kernel come from the ncu captures
 # summarised in this file's table (one row per workload, kernel and tile configuration); a
@@ -497,30 +497,36 @@ def views_tiles(wl, tuned) -> int:
                    for c in wl.cameras))
 
 
-def phase_rooflines(phases, stats, n, V, K, tiles, hbm_peak, fp32_peak):
+def views_cells(wl, tuned) -> int:
+    """Cells of 4 x 4 tiles of the workload's views at the tuned tile shape."""
+    return int(sum(-(-c["width"] // (4 * tuned["tile_w"])) * -(-c["height"] // (4 * tuned["tile_h"]))
+                   for c in wl.cameras))
+
+
+def phase_rooflines(phases, stats, n, V, K, tiles, hbm_peak, fp32_peak, cells=None):
     """Every phase of the step against its roofline: the blends by their FP32 work (15 and 40
     FLOP per visited position), the others by their algorithmic bytes, the minimum each must
     move (inputs read once, outputs written once, sort passes as the radix digits require):
     - preprocess: the cull reads mean, log-scales, quaternion and opacity logit (44 B) per
       Gaussian and clears one visibility bit per (view, Gaussian); the projection reads those and
-      the SH coefficients (12K B) and writes a 48 B record and a 4 B tile count per visible entry;
-    - compact: the visibility bits, and a key, a value and a list entry (12 B) written plus a
-      16 B record read per visible entry;
-    - depth sort: 4 passes of 8-bit digits over the 31-bit depth keys, each reading the key
-      twice and the value once and writing both (20 B per entry);
-    - offsets: a tile count gathered and an offset written per visible entry (8 B);
-    - duplicate: a (tile, entry) pair written (8 B) per pair, order, offset, count and two
-      records read (44 B) per visible entry;
-    - tile sort: ceil(bits / 9) passes of the wide radix sort from 4M pairs on, else ceil(bits /
-      8) passes of the small one, 20 B per pair each;
-    - ranges: every pair's key read, two words written per tile, and the tile order's keys and
-      values sorted (one pass, 24 B per tile);
+      the SH coefficients (12K B) and writes 56 B of the record and a 4 B depth per visible entry;
+    - compact: the visibility bits, and per visible entry a depth read (4 B) and a key, a value and
+      a list entry written (12 B);
+    - depth sort: 4 passes over the 31-bit depth keys, each reading the key twice and the value
+      once and writing both (20 B per entry);
+    - duplicate: per visible entry the order, the counts and the two footprint words of the record
+      read (44 B), per cell entry a key and a value written (8 B);
+    - tile sort: the cell entries by cell, ceil(bits / 9) passes of the wide radix sort from 2^20
+      entries on, else ceil(bits / 8) passes of the small one, 20 B per entry each;
+    - ranges: per cell entry the key read for the cells' ranges, again to count and, with the value,
+      to expand (16 B), per cell a range written and read twice (24 B), per pair its index written
+      (4 B), per tile a count written and read twice, a range written and read and a place in the
+      launch order written (32 B);
     - preprocess backward: a 64 B record read and written per visible entry, the parameters read
       and their gradients written once per Gaussian (11 + 3K floats each).
-    Offsets, duplicate, tile sort and ranges are counted as a sort of every (tile, entry) pair
-    would move them. The library builds its lists in two levels (one entry per cell of 4x4 tiles is
-    sorted and then expanded) and moves fewer bytes, so their fractions compare with that sort and
-    can exceed 1."""
+    `cells`: (cell entries, cells) of the step. The phase "offsets" does nothing and has no entry.
+    Without `cells` the lists are modelled as a sort of every (tile, entry) pair, with a 52 B record
+    and a 16 B read to compact it: what a library without cells moves."""
     nv, pairs, n_eval = stats["n_visible"], stats["n_pairs"], stats["n_eval"]
     tile_bits = max(1, int(np.ceil(np.log2(tiles + 2))))
     bytes_model = {
@@ -534,6 +540,18 @@ def phase_rooflines(phases, stats, n, V, K, tiles, hbm_peak, fp32_peak):
         "ranges": 4 * pairs + 8 * tiles + 24 * tiles,
         "preprocess_backward": 2 * 64 * nv + 2 * 4 * (11 + 3 * K) * n,
     }
+    if cells is not None:
+        entries, total_cells = cells
+        cell_bits = max(1, int(total_cells).bit_length())  # ids 0 .. total_cells
+        passes = int(np.ceil(cell_bits / (9 if entries >= WIDE_SORT_MIN_PAIRS else 8)))
+        del bytes_model["offsets"]
+        bytes_model.update({
+            "preprocess": 44 * n + n * V / 8 + nv * (44 + 12 * K + 60),
+            "compact": n * V / 8 + 16 * nv,
+            "duplicate": 44 * nv + 8 * entries,
+            "tile_sort": passes * 20 * entries,
+            "ranges": 16 * entries + 24 * total_cells + 4 * pairs + 32 * tiles,
+        })
     flop_model = {"blend_forward": FWD_FLOP_PER_EVAL * n_eval,
                   "blend_backward": BWD_FLOP_PER_EVAL * n_eval}
     out = {}
@@ -750,6 +768,7 @@ def run_ours(args, world, rank, local):
     ms_per_step = total_ms / args.steps
     value = throughput(world, pixels, args.steps, total_ms)
     stats = r.stats(state)
+    cell_entries = r.ctx.cell_entries(state, r.stream_handle())
     # Spread of the per-tile work: the run length of each non-empty tile (its Gaussians), the
     # quantity a blend CTA's time follows.
     runs = np.diff(r.ctx.tile_ranges(state, int(sum(
@@ -964,11 +983,11 @@ def run_ours(args, world, rank, local):
         # Byte models of the other phases (algorithmic bytes per step): the backward preprocess
         # reads and writes a 64-byte record per visible entry and reads the parameters and
         # writes their gradients once per Gaussian (11 + 3K floats each way); the forward
-        # preprocess reads the parameters once and writes 52 bytes per candidate entry.
+        # preprocess reads the parameters once and writes 60 bytes per visible entry.
         param_bytes = 4 * (11 + 3 * K)
         bytes_model = {
             "preprocess_backward": 64 * stats["n_visible"] + 2 * param_bytes * n,
-            "preprocess": param_bytes * n + 4 * V * n + 52 * stats["n_visible"],
+            "preprocess": param_bytes * n + V * n / 8 + 60 * stats["n_visible"],
         }
         hbm = float(peaks.get("hbm_gbs", 6800.0))
         achieved = (bytes_model[dominant] / (phases[dominant] / 1e3) / 1e9
@@ -978,7 +997,8 @@ def run_ours(args, world, rank, local):
                     "traffic": None}
 
     phase_roofline = phase_rooflines(phases, stats, n, V, K, views_tiles(wl, tuned),
-                                     float(peaks.get("hbm_gbs", 6800.0)), fp32_peak)
+                                     float(peaks.get("hbm_gbs", 6800.0)), fp32_peak,
+                                     (cell_entries, views_cells(wl, tuned)))
 
     line = {
         "metric": METRIC, "value": value, "unit": "Mpix/s", "n_gpus": world,
@@ -1009,6 +1029,7 @@ def run_ours(args, world, rank, local):
                                 "speedup": loop_ms_per_step / ms_per_step},
         "phases_ms": phases,
         "counts": {"visible": stats["n_visible"], "pairs": stats["n_pairs"],
+                   "cell_entries": cell_entries,
                    "evaluated": n_eval},
     }
     line["tracking"] = measure_tracking(r, params, wl.cameras, images,

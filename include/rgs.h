@@ -352,6 +352,8 @@ rgs_status rgs_set_phase_timing(rgs_ctx* ctx, int32_t enable);
 rgs_status rgs_phase_times(rgs_ctx* ctx, uint64_t state, float* ms, int32_t n, void* stream);
 
 /* ---- Diagnostics: copies of a state's binning results (synchronise `stream`). ----
+ * rgs_cell_entries: the number of (cell of 4 x 4 tiles, entry) list entries of the last forward,
+ * what its emission writes and its cell sort moves, into *n_entries.
  * rgs_copy_tile_lists: the sorted pair list (the (view, Gaussian) index vi = view * n + i of each
  * pair, tile runs in near-to-far order) into host_vals (capacity vals_cap entries; the number of
  * pairs is written to *n_pairs even when it exceeds vals_cap, in which case nothing is copied),
@@ -362,6 +364,7 @@ rgs_status rgs_phase_times(rgs_ctx* ctx, uint64_t state, float* ms, int32_t n, v
  * triangular with L L^T = (log2 e / 2) (Sigma^I)^-1, and log2 o; r, g, b and camera-space depth),
  * and the touched-tile counts into host_ntiles (may be NULL).
  * A record is meaningful only where its tile count is non-zero. */
+rgs_status rgs_cell_entries(rgs_ctx* ctx, uint64_t state, int64_t* n_entries, void* stream);
 rgs_status rgs_copy_tile_lists(rgs_ctx* ctx, uint64_t state, uint32_t* host_vals, int64_t vals_cap,
                                uint32_t* host_ranges, int64_t* n_pairs, void* stream);
 rgs_status rgs_copy_records(rgs_ctx* ctx, uint64_t state, float* host_rec, uint32_t* host_ntiles,

@@ -26,7 +26,7 @@ EXPORTED = ("rgs_create", "rgs_destroy", "rgs_config_default", "rgs_last_error",
             "rgs_render_forward", "rgs_render_backward", "rgs_release_state", "rgs_trim", "rgs_reserve",
             "rgs_query_stats", "rgs_set_phase_timing", "rgs_phase_times", "rgs_radix_sort_u32",
             "rgs_exclusive_scan_u32", "rgs_exclusive_scan_u32_static", "rgs_copy_tile_lists",
-            "rgs_copy_records", "rgs_autotune", "rgs_render_forward_posed",
+            "rgs_copy_records", "rgs_cell_entries", "rgs_autotune", "rgs_render_forward_posed",
             "rgs_track_config_default", "rgs_adam_config_default", "rgs_track_grad_weight",
             "rgs_track_loss", "rgs_pose_adam_step", "rgs_seed_config_default", "rgs_triangulate",
             "rgs_init_seeds", "rgs_covisibility", "rgs_render_backward_mapping", "rgs_map_ema",
@@ -138,6 +138,7 @@ def load(build_if_needed: bool = True):
                                         P]),
             "rgs_release_state": (S, [P, U64]),
             "rgs_trim": (S, [P]),
+            "rgs_cell_entries": (S, [P, U64, ctypes.POINTER(I64), P]),
             "rgs_reserve": (S, [P, ctypes.POINTER(U64), I64, P]),
             "rgs_query_stats": (S, [P, U64, ctypes.POINTER(Stats), P]),
             "rgs_set_phase_timing": (S, [P, I32]),
@@ -417,6 +418,13 @@ class Context:
         self._check(self.lib.rgs_phase_times(self.handle, ctypes.c_uint64(state), ms, len(PHASES),
                                              ctypes.c_void_p(stream)))
         return dict(zip(PHASES, [float(x) for x in ms]))
+
+    def cell_entries(self, state: int, stream: int = 0) -> int:
+        """Number of (cell, entry) list entries of a state's last forward."""
+        n = ctypes.c_int64()
+        self._check(self.lib.rgs_cell_entries(self.handle, ctypes.c_uint64(state),
+                                              ctypes.byref(n), ctypes.c_void_p(stream)))
+        return n.value
 
     def tile_lists(self, state: int, total_tiles: int, stream: int = 0):
         """(pair values [P] u32, ranges [total_tiles, 2] u32) of a state's sorted pair list."""

@@ -1251,6 +1251,20 @@ rgs_status rgs_query_stats(rgs_ctx* ctx, uint64_t handle, rgs_stats* out, void* 
   return RGS_OK;
 }
 
+rgs_status rgs_cell_entries(rgs_ctx* ctx, uint64_t handle, int64_t* n_entries, void* stream_ptr) {
+  if (!ctx || !n_entries) return RGS_ERR_INVALID_ARG;
+  State* s = find_state(ctx, handle);
+  if (!s || !s->has_forward) return fail(ctx, RGS_ERR_STATE, "state holds no completed forward");
+  cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);
+  cudaSetDevice(ctx->device);
+  RGS_CUDA(cudaMemcpyAsync(ctx->host_counters, s->counters, sizeof(Counters),
+                           cudaMemcpyDeviceToHost, stream),
+           "read counters");
+  RGS_CUDA(cudaStreamSynchronize(stream), "sync");
+  *n_entries = ctx->host_counters->n_cells_stored;
+  return RGS_OK;
+}
+
 rgs_status rgs_copy_tile_lists(rgs_ctx* ctx, uint64_t handle, uint32_t* host_vals,
                                int64_t vals_cap, uint32_t* host_ranges, int64_t* n_pairs,
                                void* stream_ptr) {
