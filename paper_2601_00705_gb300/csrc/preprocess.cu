@@ -870,8 +870,8 @@ __global__ void __launch_bounds__(kPreThreads) backward_view_kernel(
 // ------------------------------------------------------------------------------------------
 template <int DEG, bool kReg>
 // At most 80 registers (6 blocks of 128 threads per SM): the kernel waits on its gathers, and
-// 24 resident warps per SM instead of 16 halve its time despite a few spilled registers (0.98
-// -> 0.50 ms over 3M Gaussians; with 64 registers the spills cost more than the warps gain).
+// 24 resident warps per SM instead of 16 halved its time (0.98 -> 0.50 ms over 3M Gaussians, when
+// each thread stored its own gradients; with 64 registers the spills cost more than the warps gain).
 __global__ void __launch_bounds__(kPreThreads, 6) backward_gaussian_kernel(
     const __grid_constant__ Views views, int n, const float* __restrict__ means,
     const float* __restrict__ log_scales, const float* __restrict__ quats,

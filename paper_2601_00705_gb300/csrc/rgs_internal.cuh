@@ -367,11 +367,11 @@ __device__ __forceinline__ float sqrt_fixed(float x) {
 
 // Every operation below is a single instruction with no contraction (explicitly rounded
 // arithmetic, hardware approximations of reciprocals and square roots), so the counting pass in
-// the projection and the emitting pass of the duplication visit exactly the same tiles. The
-// approximations err by a few ulp, far inside the 1-pixel padding.
+// the projection and the emission of the cell entries visit exactly the same tiles. The
+// approximations err by a few ulp, far inside the padding of 1/16 px.
 //
 // TileCover holds the per-footprint constants; span(ty) gives the column span of one tile row,
-// so that rows can be walked in sequence (for_each_tile_row) or in parallel, one per lane.
+// which cell_row collects for the rows of a cell.
 struct TileCover {
   int ty0, ty1, bx0, bx1;
   bool box_only;  // a single row or column of tiles: every row spans the padded box
@@ -577,7 +577,7 @@ inline int64_t vis_bit_words_cap(int64_t vn_cap) { return (vn_cap + 31) / 32 + k
 
 // Tile states of one Lookback area serving up to n_cap elements: a scan of n_cap elements
 // takes scan_blocks(n_cap) tiles; the bitmask compaction of n_views x n <= n_cap entries
-// (tiles of 256 words, n_views <= RGS_MAX_VIEWS <= 256) takes at most n_cap / 8192 + 2.
+// (tiles of 512 words, n_views <= RGS_MAX_VIEWS <= 256) takes at most n_cap / 16384 + 2.
 static_assert(RGS_MAX_VIEWS <= 256, "bound of the bitmask compaction's tiles");
 inline int64_t lookback_tiles(int64_t n_cap) { return scan_blocks(n_cap) + 2; }
 // Bytes of one Lookback area (a 16-byte header, then the tile states).

@@ -10,7 +10,7 @@
 //   * co-visibility of frame pairs for the keyframe test (Eq. iou): intersection and union of
 //     the pixels whose accumulated opacity exceeds a threshold.
 // All passes are elementwise or reductions over the images (HBM-bound) except the pose update
-// (one thread per view).
+// (six lanes per view).
 #include <math.h>
 
 #include <algorithm>
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kLossThreads) track_loss_kernel(
 // Six lanes per view (five views per warp), lane j with component j: a double-precision
 // instruction costs a warp 64 cycles whatever its lanes do, so the views' components go through
 // each one together and what a view shares is computed by its six lanes alike (27 us with a thread
-// per view and the pow, sin and cos of the general case, 6 us).
+// per view and the pow, sin and cos of the general case, now 10).
 constexpr int kAdamViews = 5;  // views per warp
 
 // x^n by squaring. n follows from the caller's step counter in device memory, so it may be anything:
