@@ -114,7 +114,8 @@ struct State {
   uint32_t* tile_order = nullptr;  // launch order of the blends' tiles (longest run first)
   uint32_t *cell_keys[2] = {nullptr, nullptr}, *cell_vals[2] = {nullptr, nullptr};
   // The pair list of the last forward: in r_pair, or, where the cell list's buffers are at least as
-  // long, in the one that the cell sort leaves free.
+  // long, in cell_keys[1]. The cell sort starts in whichever buffers make it end in cell_keys[0], so
+  // eager and captured forwards (whose sorts differ in length, and so in passes) agree on the place.
   uint32_t* pairs = nullptr;
   // Scratch.
   uint32_t* hist = nullptr;
@@ -1047,26 +1048,29 @@ rgs_status forward_on_state(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_came
   s->order = s->vis_vals[alt ? 1 : 0];
   RGS_CUDA(mark(ctx, *s, 3, stream, capturing), "event");
   RGS_CUDA(mark(ctx, *s, 4, stream, capturing), "event");
+  // The cell ids are [0, total_cells]; total_cells itself marks an unused slot.
+  const int cell_bits = bits_for((uint32_t)views.total_cells + 1u);
+  const int key_shift = cells_masked(views.total_cells) ? 16 : 0;
+  const int cell_items = n_cells <= kSmallBlockSort ? kSortItemsSmall : kSortItems;
+  const int from = radix_sort_in_alt(n_cells, key_shift, key_shift + cell_bits, cell_items) ? 1 : 0;
   // 4. Cell entries in depth order.
   RGS_CUDA(launch_emit_cells(views, g->n, s->order, s->rec,
                              consts.log2_alpha_min, vis_cap, (uint32_t)s->cell_cap,
-                             s->cell_keys[0], s->cell_vals[0],
+                             s->cell_keys[from], s->cell_vals[from],
                              lookback_at(lb_emit, &cnt->status, emit_items), cnt, stream),
            "emit cells");
   RGS_CUDA(mark(ctx, *s, 5, stream, capturing), "event");
-  // 5. Stable sort by cell. The ids are [0, total_cells]; total_cells itself marks an unused slot.
+  // 5. Stable sort by cell, into buffers 0.
   alt = false;
-  const int cell_bits = bits_for((uint32_t)views.total_cells + 1u);
-  const int key_shift = cells_masked(views.total_cells) ? 16 : 0;
-  RGS_CUDA(launch_radix_sort(s->cell_keys[0], s->cell_vals[0], s->cell_keys[1], s->cell_vals[1],
-                             n_cells, &cnt->n_cells_stored, key_shift, key_shift + cell_bits,
-                             s->hist, s->block_sums, &alt, stream,
-                             n_cells <= kSmallBlockSort ? kSortItemsSmall : kSortItems),
+  RGS_CUDA(launch_radix_sort(s->cell_keys[from], s->cell_vals[from], s->cell_keys[1 - from],
+                             s->cell_vals[1 - from], n_cells, &cnt->n_cells_stored, key_shift,
+                             key_shift + cell_bits, s->hist, s->block_sums, &alt, stream,
+                             cell_items),
            "cell sort");
-  const uint32_t* keys = s->cell_keys[alt ? 1 : 0];
-  const uint32_t* vals = s->cell_vals[alt ? 1 : 0];
-  s->pairs = s->pair_cap >= s->cell_cap ? static_cast<uint32_t*>(s->r_pair.base)
-                                        : s->cell_keys[alt ? 0 : 1];
+  if (alt != (from == 1)) return fail(ctx, RGS_ERR_CUDA, "cell sort ended in the wrong buffers");
+  const uint32_t* keys = s->cell_keys[0];
+  const uint32_t* vals = s->cell_vals[0];
+  s->pairs = s->pair_cap >= s->cell_cap ? static_cast<uint32_t*>(s->r_pair.base) : s->cell_keys[1];
   const uint32_t pair_cap = (uint32_t)s->pair_capacity();
   RGS_CUDA(mark(ctx, *s, 6, stream, capturing), "event");
   // 6. The tiles' lists, their ranges and launch order.

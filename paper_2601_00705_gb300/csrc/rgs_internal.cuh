@@ -718,5 +718,7 @@ cudaError_t launch_radix_sort(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt
                               int begin_bit, int end_bit, uint32_t* hist, uint32_t* block_sums,
                               bool* result_in_alt, cudaStream_t stream,
                               int items = kSortItems);
+// What such a call will return in *result_in_alt (buffers aligned to 16 bytes).
+bool radix_sort_in_alt(int64_t n_cap, int begin_bit, int end_bit, int items);
 
 }  // namespace rgs

@@ -1111,38 +1111,52 @@ int64_t cluster_sort_capacity(int device) {
   return std::min<int64_t>((int64_t)cluster_sort_blocks(device) * kCsSlice, kCsMaxN);
 }
 
+namespace {
+bool one_cluster(int64_t n_cap, int begin_bit, int end_bit, int* blocks) {
+  int device = 0;
+  if (n_cap <= 0 || end_bit <= begin_bit || cudaGetDevice(&device) != cudaSuccess) return false;
+  *blocks = cluster_sort_blocks(device);
+  return *blocks > 0 && n_cap <= std::min<int64_t>((int64_t)*blocks * kCsSlice, kCsMaxN);
+}
+}  // namespace
+
+bool radix_sort_in_alt(int64_t n_cap, int begin_bit, int end_bit, int items) {
+  int blocks = 0;
+  if (n_cap <= 0 || end_bit <= begin_bit) return false;
+  if (one_cluster(n_cap, begin_bit, end_bit, &blocks)) return true;
+  const int digit = n_cap >= kWideMinN && items == kSortItems ? kWideBits : 8;
+  return (end_bit - begin_bit + digit - 1) / digit % 2 != 0;
+}
+
 cudaError_t launch_radix_sort(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
                               uint32_t* vals_alt, int64_t n_cap, const uint32_t* n_dev,
                               int begin_bit, int end_bit, uint32_t* hist, uint32_t* block_sums,
                               bool* result_in_alt, cudaStream_t stream, int items) {
   (void)block_sums;
-  int device = 0;
-  if (n_cap > 0 && end_bit > begin_bit && cudaGetDevice(&device) == cudaSuccess) {
-    const int blocks = cluster_sort_blocks(device);
-    if (blocks > 0 && n_cap <= std::min<int64_t>((int64_t)blocks * kCsSlice, kCsMaxN)) {
-      // One launch: (keys, vals) -> (keys_alt, vals_alt).
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(blocks);
-      cfg.blockDim = dim3(kCsThreads);
-      cfg.dynamicSmemBytes = kCsSmemBytes;
-      cfg.stream = stream;
-      cudaLaunchAttribute attr[2];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = blocks;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[1].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 2;
-      const cudaError_t e = cudaLaunchKernelEx(&cfg, cluster_sort_kernel, (const uint32_t*)keys,
-                                               (const uint32_t*)vals, keys_alt,
-                                               vals ? vals_alt : nullptr, n_cap, n_dev,
-                                               begin_bit, end_bit);
-      RGS_LAUNCHED();
-      *result_in_alt = true;
-      return e;
-    }
+  int blocks = 0;
+  if (one_cluster(n_cap, begin_bit, end_bit, &blocks)) {
+    // One launch: (keys, vals) -> (keys_alt, vals_alt).
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kCsThreads);
+    cfg.dynamicSmemBytes = kCsSmemBytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = blocks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, cluster_sort_kernel, (const uint32_t*)keys,
+                                             (const uint32_t*)vals, keys_alt,
+                                             vals ? vals_alt : nullptr, n_cap, n_dev,
+                                             begin_bit, end_bit);
+    RGS_LAUNCHED();
+    *result_in_alt = true;
+    return e;
   }
   // The wide upsweep reads keys with 16-byte loads: both key buffers must be 16-byte aligned.
   const bool aligned16 = reinterpret_cast<uintptr_t>(keys) % 16 == 0 &&

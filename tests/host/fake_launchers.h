@@ -49,9 +49,10 @@ cudaError_t launch_radix_sort(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt
     if (p) check(p, 4 * (size_t)n, "sort buffer");
   check(hist, 4 * (size_t)sort_hist_entries(n, items), "sort counts");
   check(sums, 4 * (size_t)(scan_blocks(sort_hist_entries(n, items)) + 1), "sort sums");
-  *alt = true;
+  *alt = n % 2 == 0;
   return cudaSuccess;
 }
+bool radix_sort_in_alt(int64_t n, int, int, int) { return n % 2 == 0; }
 cudaError_t launch_emit_cells(const Views&, int, const uint32_t*, const Record*, float, int64_t,
                               uint32_t capacity, uint32_t* keys, uint32_t* vals, Lookback,
                               Counters*, cudaStream_t) {
@@ -72,6 +73,9 @@ cudaError_t launch_tile_lists(const Views& views, const uint2*, const uint32_t* 
   check(ranges, 8 * (size_t)views.total_tiles, "tile ranges");
   check(tile_order, 4 * (size_t)views.total_tiles, "tile order");
   if (capacity) check(pairs, 4 * (size_t)capacity, "pairs");
+  if (fake::one_place && fake::wrote_pairs && pairs != fake::wrote_pairs)
+    check(nullptr, 0, "pairs written to another place than before");
+  if (fake::one_place) fake::wrote_pairs = pairs;
   const char *a = reinterpret_cast<const char*>(pairs), *b = a + 4 * (size_t)capacity;
   for (const uint32_t* in : {keys, vals}) {  // the lists are read while the pairs are written
     const char* c = reinterpret_cast<const char*>(in);
@@ -80,11 +84,14 @@ cudaError_t launch_tile_lists(const Views& views, const uint2*, const uint32_t* 
   return cudaSuccess;
 }
 cudaError_t launch_blend(bool forward, const Views& views, const Consts&, const uint2* ranges,
-                         const uint32_t*, const Record* rec, float*, float*, float*,
+                         const uint32_t* pairs, const Record* rec, float*, float*, float*,
                          float* t_final, int32_t* last, const float*, const float*, const float*,
                          float* g2d, const uint32_t*, Counters*, cudaStream_t) {
   check(ranges, 8 * (size_t)views.total_tiles, "blend's ranges");
   check(rec, sizeof(Record), "blend's records");
+  check(pairs, 4 * (size_t)fake::pairs, "blend's pairs");
+  if (fake::wrote_pairs && pairs != fake::wrote_pairs)
+    check(nullptr, 0, "blend's pairs are not where a forward on this state wrote them");
   check(t_final, 4 * (size_t)views.total_pixels, "transmittances");
   check(last, 4 * (size_t)views.total_pixels, "last indices");
   if (!forward) check(g2d, 64, "gradient records");

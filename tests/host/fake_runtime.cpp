@@ -15,7 +15,8 @@ static std::map<char*, size_t>& blocks() {
   return m;
 }
 size_t live = 0, limit = SIZE_MAX, total = 288ull << 30;
-bool capturing = false;
+bool capturing = false, one_place = false;
+const void* wrote_pairs = nullptr;
 int stale = 0, unsafe = 0;
 unsigned long long visible = 0, cells = 0, pairs = 0, pairs_per_cell = 1;
 

@@ -225,6 +225,17 @@ void reserved_pairs() {
     EXPECT(backward(ctx, s) == RGS_OK);
     EXPECT(fake::live - before == grown);
   }
+  // Eager and captured forwards write to one place: a backward after a replay reads what it wrote.
+  fake::one_place = true;
+  for (unsigned long long count : {50ull, 51ull, 999999ull}) {
+    EXPECT(forward(ctx, 1000, 64, count, &s) == RGS_OK);
+    fake::capturing = true;
+    EXPECT(forward(ctx, 1000, 64, count, &s) == RGS_OK);
+    fake::capturing = false;
+    EXPECT(backward(ctx, s) == RGS_OK);
+  }
+  fake::one_place = false;
+  fake::wrote_pairs = nullptr;
   fake::pairs_per_cell = 8;
   EXPECT(forward(ctx, 1000, 64, asked, &s) == RGS_OK);
   EXPECT(rgs_query_stats(ctx, s, &stats, nullptr) == RGS_OK);
