@@ -394,6 +394,19 @@ rgs_status ensure_cells(rgs_ctx* ctx, State& s, int64_t cells) {
   return RGS_OK;
 }
 
+// Before the cell list grows to `cells` outside a forward: the last forward's pairs move out of it,
+// so that its backward still finds them.
+rgs_status keep_pairs(rgs_ctx* ctx, State& s, int64_t cells) {
+  if (cells <= s.cell_cap || !s.has_forward || s.pairs != s.cell_keys[1]) return RGS_OK;
+  RGS_CUDA(cudaDeviceSynchronize(), "sync before growth");
+  const size_t bytes = sizeof(uint32_t) * s.cell_cap;
+  RGS_CUDA(alloc_region(ctx, s.r_pair, align_up(bytes), {&s.pair_cap}), "allocate pair list");
+  RGS_CUDA(cudaMemcpy(s.r_pair.base, s.pairs, bytes, cudaMemcpyDeviceToDevice), "move pair list");
+  s.pairs = static_cast<uint32_t*>(s.r_pair.base);
+  s.pair_cap = s.cell_cap;
+  return RGS_OK;
+}
+
 State* find_state(rgs_ctx* ctx, uint64_t id) {
   auto it = ctx->states.find(id);
   return it == ctx->states.end() ? nullptr : it->second;
@@ -472,6 +485,16 @@ void drop_spares(rgs_ctx* ctx) {
   cudaDeviceSynchronize();  // queued work may still use their buffers
   for (State* s : ctx->spare) destroy_state(s);
   ctx->spare.clear();
+}
+
+// Ends the state that a call created and then failed on: its caller has none. (Under stream capture
+// such a state holds no memory, and nothing here may disturb the capture.)
+void end_state(rgs_ctx* ctx, uint64_t* handle) {
+  State* s = find_state(ctx, *handle);
+  ctx->states.erase(*handle);
+  *handle = 0;
+  if (s->bytes() > 0) cudaDeviceSynchronize();  // queued work may still use its buffers
+  destroy_state(s);
 }
 
 // Brackets the work that a forward or backward queues on a state.
@@ -848,6 +871,7 @@ rgs_status rgs_reserve(rgs_ctx* ctx, uint64_t* handle, int64_t pair_capacity, vo
   if (!ctx) return RGS_ERR_INVALID_ARG;
   if (pair_capacity > kMaxListed)
     return fail(ctx, RGS_ERR_INVALID_ARG, "pair list exceeds 2^31 - 1");
+  const bool creates = handle && *handle == 0;
   State* s = nullptr;
   rgs_status st = get_or_create_state(ctx, handle, &s);
   if (st != RGS_OK) return st;
@@ -856,12 +880,13 @@ rgs_status rgs_reserve(rgs_ctx* ctx, uint64_t* handle, int64_t pair_capacity, vo
     // As many cell entries, whose buffers hold the pair list too. No footprint has more cell
     // entries than pairs, unless it skips whole cells between two pixel rows: only a needle of an
     // opacity below 1.4 alpha_min can (the dilation makes every other one too thick).
-    st = ensure_cells(ctx, *s, pair_capacity);
-    if (st != RGS_OK) return st;
-    st = ensure_scratch(ctx, *s, std::max<int64_t>(s->cell_cap, s->vn_cap), false);
-    if (st != RGS_OK) return st;
+    st = keep_pairs(ctx, *s, pair_capacity);
+    if (st == RGS_OK) st = ensure_cells(ctx, *s, pair_capacity);
+    if (st == RGS_OK)
+      st = ensure_scratch(ctx, *s, std::max<int64_t>(s->cell_cap, s->vn_cap), false);
   }
-  return RGS_OK;
+  if (st != RGS_OK && creates) end_state(ctx, handle);
+  return st;
 }
 
 namespace {
@@ -899,15 +924,7 @@ rgs_status render_forward(rgs_ctx* ctx, const rgs_gaussians* g, const rgs_camera
   const bool creates = handle && *handle == 0;
   const rgs_status st = forward_on_state(ctx, g, cams, n_views, world_to_cam, cfg_in, out, handle,
                                          stream_ptr);
-  if (st != RGS_OK && creates && *handle != 0) {
-    // The caller has no state from a call that failed: what it created ends here. (Under stream
-    // capture the state holds no memory, and nothing here may disturb the capture.)
-    State* s = find_state(ctx, *handle);
-    ctx->states.erase(*handle);
-    *handle = 0;
-    if (s->bytes() > 0) cudaDeviceSynchronize();  // queued work may still use its buffers
-    destroy_state(s);
-  }
+  if (st != RGS_OK && creates && *handle != 0) end_state(ctx, handle);
   return st;
 }
 

@@ -246,6 +246,37 @@ void reserved_pairs() {
   rgs_destroy(ctx);
 }
 
+// A reserve between a forward and its backward leaves the forward's pairs readable, wherever they
+// lie, also when it fails; one that fails on a state it created leaves none.
+void reserve_after_forward() {
+  for (unsigned long long per_cell : {1ull, 8ull}) {
+    for (size_t room = 0;; room += 1 << 16) {
+      fake::pairs_per_cell = per_cell;
+      rgs_ctx* ctx = make_context();
+      uint64_t s = 0;
+      EXPECT(forward(ctx, 1000, 64, 20000, &s) == RGS_OK);
+      fake::limit = fake::live + room;
+      const rgs_status st = rgs_reserve(ctx, &s, 1000000, nullptr);
+      fake::limit = SIZE_MAX;
+      EXPECT(st == RGS_OK || st == RGS_ERR_NOMEM);
+      EXPECT(backward(ctx, s) == RGS_OK);
+      EXPECT(forward(ctx, 1000, 64, 20000, &s) == RGS_OK);
+      EXPECT(backward(ctx, s) == RGS_OK);
+      rgs_destroy(ctx);
+      EXPECT(fake::live == 0);
+      if (st == RGS_OK) break;
+    }
+  }
+  fake::pairs_per_cell = 1;
+  rgs_ctx* ctx = make_context();
+  const size_t bare = fake::live;
+  uint64_t s = 0;
+  fake::limit = bare + 1000;
+  EXPECT(rgs_reserve(ctx, &s, 1000000, nullptr) == RGS_ERR_NOMEM && s == 0 && fake::live == bare);
+  fake::limit = SIZE_MAX;
+  rgs_destroy(ctx);
+}
+
 // What is kept after a release is bounded, is not kept while memory is scarce, and is given back.
 void kept_memory() {
   for (size_t room : {(size_t)0, fake::total / 8 - (1u << 20), fake::total / 8 + (1u << 20)}) {
@@ -287,6 +318,7 @@ int main(int argc, char** argv) {
   else if (which == "list_limits") list_limits();
   else if (which == "reserved_pairs") reserved_pairs();
   else if (which == "kept_memory") kept_memory();
+  else if (which == "reserve_after_forward") reserve_after_forward();
   else return 2;
   EXPECT(fake::stale == 0);
   return failures ? 1 : 0;

@@ -53,3 +53,31 @@ def test_reserved_states_give_the_same_results(n, width, height, tile_w, tile_h,
             assert rel_l2(g.cpu().numpy(), ref_grads[k].cpu().numpy()) <= GRAD_REL_L2, k
     r.release(state)
     r.release(plain)
+
+
+def test_a_backward_after_a_replay_reads_the_replayed_lists():
+    # The eager cell sort is short (one cluster), the captured one as long as the reserve.
+    n, wl = 3000, synthetic.tiny(seed=9, n=3000, width=320, height=240)
+    p = [to_dev(wl.gaussians.as_dict()[k]) for k in KEYS]
+    up = torch.randn((wl.n_pixels, 3), generator=torch.Generator("cuda").manual_seed(1),
+                     device="cuda") / wl.n_pixels
+    for reserve in (60_000, 300_000, 600_000, 2_000_000):
+        r = Renderer(0)
+        state = r.ctx.reserve(0, reserve, r.stream_handle())
+        *out, state = r.forward_raw(*p, wl.cameras, state=state)
+        ref = r.backward_raw(state, n, 1, 1, up)
+        graph, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(s), torch.cuda.graph(graph, stream=s):
+            r.forward_raw(*p, wl.cameras, state=state, out=tuple(out))
+        torch.cuda.current_stream().wait_stream(s)
+        r.forward_raw(*p, wl.cameras, state=state, out=tuple(out))
+        graph.replay()
+        torch.cuda.synchronize()
+        vals, _ = r.ctx.tile_lists(state, 20 * 15)
+        assert r.stats(state)["status"] == 0 and vals.size and vals.max() < n
+        grads = r.backward_raw(state, n, 1, 1, up)
+        torch.cuda.synchronize()
+        for k, g in grads.items():
+            assert rel_l2(g.cpu().numpy(), ref[k].cpu().numpy()) <= GRAD_REL_L2, (reserve, k)
+        r.release(state)

@@ -52,3 +52,7 @@ def test_reserved_pairs_take_their_documented_memory_and_serve_captures(program)
 
 def test_kept_memory_is_bounded_and_given_back(program):
     _run(program, "kept_memory")
+
+
+def test_a_reserve_between_a_forward_and_its_backward_keeps_the_pairs(program):
+    _run(program, "reserve_after_forward")
