@@ -243,7 +243,8 @@ rgs_status rgs_trim(rgs_ctx* ctx);
 /* Grows a state's pair-list capacity to at least `pair_capacity` entries (0 = leave) and the list of
  * touched cells behind it (at most one entry per pair) to as many, so that a later forward under
  * stream capture does not overflow. Takes 20 bytes per entry asked for (16, and a quarter more). Creates the state if *state is 0. At most
- * 2^31 - 1 (RGS_ERR_INVALID_ARG beyond). */
+ * 2^31 - 1 (RGS_ERR_INVALID_ARG beyond). The state's last forward keeps its data. When the call
+ * fails, *state stays 0 if it was. */
 rgs_status rgs_reserve(rgs_ctx* ctx, uint64_t* state, int64_t pair_capacity, void* stream);
 
 /* Reads the counters of the last forward on `state` (synchronises `stream`). */

@@ -182,12 +182,13 @@ struct rgs_ctx {
   std::map<uint64_t, State*> states;
   uint64_t next_id = 1;
   // Released states kept for the next one (oldest first): at most kSpareStates of them, together
-  // at most 1/kSpareShare of the device (spare_limit). A forward that creates its state (every `render` call does) then
-  // takes buffers that are already there: allocating and freeing them with a device
-  // synchronisation cost 0.55 ms of a 0.82 ms 1200x680 frame and 1.0 ms of a 1.7 ms ten-view
-  // training step. Freed by rgs_trim, with the context, and whenever one of its allocations fails.
-  // Other allocators of the process cannot ask for them, so a state of kSmallSpare and more is kept
-  // only while 1/kSpareFree of the device is free: a program near the limit finds nothing withheld.
+  // at most 1/kSpareShare of the device (spare_limit). A forward that creates its state (every
+  // `render` call does) then takes buffers that are already there: allocating and freeing them with
+  // a device synchronisation cost 0.55 ms of a 0.82 ms 1200x680 frame and 1.0 ms of a 1.7 ms
+  // ten-view training step. Freed by rgs_trim, with the context, and whenever one of its allocations
+  // fails. Other allocators of the process cannot ask for them, so a state of kSmallSpare and more
+  // is kept only while 1/kSpareFree of the device is free: a program near the limit finds nothing
+  // withheld.
   std::vector<State*> spare;
   size_t spare_limit = 0;
   Counters* host_counters = nullptr;  // pinned
